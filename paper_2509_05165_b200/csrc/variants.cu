@@ -5,27 +5,39 @@
 namespace kvc {
 namespace {
 
-// One warp per value row: lanes take 16-byte pieces, squares are added in fp32, then over the warp.
-template <typename T>
+// ||v|| of every value row.  Bound by HBM: V is read once.  A row is kLpr = row bytes / 16 lanes wide (16 for the
+// 256-byte rows of a bf16 head of 128), so a warp carries 32 / kLpr rows at a time and every lane loads; each lane has
+// kNormRows such rows in flight (one 16-byte load each) before it adds anything, and a warp's rows are consecutive, so
+// that its norms leave in one store.  A warp per row with half of its lanes idle and one load in flight took 807 us for
+// 1.07 GB (1.3 TB/s); this form takes 194 us (5.5 TB/s).  The squares are added in the order they always were:
+// a lane's elements in ascending order, then the lanes by halving distances.
+constexpr int kNormRows = 8;
+
+template <typename T, int kLpr>
 __global__ void __launch_bounds__(256)
-value_norm_kernel(LayerPtrs vp, float* __restrict__ vnorm, int L, int Bt, int Hkv, int d, long long N,
-                  long long vs0, long long vs1, long long vs2) {
+value_norm_kernel(LayerPtrs vp, float* __restrict__ vnorm, int Bt, int Hkv, long long segs, long long N, long long vs0,
+                  long long vs1, long long vs2) {
   grid_dependency_wait();
-  const int lane = threadIdx.x & 31;
-  const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-  const long long rows = (long long)L * Bt * Hkv * N;
-  constexpr int kPer16 = 16 / (int)sizeof(T);
-  for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps) {
-    const long long c = r % N;
-    long long t = r / N;
-    const int h = (int)(t % Hkv); t /= Hkv;
-    const int b = (int)(t % Bt);
-    const int l = (int)(t / Bt);
-    const T* row = reinterpret_cast<const T*>(vp.p[l]) + b * vs0 + h * vs1 + c * vs2;
-    float acc = 0.f;
-    for (int piece = lane; piece * kPer16 < d; piece += 32) {
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(row) + piece);
-      const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+  constexpr int kGroups = 32 / kLpr;                         // rows a warp loads at once
+  static_assert(kNormRows <= kLpr, "a lane of the row's group holds each norm");
+  const int lane = threadIdx.x & 31, sub = lane & (kLpr - 1), grp = lane / kLpr;
+  const long long row0 = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * (kNormRows * kGroups) + grp;
+  for (long long seg = blockIdx.y; seg < segs; seg += gridDim.y) {      // (l * Bt + b) * Hkv + h
+    const int h = (int)(seg % Hkv);
+    const int b = (int)(seg / Hkv % Bt);
+    const int l = (int)(seg / Hkv / Bt);
+    const T* base = reinterpret_cast<const T*>(vp.p[l]) + b * vs0 + h * vs1;
+    uint4 w[kNormRows];
+#pragma unroll
+    for (int u = 0; u < kNormRows; ++u) {
+      const long long c = min(row0 + u * kGroups, N - 1);
+      w[u] = __ldg(reinterpret_cast<const uint4*>(base + c * vs2) + sub);
+    }
+    float mine = 0.f;
+#pragma unroll
+    for (int u = 0; u < kNormRows; ++u) {
+      const uint32_t ws[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+      float acc = 0.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         if (sizeof(T) == 2) {
@@ -38,11 +50,24 @@ value_norm_kernel(LayerPtrs vp, float* __restrict__ vnorm, int L, int Bt, int Hk
           acc = fmaf(x, x, acc);
         }
       }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) vnorm[r] = sqrtf(acc);
+      for (int o = kLpr / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (sub == u) mine = acc;
+    }
+    const long long c = row0 + sub * kGroups;
+    if (sub < kNormRows && c < N) vnorm[seg * N + c] = sqrtf(mine);
   }
+}
+
+template <typename T, int kLpr>
+kvc_status launch_norm_t(const Problem& P, const LayerPtrs& v, float* vnorm, cudaStream_t st) {
+  const long long per_cta = 8LL * kNormRows * (32 / kLpr);
+  const long long segs = (long long)P.L * P.Bt * P.Hkv;
+  const dim3 grid((unsigned)((P.N + per_cta - 1) / per_cta), (unsigned)(segs < 65535 ? segs : 65535));
+  KVC_CUDA(launch_dependent(value_norm_kernel<T, kLpr>, grid, dim3(256), 0, st, v, vnorm, P.Bt, P.Hkv, segs, P.N,
+                            P.kvs[0], P.kvs[1], P.kvs[2]));
+  KVC_LAUNCH_CHECK("value_norm_kernel");
+  return KVC_OK;
 }
 
 // One CTA per (layer, sequence, head): marks the kept positions in a bitmap (global scratch, one
@@ -156,23 +181,9 @@ kvc_status launch_scale(float* x, long long n, float f, cudaStream_t st) {
 }
 
 kvc_status launch_value_norm(const Problem& P, const LayerPtrs& v, float* vnorm, cudaStream_t st) {
-  const long long rows = (long long)P.L * P.Bt * P.Hkv * P.N;
-  long long blocks = (rows + 7) / 8;
-  int dev = 0, sms = 0;
-  KVC_CUDA(cudaGetDevice(&dev));
-  KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const long long cap = (long long)sms * 32;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  if (P.dtype == KVC_BF16) {
-    KVC_CUDA(launch_dependent(value_norm_kernel<__nv_bfloat16>, dim3((unsigned)blocks), dim3(256), 0, st, v, vnorm,
-                              P.L, P.Bt, P.Hkv, P.d, P.N, P.kvs[0], P.kvs[1], P.kvs[2]));
-  } else {
-    KVC_CUDA(launch_dependent(value_norm_kernel<float>, dim3((unsigned)blocks), dim3(256), 0, st, v, vnorm,
-                              P.L, P.Bt, P.Hkv, P.d, P.N, P.kvs[0], P.kvs[1], P.kvs[2]));
-  }
-  KVC_LAUNCH_CHECK("value_norm_kernel");
-  return KVC_OK;
+  if (P.dtype == KVC_BF16)
+    return P.d == 128 ? launch_norm_t<__nv_bfloat16, 16>(P, v, vnorm, st) : launch_norm_t<__nv_bfloat16, 8>(P, v, vnorm, st);
+  return P.d == 128 ? launch_norm_t<float, 32>(P, v, vnorm, st) : launch_norm_t<float, 16>(P, v, vnorm, st);
 }
 
 size_t order_kept_workspace_bytes(const Problem& P) {
