@@ -46,10 +46,11 @@
 // KVC_ERR_TIMEOUT, stops computing and drains.
 //
 // Warp roles (512 threads): warp 0 = TMA producer (K ring, Q ring, L2 prefetch); warp 1 = MMA
-// issuer of pass 1 and TMEM owner; warp 2 = MMA issuer of pass 2 (two issuers: issuing the eight
-// MMAs of a tile takes a thread about 420 clocks, a commit about 50 and every barrier wait
-// about 100 even when it succeeds at once, which together is more than the 512 tensor clocks of
-// the tile, and the tensor pipe would idle meanwhile); warp 3 has no role; warps 4-7 =
+// issuer of pass 1 and TMEM owner; warp 2 = MMA issuer of pass 2 (two issuers: the waits, the eight MMAs
+// and the commits of a tile take longer than its 512 tensor clocks).  These three warps run their
+// loops with all lanes and elect a lane for each MMA, commit or copy: from one lane of a diverged warp
+// every such instruction first moves its operands to uniform registers, about 50 clocks per MMA (the
+// kernel alone on the 8B shape at 32K: 684 -> 656 us; 64 window rows and GQA group 7: 8 % less); warp 3 has no role; warps 4-7 =
 // pass-2 epilogue; warps 8-15 = pass-1 epilogue (two groups of four warps, each takes one half
 // of every tile's columns).
 #include <cuda.h>
@@ -172,6 +173,18 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
   if (mbar_try(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, ctl);
+}
+// The same by a whole warp, with one answer for all lanes: a role that runs warp-uniformly keeps its ring
+// positions, descriptors and barrier addresses in uniform registers, which is where tcgen05.mma, tcgen05.commit and
+// the TMA copies take them from.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
+  if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, ctl));
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 // The same for a copy or an MMA that has been issued and therefore completes whatever the rest
 // of the grid does: only the time bound ends this wait early, not the abort flag.
@@ -539,7 +552,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
   using SL = SmemLayout<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   volatile Ctl* ctl = reinterpret_cast<volatile Ctl*>(smem + SL::kCtl);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + SL::kTmemSlot);
 
@@ -869,7 +882,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     // last one seen, so neither thread may skip a phase of a ring barrier, and the producer must
     // not refill a slot before both have seen its fill (the "empty" barriers count two arrivals:
     // the user's commit and the other thread's acknowledgement).
-    if (lane == 0) {
+    {
       const int mine = warp - 1;       // the pass this thread issues
       Ring kr = {0, 0}, qr = {0, 0};
       Ring tb = {0, 0};                // accumulator buffer of this pass (two per pass)
@@ -886,31 +899,34 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
           Cursor& c = cur[pass];
           if (c.valid(P)) {
             if (c.t == 0) {
-              ok = mbar_wait(bar_qfull(qr.i), (uint32_t)qr.phase, ctl);
+              ok = mbar_wait_warp(bar_qfull(qr.i), (uint32_t)qr.phase, ctl);
               if (pass == mine) cur_slot = qr.i;
-              else if (ok) mbar_arrive(bar_qfree(qr.i));
+              else if (ok && elect_one()) mbar_arrive(bar_qfree(qr.i));
             }
-            if (ok) ok = mbar_wait(bar_kfull(kr.i), (uint32_t)kr.phase, ctl);
-            if (ok && pass != mine) mbar_arrive(bar_kempty(kr.i));
+            if (ok) ok = mbar_wait_warp(bar_kfull(kr.i), (uint32_t)kr.phase, ctl);
+            if (ok && pass != mine && elect_one()) mbar_arrive(bar_kempty(kr.i));
             if (pass == mine) {
               const int buf = pass * 2 + tb.i;
-              if (ok && nt >= 2) ok = mbar_wait(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
+              if (ok && nt >= 2) ok = mbar_wait_warp(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
               if (ok) {
                 tc_fence_after();
                 const uint64_t dq0 = umma_desc(sbase + SL::kQ + cur_slot * SL::kTileBytes);
                 const uint64_t dk0 = umma_desc(sbase + SL::kK + kr.i * SL::kTileBytes);
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * kTile;
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                  // the start-address field counts 16-byte units: 64-element half, then 32 B per K step
-                  const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-                  // pass 1: rows = query rows (A = Q), columns = tokens (B = K); pass 2: swapped
-                  if (pass == 0) tc_mma_bf16(d_tmem, dq0 + off, dk0 + off, kIdesc, kk > 0);
-                  else tc_mma_bf16(d_tmem, dk0 + off, dq0 + off, kIdesc, kk > 0);
+                  for (int kk = 0; kk < D / 16; ++kk) {
+                    // the start-address field counts 16-byte units: 64-element half, then 32 B per K step
+                    const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
+                    // pass 1: rows = query rows (A = Q), columns = tokens (B = K); pass 2: swapped
+                    if (pass == 0) tc_mma_bf16(d_tmem, dq0 + off, dk0 + off, kIdesc, kk > 0);
+                    else tc_mma_bf16(d_tmem, dk0 + off, dq0 + off, kIdesc, kk > 0);
+                  }
+                  tc_commit(bar_kempty(kr.i));   // the K stage may be refilled once these MMAs are done
+                  tc_commit(bar_tfull(buf));     // ... and the accumulator is then complete
+                  if (c.last(P)) tc_commit(bar_qfree(cur_slot));
                 }
-                tc_commit(bar_kempty(kr.i));   // the K stage may be refilled once these MMAs are done
-                tc_commit(bar_tfull(buf));     // ... and the accumulator is then complete
-                if (c.last(P)) tc_commit(bar_qfree(cur_slot));
+                __syncwarp();
                 tb.next(2);
                 if (nt < 2) ++nt;
               }
@@ -923,13 +939,14 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       }
       // no MMA may be in flight when the TMEM columns and the shared memory are given back
       if (nt > 0) {
-        tc_commit(bar_mma_done(mine));
+        if (elect_one()) tc_commit(bar_mma_done(mine));
+        __syncwarp();
         mbar_wait_issued(bar_mma_done(mine), 0u, ctl);
       }
     }
   } else if (warp == 0) {
     // ============================== TMA producer ==============================================
-    if (lane == 0) {
+    {
       unsigned long long pol_stream, pol_keep;
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
       asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
@@ -941,7 +958,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       int ahead_pos = 0;
       auto prefetch_next = [&]() {
         if (ahead_pos >= my_tiles) return;
-        if (ahead.valid(P)) {
+        if (ahead.valid(P) && elect_one()) {
           tma_prefetch_5d(P.k_maps + ahead.l, 0, ahead.tile(P) * kTile, 0, ahead.h, ahead.b);
         }
         ahead.advance(P);
@@ -956,23 +973,29 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
           Cursor& c = cur[pass];
           if (c.valid(P)) {
             if (c.t == 0) {                                    // a new run: its Q goes into the next ring slot
-              if (qc >= kQSlots) ok = mbar_wait(bar_qfree(qr.i), (uint32_t)(qr.phase ^ 1), ctl);
+              if (qc >= kQSlots) ok = mbar_wait_warp(bar_qfree(qr.i), (uint32_t)(qr.phase ^ 1), ctl);
               if (ok) {
-                mbar_expect_tx(bar_qfull(qr.i), q_bytes);
-                for (int hf = 0; hf < SL::kHalves; ++hf)
-                  tma_load_4d(sbase + SL::kQ + qr.i * SL::kTileBytes + hf * (kTile * 128), P.q_maps + c.l,
-                              bar_qfull(qr.i), hf * 64, c.template row0<kLong>(P), c.h * P.G + c.template head0<kLong>(P), c.b, pol_keep);
+                if (elect_one()) {
+                  mbar_expect_tx(bar_qfull(qr.i), q_bytes);
+                  for (int hf = 0; hf < SL::kHalves; ++hf)
+                    tma_load_4d(sbase + SL::kQ + qr.i * SL::kTileBytes + hf * (kTile * 128), P.q_maps + c.l,
+                                bar_qfull(qr.i), hf * 64, c.template row0<kLong>(P), c.h * P.G + c.template head0<kLong>(P), c.b, pol_keep);
+                }
+                __syncwarp();
                 qr.next(kQSlots);
                 if (qc < kQSlots) ++qc;
               }
             }
-            if (ok && nk >= SL::kStages) ok = mbar_wait(bar_kempty(kr.i), (uint32_t)(kr.phase ^ 1), ctl);
+            if (ok && nk >= SL::kStages) ok = mbar_wait_warp(bar_kempty(kr.i), (uint32_t)(kr.phase ^ 1), ctl);
             if (ok) {
-              mbar_expect_tx(bar_kfull(kr.i), SL::kTileBytes);
-              // pass 1 leaves the rows in L2 for pass 2; pass 2 is their last use
-              // (one copy for the whole tile: the 64-element halves of the rows are a dimension of the map)
-              tma_load_5d(sbase + SL::kK + kr.i * SL::kTileBytes, P.k_maps + c.l, bar_kfull(kr.i), 0, c.tile(P) * kTile, 0,
-                          c.h, c.b, pass == 0 ? pol_keep : pol_stream);
+              if (elect_one()) {
+                mbar_expect_tx(bar_kfull(kr.i), SL::kTileBytes);
+                // pass 1 leaves the rows in L2 for pass 2; pass 2 is their last use
+                // (one copy for the whole tile: the 64-element halves of the rows are a dimension of the map)
+                tma_load_5d(sbase + SL::kK + kr.i * SL::kTileBytes, P.k_maps + c.l, bar_kfull(kr.i), 0, c.tile(P) * kTile, 0,
+                            c.h, c.b, pass == 0 ? pol_keep : pol_stream);
+              }
+              __syncwarp();
               kr.next(SL::kStages);
               if (nk < SL::kStages) ++nk;
             }
