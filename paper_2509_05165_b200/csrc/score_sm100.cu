@@ -24,8 +24,8 @@
 //                        else); a pass-2 thread whose word shows such runs acquires the complete
 //                        word and folds their records, in run order (the same order for every
 //                        reader), into the fixed-point sum of the others.
-//   pass 2 (emit)        the same CTA revisits its tiles a fixed number of runs later, when their
-//                        K rows are still in L2.  D[token, query row] = K Q^T (operands swapped:
+//   pass 2 (emit)        the same CTA revisits its tiles as soon as their unit's statistics are
+//                        complete, when their K rows are still in L2.  D[token, query row] = K Q^T (operands swapped:
 //                        tokens on TMEM lanes), so the max over the window rows (Eq. 14) and the
 //                        mean/max over the query heads of the group (Eq. 15) are in-thread and
 //                        the score store is coalesced.  max_m exp(s_m - lse_m) is evaluated as
@@ -37,22 +37,24 @@
 // length through one variant that reads it at run time); with more than one row tile the
 // pass-2 results are partial group aggregates that the Eq. 16 kernel combines in a fixed order.
 //
-// Every CTA walks one static sequence that alternates a pass-1 tile with a pass-2 tile; the
-// pass-2 stream trails the pass-1 stream by `shift` tiles (two runs where a unit has no more
-// runs than there are CTAs: 38 MB of K at 148 CTAs, which L2 still holds).  A pass-2 tile only
-// ever waits for pass-1 tiles that lie earlier in every CTA's sequence, so the walk cannot
-// deadlock while all CTAs are resident (the host checks that they can be).  Every wait
-// (mbarrier or global word) is bounded; on expiry the kernel records
-// KVC_ERR_TIMEOUT, stops computing and drains.
+// The two passes of a CTA are two pipelines of their own (copies -> K stages and Q slots -> MMAs -> two
+// accumulators -> epilogue) over the same list of runs; they share nothing but the issue slots and the
+// tensor pipe.  Pass 2 goes as fast as the statistics arrive; pass 1 is held to at most `lead` tiles ahead
+// of it (two runs where a unit has no more runs than there are CTAs: 38 MB of K at 148 CTAs, which L2 still
+// holds), exactly what the statistics need: they need every run of a unit, and the other CTAs' runs of
+// it lie that far ahead at most, so the CTAs cannot wait for each other in a circle while all of them are
+// resident (the host checks that they can be).  Every wait (mbarrier or global word) is bounded; on expiry
+// the kernel records KVC_ERR_TIMEOUT, stops computing and drains.
 //
-// Warp roles (512 threads): warp 0 = TMA producer (K ring, Q ring, L2 prefetch); warp 1 = MMA
-// issuer of pass 1 and TMEM owner; warp 2 = MMA issuer of pass 2 (two issuers: the waits, the eight MMAs
-// and the commits of a tile take longer than its 512 tensor clocks).  These three warps run their
-// loops with all lanes and elect a lane for each MMA, commit or copy: from one lane of a diverged warp
-// every such instruction first moves its operands to uniform registers, about 50 clocks per MMA (the
-// kernel alone on the 8B shape at 32K: 684 -> 656 us; 64 window rows and GQA group 7: 8 % less); warp 3 has no role; warps 4-7 =
-// pass-2 epilogue; warps 8-15 = pass-1 epilogue (two groups of four warps, each takes one half
-// of every tile's columns).
+// Warp roles (512 threads): warp 0 = TMA producer of pass 1 (K, Q, L2 prefetch), warp 3 = of pass 2; warp
+// 1 = MMA issuer of pass 1 and TMEM owner, warp 2 = of pass 2; warps 4-7 = pass-2 epilogue; warps 8-15 = pass-1
+// epilogue (two groups of four warps, each takes one half of every tile's columns).  The four single warps
+// run their loops with all lanes and elect a lane for each MMA, commit or copy: from one lane of a diverged
+// warp every such instruction first moves its operands to uniform registers, about 50 clocks per MMA (the
+// scoring of the 8B shape at 32K: 684 -> 656 us).  With one producer and one K and Q ring for both passes,
+// every one of these warps had to follow both passes tile by tile, 1100 (issuers) to 1500 (producer) clocks
+// of bookkeeping out of the 2160 that a pair of tiles took; with a pipeline per pass a pair takes 1890 (32K: 656 ->
+// 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers), and the epilogues are what it waits for.
 #include <cuda.h>
 
 #include <atomic>
@@ -60,25 +62,14 @@
 
 #include "kvc_internal.cuh"
 
-#ifndef KVC_SCORE_RUN_TILES
-#define KVC_SCORE_RUN_TILES 4      // tiles per run
-#endif
-#ifndef KVC_SCORE_LAG_TILES
-#define KVC_SCORE_LAG_TILES 0      // tiles of slack beyond the runs a unit's statistics have to wait for
-#endif
-#ifndef KVC_SCORE_PREFETCH
-#define KVC_SCORE_PREFETCH 2       // pass-1 tiles prefetched into L2 ahead of their load
-#endif
-
 namespace kvc {
 namespace {
 
 constexpr int kTile = 128;            // tokens per tile = MMA M = MMA N
 constexpr int kFastThreads = 512;
 constexpr int kRows = 128;            // query rows per unit handled by one MMA (R <= 128)
-constexpr int kMinRunTiles = KVC_SCORE_RUN_TILES;   // runs are longer only where a unit would otherwise have more than 255
-constexpr int kQSlots = 3;
-constexpr int kPrefetch = KVC_SCORE_PREFETCH;
+constexpr int kMinRunTiles = 4;       // tiles per run; runs are longer only where a unit would otherwise have more than 255
+constexpr int kPrefetch = 2;          // pass-1 tiles prefetched into L2 ahead of their load
 constexpr float kLog2eF = 1.4426950408889634f;
 constexpr float kRescaleLimit = 1.8446744e19f;               // 2^64: a chunk sum beyond it restarts with a new reference
 constexpr unsigned long long kDefaultWaitLimitNs = 2000000000ull;   // 2 s: far beyond any healthy wait
@@ -107,7 +98,7 @@ struct FastParams {
   int step_u, step_j;          // grid = step_u * RPU + step_j: how a CTA's next run moves (unit, run in unit)
   int step_l, step_b, step_h, step_q;  // step_u = ((step_l * Bt + step_b) * Hkv + step_h) * QT + step_q
   unsigned int total_runs;     // U * RPU
-  int shift;                   // tiles by which the pass-2 stream trails the pass-1 stream
+  int lead;                    // tiles by which pass 1 may be ahead of pass 2 (their K copies)
   float sl2e;                  // scale * log2(e)
   int agg_group;
   unsigned long long wait_limit_ns;   // bound of every device-side wait
@@ -147,7 +138,7 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
 // Per-CTA control block in shared memory.
 struct Ctl {
   int abort;                       // set by the first wait of this CTA that gives up
-  int pad;
+  int p2_tiles;                    // pass-2 tiles whose copies have been issued
   unsigned long long limit_ns;     // bound of every wait
   const int* grid_status;          // the device status word (may be null): non-zero once any CTA gave up
 };
@@ -180,6 +171,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
   if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
   return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, ctl));
+}
+// Pass 1 may copy tile `pos` once fewer than `lead` tiles lie between it and pass 2 (bounded; one answer per warp).
+__device__ __noinline__ bool wait_lead_slow(int pos, int lead, volatile Ctl* ctl) {
+  const unsigned long long t0 = globaltimer_ns();
+  uint32_t spins = 0;
+  while (pos - ctl->p2_tiles >= lead) {
+    __nanosleep(20);
+    if ((++spins & 1023u) == 0 && give_up(ctl, t0)) return false;
+  }
+  return true;
+}
+__device__ __forceinline__ bool wait_lead(int pos, int lead, volatile Ctl* ctl) {
+  if (__all_sync(0xffffffffu, pos - ctl->p2_tiles < lead)) return true;
+  return __all_sync(0xffffffffu, wait_lead_slow(pos, lead, ctl));
 }
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
@@ -286,6 +291,9 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 __device__ __forceinline__ void named_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+__device__ __forceinline__ void named_bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 // (release: what this thread wrote before -- the run's record of the row -- is visible to whoever
 // acquires a value of the word that includes this addition)
 __device__ __forceinline__ void red_add_release_u64(unsigned long long* p, unsigned long long v) {
@@ -330,19 +338,15 @@ __device__ __forceinline__ void combine(float& M, float& Ls, float m, float l) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// The static per-CTA sequence.  Stream position idx -> (run ordinal, tile); a run is RT
-// consecutive tiles of one unit, runs are dealt to the CTAs round-robin.
+// The runs of a CTA.  A run is RT consecutive tiles of one unit (the last run of a unit may be
+// shorter); run k of the CTA is the global run blockIdx.x + k * grid.  The cursor moves from run to run
+// by additions only (the increments come from the host): a division would queue behind the
+// exponentials in the special-function pipe.
 // ------------------------------------------------------------------------------------------------
-// Walks one stream of this CTA: position -> (run, tile).  Run k of the CTA is the global run
-// blockIdx.x + k * grid; the cursor moves from run to run by additions only (the per-run
-// increments come from the host), because a division would queue behind the exponentials in the
-// special-function pipe.
-struct Cursor {
-  int t;            // position inside the run, 0 .. RT-1
+struct RunCursor {
   int u, j;         // unit, run inside the unit
   int l, b, h, q;   // the unit's layer, sequence, KV head, row tile
   __device__ __forceinline__ void init(const FastParams& P) {
-    t = 0;
     u = (int)(blockIdx.x / (unsigned int)P.RPU);
     j = (int)(blockIdx.x - (unsigned int)u * (unsigned int)P.RPU);
     const int uh = u / P.QT;
@@ -366,11 +370,9 @@ struct Cursor {
   __device__ __forceinline__ int head0(const FastParams& P) const { return (!kLong || P.CH == 1) ? q * P.HPT : q / P.CH; }
   // index of the (layer, sequence, KV head)
   __device__ __forceinline__ int kv_unit(const FastParams& P) const { return (l * P.Bt + b) * P.Hkv + h; }
-  __device__ __forceinline__ int tile(const FastParams& P) const { return j * P.RT + t; }
-  __device__ __forceinline__ bool valid(const FastParams& P) const { return tile(P) < P.NT; }
-  // last valid tile of its run
-  __device__ __forceinline__ bool last(const FastParams& P) const { return t == P.RT - 1 || tile(P) + 1 >= P.NT; }
-  __device__ __forceinline__ void next_run(const FastParams& P) {
+  __device__ __forceinline__ int tiles(const FastParams& P) const { return min(P.RT, P.NT - j * P.RT); }
+  __device__ __forceinline__ int first_token(const FastParams& P) const { return j * P.RT * kTile; }
+  __device__ __forceinline__ void next(const FastParams& P) {
     j += P.step_j;
     int c = 0;
     if (j >= P.RPU) { j -= P.RPU; c = 1; }
@@ -383,9 +385,6 @@ struct Cursor {
     if (b >= P.Bt) { b -= P.Bt; c = 1; }
     l += P.step_l + c;
   }
-  __device__ __forceinline__ void advance(const FastParams& P) {
-    if (++t == P.RT) { t = 0; next_run(P); }
-  }
 };
 
 // A ring position with its mbarrier phase bit.
@@ -394,27 +393,39 @@ struct Ring {
   __device__ __forceinline__ void next(int n) { if (++i == n) { i = 0; phase ^= 1; } }
 };
 
+// K stages and Q slots per pass: what 227 KB hold, and pass 1, whose rows come from HBM, gets the odd stage.  (With two
+// and two stages and another Q slot for either pass, or with two and three, the kernel takes the same time within 1 %;
+// with three and one it is 5 % slower.)
+template <int K1, int K2, int Q1, int Q2>
+struct RingSizes {
+  static constexpr int kK1 = K1, kK2 = K2, kQ1 = Q1, kQ2 = Q2;
+};
+template <int D> struct Rings;
+template <> struct Rings<128> : RingSizes<3, 2, 1, 1> {};
+template <> struct Rings<64> : RingSizes<5, 5, 2, 2> {};
+
 template <int D>
-struct SmemLayout {
+struct SmemLayout : Rings<D> {
+  using R = Rings<D>;
   static constexpr int kHalves = D / 64;
   static constexpr int kTileBytes = kTile * D * 2;
-  static constexpr int kStages = (D == 128) ? 4 : 8;
-  static constexpr int kQ = 0;                                 // Q ring
-  static constexpr int kK = kQSlots * kTileBytes;              // K stage ring
+  static constexpr int kStages = R::kK1 + R::kK2, kSlots = R::kQ1 + R::kQ2;
+  static constexpr int kQ = 0;                                 // Q slots, pass 1's first
+  static constexpr int kK = kSlots * kTileBytes;               // K stages, pass 1's first
   static constexpr int kMisc = kK + kStages * kTileBytes;
   static constexpr int kBarKFull = kMisc;                      // kStages x 8
   static constexpr int kBarKEmpty = kBarKFull + 8 * kStages;
   static constexpr int kBarTFull = kBarKEmpty + 8 * kStages;   // 4 x 8
   static constexpr int kBarTEmpty = kBarTFull + 32;
-  static constexpr int kBarQFull = kBarTEmpty + 32;            // kQSlots x 8
-  static constexpr int kBarQFree = kBarQFull + 8 * kQSlots;
-  static constexpr int kBarMmaDone = kBarQFree + 8 * kQSlots;  // 2 x 8
+  static constexpr int kBarQFull = kBarTEmpty + 32;            // kSlots x 8
+  static constexpr int kBarQFree = kBarQFull + 8 * kSlots;
+  static constexpr int kBarMmaDone = kBarQFree + 8 * kSlots;   // 2 x 8
   static constexpr int kTmemSlot = kBarMmaDone + 16;           // 4 B (+ padding)
   static constexpr int kCtl = kTmemSlot + 8;                   // Ctl, 24 B
   static constexpr int kNegLse = (kCtl + 24 + 15) / 16 * 16;   // 128 floats, read as 16-byte vectors:
                                                                // -log-sum-exp of the pass-2 unit
-  static constexpr int kStats = kNegLse + kRows * 4;           // 128 rows x float2: the upper half's statistics
-  static constexpr int kTotal = kStats + kRows * 8;
+  static constexpr int kStats = kNegLse + kRows * 4;           // 2 x 128 rows x float2: the upper half's statistics
+  static constexpr int kTotal = kStats + 2 * kRows * 8;
   static_assert(kCtl % 8 == 0 && kNegLse % 16 == 0 && kStats % 8 == 0 && kTotal <= 232448, "shared-memory layout");
 };
 
@@ -566,12 +577,13 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
 
   const bool aligned = (sbase & 1023u) == 0;     // the swizzled tiles need a 1024-byte aligned base
   if (threadIdx.x == 0) {
-    for (int s = 0; s < SL::kStages; ++s) { mbar_init(bar_kfull(s), 1); mbar_init(bar_kempty(s), 2); }
+    for (int s = 0; s < SL::kStages; ++s) { mbar_init(bar_kfull(s), 1); mbar_init(bar_kempty(s), 1); }
     // the accumulators of pass 1 are read by eight warps (two column halves), those of pass 2 by four
     for (int b = 0; b < 4; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), b < 2 ? 8 : 4); }
-    for (int q = 0; q < kQSlots; ++q) { mbar_init(bar_qfull(q), 1); mbar_init(bar_qfree(q), 2); }
+    for (int q = 0; q < SL::kSlots; ++q) { mbar_init(bar_qfull(q), 1); mbar_init(bar_qfree(q), 1); }
     mbar_init(bar_mma_done(0), 1); mbar_init(bar_mma_done(1), 1);
     ctl->abort = 0;
+    ctl->p2_tiles = 0;
     ctl->limit_ns = P.wait_limit_ns;
     ctl->grid_status = P.status;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -587,15 +599,12 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
   const uint32_t tmem_base = *tmem_slot;
   grid_dependency_wait();      // everything above overlapped the end of the kernel before this one
 
-  // this CTA's share of the runs and the length of its sequence
-  // (the host keeps all of these below 2^31)
+  // this CTA's share of the runs
   int my_runs = (P.total_runs > blockIdx.x) ? (int)((P.total_runs - blockIdx.x + P.grid - 1) / P.grid) : 0;
   if (!aligned) {
     if (threadIdx.x == 0 && P.status) atomicCAS(P.status, 0, (int)KVC_ERR_CUDA);
     my_runs = 0;               // nothing is computed; the teardown below still frees the TMEM columns
   }
-  const int my_tiles = my_runs * P.RT;                  // stream length (some positions hold no tile)
-  const int n_steps = my_tiles > 0 ? my_tiles + P.shift : 0;
   constexpr bool kLong = (W == 0);   // only the run-time window variant has windows longer than 128 rows
   // the whole box arrives (rows outside the tensor as zeros)
   const uint32_t q_bytes = (uint32_t)((!kLong || P.CH == 1) ? P.HPT * P.w : kRows) * D * 2;
@@ -609,7 +618,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     const int quarter = warp & 3;                     // TMEM lane quarter this warp may read
     const int row = quarter * 32 + lane;              // TMEM lane = query row
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    float2* stage = reinterpret_cast<float2*>(smem + SL::kStats) + row;
+    float2* const stage = reinterpret_cast<float2*>(smem + SL::kStats) + row;
     const int row_m = row % (W > 0 ? W : P.w);        // the row inside its query head (windows of up to 128 rows)
     const unsigned long long scale2 = pack2(P.sl2e, P.sl2e);
 
@@ -647,24 +656,22 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       }
     };
 
-    Cursor c;
+    RunCursor c;
     c.init(P);
-    for (int idx = 0; idx < my_tiles; ++idx, c.advance(P)) {
-      if (!c.valid(P)) continue;
-      const int tile = c.tile(P);
-      const bool run_ends = c.last(P);
+    for (int k = 0; k < my_runs; ++k, c.next(P)) {
       const bool row_used = row < c.template rows<kLong>(P);
-      if (c.t == 0 && half == 0) row_ref = __ldg(P.ref + (long long)c.u * kRows + row);   // used at the run's end
-      const int buf = n1 & 1;
-      // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
-      ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(buf), (uint32_t)((n1 >> 1) & 1), ctl));
-      ++n1;
-      if (ok) {
+      if (half == 0) row_ref = __ldg(P.ref + (long long)c.u * kRows + row);   // used at the run's end
+      const int nt = c.tiles(P);
+      int tok0 = c.first_token(P);                      // first token of the tile
+      for (int t = 0; t < nt; ++t, tok0 += kTile) {
+        const int buf = n1 & 1;
+        // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
+        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(buf), (uint32_t)((n1 >> 1) & 1), ctl));
+        ++n1;
+        if (!ok) continue;
         tc_fence_after();
-        const long long c0 = (long long)tile * kTile + half * 64;
-        const bool full = (long long)tile * kTile + kTile - 1 <= vis_all;       // no masking anywhere in the tile
         const uint32_t taddr = lane_addr + (uint32_t)buf * kTile + half * 64;
-        if (full) {
+        if (tok0 + kTile - 1 <= vis_all) {              // no masking anywhere in the tile
           uint32_t ra[32], rb[32];
           tc_ld32_nowait(taddr, ra);
           tc_ld32_nowait(taddr + 32, rb);
@@ -677,21 +684,25 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         } else {
           float m2 = mref, l2 = lsum;                     // (the whole warp takes part in the TMEM loads)
           const long long row_vis = min(P.N - 1, P.q_pos0 + ((!kLong || P.CH == 1) ? row_m : c.template row0<kLong>(P) + row));   // last key this row sees
-          p1_masked_half(taddr, c0, row_vis, P.sl2e, &m2, &l2);
+          p1_masked_half(taddr, (long long)tok0 + half * 64, row_vis, P.sl2e, &m2, &l2);
           if (row_used) { mref = m2; lsum = l2; }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(bar_tempty(buf));
         }
       }
-      if (run_ends) {
-        // the two halves of every row meet through shared memory; the lower half's warps send the
-        // run's sum of every row
-        if (half == 1) *stage = make_float2(row_used ? mref : -INFINITY, row_used ? lsum : 0.f);
-        named_bar(3, 256);
-        const float2 other = *stage;
-        named_bar(3, 256);                                // the stage may be written again
-        if (half == 0 && ok && c.u != P.withhold_unit) {
+      // the end of the run: the two halves of every row meet through shared memory (two buffers in turn); the lower
+      // half's warps send the run's sum of every row, the upper half's go on to the next run
+      const int par = k & 1;
+      if (half == 1) {
+        if (k >= 2) named_bar(5 + par, 256);              // the buffer has been read
+        stage[par * kRows] = make_float2(row_used ? mref : -INFINITY, row_used ? lsum : 0.f);
+        named_bar_arrive(3 + par, 256);
+      } else {
+        named_bar(3 + par, 256);
+        const float2 other = stage[par * kRows];
+        if (k + 2 < my_runs) named_bar_arrive(5 + par, 256);
+        if (ok && c.u != P.withhold_unit) {
           float M = row_used ? mref : -INFINITY, Ls = row_used ? lsum : 0.f;
           combine(M, Ls, other.x, other.y);
           // the short way: add the run's sum, rescaled to the row's fixed reference, to the row's
@@ -710,8 +721,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
             red_add_release_u64(word, kAccArrival + kAccOverflow);
           }
         }
-        mref = -INFINITY; lsum = 0.f;
       }
+      mref = -INFINITY; lsum = 0.f;
     }
   } else if (warp >= 4 && warp < 8) {
     // ============================== pass-2 epilogue ============================================
@@ -727,26 +738,23 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     const float inv_g = (P.QT == 1 && !gmax) ? 1.f / (float)P.G : 1.f;   // one row tile: the mean of Eq. 15 is finished here
     const int vis_all_i = (int)vis_all;                // (N < 2^30)
     const int n_ctx = (int)P.N;
-    int rows_u = 0, n_chunks = 0;                      // of the current run's unit
-    float* score_row = nullptr;                        // where that unit's scores (or partial aggregates) go
-
-    Cursor cu;
+    RunCursor cu;
     cu.init(P);
     unsigned long long early_word = 0ull;             // a coming run's pushed word and reference, fetched ahead
     float early_ref = 0.f;
-    int early_u = -1;                                 // ... and the unit they belong to
-    if (my_tiles > 0) {
+    if (my_runs > 0) {
       early_word = ld_relaxed_u64(P.acc + (long long)cu.u * kRows + trow);
       early_ref = __ldg(P.ref + (long long)cu.u * kRows + trow);
-      early_u = cu.u;
     }
-    for (int idx = 0; idx < my_tiles; ++idx, cu.advance(P)) {
-      if (!cu.valid(P)) continue;
-      const int tok0 = cu.tile(P) * kTile;             // first token of the tile
-      if (cu.t == 0) {
-        rows_u = cu.template rows<kLong>(P);
-        n_chunks = (rows_u + 31) / 32;
-        score_row = P.scores + ((long long)cu.q * ((long long)P.L * P.Bt * P.Hkv) + cu.kv_unit(P)) * P.N;
+    for (int k = 0; k < my_runs; ++k) {
+      const int rows_u = cu.template rows<kLong>(P);
+      const int n_chunks = (rows_u + 31) / 32;
+      const int row0 = cu.template row0<kLong>(P);
+      // where the unit's scores (or partial aggregates) go
+      float* const score_row = P.scores + ((long long)cu.q * ((long long)P.L * P.Bt * P.Hkv) + cu.kv_unit(P)) * P.N;
+      const int nt = cu.tiles(P);
+      int tok0 = cu.first_token(P);                    // first token of the tile
+      {
         // a new run: its unit's log-sum-exp.  The short way: the row's pushed word, complete once
         // every run of the unit has arrived (fetched a tile or two ago; polled if it was not
         // complete then).  If a run's sum did not fit, the runs' records decide.
@@ -754,7 +762,6 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         if (ok && trow < rows_u) {
           bool pushed = false;
           {
-            if (early_u != cu.u) { early_word = 0ull; early_ref = __ldg(P.ref + (long long)cu.u * kRows + trow); }
             unsigned long long word = early_word;
             if ((unsigned int)(word >> 56) != (unsigned int)P.RPU)
               word = poll_acc_slow(P.acc + (long long)cu.u * kRows + trow, (unsigned int)P.RPU, ctl);
@@ -788,19 +795,17 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
             lse = M + log2f(Ls);
           }
         }
-        early_u = -1;
         named_bar(1, 128);                             // everyone is done with the previous unit's values
         neg_lse[trow] = (trow < rows_u) ? -lse : 0.f;
         named_bar(1, 128);
         ok = !__any_sync(0xffffffffu, ctl->abort != 0) && ok;
       }
-      if (early_u < 0 && cu.t >= P.RT - 2 && idx + (P.RT - cu.t) < my_tiles) {
+      cu.next(P);
+      for (int t = 0; t < nt; ++t, tok0 += kTile) {
+      if (t == max(nt - 2, 0) && k + 1 < my_runs) {
         // the next run's word and reference: in flight while the rest of this run is computed
-        Cursor nx = cu;
-        nx.next_run(P);
-        early_word = ld_relaxed_u64(P.acc + (long long)nx.u * kRows + trow);
-        early_ref = __ldg(P.ref + (long long)nx.u * kRows + trow);
-        early_u = nx.u;
+        early_word = ld_relaxed_u64(P.acc + (long long)cu.u * kRows + trow);
+        early_ref = __ldg(P.ref + (long long)cu.u * kRows + trow);
       }
       const int buf = 2 + (n2 & 1);
       const uint32_t tmem_col = (uint32_t)buf * kTile;
@@ -860,7 +865,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         // a window longer than 128 rows: the tile holds rows row0 .. of one query head and yields
         // that head's partial Eq. 14 (the maximum, or the sum, over these rows)
         gacc = p2_long_tile<kTaskMean>(lane_addr + tmem_col, neg_lse, n_chunks, rows_u, P.sl2e, full,
-                                       (long long)c - P.q_pos0 - cu.template row0<kLong>(P));
+                                       (long long)c - P.q_pos0 - row0);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty(buf));
@@ -873,154 +878,133 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       }
       // one row tile: the group aggregate itself; several: this tile's part of it
       if (c < n_ctx) score_row[c] = gacc * inv_g;
+      }
     }
   } else if (warp == 1 || warp == 2) {
     // ============================== MMA issuers ================================================
-    // Both walk the whole sequence (the rings are shared and filled in sequence order) and each
-    // issues the tiles of its own pass.  Each also waits for the fills that belong to the other
-    // pass and acknowledges them: a parity wait is only meaningful for the phase that follows the
-    // last one seen, so neither thread may skip a phase of a ring barrier, and the producer must
-    // not refill a slot before both have seen its fill (the "empty" barriers count two arrivals:
-    // the user's commit and the other thread's acknowledgement).
-    {
-      const int mine = warp - 1;       // the pass this thread issues
-      Ring kr = {0, 0}, qr = {0, 0};
-      Ring tb = {0, 0};                // accumulator buffer of this pass (two per pass)
-      int nt = 0;                      // tiles issued (saturating at 2)
-      int cur_slot = 0;
-      bool ok = true;
-      Cursor cur[2];
-      cur[0].init(P); cur[1].init(P);
-      for (int i = 0; i < n_steps && ok; ++i) {
+    // One warp per pass, the same code: it walks its pass's runs, all lanes together.
+    const int pass = warp - 1;
+    const int stage0 = pass == 0 ? 0 : SL::kK1, stages = pass == 0 ? SL::kK1 : SL::kK2;
+    const int slot0 = pass == 0 ? 0 : SL::kQ1, slots = pass == 0 ? SL::kQ1 : SL::kQ2;
+    Ring kr = {0, 0}, qr = {0, 0}, tb = {0, 0};        // K stage, Q slot, accumulator (two per pass)
+    bool ok = true, issued = false;
+    RunCursor c;
+    c.init(P);
+    for (int k = 0; k < my_runs && ok; ++k, c.next(P)) {
+      const int nt = c.tiles(P);
+      const int slot = slot0 + qr.i;
+      ok = mbar_wait_warp(bar_qfull(slot), (uint32_t)qr.phase, ctl);
+      const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
+      qr.next(slots);
+      for (int t = 0; t < nt && ok; ++t) {
+        const int st = stage0 + kr.i, buf = pass * 2 + tb.i;
+        ok = mbar_wait_warp(bar_kfull(st), (uint32_t)kr.phase, ctl);
+        if (ok) ok = mbar_wait_warp(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t dk = umma_desc(sbase + SL::kK + st * SL::kTileBytes);
+        // pass 1: rows = query rows (A = Q), columns = tokens (B = K); pass 2: swapped
+        const uint64_t da = pass == 0 ? dq : dk, db = pass == 0 ? dk : dq;
+        const uint32_t d_tmem = tmem_base + (uint32_t)buf * kTile;
+        if (elect_one()) {
 #pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-          const int idx = pass == 0 ? i : i - P.shift;
-          if (!ok || idx < 0 || idx >= my_tiles) continue;
-          Cursor& c = cur[pass];
-          if (c.valid(P)) {
-            if (c.t == 0) {
-              ok = mbar_wait_warp(bar_qfull(qr.i), (uint32_t)qr.phase, ctl);
-              if (pass == mine) cur_slot = qr.i;
-              else if (ok && elect_one()) mbar_arrive(bar_qfree(qr.i));
-            }
-            if (ok) ok = mbar_wait_warp(bar_kfull(kr.i), (uint32_t)kr.phase, ctl);
-            if (ok && pass != mine && elect_one()) mbar_arrive(bar_kempty(kr.i));
-            if (pass == mine) {
-              const int buf = pass * 2 + tb.i;
-              if (ok && nt >= 2) ok = mbar_wait_warp(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
-              if (ok) {
-                tc_fence_after();
-                const uint64_t dq0 = umma_desc(sbase + SL::kQ + cur_slot * SL::kTileBytes);
-                const uint64_t dk0 = umma_desc(sbase + SL::kK + kr.i * SL::kTileBytes);
-                const uint32_t d_tmem = tmem_base + (uint32_t)buf * kTile;
-                if (elect_one()) {
-#pragma unroll
-                  for (int kk = 0; kk < D / 16; ++kk) {
-                    // the start-address field counts 16-byte units: 64-element half, then 32 B per K step
-                    const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-                    // pass 1: rows = query rows (A = Q), columns = tokens (B = K); pass 2: swapped
-                    if (pass == 0) tc_mma_bf16(d_tmem, dq0 + off, dk0 + off, kIdesc, kk > 0);
-                    else tc_mma_bf16(d_tmem, dk0 + off, dq0 + off, kIdesc, kk > 0);
-                  }
-                  tc_commit(bar_kempty(kr.i));   // the K stage may be refilled once these MMAs are done
-                  tc_commit(bar_tfull(buf));     // ... and the accumulator is then complete
-                  if (c.last(P)) tc_commit(bar_qfree(cur_slot));
-                }
-                __syncwarp();
-                tb.next(2);
-                if (nt < 2) ++nt;
-              }
-            }
-            if (c.t == 0) qr.next(kQSlots);
-            kr.next(SL::kStages);
+          for (int kk = 0; kk < D / 16; ++kk) {
+            // the start-address field counts 16-byte units: 64-element half, then 32 B per K step
+            const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
+            tc_mma_bf16(d_tmem, da + off, db + off, kIdesc, kk > 0);
           }
-          c.advance(P);
+          tc_commit(bar_kempty(st));            // the K stage may be refilled once these MMAs are done
+          tc_commit(bar_tfull(buf));            // ... and the accumulator is then complete
+          if (t + 1 == nt) tc_commit(bar_qfree(slot));
         }
-      }
-      // no MMA may be in flight when the TMEM columns and the shared memory are given back
-      if (nt > 0) {
-        if (elect_one()) tc_commit(bar_mma_done(mine));
         __syncwarp();
-        mbar_wait_issued(bar_mma_done(mine), 0u, ctl);
+        issued = true;
+        kr.next(stages);
+        tb.next(2);
       }
     }
-  } else if (warp == 0) {
-    // ============================== TMA producer ==============================================
-    {
-      unsigned long long pol_stream, pol_keep;
-      asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
-      asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
-      Ring kr = {0, 0}, qr = {0, 0};   // next K stage / Q slot to fill; phase = parity of the fill count / ring size
-      int nk = 0, qc = 0;              // K tiles / Q tiles issued (saturating small counts are all that is needed)
-      bool ok = true;
-      Cursor cur[2], ahead;            // the two streams, and the pass-1 stream kPrefetch tiles ahead
-      cur[0].init(P); cur[1].init(P); ahead.init(P);
-      int ahead_pos = 0;
-      auto prefetch_next = [&]() {
-        if (ahead_pos >= my_tiles) return;
-        if (ahead.valid(P) && elect_one()) {
-          tma_prefetch_5d(P.k_maps + ahead.l, 0, ahead.tile(P) * kTile, 0, ahead.h, ahead.b);
-        }
-        ahead.advance(P);
-        ++ahead_pos;
-      };
-      for (int i = 0; i < kPrefetch; ++i) prefetch_next();
-      for (int i = 0; i < n_steps && ok; ++i) {
-#pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-          const int idx = pass == 0 ? i : i - P.shift;
-          if (!ok || idx < 0 || idx >= my_tiles) continue;
-          Cursor& c = cur[pass];
-          if (c.valid(P)) {
-            if (c.t == 0) {                                    // a new run: its Q goes into the next ring slot
-              if (qc >= kQSlots) ok = mbar_wait_warp(bar_qfree(qr.i), (uint32_t)(qr.phase ^ 1), ctl);
-              if (ok) {
-                if (elect_one()) {
-                  mbar_expect_tx(bar_qfull(qr.i), q_bytes);
-                  for (int hf = 0; hf < SL::kHalves; ++hf)
-                    tma_load_4d(sbase + SL::kQ + qr.i * SL::kTileBytes + hf * (kTile * 128), P.q_maps + c.l,
-                                bar_qfull(qr.i), hf * 64, c.template row0<kLong>(P), c.h * P.G + c.template head0<kLong>(P), c.b, pol_keep);
-                }
-                __syncwarp();
-                qr.next(kQSlots);
-                if (qc < kQSlots) ++qc;
-              }
-            }
-            if (ok && nk >= SL::kStages) ok = mbar_wait_warp(bar_kempty(kr.i), (uint32_t)(kr.phase ^ 1), ctl);
-            if (ok) {
-              if (elect_one()) {
-                mbar_expect_tx(bar_kfull(kr.i), SL::kTileBytes);
-                // pass 1 leaves the rows in L2 for pass 2; pass 2 is their last use
-                // (one copy for the whole tile: the 64-element halves of the rows are a dimension of the map)
-                tma_load_5d(sbase + SL::kK + kr.i * SL::kTileBytes, P.k_maps + c.l, bar_kfull(kr.i), 0, c.tile(P) * kTile, 0,
-                            c.h, c.b, pass == 0 ? pol_keep : pol_stream);
-              }
-              __syncwarp();
-              kr.next(SL::kStages);
-              if (nk < SL::kStages) ++nk;
-            }
+    // no MMA may be in flight when the TMEM columns and the shared memory are given back
+    if (issued) {
+      if (elect_one()) tc_commit(bar_mma_done(pass));
+      __syncwarp();
+      mbar_wait_issued(bar_mma_done(pass), 0u, ctl);
+    }
+  } else {
+    // ============================== TMA producers =============================================
+    // Warp 0 for pass 1, warp 3 for pass 2, the same code.  Pass 1 leaves the rows in L2 for pass 2; pass 2 is
+    // their last use.  Pass 1's producer stays at most P.lead tiles ahead of pass 2's.
+    const int pass = warp == 0 ? 0 : 1;
+    const int stage0 = pass == 0 ? 0 : SL::kK1, stages = pass == 0 ? SL::kK1 : SL::kK2;
+    const int slot0 = pass == 0 ? 0 : SL::kQ1, slots = pass == 0 ? SL::kQ1 : SL::kQ2;
+    unsigned long long pol_stream, pol_keep;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
+    const unsigned long long pol_k = pass == 0 ? pol_keep : pol_stream;
+    Ring kr = {0, 0}, qr = {0, 0};
+    int pos = 0, nq = 0;               // K tiles and Q tiles issued
+    bool ok = true;
+    RunCursor c, nx;
+    c.init(P);
+    for (int k = 0; k < my_runs && ok; ++k) {
+      nx = c;
+      nx.next(P);
+      const int nt = c.tiles(P);
+      const int ntn = k + 1 < my_runs ? nx.tiles(P) : 0;
+      const int tok0 = c.first_token(P);
+      for (int t = 0; t < nt; ++t) {
+        if (pass == 0) ok = wait_lead(pos, P.lead, ctl);
+        const int st = stage0 + kr.i;
+        if (ok) ok = mbar_wait_warp(bar_kempty(st), (uint32_t)(kr.phase ^ 1), ctl);
+        if (!ok) break;
+        if (elect_one()) {
+          mbar_expect_tx(bar_kfull(st), SL::kTileBytes);
+          // (one copy for the whole tile: the 64-element halves of the rows are a dimension of the map)
+          tma_load_5d(sbase + SL::kK + st * SL::kTileBytes, P.k_maps + c.l, bar_kfull(st), 0, tok0 + t * kTile, 0, c.h, c.b,
+                      pol_k);
+          if (pass == 0) {
+            const int ta = t + kPrefetch;
+            if (ta < nt) tma_prefetch_5d(P.k_maps + c.l, 0, tok0 + ta * kTile, 0, c.h, c.b);
+            else if (ta - nt < ntn) tma_prefetch_5d(P.k_maps + nx.l, 0, nx.first_token(P) + (ta - nt) * kTile, 0, nx.h, nx.b);
+          } else {
+            ctl->p2_tiles = pos + 1;
           }
-          c.advance(P);
-          if (pass == 0) prefetch_next();
+        }
+        __syncwarp();
+        kr.next(stages);
+        ++pos;
+        if (t == 0) {
+          // the run's Q (after its first K tile: with a single slot it has to wait for the MMAs of the run before)
+          const int slot = slot0 + qr.i;
+          ok = mbar_wait_warp(bar_qfree(slot), (uint32_t)(qr.phase ^ 1), ctl);
+          if (!ok) break;
+          if (elect_one()) {
+            mbar_expect_tx(bar_qfull(slot), q_bytes);
+            for (int hf = 0; hf < SL::kHalves; ++hf)
+              tma_load_4d(sbase + SL::kQ + slot * SL::kTileBytes + hf * (kTile * 128), P.q_maps + c.l, bar_qfull(slot), hf * 64,
+                          c.template row0<kLong>(P), c.h * P.G + c.template head0<kLong>(P), c.b, pol_keep);
+          }
+          __syncwarp();
+          qr.next(slots);
+          ++nq;
         }
       }
-      // drain: every issued copy must have landed before the CTA's shared memory is released
-      // (an issued copy always completes, so these waits do not take the abort shortcut).
-      // The last fill of stage i is complete once its full barrier has left the phase of that fill.
-      for (int n = 0; n < nk; ++n) {
-        // walk the ring backwards from the slot before kr
-        int i2 = kr.i - 1 - n, ph = kr.phase;
-        if (i2 < 0) { i2 += SL::kStages; ph ^= 1; }
-        mbar_wait_issued(bar_kfull(i2), (uint32_t)ph, ctl);
-      }
-      for (int n = 0; n < qc; ++n) {
-        int i2 = qr.i - 1 - n, ph = qr.phase;
-        if (i2 < 0) { i2 += kQSlots; ph ^= 1; }
-        mbar_wait_issued(bar_qfull(i2), (uint32_t)ph, ctl);
-      }
+      c = nx;
+    }
+    // drain: every issued copy must have landed before the CTA's shared memory is released
+    // (an issued copy always completes, so these waits do not take the abort shortcut).
+    // The last fill of a stage is complete once its full barrier has left the phase of that fill.
+    for (int n = 0; n < min(pos, stages); ++n) {
+      // walk the ring backwards from the slot before kr
+      int i2 = kr.i - 1 - n, ph = kr.phase;
+      if (i2 < 0) { i2 += stages; ph ^= 1; }
+      mbar_wait_issued(bar_kfull(stage0 + i2), (uint32_t)ph, ctl);
+    }
+    for (int n = 0; n < min(nq, slots); ++n) {
+      int i2 = qr.i - 1 - n, ph = qr.phase;
+      if (i2 < 0) { i2 += slots; ph ^= 1; }
+      mbar_wait_issued(bar_qfull(slot0 + i2), (uint32_t)ph, ctl);
     }
   }
-  // (warp 3 has no role)
 
   // ---------------- teardown ----------------
   tc_fence_before();
@@ -1121,7 +1105,8 @@ bool encode_map(CUtensorMap* m, const void* base, int rank, const long long* dim
 struct FastPlan {
   int U, NT, RPU, grid, RT;
   int HPT, QT, CH;             // query heads per row tile, row tiles per KV head, row tiles per query head
-  long long total_runs, shift;
+  long long total_runs;
+  int lead;
   size_t off_partial, off_parts, off_acc, off_ovf, off_ref, off_total;
 };
 
@@ -1144,11 +1129,10 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   pl->RPU = (pl->NT + pl->RT - 1) / pl->RT;
   pl->total_runs = (long long)pl->U * pl->RPU;
   pl->grid = sms > 0 ? (int)(pl->total_runs < sms ? pl->total_runs : sms) : 1;
-  // pass 2 of a run starts once every CTA has been through the rest of the run's unit, at most
-  // ceil(RPU / grid) runs later, and through one run more, which covers the exchange (the pushed
-  // sums take two round trips to L2); the K rows of that many tiles are still in L2 then
-  const long long lag_runs = (pl->RPU + pl->grid - 1) / pl->grid + 1;
-  pl->shift = lag_runs * pl->RT + KVC_SCORE_LAG_TILES;
+  // Pass 2 of a run starts once every run of its unit has been through pass 1: at other CTAs these lie at most
+  // (grid + RPU - 2) / grid runs later in their order.  Pass 1 must be allowed that far ahead of pass 2 (or the CTAs
+  // would wait for each other), and no further: the rows in between should still be in L2 when pass 2 reads them.
+  pl->lead = (1 + (pl->grid + pl->RPU - 2) / pl->grid) * pl->RT;
   size_t off = 0;
   pl->off_partial = off; off += align_up((size_t)pl->total_runs * kRows * sizeof(float2));
   pl->off_acc = off; off += align_up((size_t)pl->U * kRows * sizeof(unsigned long long));
@@ -1230,7 +1214,7 @@ bool score_sm100_shape_ok(const Problem& P) {
   FastPlan pl;
   make_plan(P, 0, &pl);
   if ((long long)P.L * P.Bt * P.Hkv * pl.QT > (1 << 24)) return false;
-  if ((pl.total_runs + 4096) * pl.RT + pl.shift >= (1LL << 31)) return false;   // 32-bit sequence indices
+  if ((pl.total_runs + 8192) * pl.RT >= (1LL << 31)) return false;   // 32-bit sequence indices
   return true;
 }
 
@@ -1292,7 +1276,7 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
   fp.HPT = pl.HPT; fp.QT = pl.QT; fp.CH = pl.CH; fp.w = P.w;
   fp.N = P.N; fp.q_pos0 = P.q_pos0;
   fp.U = pl.U; fp.NT = pl.NT; fp.RPU = pl.RPU; fp.RT = pl.RT; fp.grid = pl.grid;
-  fp.total_runs = (unsigned int)pl.total_runs; fp.shift = (int)pl.shift;
+  fp.total_runs = (unsigned int)pl.total_runs; fp.lead = pl.lead;
   fp.step_u = pl.grid / pl.RPU; fp.step_j = pl.grid % pl.RPU;
   fp.step_q = fp.step_u % pl.QT;
   fp.step_h = (fp.step_u / pl.QT) % P.Hkv;
