@@ -531,6 +531,57 @@ __device__ __noinline__ float p2_generic_tile(uint32_t taddr, const float* neg_l
   return gacc;
 }
 
+// kC consecutive accumulator columns of this thread's TMEM lane, loaded.
+template <int kC>
+__device__ __forceinline__ void tc_ld_cols(uint32_t taddr, uint32_t (&r)[kC]) {
+  static_assert(kC == 8 || kC == 16 || kC == 32, "columns");
+  if constexpr (kC == 32) {
+    tc_ld32_nowait(taddr, r);
+    tc_wait_ld(r);
+  } else if constexpr (kC == 16) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+  } else {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr) : "memory");
+  }
+}
+
+// Pass 2, one token, max over a window of w <= 128 rows that is no power of two, on a tile no mask touches.  A query
+// head's columns are taken kC at a time (kC <= w, the largest of 8, 16, 32), the last kC ending with the head and
+// overlapping the ones before: a maximum does not mind.  (Column by column with a run-time count of the rows, as the
+// masked tiles still are, the scoring of the 8B shape at 16K takes 886 us with w = 24, 2071 with 49 and 4097 with 100; so it
+// takes 386, 649 and 1240.)  Returns the group aggregate before the division of the mean.
+template <int kC>
+__device__ __noinline__ float p2_odd_tile(uint32_t taddr, const float* neg_lse, int R, int w, float sl2e, bool gmax) {
+  float gacc = gmax ? -INFINITY : 0.f;
+#pragma unroll 1
+  for (int h0 = 0; h0 < R; h0 += w) {
+    float hacc = -INFINITY;
+#pragma unroll 1
+    for (int c = 0; c < w; c += kC) {
+      const int col = h0 + min(c, w - kC);
+      uint32_t r[kC];
+      tc_ld_cols<kC>(taddr + col, r);
+#pragma unroll
+      for (int i = 0; i < kC; i += 2)
+        hacc = max3(hacc, fmaf(__uint_as_float(r[i]), sl2e, neg_lse[col + i]),
+                    fmaf(__uint_as_float(r[i + 1]), sl2e, neg_lse[col + i + 1]));
+    }
+    const float s_task = ex2(hacc);
+    gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
+  }
+  return gacc;
+}
+
 // Pass 2, one token against the R rows of one query head that this row tile holds (windows longer
 // than 128 rows), with masking: rows below m_min do not see the token.  Returns the tile's part of
 // Eq. 14 for the token: the largest attention weight, or the sum of the weights, over these rows.
@@ -796,7 +847,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
           }
         }
         named_bar(1, 128);                             // everyone is done with the previous unit's values
-        neg_lse[trow] = (trow < rows_u) ? -lse : 0.f;
+        neg_lse[trow] = (trow < rows_u) ? -lse : -INFINITY;    // (a row that is not there never wins a maximum)
         named_bar(1, 128);
         ok = !__any_sync(0xffffffffu, ctl->abort != 0) && ok;
       }
@@ -817,9 +868,11 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       const int c = tok0 + trow;                                     // this thread's token
       const bool full = tok0 + kTile - 1 <= vis_all_i;
       float gacc;
-      if (!kTaskMean && W >= 32 && full) {
-        // the paper's default (max over the window) on a tile no mask touches: every 32-column
-        // chunk belongs to one query head
+      if (!kTaskMean && full && (W > 0 || P.CH > 1)) {
+        // the paper's default (max over the window) on a tile no mask touches: every 32-column chunk belongs to
+        // one query head, or holds whole query heads (W = 8, 16); a row tile of a window longer than 128 rows
+        // belongs to one head throughout (a window of 500 rows at 4K: 1849 -> 1036 us for the scoring against the
+        // column-by-column loop of the masked tiles)
         gacc = gmax ? -INFINITY : 0.f;
         float hacc = -INFINITY;
         uint32_t r[32];
@@ -848,12 +901,26 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty(buf));
           }
+          if (W == 8 || W == 16) {
+            constexpr int kW = W > 0 ? W : 32;
+#pragma unroll
+            for (int h0 = 0; h0 < 32; h0 += kW) {
+              float a = fmaxf(x[h0], x[h0 + 1]);
+#pragma unroll
+              for (int i = 2; i < kW; i += 2) a = max3(a, x[h0 + i], x[h0 + i + 1]);
+              if (j * 32 + h0 < rows_u) {
+                const float s_task = ex2(a);
+                gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
+              }
+            }
+            return;
+          }
           float a = x[0], b = x[1];
 #pragma unroll
           for (int i = 2; i < 30; i += 4) { a = max3(a, x[i], x[i + 1]); b = max3(b, x[i + 2], x[i + 3]); }
           hacc = max3(hacc, a, b);
           hacc = max3(hacc, x[30], x[31]);
-          if (((j + 1) * 32) % (W > 0 ? W : 1) == 0) {
+          if (W > 0 && ((j + 1) * 32) % (W > 0 ? W : 1) == 0) {
             const float s_task = ex2(hacc);
             gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
             hacc = -INFINITY;
@@ -861,6 +928,14 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         };
 #pragma unroll 1
         for (int j = 0; j < n_chunks; ++j) chunk(j, j + 1 == n_chunks);
+        if (W == 0) gacc = ex2(hacc);                                  // the head's maximum over these rows
+      } else if (!kTaskMean && W == 0 && full && P.w >= 8) {
+        gacc = P.w >= 32 ? p2_odd_tile<32>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
+             : P.w >= 16 ? p2_odd_tile<16>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
+                         : p2_odd_tile<8>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tempty(buf));
       } else if (W == 0 && P.CH > 1) {
         // a window longer than 128 rows: the tile holds rows row0 .. of one query head and yields
         // that head's partial Eq. 14 (the maximum, or the sum, over these rows)

@@ -35,3 +35,19 @@ def test_value_norms_at_tile_edges(dtype, d, N):
             ref = oracle.score_layer_vnorm(Pz.to_f32_numpy(wl.q[l][b]), Pz.to_f32_numpy(wl.k[l][b]), Pz.to_f32_numpy(wl.v[l][b]),
                                            1.0 / np.sqrt(d), desc.q_pos0, desc.agg_task, desc.agg_group, bool(desc.augment_head_mean))
             Pz.assert_scores_close(S[l, b], ref)
+
+
+@pytest.mark.parametrize("Hq,Hkv,w,agg_group", [
+    (4, 2, 8, 1), (6, 2, 16, 0),        # whole heads inside a 32-column chunk, the last of them not there
+    (8, 2, 9, 1), (8, 2, 31, 0),        # columns taken 8 and 16 at a time, the last ones overlapping
+    (14, 2, 33, 1), (4, 2, 127, 0),     # ... and 32 at a time; row tiles of three heads and of one
+    (2, 1, 129, 1), (4, 2, 256, 0),     # row tiles of 128 rows and one row; of exactly 128
+])
+def test_max_over_windows_of_any_length(Hq, Hkv, w, agg_group):
+    """Pass 2 on tiles no mask touches: every way a tile's columns are split into query heads."""
+    cfg = W.WorkloadConfig("windows", 2, Hq, Hkv, 128, 700, w, dtype="bf16", elem_std=1.0, hh_frac=0.01)
+    dev, wl, desc = _setup(cfg, agg_group=agg_group, q_pos0=700)
+    out = alloc_outputs(desc, 1, wl.k[0].dtype, dev)
+    kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
+    torch.cuda.synchronize()
+    Pz.assert_scores_close(out.scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
