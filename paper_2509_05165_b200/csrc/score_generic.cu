@@ -1,7 +1,8 @@
 // Token-importance scoring on the CUDA cores (Eqs. 3, 14-16).
 //
 // This is the shape-agnostic path: fp32 or bf16 inputs, head_dim 64 or 128, any window length,
-// any GQA map.  It makes two sweeps over K.  Sweep 1 produces, for every query row, the
+// any GQA map.  Where the logits of a (layer, sequence, KV head) fit a bounded buffer they are computed once and kept
+// (second part of this file); otherwise it makes two sweeps over K.  Sweep 1 produces, for every query row, the
 // log-sum-exp of its logits over the visible keys (per-chunk partials, then a combine kernel).
 // Sweep 2 recomputes the logits and emits exp(s - lse) -- the softmax weight of Eq. 3 -- reduced
 // over the window rows (Eq. 14) and over the query heads of the KV head (Eq. 15).  A last kernel
@@ -239,6 +240,306 @@ score_emit_kernel(ScoreParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp,
   if (valid) s_group[((long long)lb * P.Hkv + h) * P.N + c] = gacc;
 }
 
+// ---- one product, its logits kept -----------------------------------------------------------------
+// The sweeps above compute every logit twice, and one token per thread makes them wait for the broadcast reads of
+// Q (a 16-byte read per four multiplications and thread).  Where the logits of a (layer, sequence, KV head) fit the
+// workspace, they are computed once, by a register-tiled product, and kept in a buffer of at most kLogitsCap bytes;
+// the statistics and the emission then read them.  Units are taken in groups that fill the buffer.  Every sum is
+// taken in the order of the sweeps (four partial products per logit, the butterfly over 32 tokens, 8 such steps per
+// warp and chunk), so the scores are the same bit for bit.  fp32, 16 layers, N = 3001, 32 / 8 heads of 128, w = 32:
+// 1342 us for the two sweeps, 424 us so (the product 335; it cannot take less than 175: 128 multiply-adds a clock and
+// SM).  A larger buffer (96 MB) gains 1 %, smaller ones mean more and shorter launches.
+constexpr int kTileTok = 128, kTileRow = 128, kLogitThreads = 256;
+constexpr size_t kLogitsCap = (size_t)64 << 20;
+constexpr int kMaxLogitChunks = 1024;           // the statistics of a row's chunks meet in shared memory
+
+struct LogitParams {
+  int Bt, Hkv, w, max_rows;                     // max_rows: of a unit (the largest group's)
+  long long N, np, q_pos0;                      // np: row stride of the buffer
+  long long qs0, qs1, qs2, kvs0, kvs1, kvs2;
+  float scale_log2e;
+  int agg_task, agg_group, nchunks, unit0;      // unit0: first unit of the group
+};
+
+// Two fp32 lanes in one 64-bit register: d = a * b + c in both.
+__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float2 unpack_f2(unsigned long long p) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
+  return r;
+}
+// Four elements of a row to four floats in shared memory: asynchronously, or through registers where they are converted.
+__device__ __forceinline__ void stage4(float* dst, const float* row, int v) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(row + 4 * v) : "memory");
+}
+__device__ __forceinline__ void stage4(float* dst, const __nv_bfloat16* row, int v) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(row) + v);
+  *reinterpret_cast<float4*>(dst) = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                                                __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+}
+
+// dots[unit - unit0][row][token] = <q row, k token>.  Work items are (unit, 128 rows, 128 tokens), tokens fastest, dealt
+// to the CTAs in even stretches, so that a CTA keeps its Q rows and streams K tiles through two buffers.  8 x 8 logits
+// per thread; the four partial products of a logit are taken two at a time (a packed pair), in two sweeps over the
+// tile.  Bound by the multiply-adds (128 clocks of a scheduler per warp and step of two elements); the operand reads
+// are what a smaller register tile would wait for: an 8-byte read costs the SM 2 clocks where neighbouring lanes read
+// different addresses (the 8 tokens) and 1 where they share one (the 8 rows), 96 for four warps' steps.  (4 x 4 logits
+// with all four products at once: 423 us in the case above.)  Rows are padded by 16 bytes to spread a read over the banks.
+template <typename T, int D>
+__global__ void __launch_bounds__(kLogitThreads, 1)
+score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, float* __restrict__ dots, int row_tiles,
+                    int tok_tiles, int items) {
+  constexpr int kPitch = D + 4, kVec = D / 4;
+  extern __shared__ __align__(16) float gsm[];
+  float* const Qs = gsm;
+  float* const Ks = gsm + kTileRow * kPitch;                   // two buffers
+  grid_dependency_wait();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tok = (warp & 1) * 64 + (lane & 7);               // tokens tok + 8 i
+  const int row = (warp >> 1) * 32 + (lane >> 3);             // rows row + 4 j
+  const int i0 = (int)((long long)items * blockIdx.x / gridDim.x), i1 = (int)((long long)items * (blockIdx.x + 1) / gridDim.x);
+  auto load_k = [&](int item, float* dst) {
+    const int ur = item / tok_tiles, tt = item - ur * tok_tiles;
+    const int unit = P.unit0 + ur / row_tiles;
+    const int h = unit % P.Hkv, lb = unit / P.Hkv;
+    const T* base = reinterpret_cast<const T*>(kp.p[lb / P.Bt]) + (lb % P.Bt) * P.kvs0 + h * P.kvs1;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < kTileTok * kVec; i += kLogitThreads) {
+      const int t = i / kVec, v = i % kVec;
+      stage4(dst + t * kPitch + 4 * v, base + min((long long)tt * kTileTok + t, P.N - 1) * P.kvs2, v);
+    }
+  };
+  if (i0 < i1) load_k(i0, Ks);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  int cur = -1, rows = 0, r0 = 0;                              // the (unit, rows) whose Q is here
+  for (int item = i0; item < i1; ++item) {
+    float* const buf = Ks + ((item - i0) & 1) * (kTileTok * kPitch);
+    const int ur = item / tok_tiles, tt = item - ur * tok_tiles;
+    if (ur != cur) {
+      cur = ur;
+      const int unit = P.unit0 + ur / row_tiles;
+      const int h = unit % P.Hkv, lb = unit / P.Hkv;
+      rows = (gm.begin[h + 1] - gm.begin[h]) * P.w;
+      r0 = (ur % row_tiles) * kTileRow;
+      const T* base = reinterpret_cast<const T*>(qp.p[lb / P.Bt]) + (lb % P.Bt) * P.qs0;
+#pragma unroll 4
+      for (int i = threadIdx.x; i < kTileRow * kVec; i += kLogitThreads) {
+        const int rr = min(r0 + i / kVec, rows - 1), v = i % kVec;
+        const int j = gm.qh[gm.begin[h] + rr / P.w];
+        stage4(Qs + (i / kVec) * kPitch + 4 * v, base + j * P.qs1 + (long long)(rr % P.w) * P.qs2, v);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if (item + 1 < i1) load_k(item + 1, Ks + ((item + 1 - i0) & 1) * (kTileTok * kPitch));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");       // all but the next item's tile
+    __syncthreads();
+    if (r0 + (warp >> 1) * 32 < rows) {
+      const float* kq = buf + tok * kPitch;
+      const float* qq = Qs + row * kPitch;
+      unsigned long long acc[8][8];                            // [token][row]: two partial products
+      float first[8][8];                                       // the sum of the first two
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+#pragma unroll 4
+        for (int v = 0; v < kVec; ++v) {
+          unsigned long long kv[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) kv[i] = *reinterpret_cast<const unsigned long long*>(kq + i * 8 * kPitch + 4 * v + 2 * half);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const unsigned long long qv = *reinterpret_cast<const unsigned long long*>(qq + j * 4 * kPitch + 4 * v + 2 * half);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i][j] = ffma2(qv, kv[i], acc[i][j]);
+          }
+        }
+        if (half == 0) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { const float2 x = unpack_f2(acc[i][j]); first[i][j] = x.x + x.y; }
+        }
+      }
+      const long long t0 = (long long)tt * kTileTok + tok;
+      float* out = dots + ((long long)(ur / row_tiles) * P.max_rows + r0 + row) * P.np + t0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (r0 + row + 4 * j < rows) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float2 y = unpack_f2(acc[i][j]);
+            if (t0 + 8 * i < P.N) out[(long long)(4 * j) * P.np + 8 * i] = first[i][j] + (y.x + y.y);
+          }
+        }
+      }
+    }
+    __syncthreads();                                           // this tile and these Q rows have been read
+  }
+}
+
+// The log-sum-exp (base 2) of four rows of a unit.  Eight lanes per row; a warp takes 8 steps of 32 tokens, 128 apart,
+// as a warp of score_stats_kernel does; the four "warps" of a chunk and then the chunks are folded as there.
+constexpr int kRowStatWarps = 4;
+__global__ void __launch_bounds__(kRowStatWarps * 32)
+score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dots, float* __restrict__ lse2) {
+  extern __shared__ float2 st_sm[];                            // [4 * nchunks][4 rows]
+  grid_dependency_wait();
+  const int unit = P.unit0 + blockIdx.y;
+  const int h = unit % P.Hkv;
+  const int rows = (gm.begin[h + 1] - gm.begin[h]) * P.w;
+  const int r0 = blockIdx.x * 4;
+  if (r0 >= rows) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 7, rl = lane >> 3;
+  const int r = min(r0 + rl, rows - 1);
+  const float* src = dots + ((long long)blockIdx.y * P.max_rows + r) * P.np;
+  const long long vis = min(P.N - 1, P.q_pos0 + r % P.w);      // the last token the row sees
+  for (int p = warp; p < 4 * P.nchunks; p += kRowStatWarps) {
+    const long long base = (long long)(p >> 2) * (kChunkIters * kThreads) + (p & 3) * 32 + sub;
+    const float* at = src + base;
+    float s[kChunkIters][4];
+    if (base + (kChunkIters - 1) * kThreads + 24 <= vis) {     // all of them are there and seen
+#pragma unroll
+      for (int it = 0; it < kChunkIters; ++it)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[it][i] = __ldg(at + it * kThreads + 8 * i);
+#pragma unroll
+      for (int it = 0; it < kChunkIters; ++it)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[it][i] = s[it][i] * P.scale_log2e;
+    } else {
+      const int left = (int)max(-1LL, min(vis - base, (long long)kChunkIters * kThreads));   // offsets up to here count
+#pragma unroll
+      for (int it = 0; it < kChunkIters; ++it)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          s[it][i] = it * kThreads + 8 * i <= left ? __ldg(at + it * kThreads + 8 * i) * P.scale_log2e : -INFINITY;
+    }
+    float m = -INFINITY, lsum = 0.f;
+#pragma unroll
+    for (int it = 0; it < kChunkIters; ++it) {
+      float m_w = fmaxf(fmaxf(s[it][0], s[it][1]), fmaxf(s[it][2], s[it][3]));
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) m_w = fmaxf(m_w, __shfl_xor_sync(0xffffffffu, m_w, o));
+      const float m_new = fmaxf(m, m_w);
+      float e[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) e[i] = (m_new == -INFINITY) ? 0.f : exp2f(s[it][i] - m_new);
+      float l_w = (e[0] + e[2]) + (e[1] + e[3]);               // distances 16 and 8 of the butterfly
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) l_w += __shfl_xor_sync(0xffffffffu, l_w, o);
+      if (m_new > -INFINITY) {
+        lsum = lsum * exp2f(m - m_new) + l_w;
+        m = m_new;
+      }
+    }
+    if (sub == 0) st_sm[p * 4 + rl] = make_float2(m, lsum);
+  }
+  __syncthreads();
+  // per chunk: the four warps' statistics
+  for (int i = threadIdx.x; i < P.nchunks * 4; i += kRowStatWarps * 32) {
+    const int ch = i >> 2, rr = i & 3;
+    float M = -INFINITY;
+#pragma unroll
+    for (int wv = 0; wv < 4; ++wv) M = fmaxf(M, st_sm[(ch * 4 + wv) * 4 + rr].x);
+    float Lsum = 0.f;
+    if (M > -INFINITY) {
+#pragma unroll
+      for (int wv = 0; wv < 4; ++wv) {
+        const float2 v = st_sm[(ch * 4 + wv) * 4 + rr];
+        Lsum += v.y * exp2f(v.x - M);
+      }
+    }
+    st_sm[ch * 16 + rr] = make_float2(M, Lsum);                // (read by nobody else: slot wv = 0 of this chunk and row)
+  }
+  __syncthreads();
+  if (threadIdx.x < 4 && r0 + threadIdx.x < rows) {
+    float M = -INFINITY;
+    for (int i = 0; i < P.nchunks; ++i) M = fmaxf(M, st_sm[i * 16 + threadIdx.x].x);
+    float Lsum = 0.f;
+    for (int i = 0; i < P.nchunks; ++i) {
+      const float2 v = st_sm[i * 16 + threadIdx.x];
+      if (v.x > -INFINITY) Lsum += v.y * exp2f(v.x - M);
+    }
+    lse2[(long long)blockIdx.y * P.max_rows + r0 + threadIdx.x] = M + log2f(Lsum);
+  }
+}
+
+// Eqs. 14-15 from the kept logits: four tokens per thread, 16 rows in flight.  kMean: agg_task is the mean.
+template <bool kMean>
+__global__ void __launch_bounds__(kThreads)
+score_emit_logits_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dots, const float* __restrict__ lse2,
+                         float* __restrict__ s_group) {
+  __shared__ float neg_lse[kThreads];
+  grid_dependency_wait();
+  const int unit = P.unit0 + blockIdx.y;
+  const int h = unit % P.Hkv;
+  const long long c = ((long long)blockIdx.x * kThreads + threadIdx.x) * 4;
+  const int members = gm.begin[h + 1] - gm.begin[h];
+  // (a thread behind the end reads the last four tokens again)
+  const float4* src = reinterpret_cast<const float4*>(dots + (long long)blockIdx.y * P.max_rows * P.np + min(c, P.np - 4));
+  const float* lse = lse2 + (long long)blockIdx.y * P.max_rows;
+  const long long step = P.np / 4;
+  const int all_from = (int)min((long long)P.w, max(0LL, c + 3 - P.q_pos0));      // window rows from here on see all four tokens
+  float gacc[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) gacc[e] = (P.agg_group == KVC_AGG_MAX) ? -INFINITY : 0.f;
+  for (int mi = 0; mi < members; ++mi) {
+    float tacc[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tacc[e] = kMean ? 0.f : -INFINITY;
+    for (int r0 = 0; r0 < P.w; r0 += kThreads) {
+      const int nr = min(kThreads, P.w - r0);
+      __syncthreads();
+      if (threadIdx.x < nr) neg_lse[threadIdx.x] = -__ldg(lse + threadIdx.x);
+      __syncthreads();
+      auto row = [&](const float4 d, const int r, const bool masked) {
+        const float nl = neg_lse[r];
+        const float dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float t = fmaf(dv[e], P.scale_log2e, nl);              // log2 of the attention weight
+          if (masked && c + e > P.q_pos0 + r0 + r) t = -INFINITY;
+          if (kMean) tacc[e] += exp2f(t); else tacc[e] = fmaxf(tacc[e], t);
+        }
+      };
+      int r = 0;
+      for (; r + 16 <= nr; r += 16) {
+        float4 d[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) d[i] = __ldg(src + i * step);
+        src += 16 * step;
+        if (r0 + r >= all_from) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) row(d[i], r + i, false);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) row(d[i], r + i, true);
+        }
+      }
+      for (; r < nr; ++r) { row(__ldg(src), r, true); src += step; }
+      lse += nr;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float s_task = kMean ? tacc[e] / (float)P.w : exp2f(tacc[e]);
+      gacc[e] = (P.agg_group == KVC_AGG_MAX) ? fmaxf(gacc[e], s_task) : gacc[e] + s_task;
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if (P.agg_group == KVC_AGG_MEAN) gacc[e] /= (float)members;
+    if (c + e < P.N) s_group[(long long)unit * P.N + c + e] = gacc[e];
+  }
+}
+
 // Eq. 16: S[h, c] = S_group[h, c] + (1/Hkv) sum_i S_group[i, c], in place.  With row tiles, first
 // Eq. 15 from the tiles' partial aggregates (sum or max over the tile's query heads), in tile order.
 // With vnorm (App. A.1.3), the group aggregate is multiplied by the token's value norm before Eq. 16.
@@ -330,6 +631,74 @@ kvc_status run(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const L
   return KVC_OK;
 }
 
+// How the units are cut into groups whose logits fit the buffer; units_per_group = 0: one unit alone does not fit (or the
+// problem belongs to the tensor cores and gets here only when its strides do not suit them): the two sweeps.
+struct LogitPlan {
+  long long np, units;
+  int max_rows, units_per_group;
+  size_t dots_bytes, lse_bytes;
+};
+LogitPlan logit_plan(const Problem& P) {
+  LogitPlan p;
+  p.np = (P.N + 3) / 4 * 4;
+  p.units = (long long)P.L * P.Bt * P.Hkv;
+  const long long rows = (long long)P.max_group * P.w;
+  const long long unit_bytes = rows * p.np * (long long)sizeof(float);
+  const long long nchunks = (P.N + kChunkIters * kThreads - 1) / (kChunkIters * kThreads);
+  p.max_rows = (int)rows;
+  p.units_per_group = 0;
+  p.dots_bytes = p.lse_bytes = 0;
+  if (unit_bytes > (long long)kLogitsCap || nchunks > kMaxLogitChunks || score_sm100_shape_ok(P)) return p;
+  const long long per = (long long)kLogitsCap / unit_bytes < 65535 ? (long long)kLogitsCap / unit_bytes : 65535;
+  const long long groups = (p.units + per - 1) / per;
+  p.units_per_group = (int)((p.units + groups - 1) / groups);   // groups of even size
+  p.dots_bytes = align_up((size_t)p.units_per_group * unit_bytes);
+  p.lse_bytes = align_up((size_t)p.units_per_group * rows * sizeof(float));
+  return p;
+}
+
+template <typename T, int D>
+kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
+                      const LogitPlan& pl, char* ws, cudaStream_t st) {
+  constexpr int kSmem = (2 * kTileTok + kTileRow) * (D + 4) * (int)sizeof(float);
+  KVC_CUDA(cudaFuncSetAttribute(score_logits_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+  int dev = 0, sms = 0;
+  KVC_CUDA(cudaGetDevice(&dev));
+  KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int row_tiles = (pl.max_rows + kTileRow - 1) / kTileRow;
+  const int tok_tiles = (int)((P.N + kTileTok - 1) / kTileTok);
+  LogitParams lp;
+  lp.Bt = P.Bt; lp.Hkv = P.Hkv; lp.w = P.w; lp.max_rows = pl.max_rows;
+  lp.N = P.N; lp.np = pl.np; lp.q_pos0 = P.q_pos0;
+  lp.qs0 = P.qs[0]; lp.qs1 = P.qs[1]; lp.qs2 = P.qs[2];
+  lp.kvs0 = P.kvs[0]; lp.kvs1 = P.kvs[1]; lp.kvs2 = P.kvs[2];
+  lp.scale_log2e = P.scale * kLog2e;
+  lp.agg_task = P.agg_task; lp.agg_group = P.agg_group;
+  lp.nchunks = (int)((P.N + kChunkIters * kThreads - 1) / (kChunkIters * kThreads));
+  const size_t stat_smem = (size_t)lp.nchunks * 16 * sizeof(float2);
+  if (stat_smem > 48 * 1024)
+    KVC_CUDA(cudaFuncSetAttribute(score_row_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kMaxLogitChunks * 16 * (int)sizeof(float2)));
+  float* dots = reinterpret_cast<float*>(ws);
+  float* lse2 = reinterpret_cast<float*>(ws + pl.dots_bytes);
+  for (long long u0 = 0; u0 < pl.units; u0 += pl.units_per_group) {
+    const unsigned n = (unsigned)(pl.units - u0 < pl.units_per_group ? pl.units - u0 : pl.units_per_group);
+    lp.unit0 = (int)u0;
+    const long long items = (long long)n * row_tiles * tok_tiles;
+    KVC_CUDA(launch_dependent(score_logits_kernel<T, D>, dim3((unsigned)(items < sms ? items : sms)), dim3(kLogitThreads),
+                              (size_t)kSmem, st, lp, gm, q, k, dots, row_tiles, tok_tiles, (int)items));
+    KVC_LAUNCH_CHECK("score_logits_kernel");
+    KVC_CUDA(launch_dependent(score_row_stats_kernel, dim3((unsigned)((pl.max_rows + 3) / 4), n), dim3(kRowStatWarps * 32),
+                              stat_smem, st, lp, gm, (const float*)dots, lse2));
+    KVC_LAUNCH_CHECK("score_row_stats_kernel");
+    KVC_CUDA(launch_dependent(P.agg_task == KVC_AGG_MEAN ? score_emit_logits_kernel<true> : score_emit_logits_kernel<false>,
+                              dim3((unsigned)((P.N + 4 * kThreads - 1) / (4 * kThreads)), n), dim3(kThreads), 0, st, lp, gm,
+                              (const float*)dots, (const float*)lse2, scores));
+    KVC_LAUNCH_CHECK("score_emit_logits_kernel");
+  }
+  return KVC_OK;
+}
+
 }  // namespace
 
 static int generic_nchunks(const Problem& P) {
@@ -338,6 +707,8 @@ static int generic_nchunks(const Problem& P) {
 }
 
 size_t score_generic_workspace_bytes(const Problem& P) {
+  const LogitPlan pl = logit_plan(P);
+  if (pl.units_per_group > 0) return pl.dots_bytes + pl.lse_bytes;
   const size_t rows = (size_t)P.L * P.Bt * P.Hq * P.w;
   return align_up(rows * generic_nchunks(P) * sizeof(float2)) + align_up(rows * sizeof(float));
 }
@@ -359,6 +730,18 @@ kvc_status launch_score_generic(const Problem& P, const GroupMap& gm, const Laye
   if (ws_bytes < score_generic_workspace_bytes(P)) {
     set_error("score: workspace too small");
     return KVC_ERR_WORKSPACE;
+  }
+  const LogitPlan pl = logit_plan(P);
+  if (pl.units_per_group > 0) {
+    char* w = reinterpret_cast<char*>(ws);
+    kvc_status r;
+    if (P.dtype == KVC_BF16)
+      r = P.d == 64 ? run_logits<__nv_bfloat16, 64>(P, gm, q, k, scores, pl, w, st)
+                    : run_logits<__nv_bfloat16, 128>(P, gm, q, k, scores, pl, w, st);
+    else
+      r = P.d == 64 ? run_logits<float, 64>(P, gm, q, k, scores, pl, w, st) : run_logits<float, 128>(P, gm, q, k, scores, pl, w, st);
+    if (r != KVC_OK) return r;
+    return launch_score_augment(P, scores, nullptr, 1, 1, vnorm, st);
   }
   const size_t rows = (size_t)P.L * P.Bt * P.Hq * P.w;
   const int nchunks = generic_nchunks(P);

@@ -51,3 +51,27 @@ def test_max_over_windows_of_any_length(Hq, Hkv, w, agg_group):
     kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
     torch.cuda.synchronize()
     Pz.assert_scores_close(out.scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
+
+
+@pytest.mark.parametrize("dtype,Hq,Hkv,w,N,agg_task,explicit", [
+    ("f32", 2, 2, 1, 129, 0, False),       # one row per unit; one token more than a tile
+    ("f32", 6, 2, 43, 1027, 1, False),     # 129 rows: a second row tile of one row; three tokens into the second chunk
+    ("f32", 8, 2, 600, 4100, 0, False),    # a unit's logits fill most of the buffer: one unit per group
+    ("f32", 8, 1, 600, 4100, 0, False),    # ... and do not fit it: the two sweeps
+    ("bf16", 5, 2, 40, 333, 0, True),      # uneven groups, converted operands
+])
+def test_scoring_on_the_cuda_cores(dtype, Hq, Hkv, w, N, agg_task, explicit):
+    import ctypes
+    heads = Hq if explicit else Hkv       # (the generator draws equal groups)
+    cfg = W.WorkloadConfig("generic", 1, Hq, heads, 64, N, w, dtype=dtype, elem_std=1.0, hh_frac=0.0)
+    dev, wl, desc = _setup(cfg, agg_task=agg_task)
+    if explicit:
+        wl = W.Workload(cfg, wl.q, [t[:, :Hkv].contiguous() for t in wl.k], [t[:, :Hkv].contiguous() for t in wl.v])
+        desc = kvc.kvc_desc_init(1, 1, Hq, Hkv, 64, N, w, kvc.BF16)
+        members = (ctypes.c_int32 * Hq)(0, 1, 0, 0, 0)
+        desc.q_to_kv = ctypes.cast(members, ctypes.POINTER(ctypes.c_int32))
+    out = alloc_outputs(desc, 1, wl.k[0].dtype, dev)
+    kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
+    torch.cuda.synchronize()
+    assert not kvc.kvc_score_uses_tensor_cores(desc)
+    Pz.assert_scores_close(out.scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
