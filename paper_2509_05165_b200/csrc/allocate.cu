@@ -6,15 +6,14 @@
 //   N_l = #{k : I[l, k] > T}  +  (a share of the entries equal to T, handed out in layer order
 //                                 until the budget is met -- the total order (I desc, l asc, k asc)).
 // Two ways to T, both over the 32-bit order-preserving keys:
-//   * pools of up to 128 rows: one kernel, one CTA per sequence, which only ever looks at a few
+//   * pools of up to 256 rows: one kernel, one CTA per sequence, which only ever looks at a few
 //     thousand entries.  Every row keeps a window of positions that must hold its boundary; per
-//     round the CTA samples each window at equal distances, sorts the samples with their block
-//     sizes as weights, and the weighted ranks bracket T between two sample values, which cuts
-//     every window to the blocks between them (about a sixteenth per round).  A value with so many
-//     copies that the windows stop shrinking is located exactly in every row (32-way searches) and
-//     either is T or leaves the windows; when at most 1024 entries are left they are sorted and T
-//     is read off.  The rounds are bounded; past the bound T is found by bisection over the key
-//     range with exact counts.
+//     round the CTA samples each window at equal distances, and the samples' weighted ranks (their
+//     block sizes as weights) bracket T between two sample values, which cuts every window to the
+//     blocks between them.  A value with so many copies that the windows stop shrinking is located
+//     exactly in every row (32-way searches) and either is T or leaves the windows; when at most
+//     2048 entries are left T is read off them.  The rounds are bounded; past the bound T is found
+//     by bisection over the key range with exact counts.
 //   * larger pools: a most-significant-digit radix select -- four histogram passes over the pool
 //     (each CTA re-derives the prefix chosen so far from the previous passes' global histograms),
 //     then one small kernel does the per-row searches and the tie hand-out.
@@ -238,94 +237,117 @@ select_finish_kernel(const float* __restrict__ composite,
 
 // ------------------------------------------------------------------------------------------------
 // Selection on the sorted rows themselves: one CTA per sequence, no scratch in global memory.
+//
+// Bound by latency and by the instructions of one CTA: a round is one round trip to L2 for the samples and a few
+// block-wide steps on them.  It takes four samples per thread (64 per row for up to 32 rows, 8 for 256) and finds the
+// two bracketing sample values by a weighted radix select: a histogram of the block sizes over 2048 equal steps of the
+// samples' key range, a scan, and again inside the bracketing bins while these still hold more than a 128th of the
+// windows.  (Sorting 1024 samples took 4300 of a round's 9000 clocks and the last step's sort 8000: the kernel takes
+// 12.7 us on 32 rows of 32768 where that took 20.2, 10.8 on 32 rows of 1000 where it took 15.5, and 25 on
+// 256 rows of 8192 where the six launches of the histogram passes took 72.  With 1024 threads a round is longer, 5200
+// clocks for a level of the select alone: all warps issue the same instructions, half of them for samples not needed.)
 // ------------------------------------------------------------------------------------------------
-constexpr int kSelThreads = 1024;
-constexpr int kSelMaxRows = 128;          // rows of a pool this kernel takes (fewer samples per row as the rows grow)
+constexpr int kSelThreads = 512;
+constexpr int kSelItems = 4;              // samples (or, in the last step, entries) per thread
+constexpr int kSelMaxRows = 256;          // rows of a pool this kernel takes (fewer samples per row as the rows grow)
+constexpr int kSelBits = 11;              // a level of the select; three make up a key
+constexpr int kSelBins = 1 << kSelBits;   // four per thread
 constexpr int kSelDefaultRounds = 40;     // sampling rounds and exact steps together, before the bisection takes over
 
 struct SelectShared {
-  uint32_t sortbuf[2][kSelThreads];             // exchange buffers of the sort
-  unsigned long long pref[kSelThreads];         // weighted inclusive ranks, in sorted order
-  long long wt[kSelThreads];                    // block size behind every sample
-  uint32_t skey[kSelThreads];                   // the samples' shortened keys in sorted order
-  uint32_t fkey[kSelThreads];                   // the samples' keys
-  long long lo[kSelMaxRows], hi[kSelMaxRows];   // the rows' windows: positions < lo are better than T, >= hi worse
-  long long gt[kSelMaxRows], ge[kSelMaxRows];   // the answer: entries better than T, and at least as good
-  long long off[kSelMaxRows + 1];               // running sum of the window lengths (last step)
-  long long row_a[kSelMaxRows], row_b[kSelMaxRows];   // per-row terms of the sums below
-  int clt[kSelMaxRows], cle[kSelMaxRows];
-  unsigned long long warp_tot[32];
-  long long rank, width;                        // T is the rank-th best entry inside the windows (1-based); their total length
-  long long slack, new_width;
+  uint32_t hist[kSelBins];                      // block sizes of the samples per bin
+  int lo[kSelMaxRows], hi[kSelMaxRows];         // the rows' windows: positions < lo are better than T, >= hi worse
+  int gt[kSelMaxRows], ge[kSelMaxRows];         // the answer: entries better than T, and at least as good
+  int off[kSelMaxRows + 1];                     // running sum of the window lengths (last step)
+  int clt[kSelMaxRows], cle[kSelMaxRows];       // entries better than T, at least as good, in the windows (last step)
+  uint32_t warp_tot[kSelThreads / 32];
   unsigned long long tot_lt, tot_le;
-  uint32_t khi, khi_key;                        // upper bracket: shortened key, and the key of the sample it came from
+  uint32_t bin[2], below[2], weight[2];         // of a level: the bin a target falls into, what lies before it, what is in it
+  uint32_t rank, width;                         // T is the rank-th best entry inside the windows (1-based); their total length
+  uint32_t slack, taken, new_width;
   uint32_t kmin, kmax;                          // range of the round's sample keys
-  int ilo;
 };
 
-// Bitonic sort of 1024 32-bit values, one per thread; returns the value of rank threadIdx.x (ascending).
-// K0 = 2 for any input; K0 = 2 m when the values arrive as runs of m neighbours that are already
-// sorted, ascending where (threadIdx.x & m) == 0 and descending elsewhere: the stages that would
-// build such runs are left out.  Exchanges closer than a warp go through shuffles, the others
-// through shared memory (two buffers in turn: one barrier per step).  Fully unrolled: every
-// step's partner and direction are constants.
-template <int K0>
-__device__ __forceinline__ uint32_t block_sort(uint32_t v, SelectShared& sh) {
-  const int i = threadIdx.x;
-  int which = 0;
-#pragma unroll
-  for (int k = K0; k <= kSelThreads; k <<= 1) {
-    const bool asc = (i & k) == 0;
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      uint32_t other;
-      if (j >= 32) {
-        sh.sortbuf[which][i] = v;
-        __syncthreads();
-        other = sh.sortbuf[which][i ^ j];
-        which ^= 1;
-      } else {
-        other = __shfl_xor_sync(0xffffffffu, v, j);
-      }
-      const bool take_min = ((i & j) == 0) == asc;
-      if ((other < v) == take_min) v = other;
-    }
-  }
-  return v;
-}
-
 // Inclusive sum over the block in thread order.
-__device__ inline unsigned long long block_scan(unsigned long long v, SelectShared& sh) {
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, SelectShared& sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long n = __shfl_up_sync(0xffffffffu, v, o);
+    const uint32_t n = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += n;
   }
-  if (lane == 31) sh.warp_tot[warp] = v;    // (last read before the barriers of the sort that precedes every scan)
+  if (lane == 31) sh.warp_tot[warp] = v;        // (the previous scan's totals were read before the caller's last barrier)
   __syncthreads();
-  if (warp == 0) {
-    const unsigned long long t = sh.warp_tot[lane];
-    unsigned long long incl = t;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long n = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += n;
-    }
-    sh.warp_tot[lane] = incl - t;
-  }
-  __syncthreads();
-  return v + sh.warp_tot[warp];
+  return v + __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp_tot[lane] : 0u);
 }
 
-// Sum of a per-row array (kSelMaxRows entries, zeros beyond the rows in use); call with the whole first warp.
-__device__ inline long long warp_sum_rows(const long long* a) {
-  const int lane = threadIdx.x & 31;
-  long long v = a[lane] + a[lane + 32] + a[lane + 64] + a[lane + 96];
+// A bracket being narrowed: the keys base .. base + 2^bits - 1 hold the target-th unit of weight (1-based), `target`
+// counted from base on.
+struct Bracket {
+  uint32_t base, target;
+  int bits;
+  bool active;
+};
+
+// One level for the brackets A and B, which are at the same place (B may be the same as A for a single one): histogram
+// over kSelBins equal steps, scan, descend into each one's bin.  A bracket stops being active when its bin is one key
+// or holds at most `enough`.  `unit`: what most of a lane's items weigh; runs of lanes with the same bin are added by
+// their first lane (lanes hold keys in ascending order inside a row; `row_start`: the lane begins a row, its weights
+// may differ from its neighbour's).
+__device__ __forceinline__ void select_level(SelectShared& sh, const uint32_t (&key)[kSelItems], const uint32_t (&wgt)[kSelItems],
+                                          uint32_t unit, bool row_start, Bracket& A, Bracket& B, uint32_t enough) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint32_t base = A.base;
+  const int bits = A.bits, shift = bits > kSelBits ? bits - kSelBits : 0;
+  const uint32_t reach = bits >= 32 ? 0xffffffffu : (1u << bits) - 1u;
+  *reinterpret_cast<uint4*>(&sh.hist[tid * 4]) = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int i = 0; i < kSelItems; ++i) {
+    const uint32_t rel = key[i] - base;
+    const bool in = wgt[i] > 0 && key[i] >= base && rel <= reach;
+    const uint32_t d = in ? rel >> shift : 0xffffffffu;
+    const uint32_t prev = __shfl_up_sync(0xffffffffu, d, 1);
+    const bool head = lane == 0 || row_start || prev != d;
+    const uint32_t heads = __ballot_sync(0xffffffffu, head);
+    if (in) {
+      if (head) {
+        const uint32_t later = lane == 31 ? 0u : heads >> (lane + 1);
+        atomicAdd(&sh.hist[d], unit * (uint32_t)(later ? __ffs(later) : 32 - lane));
+      }
+      if (wgt[i] != unit) atomicAdd(&sh.hist[d], wgt[i] - unit);       // (modulo 2^32)
+    }
+  }
+  __syncthreads();
+  const uint4 h4 = *reinterpret_cast<const uint4*>(&sh.hist[tid * 4]);
+  const uint32_t h[4] = {h4.x, h4.y, h4.z, h4.w};
+  const uint32_t sum = h[0] + h[1] + h[2] + h[3];
+  const uint32_t top = block_scan(sum, sh);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const Bracket& X = q == 0 ? A : B;
+    uint32_t before = top - sum;
+    if (X.active && before < X.target && X.target <= top) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (before < X.target && X.target <= before + h[j]) { sh.bin[q] = tid * 4 + j; sh.below[q] = before; sh.weight[q] = h[j]; }
+        before += h[j];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    Bracket& X = q == 0 ? A : B;
+    if (!X.active) continue;
+    X.base = base + (sh.bin[q] << shift);
+    X.target -= sh.below[q];
+    X.bits = shift;
+    X.active = shift > 0 && sh.weight[q] > enough;
+  }
 }
+
+__device__ __forceinline__ int bits_of_range(uint32_t lo, uint32_t hi) { return hi > lo ? 32 - __clz(hi - lo) : 0; }
 
 // Exact position of key T in every row's window (32-way searches, one warp per row): gt / ge of
 // the row as absolute pool positions, and their sums over the rows relative to the windows.
@@ -335,12 +357,12 @@ __device__ inline void locate_in_windows(const float* __restrict__ composite, Se
   if (threadIdx.x == 0) { sh.tot_lt = 0; sh.tot_le = 0; }
   __syncthreads();
   for (int r = warp; r < R; r += kSelThreads / 32) {
-    const long long lo = sh.lo[r], w = sh.hi[r] - lo;
+    const int lo = sh.lo[r], w = sh.hi[r] - lo;
     long long lt = 0, le = 0;
     if (w > 0) count_layer_warp(composite + row_start(r, b, Bt, hpr, N) + floor + lo, w, T, &lt, &le);
     if (lane == 0) {
-      sh.gt[r] = lo + lt;
-      sh.ge[r] = lo + le;
+      sh.gt[r] = lo + (int)lt;
+      sh.ge[r] = lo + (int)le;
       atomicAdd(&sh.tot_lt, (unsigned long long)lt);
       atomicAdd(&sh.tot_le, (unsigned long long)le);
     }
@@ -348,250 +370,242 @@ __device__ inline void locate_in_windows(const float* __restrict__ composite, Se
   __syncthreads();
 }
 
+// (the host keeps R * (N - floor) below 2^32)
 __global__ void __launch_bounds__(kSelThreads)
 select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr, long long N, long long floor,
                      long long budget, int max_rounds, int32_t* __restrict__ n_keep,
                      long long* __restrict__ offsets) {
-  __shared__ SelectShared sh;
+  __shared__ __align__(16) SelectShared sh;
   grid_dependency_wait();
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
-  const long long M = N - floor;                       // pooled entries per row
-  // samples per row and round: 32 for up to 32 rows, 16 for up to 64, 8 beyond
-  const int sshift = R <= 32 ? 5 : (R <= 64 ? 4 : 3);
-  const int S = 1 << sshift;
-  const int r = tid >> sshift, k = tid & (S - 1);      // this thread's row and its place among the row's threads
-  // the row's samples are sorted already: every other row takes them in reverse, so that the sort can
-  // start from runs of S
-  const int ks = (tid & S) ? S - 1 - k : k;            // which sample of the row this thread takes
-  const unsigned int sample_id = (unsigned int)((r << sshift) | ks);
+  const int M = (int)(N - floor);                      // pooled entries per row
+  // threads per row in a round: 16 for up to 32 rows, 2 for 256; kSelItems samples each
+  int tshift = 4;
+  while ((kSelThreads >> tshift) < R) --tshift;
+  const int tpr = 1 << tshift, sshift = tshift + 2;
+  static_assert(kSelItems == 4, "sshift");
+  const int r = tid >> tshift, sub = tid & (tpr - 1);  // this thread's row and its place among the row's threads
   const int rr0 = r < R ? r : 0, rl = rr0 / hpr;       // (32-bit: the 64-bit division of row_start is slow)
   const float* row = composite + (((long long)rl * Bt + b) * hpr + (rr0 - rl * hpr)) * N + floor;
   if (tid < R) { sh.lo[tid] = 0; sh.hi[tid] = M; sh.gt[tid] = 0; sh.ge[tid] = 0; }
-  if (tid < kSelMaxRows) { sh.row_a[tid] = 0; sh.row_b[tid] = 0; }
   if (tid == 0) {
-    sh.width = (long long)R * M;
-    sh.rank = budget < sh.width ? budget : sh.width;
+    sh.width = (uint32_t)((unsigned long long)R * (unsigned long long)M);
+    sh.rank = budget < (long long)R * M ? (uint32_t)budget : sh.width;
     sh.kmin = 0xffffffffu;
     sh.kmax = 0u;
+    sh.slack = sh.taken = sh.new_width = 0u;
   }
   __syncthreads();
   if (budget > 0 && M > 0) {
     bool found = false;                                // sh.gt / sh.ge hold the answer
     for (int round = 0; round < max_rounds; ++round) {
-      const long long width = sh.width, rank = sh.rank;
-      if (width <= kSelThreads) break;
-      __syncthreads();                                 // (everyone has read width and rank)
-      if (tid == 0) sh.ilo = 0;
-      // this thread's sample: the last (worst) entry of block k of its row's window
-      long long lo = 0, w = 0, s = 0, wgt = 0;
-      uint32_t key = 0xffffffffu;
+      const uint32_t width = sh.width, rank = sh.rank;
+      if (width <= kSelThreads * kSelItems) break;
+      // this thread's samples: the last (worst) entries of blocks kSelItems * sub .. of its row's window
+      int lo = 0, w = 0, s = 0;
+      uint32_t key[kSelItems], wgt[kSelItems];
       if (r < R) {
         lo = sh.lo[r];
         w = sh.hi[r] - lo;
-        if (w > 0) {
-          s = (w + S - 1) >> sshift;
-          const long long b0 = ks * s;
-          if (b0 < w) {
-            const long long b1 = b0 + s < w ? b0 + s : w;
-            wgt = b1 - b0;
-            key = score_to_key(row[lo + b1 - 1]);
-          }
-        }
-        if (k == 0) sh.row_a[r] = w > 0 ? s - 1 : 0;   // what a partial block can hide
+        s = (int)(((unsigned)w + (1u << sshift) - 1u) >> sshift);
       }
-      sh.wt[sample_id] = wgt;
-      sh.fkey[sample_id] = key;
-      // The samples are sorted as 32-bit words: the key, taken relative to the smallest sample key and
-      // shortened to its leading 22 bits of the samples' range, above the sample's number (which breaks
-      // ties so that the rows' runs stay sorted).  Shortening is monotone, so every bound below holds
-      // for the shortened keys as it would for the keys; samples that fall together just make the
-      // brackets a little wider.
-      const bool real = wgt > 0;
+#pragma unroll
+      for (int i = 0; i < kSelItems; ++i) {
+        key[i] = 0xffffffffu;
+        wgt[i] = 0u;
+        const long long b0 = (long long)(kSelItems * sub + i) * s;
+        if (b0 < w) {
+          const int b1 = (int)min(b0 + s, (long long)w);
+          wgt[i] = (uint32_t)(b1 - (int)b0);
+          key[i] = score_to_key(row[lo + b1 - 1]);
+        }
+      }
       {
-        const uint32_t wmin = __reduce_min_sync(0xffffffffu, real ? key : 0xffffffffu);
-        const uint32_t wmax = __reduce_max_sync(0xffffffffu, real ? key : 0u);
-        if (lane == 0) { atomicMin(&sh.kmin, wmin); atomicMax(&sh.kmax, wmax); }
+        uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+        for (int i = 0; i < kSelItems; ++i)
+          if (wgt[i]) { kmin = min(kmin, key[i]); kmax = max(kmax, key[i]); }
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        const uint32_t hidden = __reduce_add_sync(0xffffffffu, sub == 0 && w > 0 ? (uint32_t)(s - 1) : 0u);   // in partial blocks
+        if (lane == 0) { atomicMin(&sh.kmin, kmin); atomicMax(&sh.kmax, kmax); atomicAdd(&sh.slack, hidden); }
       }
       __syncthreads();
-      const uint32_t base = sh.kmin, span = sh.kmax - base;
-      const int cut = (span >> 22) ? (32 - __clz(span)) - 22 : 0;
-      const uint32_t tkey = real ? ((key - base) >> cut) : 0x3fffffu;
-      const uint32_t packed = (tkey << 10) | sample_id;
-      const uint32_t e = sshift == 5 ? block_sort<64>(packed, sh)
-                       : sshift == 4 ? block_sort<32>(packed, sh) : block_sort<16>(packed, sh);
-      const uint32_t ekey = e >> 10;
-      // weighted rank: entries known to be at least as good as this sample (whole blocks only)
-      const unsigned long long P = block_scan((unsigned long long)sh.wt[e & 1023u], sh);
-      sh.skey[tid] = ekey;
-      sh.pref[tid] = P;
-      if (tid < 32) { const long long v = warp_sum_rows(sh.row_a); if (tid == 0) sh.slack = v; }
+      // upper bracket: the first sample value whose whole blocks already hold `rank` entries: T is at least as good.
+      // lower bracket: sample values for which even whole blocks plus one partial block per row hold fewer than
+      // `rank` entries at least as good: T is worse than those, the ones before the first that may hold them.
+      const uint32_t slack = sh.slack;
+      Bracket A = {sh.kmin, rank, bits_of_range(sh.kmin, sh.kmax), true};
+      Bracket B = {sh.kmin, rank > slack ? rank - slack : 0u, A.bits, rank > slack};
+      const bool has_lo = B.active;
+      // (at most three levels each: 11 + 11 + 10 bits)
+      const uint32_t enough = width / 128;
+      for (int level = 0; level < 6 && (A.active || B.active); ++level) {
+        // together as long as they are at the same place, then the upper one first
+        const bool one = A.active, two = !A.active || (B.active && A.base == B.base && A.bits == B.bits);
+        Bracket X = one ? A : B, Y = B;
+        X.active = one;
+        Y.active = two;
+        select_level(sh, key, wgt, (uint32_t)s, sub == 0, X, Y, enough);
+        if (one) A = X;
+        if (two) B = Y;
+      }
+      const uint32_t reach = A.bits >= 32 ? 0xffffffffu : (1u << A.bits) - 1u;
+      const uint32_t khi = A.base > 0xffffffffu - reach ? 0xffffffffu : A.base + reach;   // T <= khi
+      const uint32_t klo = B.base;                     // T is worse than the sample values before klo
+      // samples of the row on the good side of either bracket
+      uint32_t good = 0u;                              // two counts in one word
+#pragma unroll
+      for (int i = 0; i < kSelItems; ++i)
+        if (wgt[i]) good += (key[i] <= khi ? 0x10000u : 0u) + (has_lo && key[i] < klo ? 1u : 0u);
+      for (int o = tpr >> 1; o > 0; o >>= 1) good += __shfl_xor_sync(0xffffffffu, good, o);
+      uint32_t took = 0u, left = 0u;
+      if (r < R && sub == 0 && w > 0) {
+        const long long jlo = good & 0xffffu, jhi = good >> 16;
+        const int nlo = lo + (int)min((long long)s * jlo, (long long)w);
+        const int nhi = lo + (int)min((long long)s * (jhi + 1), (long long)w);
+        sh.lo[r] = nlo;
+        sh.hi[r] = nhi;
+        took = (uint32_t)(nlo - lo);                   // entries now known to be better than T
+        left = (uint32_t)(nhi - nlo);
+      }
+      took = __reduce_add_sync(0xffffffffu, took);
+      left = __reduce_add_sync(0xffffffffu, left);
+      if (lane == 0) { atomicAdd(&sh.taken, took); atomicAdd(&sh.new_width, left); }
       __syncthreads();
-      // upper bracket: the first sample whose whole blocks already hold `rank` entries: T is at least as good.
-      // lower bracket: the last sample value v for which even whole blocks plus one partial block per row
-      // hold fewer than `rank` entries at least as good as v: T is worse than v.
-      const unsigned long long Pprev = tid ? sh.pref[tid - 1] : 0ull;
-      if (Pprev < (unsigned long long)rank && (unsigned long long)rank <= P) { sh.khi = ekey; sh.khi_key = sh.fkey[e & 1023u]; }
-      const long long bound = rank - sh.slack - 1;
-      const bool last_of_value = tid == kSelThreads - 1 || sh.skey[tid + 1] != ekey;
-      if (last_of_value && (long long)P <= bound) atomicMax(&sh.ilo, tid + 1);
+      const uint32_t new_width = sh.new_width, new_rank = rank - sh.taken;
       __syncthreads();
-      const uint32_t khi = sh.khi;
-      const int ilo = sh.ilo;
-      const uint32_t klo = ilo ? sh.skey[ilo - 1] : 0u;
-      // samples of the row on the good side of either bracket (the lanes of a row are neighbours)
-      const uint32_t mlo = __ballot_sync(0xffffffffu, real && ilo > 0 && tkey <= klo);
-      const uint32_t mhi = __ballot_sync(0xffffffffu, real && tkey <= khi);
-      if (r < R && k == 0) {
-        long long nlo = lo, nhi = lo;
-        if (w > 0) {
-          const uint32_t gmask = (S == 32 ? 0xffffffffu : ((1u << S) - 1u)) << (lane & ~(S - 1));
-          const long long jlo = __popc(mlo & gmask), jhi = __popc(mhi & gmask);
-          nlo = lo + (s * jlo < w ? s * jlo : w);
-          nhi = lo + (s * (jhi + 1) < w ? s * (jhi + 1) : w);
-          sh.lo[r] = nlo;
-          sh.hi[r] = nhi;
-        }
-        sh.row_a[r] = nlo - lo;                        // entries now known to be better than T
-        sh.row_b[r] = nhi - nlo;
+      if (tid == 0) {
+        sh.width = new_width;
+        sh.rank = new_rank;
+        sh.kmin = 0xffffffffu;
+        sh.kmax = 0u;
+        sh.slack = sh.taken = sh.new_width = 0u;
       }
       __syncthreads();
-      if (tid < 32) {
-        const long long taken = warp_sum_rows(sh.row_a), nw = warp_sum_rows(sh.row_b);
-        if (tid == 0) { sh.rank = rank - taken; sh.width = nw; sh.new_width = nw; sh.kmin = 0xffffffffu; sh.kmax = 0u; }
-      }
-      __syncthreads();
-      const long long new_width = sh.new_width;
       if (new_width > width / 2) {
-        // the windows did not shrink: some value has very many copies (or many keys fell together when
-        // they were shortened).  Locate the key of the upper bracket's sample exactly.
-        locate_in_windows(composite, sh, R, b, Bt, hpr, N, floor, sh.khi_key);
-        const long long rk = sh.rank, lt = (long long)sh.tot_lt, le = (long long)sh.tot_le;
+        // the windows did not shrink: some value has very many copies.  Locate the upper bracket exactly.
+        locate_in_windows(composite, sh, R, b, Bt, hpr, N, floor, khi);
+        const uint32_t lt = (uint32_t)sh.tot_lt, le = (uint32_t)sh.tot_le;
         __syncthreads();
-        if (rk > lt && rk <= le) { found = true; break; }            // it is T
-        if (rk <= lt) {                                               // T is better: the copies leave the windows
+        if (new_rank > lt && new_rank <= le && A.bits == 0) { found = true; break; }   // it is T
+        if (new_rank <= lt) {                                         // T is better: the copies leave the windows
           if (tid < R) sh.hi[tid] = sh.gt[tid];
           if (tid == 0) sh.width = lt;
-        } else {                                                      // T is worse (only among keys that were shortened alike)
+        } else if (new_rank > le) {                                   // T is worse
           if (tid < R) sh.lo[tid] = sh.ge[tid];
-          if (tid == 0) { sh.rank = rk - le; sh.width = new_width - le; }
+          if (tid == 0) { sh.rank = new_rank - le; sh.width = new_width - le; }
+        } else {                                                      // T is not worse
+          if (tid < R) sh.hi[tid] = sh.ge[tid];
+          if (tid == 0) sh.width = le;
         }
         __syncthreads();
       }
     }
     if (!found) {
       __syncthreads();
-      const long long width = sh.width, rank = sh.rank;
-      uint32_t T;
-      if (width <= kSelThreads) {
-        // few enough entries left: sort them all, T is the rank-th
-        if (tid < 32) {
-          long long a[4], sum = 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int rr = 4 * tid + i;
-            a[i] = rr < R ? sh.hi[rr] - sh.lo[rr] : 0;
-            sum += a[i];
-          }
-          long long incl = sum;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const long long n = __shfl_up_sync(0xffffffffu, incl, o);
-            if (tid >= o) incl += n;
-          }
-          long long run = incl - sum;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) { sh.off[4 * tid + i] = run; run += a[i]; }
-          if (tid == 31) sh.off[kSelMaxRows] = run;
-        }
-        if (tid < kSelMaxRows) { sh.clt[tid] = 0; sh.cle[tid] = 0; }
+      const uint32_t width = sh.width, rank = sh.rank;
+      if (width <= kSelThreads * kSelItems) {
+        // few enough entries left: all of them are looked at, T is the rank-th
+        const uint32_t end = block_scan(tid < R ? (uint32_t)(sh.hi[tid] - sh.lo[tid]) : 0u, sh);
+        if (tid < R) { sh.off[tid + 1] = (int)end; sh.clt[tid] = 0; sh.cle[tid] = 0; }
+        if (tid == 0) sh.off[0] = 0;
         __syncthreads();
-        uint32_t key = 0xffffffffu;
-        int rr = 0;
-        if (tid < width) {
-          int a = 0, c = R - 1;                        // the row with off[rr] <= tid < off[rr + 1]
-          while (a < c) {
-            const int m = (a + c) >> 1;
-            if (sh.off[m + 1] > tid) c = m; else a = m + 1;
+        uint32_t key[kSelItems], wgt[kSelItems];
+        int at[kSelItems];
+        uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+        for (int i = 0; i < kSelItems; ++i) {
+          const int e = i * kSelThreads + tid;
+          key[i] = 0xffffffffu;
+          wgt[i] = 0u;
+          at[i] = 0;
+          if (e < (int)width) {
+            int x = 0, y = R - 1;                      // the row with off[row] <= e < off[row + 1]
+            while (x < y) {
+              const int m = (x + y) >> 1;
+              if (sh.off[m + 1] > e) y = m; else x = m + 1;
+            }
+            at[i] = x;
+            wgt[i] = 1u;
+            key[i] = score_to_key(composite[row_start(x, b, Bt, hpr, N) + floor + sh.lo[x] + (e - sh.off[x])]);
           }
-          rr = a;
-          key = score_to_key(composite[row_start(rr, b, Bt, hpr, N) + floor + sh.lo[rr] + (tid - sh.off[rr])]);
         }
-        const uint32_t e = block_sort<2>(tid < width ? key : 0xffffffffu, sh);    // (keys alone: T is a value)
-        if (tid == rank - 1) sh.khi = e;
+#pragma unroll
+        for (int i = 0; i < kSelItems; ++i)
+          if (wgt[i]) { kmin = min(kmin, key[i]); kmax = max(kmax, key[i]); }
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        if (lane == 0) { atomicMin(&sh.kmin, kmin); atomicMax(&sh.kmax, kmax); }
         __syncthreads();
-        T = sh.khi;
-        if (tid < width) {
-          if (key < T) atomicAdd(&sh.clt[rr], 1);
-          if (key <= T) atomicAdd(&sh.cle[rr], 1);
+        Bracket A = {sh.kmin, rank, bits_of_range(sh.kmin, sh.kmax), true}, B = {0u, 0u, 0, false};
+        for (int level = 0; level < 3 && A.active; ++level) select_level(sh, key, wgt, 1u, false, A, B, 0u);
+        const uint32_t T = A.base;
+#pragma unroll
+        for (int i = 0; i < kSelItems; ++i) {
+          const bool lt = wgt[i] && key[i] < T, le = wgt[i] && key[i] <= T;
+          const int x0 = __shfl_sync(0xffffffffu, at[i], 0);
+          const uint32_t mlt = __ballot_sync(0xffffffffu, lt), mle = __ballot_sync(0xffffffffu, le);
+          if (__all_sync(0xffffffffu, at[i] == x0 || !wgt[i])) {        // the whole warp in one row
+            if (lane == 0 && mle) { atomicAdd(&sh.clt[x0], __popc(mlt)); atomicAdd(&sh.cle[x0], __popc(mle)); }
+          } else {
+            if (lt) atomicAdd(&sh.clt[at[i]], 1);
+            if (le) atomicAdd(&sh.cle[at[i]], 1);
+          }
         }
         __syncthreads();
         if (tid < R) { sh.gt[tid] = sh.lo[tid] + sh.clt[tid]; sh.ge[tid] = sh.lo[tid] + sh.cle[tid]; }
       } else {
         // out of rounds: bisection over the keys, exact counts inside the windows
-        uint32_t a = 0u, c = 0xffffffffu;              // T lies in [a, c]
-        for (int it = 0; it < 32 && a < c; ++it) {
-          const uint32_t mid = a + (c - a) / 2;
+        uint32_t x = 0u, y = 0xffffffffu;              // T lies in [x, y]
+        for (int it = 0; it < 32 && x < y; ++it) {
+          const uint32_t mid = x + (y - x) / 2;
           locate_in_windows(composite, sh, R, b, Bt, hpr, N, floor, mid);
-          const long long le = (long long)sh.tot_le;
+          const uint32_t le = (uint32_t)sh.tot_le;
           __syncthreads();
-          if (le >= rank) c = mid; else a = mid + 1;
+          if (le >= rank) y = mid; else x = mid + 1;
         }
-        T = a;
-        locate_in_windows(composite, sh, R, b, Bt, hpr, N, floor, T);
+        locate_in_windows(composite, sh, R, b, Bt, hpr, N, floor, x);
       }
     }
   }
   __syncthreads();
-  if (tid < 32) {
-    // the entries equal to T go to the rows in row order until the budget is met; lane i has rows 4i .. 4i + 3
-    long long g[4], tie[4], gsum = 0, tsum = 0;
+  if (tid >= 32) return;
+  // the entries equal to T go to the rows in row order until the budget is met; a lane has `per` neighbouring rows
+  const int per = (R + 31) / 32, first = tid * per;
+  long long gsum = 0, tsum = 0;
+  for (int i = 0; i < per; ++i) {
+    if (first + i < R) { gsum += sh.gt[first + i]; tsum += sh.ge[first + i] - sh.gt[first + i]; }
+  }
+  long long used = gsum, ties_incl = tsum;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int rr = 4 * tid + i;
-      g[i] = rr < R ? sh.gt[rr] : 0;
-      tie[i] = rr < R ? sh.ge[rr] - sh.gt[rr] : 0;
-      gsum += g[i];
-      tsum += tie[i];
+  for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(0xffffffffu, used, o);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long n = __shfl_up_sync(0xffffffffu, ties_incl, o);
+    if (tid >= o) ties_incl += n;
+  }
+  long long rem = budget - used - (ties_incl - tsum);      // what is left when this lane's rows are served
+  // (what the rows before this lane's took of the ties follows from the same numbers)
+  const long long ties_taken = min(max(budget - used, 0LL), ties_incl - tsum);
+  long long gt_incl = gsum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long n = __shfl_up_sync(0xffffffffu, gt_incl, o);
+    if (tid >= o) gt_incl += n;
+  }
+  long long off = (gt_incl - gsum) + ties_taken + floor * min(first, R);
+  for (int i = 0; i < per; ++i) {
+    const int rr = first + i;
+    if (rr < R) {
+      const long long tie = sh.ge[rr] - sh.gt[rr];
+      const long long n = floor + sh.gt[rr] + max(0LL, min(tie, rem));
+      rem -= tie;
+      n_keep[(long long)b * R + rr] = (int32_t)n;
+      offsets[(long long)b * (R + 1) + rr] = off;
+      off += n;
+      if (rr == R - 1) offsets[(long long)b * (R + 1) + R] = off;
     }
-    long long used = gsum, ties_before = tsum;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(0xffffffffu, used, o);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long n = __shfl_up_sync(0xffffffffu, ties_before, o);
-      if (tid >= o) ties_before += n;
-    }
-    ties_before -= tsum;                               // ties in the rows before this lane's
-    long long rem = budget - used - ties_before;       // what is left when this lane's rows are served
-    long long n[4], nsum = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      long long take = tie[i];
-      if (take > rem) take = rem;
-      if (take < 0) take = 0;
-      rem -= tie[i];
-      n[i] = floor + g[i] + take;
-      if (4 * tid + i >= R) n[i] = 0;
-      nsum += n[i];
-    }
-    long long off = nsum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long v = __shfl_up_sync(0xffffffffu, off, o);
-      if (tid >= o) off += v;
-    }
-    const long long total = __shfl_sync(0xffffffffu, off, 31);
-    off -= nsum;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int rr = 4 * tid + i;
-      if (rr < R) {
-        n_keep[(long long)b * R + rr] = (int32_t)n[i];
-        offsets[(long long)b * (R + 1) + rr] = off;
-      }
-      off += n[i];
-    }
-    if (tid == 0) offsets[(long long)b * (R + 1) + R] = total;
   }
 }
 
@@ -633,7 +647,8 @@ kvc_status launch_allocate(const Problem& P, const float* composite, long long b
     if (hook == 1) path = SelectPath::kHistograms;
     if (hook == 2) path = SelectPath::kSortedRows;
   }
-  if (path != SelectPath::kHistograms && R <= kSelMaxRows) {
+  // (with fewer than 8 samples per row a round would hardly cut the windows; the kernel counts in 32 bits)
+  if (path != SelectPath::kHistograms && R <= kSelMaxRows && (long long)R * (P.N - min_keep) < (1LL << 32)) {
     const int hook_rounds = g_select_rounds.load();
     const int rounds = hook_rounds >= 0 ? hook_rounds : kSelDefaultRounds;
     KVC_CUDA(launch_dependent(select_sorted_kernel, dim3(P.Bt), dim3(kSelThreads), 0, st, composite, R, P.Bt,

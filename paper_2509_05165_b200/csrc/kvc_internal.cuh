@@ -133,7 +133,7 @@ size_t allocate_workspace_bytes(const Problem& P);
 // heads_per_row = 1: the pool's rows are the layers, composite [L, Bt, N].  heads_per_row = Hkv (the
 // unstructured variant, App. A.2): the rows are the (layer, head) pairs, composite = the heads'
 // sorted scores [L, Bt, Hkv, N], n_keep [Bt, L * Hkv], offsets [Bt, L * Hkv + 1].
-// How the budget's threshold is found: on the sorted rows by one CTA per sequence (pools of up to 128
+// How the budget's threshold is found: on the sorted rows by one CTA per sequence (pools of up to 256
 // rows; uses no workspace), or by the histogram passes of a radix select over the workspace.
 enum class SelectPath { kAuto, kHistograms, kSortedRows };
 kvc_status launch_allocate(const Problem& P, const float* composite, long long budget, int heads_per_row,

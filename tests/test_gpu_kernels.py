@@ -75,3 +75,31 @@ def test_scoring_on_the_cuda_cores(dtype, Hq, Hkv, w, N, agg_task, explicit):
     torch.cuda.synchronize()
     assert not kvc.kvc_score_uses_tensor_cores(desc)
     Pz.assert_scores_close(out.scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
+
+
+@pytest.mark.parametrize("L,Hkv,N,kind", [
+    (32, 8, 1500, "uniform"), (32, 8, 1500, "ties"),      # 256 rows: the most that one CTA selects from, 8 samples each
+    (43, 6, 400, "uniform"),                              # 258 rows: the histogram passes
+    (17, 2, 61, "uniform"), (33, 1, 63, "ties"),          # 2074 and 2079 entries: one round before the last step
+    (32, 1, 64, "uniform"),                               # 2048 entries: the last step alone
+])
+def test_selection_at_the_limits_of_its_kernel(L, Hkv, N, kind):
+    import oracle
+    cfg = W.WorkloadConfig("select_limits", L, Hkv, Hkv, 64, N, 1, dtype="f32", elem_std=1.0)
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    desc = kvc.desc_from_config(cfg)
+    g = np.random.default_rng(N)
+    S = g.random((L, 1, Hkv, N), dtype=np.float32) if kind == "uniform" else \
+        (np.round(g.random((L, 1, Hkv, N)) * 3) / 4).astype(np.float32)
+    scores = torch.from_numpy(S).to(dev)
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+    idx = torch.empty((L, 1, Hkv, N), dtype=torch.int32, device=dev)
+    n_keep = torch.empty((1, L, Hkv), dtype=torch.int32, device=dev)
+    off = torch.empty((1, L * Hkv + 1), dtype=torch.int64, device=dev)
+    for B in (1, L * Hkv * N // 5, L * Hkv * N - 1):
+        kvc.kvc_select_unstructured(desc, scores, B, idx, n_keep, off, ws)
+        torch.cuda.synchronize()
+        n_ref, off_ref = oracle.select_unstructured(S[:, 0].astype(np.float64), B)
+        assert np.array_equal(n_ref, n_keep.cpu().numpy()[0]) and np.array_equal(off_ref, off.cpu().numpy()[0])
