@@ -38,7 +38,6 @@ namespace {
 // top one).  After the last pass positions and keys go out through the permutation, coalesced.
 // Global traffic: scores read once, idx and sorted keys written once; one launch.
 constexpr int kSegMaxN = 32768;
-constexpr int kSegMaxIpt = 32;                 // places per thread
 constexpr int kSegBatch = 4;                   // key lookups in flight per thread
 constexpr int kMaxDevices = 64;
 
@@ -59,7 +58,6 @@ __device__ __forceinline__ void sts_v4(uint32_t a, uint4 v) {
 // Shared-memory map of a segment of N elements sorted by T threads (byte offsets).
 struct SegLayout {
   int n_pad;            // N rounded up to 32: key_slot and place_slot permute inside aligned blocks of 32
-  int lg;               // log2 of the places per thread
   uint32_t keys;        // uint32[n_pad]: the keys, by position
   uint32_t perm;        // uint16[n_pad]: the key slot (key_slot of the position) at every place
   uint32_t cnt;         // uint16[8][T][2]: thread t's counter of digit d in row d & 7, half d >> 3
@@ -69,8 +67,6 @@ struct SegLayout {
 __host__ __device__ inline SegLayout seg_layout(long long N, int T) {
   SegLayout s;
   s.n_pad = (int)((N + 31) / 32 * 32);
-  s.lg = 0;
-  while (((long long)T << s.lg) < N) ++s.lg;
   s.keys = 0;
   s.perm = 4u * s.n_pad;
   s.cnt = s.perm + 2u * s.n_pad;
@@ -96,9 +92,9 @@ __device__ __forceinline__ uint32_t seg_key(float f) {
 // Every group of 4 consecutive keys of the segment goes to use(i, k0, k1, k2, k3, n): i = position
 // of the first (a multiple of 4), n = how many of the 4 exist.  With 16-byte aligned scores all of
 // a thread's loads are issued before the first use.
-template <int T, typename F>
+template <int T, int kIpt, typename F>
 __device__ __forceinline__ void seg_for_keys(const float* s_in, int N, int tid, F use) {
-  constexpr int kGroups = kSegMaxIpt / 4;
+  constexpr int kGroups = kIpt / 4;
   const bool wide = (reinterpret_cast<uintptr_t>(s_in) & 15u) == 0 && N >= 4;
   if (wide) {
     const int last = (N & ~3) - 4;                           // first position of the last whole group
@@ -121,8 +117,8 @@ __device__ __forceinline__ void seg_for_keys(const float* s_in, int N, int tid, 
   }
 }
 
-template <int T>
-__global__ void __launch_bounds__(T, T == 1024 ? 1 : 4)
+template <int T, int kIpt>
+__global__ void __launch_bounds__(T, 1024 / T)
 segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ keys_out,
                     int32_t* __restrict__ idx_out, long long seg_len, int chunks) {
   // CTA x sorts chunk x % chunks of segment x / chunks: the positions from chunk * kSegMaxN on (a segment of
@@ -131,8 +127,8 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   const int chunk = (int)(blockIdx.x - seg * chunks);
   const long long first = seg * seg_len + (long long)chunk * kSegMaxN;      // of this chunk, in all three arrays
   const int N = (int)min((long long)kSegMaxN, seg_len - (long long)chunk * kSegMaxN);
-  constexpr int kRowShift = (T == 1024) ? 12 : 10;          // log2 of a row of counters in bytes
-  static_assert(T == 1024 || T == 256, "row shift");
+  constexpr int kRowShift = T == 1024 ? 12 : T == 512 ? 11 : T == 256 ? 10 : 9;   // log2 of a row of counters in bytes
+  static_assert((4 * T) >> kRowShift == 1 && kIpt % 8 == 0 && kIpt <= 32, "rows of counters, groups of places");
   constexpr int kScanWarps = T / 64;                        // the scan runs on the first T / 2 threads
   extern __shared__ __align__(16) unsigned char seg_smem[];
   const SegLayout lay = seg_layout(N, T);
@@ -140,10 +136,9 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   const uint32_t keys = sbase + lay.keys, perm = sbase + lay.perm, cnt = sbase + lay.cnt, wtot = sbase + lay.wtot;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int lg = lay.lg, ipt = 1 << lg;
-  const int j0 = tid << lg;
-  const int nv = max(0, min(ipt, N - j0));                   // my places: j0 .. j0 + nv - 1
-  const bool full = __all_sync(0xffffffffu, nv == kSegMaxIpt);   // the warp's decision
+  const int j0 = tid * kIpt;
+  const int nv = max(0, min(kIpt, N - j0));                  // my places: j0 .. j0 + nv - 1
+  const bool full = __all_sync(0xffffffffu, nv == kIpt);     // the warp's decision
   // My counter of digit d: + ((d & 7) << kRowShift) + ((d >> 3) << 1).  Inside a warp's 32 columns, groups
   // of 4 are permuted by the warp number so that the scan's 16-byte reads of neighbouring columns spread
   // over the banks; a lane keeps a bank of its own.
@@ -157,7 +152,7 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   {
     const uint32_t ref = seg_key(s_in[0]);
     if (tid == 0) sts_u32(wtot + 128, 0u);
-    seg_for_keys<T>(s_in, N, tid, [&](int i, uint32_t k0, uint32_t k1, uint32_t k2, uint32_t k3, int n) {
+    seg_for_keys<T, kIpt>(s_in, N, tid, [&](int i, uint32_t k0, uint32_t k1, uint32_t k2, uint32_t k3, int n) {
       const uint32_t sw = ((uint32_t)i >> 5) & 31u;          // the four stay inside their 16 bytes; the table is padded
       sts_u32(keys + (((uint32_t)i) ^ sw) * 4u, k0);
       sts_u32(keys + (((uint32_t)i + 1u) ^ sw) * 4u, k1);
@@ -169,20 +164,16 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
       if (n > 3) diff |= k3 ^ ref;
     });
     // (the permutation holds key slots, not positions: a lookup needs no translation)
-    if (lg >= 3) {
 #pragma unroll
-      for (int q = 0; q < kSegMaxIpt / 8; ++q) {
-        if (q * 8 < nv) {
-          const uint32_t j = (uint32_t)(j0 + q * 8);
-          // j is a multiple of 8: the eight slots are (j ^ m's high bits) | (e ^ m's low 3 bits), e = 0..7
-          const uint32_t m = (j >> 5) & 31u;
-          const uint32_t bb = (j ^ (m & 24u)) * 0x10001u, mm = (m & 7u) * 0x10001u;
-          sts_v4(perm + place_slot(j) * 2u, make_uint4(bb | (0x10000u ^ mm), bb | (0x30002u ^ mm),
-                                                         bb | (0x50004u ^ mm), bb | (0x70006u ^ mm)));
-        }
+    for (int q = 0; q < kIpt / 8; ++q) {
+      if (q * 8 < nv) {
+        const uint32_t j = (uint32_t)(j0 + q * 8);
+        // j is a multiple of 8: the eight slots are (j ^ m's high bits) | (e ^ m's low 3 bits), e = 0..7
+        const uint32_t m = (j >> 5) & 31u;
+        const uint32_t bb = (j ^ (m & 24u)) * 0x10001u, mm = (m & 7u) * 0x10001u;
+        sts_v4(perm + place_slot(j) * 2u, make_uint4(bb | (0x10000u ^ mm), bb | (0x30002u ^ mm),
+                                                       bb | (0x50004u ^ mm), bb | (0x70006u ^ mm)));
       }
-    } else {
-      for (int k = 0; k < nv; ++k) sts_u16(perm + place_slot((uint32_t)(j0 + k)) * 2u, key_slot((uint32_t)(j0 + k)));
     }
     diff = __reduce_or_sync(0xffffffffu, diff);
     __syncthreads();
@@ -201,29 +192,24 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
       constexpr uint32_t kRowMask = 7u << kRowShift;
       const int sh_row = 16 + 4 * h - kRowShift, sh_half = 18 + 4 * h;
 
-      // ---- count (threads whose 32 places all exist take the copy without the per-place tests)
+      // ---- count (warps whose places all exist take the copy without the per-place tests)
 #pragma unroll
       for (int d = 0; d < 8; ++d) sts_u32(cbase + ((uint32_t)d << kRowShift), 0u);
-      uint32_t packed[kSegMaxIpt];
+      uint32_t packed[kIpt];
       auto count = [&](auto full_tag) {
         constexpr bool kFull = decltype(full_tag)::value;
-        if (kFull || lg >= 3) {
 #pragma unroll
-          for (int q = 0; q < kSegMaxIpt / 8; ++q) {
-            if (kFull || q * 8 < nv) {
-              const uint4 w = lds_v4(perm + place_slot((uint32_t)(j0 + q * 8)) * 2u);
-              packed[q * 8 + 0] = w.x & 0xffffu; packed[q * 8 + 1] = w.x >> 16;
-              packed[q * 8 + 2] = w.y & 0xffffu; packed[q * 8 + 3] = w.y >> 16;
-              packed[q * 8 + 4] = w.z & 0xffffu; packed[q * 8 + 5] = w.z >> 16;
-              packed[q * 8 + 6] = w.w & 0xffffu; packed[q * 8 + 7] = w.w >> 16;
-            }
+        for (int q = 0; q < kIpt / 8; ++q) {
+          if (kFull || q * 8 < nv) {
+            const uint4 w = lds_v4(perm + place_slot((uint32_t)(j0 + q * 8)) * 2u);
+            packed[q * 8 + 0] = w.x & 0xffffu; packed[q * 8 + 1] = w.x >> 16;
+            packed[q * 8 + 2] = w.y & 0xffffu; packed[q * 8 + 3] = w.y >> 16;
+            packed[q * 8 + 4] = w.z & 0xffffu; packed[q * 8 + 5] = w.z >> 16;
+            packed[q * 8 + 6] = w.w & 0xffffu; packed[q * 8 + 7] = w.w >> 16;
           }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) if (k < nv) packed[k] = lds_u16(perm + place_slot((uint32_t)(j0 + k)) * 2u);
         }
 #pragma unroll
-        for (int k0 = 0; k0 < kSegMaxIpt; k0 += kSegBatch) {
+        for (int k0 = 0; k0 < kIpt; k0 += kSegBatch) {
           uint32_t b[kSegBatch];
 #pragma unroll
           for (int k = 0; k < kSegBatch; ++k) if (kFull || k0 + k < nv) b[k] = lds_u8(kb + packed[k0 + k] * 4u);
@@ -295,7 +281,7 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
       auto scatter = [&](auto full_tag) {
         constexpr bool kFull = decltype(full_tag)::value;
 #pragma unroll
-        for (int k = 0; k < kSegMaxIpt; ++k) {
+        for (int k = 0; k < kIpt; ++k) {
           if (kFull || k < nv) {
             const uint32_t pk = packed[k];
             const uint32_t off = lds_u16(cbase + (((pk >> sh_row) & kRowMask) | ((pk >> sh_half) & 2u)));
@@ -459,27 +445,50 @@ __global__ void sorted_scores_kernel(const uint32_t* __restrict__ keys, float* _
 
 }  // namespace
 
+typedef void (*SegmentSort)(const float*, uint32_t*, int32_t*, long long, int);
+struct SegmentPlan {
+  SegmentSort kernel;
+  int threads;
+};
+// CTA size and places per thread for a segment of N elements.  The number of places is a constant of the kernel and fits
+// the segment: all but the last warp take the loops without per-place tests, and no warp idles.  Up to 4096 elements
+// few places and more threads (a pass is a chain of look-ups per thread): 256 segments of 1000: 15.0 us with 128 x 8, 15.8
+// with 256 x 8, 21.5 with 128 x 16 (23.4 with 256 x 4 of 32 tested places); of 4096: 20.9 with 256 x 16, 23.3 with 512 x 8, 24.3
+// with 128 x 32 (31.7 tested).  Beyond, 24 or 32 places, which move the most elements per SM: 1024 segments of 5003: 92 with
+// 256 x 24, 108 with 512 x 16, 113 with 256 x 32 (116 before); 256 of 8192: 33.7 with 256 x 32, 35.3 with 512 x 16; of 16384: 60 with
+// 512 x 32, of which two fit an SM, 71 with 1024 x 16 (98 before).
+static SegmentPlan segment_plan(long long N) {
+  if (N <= 1024) return {segment_sort_kernel<128, 8>, 128};
+  if (N <= 2048) return {segment_sort_kernel<128, 16>, 128};
+  if (N <= 4096) return {segment_sort_kernel<256, 16>, 256};
+  if (N <= 6144) return {segment_sort_kernel<256, 24>, 256};
+  if (N <= 8192) return {segment_sort_kernel<256, 32>, 256};
+  if (N <= 12288) return {segment_sort_kernel<512, 24>, 512};
+  if (N <= 16384) return {segment_sort_kernel<512, 32>, 512};
+  if (N <= 24576) return {segment_sort_kernel<1024, 24>, 1024};
+  return {segment_sort_kernel<1024, 32>, 1024};
+}
+
 // Can a segment of N elements be sorted inside one SM here?  Sets the shared-memory attribute once
-// per device (it is per device), under a lock.  *threads = the CTA size to launch.
-static kvc_status segment_sort_prepare(long long N, int* threads) {
+// per device (it is per device), under a lock.
+static kvc_status segment_sort_prepare(long long N, SegmentPlan* plan) {
   if (N > kSegMaxN) return KVC_ERR_UNSUPPORTED;
   static std::mutex mu;
   static int optin[kMaxDevices];           // 0: not looked at, else the device's opt-in bytes (or -1)
   int dev = 0;
   KVC_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return KVC_ERR_UNSUPPORTED;
-  const int T = N > 8192 ? 1024 : 256;
-  const size_t need = seg_layout(N, T).total;
+  *plan = segment_plan(N);
+  const size_t need = seg_layout(N, plan->threads).total;
   std::lock_guard<std::mutex> lock(mu);
   if (optin[dev] == 0) {
     int bytes = 0;
     KVC_CUDA(cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    KVC_CUDA(cudaFuncSetAttribute(segment_sort_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    KVC_CUDA(cudaFuncSetAttribute(segment_sort_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    for (long long n : {1024LL, 2048LL, 4096LL, 6144LL, 8192LL, 12288LL, 16384LL, 24576LL, (long long)kSegMaxN})
+      KVC_CUDA(cudaFuncSetAttribute(segment_plan(n).kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     optin[dev] = bytes > 0 ? bytes : -1;
   }
   if (optin[dev] < 0 || need > (size_t)optin[dev]) return KVC_ERR_UNSUPPORTED;
-  *threads = T;
   return KVC_OK;
 }
 
@@ -519,13 +528,13 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
   int32_t* const vals_a = reinterpret_cast<int32_t*>(w + reg.vals_a);
   uint32_t* const keys_b = reinterpret_cast<uint32_t*>(w + reg.keys_b);
   const long long segments = (long long)P.L * P.Bt * P.Hkv;
-  int seg_threads = 0;
+  SegmentPlan plan;
   const long long chunk_len = P.N < kSegMaxN ? P.N : (long long)kSegMaxN;
-  const kvc_status seg_state = segment_sort_prepare(chunk_len, &seg_threads);
+  const kvc_status seg_state = segment_sort_prepare(chunk_len, &plan);
   if (seg_state != KVC_OK && seg_state != KVC_ERR_UNSUPPORTED) return seg_state;
   if (seg_state != KVC_OK) {
     set_error("compose: this device cannot give a CTA the %zu bytes of shared memory the ranking needs",
-              (size_t)seg_layout(chunk_len, chunk_len > 8192 ? 1024 : 256).total);
+              (size_t)seg_layout(chunk_len, segment_plan(chunk_len).threads).total);
     return KVC_ERR_UNSUPPORTED;
   }
   {
@@ -543,15 +552,9 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
     bool in_b = (levels % 2) == 0;                 // where the sorted chunks go
     uint32_t* k_cur = in_b ? keys_b : keys_a;
     int32_t* v_cur = in_b ? idx : vals_a;
-    const size_t smem = seg_layout(chunk_len, seg_threads).total;
+    const size_t smem = seg_layout(chunk_len, plan.threads).total;
     const unsigned grid = (unsigned)(segments * chunks);
-    if (seg_threads == 1024) {
-      KVC_CUDA(launch_dependent(segment_sort_kernel<1024>, dim3(grid), dim3(1024), smem, st,
-                                scores, k_cur, v_cur, P.N, (int)chunks));
-    } else {
-      KVC_CUDA(launch_dependent(segment_sort_kernel<256>, dim3(grid), dim3(256), smem, st,
-                                scores, k_cur, v_cur, P.N, (int)chunks));
-    }
+    KVC_CUDA(launch_dependent(plan.kernel, dim3(grid), dim3(plan.threads), smem, st, scores, k_cur, v_cur, P.N, (int)chunks));
     KVC_LAUNCH_CHECK("segment_sort_kernel");
     for (int level = 0; level < levels; ++level) {
       in_b = !in_b;

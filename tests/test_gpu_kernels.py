@@ -103,3 +103,22 @@ def test_selection_at_the_limits_of_its_kernel(L, Hkv, N, kind):
         torch.cuda.synchronize()
         n_ref, off_ref = oracle.select_unstructured(S[:, 0].astype(np.float64), B)
         assert np.array_equal(n_ref, n_keep.cpu().numpy()[0]) and np.array_equal(off_ref, off.cpu().numpy()[0])
+
+
+@pytest.mark.parametrize("N", [8, 1024, 1025, 2048, 2049, 6144, 6145, 12288, 12289, 16384, 16385, 24576, 24577])
+def test_ranking_at_the_switches_of_the_cta_size(N):
+    """Eq. 17 on random and heavily tied scores: full and barely started CTAs of every size."""
+    cfg = W.WorkloadConfig("rank_switch", 1, 2, 2, 64, N, 1, dtype="f32", elem_std=1.0)
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    desc = kvc.desc_from_config(cfg)
+    g = np.random.default_rng(N)
+    S = np.stack([g.random(N, dtype=np.float32), (np.round(g.random(N) * 5) / 8).astype(np.float32)])[None, None]
+    idx = torch.empty((1, 1, 2, N), dtype=torch.int32, device=dev)
+    comp = torch.empty((1, 1, N), dtype=torch.float32, device=dev)
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+    kvc.kvc_compose(desc, torch.from_numpy(S).to(dev), idx, comp, ws)
+    torch.cuda.synchronize()
+    Pz.assert_rank_exact(S, idx.cpu().numpy())
+    Pz.assert_compose_exact(S, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
