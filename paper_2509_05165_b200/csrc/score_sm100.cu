@@ -326,9 +326,10 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr) {
   d |= (uint64_t)2 << 61;                          // SWIZZLE_128B
   return d;
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = N = 128.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTile >> 3) << 17) |
-                            ((uint32_t)(kTile >> 4) << 24);
+// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
+__device__ __forceinline__ uint32_t umma_idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+}
 
 // (reference, sum) pairs of the same row: fold (m, l) into (M, Ls).  Exponents are base 2.
 __device__ __forceinline__ void combine(float& M, float& Ls, float m, float l) {
@@ -970,6 +971,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       const int slot = slot0 + qr.i;
       ok = mbar_wait_warp(bar_qfull(slot), (uint32_t)qr.phase, ctl);
       const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
+      // pass 2 leaves out the columns (query rows) that its epilogue does not read
+      const uint32_t idesc = umma_idesc(pass == 0 ? kTile : (c.template rows<kLong>(P) + 31) / 32 * 32);
       qr.next(slots);
       for (int t = 0; t < nt && ok; ++t) {
         const int st = stage0 + kr.i, buf = pass * 2 + tb.i;
@@ -986,7 +989,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
           for (int kk = 0; kk < D / 16; ++kk) {
             // the start-address field counts 16-byte units: 64-element half, then 32 B per K step
             const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-            tc_mma_bf16(d_tmem, da + off, db + off, kIdesc, kk > 0);
+            tc_mma_bf16(d_tmem, da + off, db + off, idesc, kk > 0);
           }
           tc_commit(bar_kempty(st));            // the K stage may be refilled once these MMAs are done
           tc_commit(bar_tfull(buf));            // ... and the accumulator is then complete
