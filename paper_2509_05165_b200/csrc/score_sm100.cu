@@ -37,14 +37,17 @@
 // length through one variant that reads it at run time); with more than one row tile the
 // pass-2 results are partial group aggregates that the Eq. 16 kernel combines in a fixed order.
 //
-// The two passes of a CTA are two pipelines of their own (copies -> K stages and Q slots -> MMAs -> two
+// The two passes of a CTA are two pipelines of their own (copies -> K stages and Q slots -> MMAs ->
 // accumulators -> epilogue) over the same list of runs; they share nothing but the issue slots and the
-// tensor pipe.  Pass 2 goes as fast as the statistics arrive; pass 1 is held to at most `lead` tiles ahead
-// of it (two runs where a unit has no more runs than there are CTAs: 38 MB of K at 148 CTAs, which L2 still
-// holds), exactly what the statistics need: they need every run of a unit, and the other CTAs' runs of
-// it lie that far ahead at most, so the CTAs cannot wait for each other in a circle while all of them are
-// resident (the host checks that they can be).  Every wait (mbarrier or global word) is bounded; on expiry
-// the kernel records KVC_ERR_TIMEOUT, stops computing and drains.
+// tensor pipe.  Pass 1 has its Q, the row operand, in TMEM (copied there once per run) and one
+// accumulator, which its epilogue empties at once: a quarter of the MMAs' operand reads leave shared
+// memory, whose data banks are busy four fifths of the time (500-row windows: 1303 -> 1277 us per pass;
+// the 8B shape gains 0.2 %).  Pass 2 goes as fast as the statistics arrive; pass 1 is held to at most
+// `lead` tiles ahead of it (two runs where a unit has no more runs than there are CTAs: 38 MB of K at
+// 148 CTAs, which L2 still holds), exactly what the statistics need: they need every run of a unit, and
+// the other CTAs' runs of it lie that far ahead at most, so the CTAs cannot wait for each other in a
+// circle while all of them are resident (the host checks that they can be).  Every wait (mbarrier or
+// global word) is bounded; on expiry the kernel records KVC_ERR_TIMEOUT, stops computing and drains.
 //
 // Warp roles (512 threads): warp 0 = TMA producer of pass 1 (K, Q, L2 prefetch), warp 3 = of pass 2; warp
 // 1 = MMA issuer of pass 1 and TMEM owner, warp 2 = of pass 2; warps 4-7 = pass-2 epilogue; warps 8-15 = pass-1
@@ -54,7 +57,9 @@
 // scoring of the 8B shape at 32K: 684 -> 656 us).  With one producer and one K and Q ring for both passes,
 // every one of these warps had to follow both passes tile by tile, 1100 (issuers) to 1500 (producer) clocks
 // of bookkeeping out of the 2160 that a pair of tiles took; with a pipeline per pass a pair takes 1890 (32K: 656 ->
-// 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers), and the epilogues are what it waits for.
+// 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers).  What bounds it now is the board's power:
+// at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds, and copies of the kernel with work left
+// out are faster by that work's energy (an eighth of the MMAs -25 %, of the exponentials -5 %, of the maxima -5 %).
 #include <cuda.h>
 
 #include <atomic>
@@ -231,6 +236,19 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// The same with A in TMEM (lane = row, 16 elements of a row in 8 columns).
+__device__ __forceinline__ void tc_mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// One K step (128 rows x 32 bytes) of a K-major operand tile from shared memory to 8 TMEM columns.
+__device__ __forceinline__ void tc_cp_256b(uint32_t d_tmem, uint64_t desc) {
+  asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;" ::"r"(d_tmem), "l"(desc) : "memory");
 }
 // 32 consecutive accumulator columns of this thread's TMEM lane; the caller waits for the load.
 __device__ __forceinline__ void tc_ld32_nowait(uint32_t taddr, uint32_t (&r)[32]) {
@@ -427,6 +445,9 @@ struct SmemLayout : Rings<D> {
                                                                // -log-sum-exp of the pass-2 unit
   static constexpr int kStats = kNegLse + kRows * 4;           // 2 x 128 rows x float2: the upper half's statistics
   static constexpr int kTotal = kStats + 2 * kRows * 8;
+  // TMEM columns: the accumulator of pass 1, the two of pass 2, pass 1's Q
+  static constexpr int kAcc1 = 0, kAcc2 = kTile, kQt = 3 * kTile;
+  static_assert(kQt + D / 2 <= 512, "TMEM columns");
   static_assert(kCtl % 8 == 0 && kNegLse % 16 == 0 && kStats % 8 == 0 && kTotal <= 232448, "shared-memory layout");
 };
 
@@ -631,7 +652,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < SL::kStages; ++s) { mbar_init(bar_kfull(s), 1); mbar_init(bar_kempty(s), 1); }
     // the accumulators of pass 1 are read by eight warps (two column halves), those of pass 2 by four
-    for (int b = 0; b < 4; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), b < 2 ? 8 : 4); }
+    for (int b = 0; b < 3; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), b == 0 ? 8 : 4); }
     for (int q = 0; q < SL::kSlots; ++q) { mbar_init(bar_qfull(q), 1); mbar_init(bar_qfree(q), 1); }
     mbar_init(bar_mma_done(0), 1); mbar_init(bar_mma_done(1), 1);
     ctl->abort = 0;
@@ -716,13 +737,12 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       const int nt = c.tiles(P);
       int tok0 = c.first_token(P);                      // first token of the tile
       for (int t = 0; t < nt; ++t, tok0 += kTile) {
-        const int buf = n1 & 1;
         // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
-        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(buf), (uint32_t)((n1 >> 1) & 1), ctl));
+        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(0), (uint32_t)(n1 & 1), ctl));
         ++n1;
         if (!ok) continue;
         tc_fence_after();
-        const uint32_t taddr = lane_addr + (uint32_t)buf * kTile + half * 64;
+        const uint32_t taddr = lane_addr + SL::kAcc1 + half * 64;
         if (tok0 + kTile - 1 <= vis_all) {              // no masking anywhere in the tile
           uint32_t ra[32], rb[32];
           tc_ld32_nowait(taddr, ra);
@@ -731,7 +751,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
           tc_wait_ld(rb);
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_tempty(buf));    // the accumulator is in registers now
+          if (lane == 0) mbar_arrive(bar_tempty(0));    // the accumulator is in registers now
           if (row_used) { fast_chunk(ra); fast_chunk(rb); }
         } else {
           float m2 = mref, l2 = lsum;                     // (the whole warp takes part in the TMEM loads)
@@ -740,7 +760,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
           if (row_used) { mref = m2; lsum = l2; }
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_tempty(buf));
+          if (lane == 0) mbar_arrive(bar_tempty(0));
         }
       }
       // the end of the run: the two halves of every row meet through shared memory (two buffers in turn); the lower
@@ -859,8 +879,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         early_word = ld_relaxed_u64(P.acc + (long long)cu.u * kRows + trow);
         early_ref = __ldg(P.ref + (long long)cu.u * kRows + trow);
       }
-      const int buf = 2 + (n2 & 1);
-      const uint32_t tmem_col = (uint32_t)buf * kTile;
+      const int buf = 1 + (n2 & 1);
+      const uint32_t tmem_col = SL::kAcc2 + (uint32_t)(n2 & 1) * kTile;
       // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
       ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(buf), (uint32_t)((n2 >> 1) & 1), ctl));
       ++n2;
@@ -962,7 +982,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     const int pass = warp - 1;
     const int stage0 = pass == 0 ? 0 : SL::kK1, stages = pass == 0 ? SL::kK1 : SL::kK2;
     const int slot0 = pass == 0 ? 0 : SL::kQ1, slots = pass == 0 ? SL::kQ1 : SL::kQ2;
-    Ring kr = {0, 0}, qr = {0, 0}, tb = {0, 0};        // K stage, Q slot, accumulator (two per pass)
+    const int bufs = pass == 0 ? 1 : 2;
+    Ring kr = {0, 0}, qr = {0, 0}, tb = {0, 0};        // K stage, Q slot, accumulator
     bool ok = true, issued = false;
     RunCursor c;
     c.init(P);
@@ -971,34 +992,52 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       const int slot = slot0 + qr.i;
       ok = mbar_wait_warp(bar_qfull(slot), (uint32_t)qr.phase, ctl);
       const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
-      // pass 2 leaves out the columns (query rows) that its epilogue does not read
       const uint32_t idesc = umma_idesc(pass == 0 ? kTile : (c.template rows<kLong>(P) + 31) / 32 * 32);
       qr.next(slots);
+      if (pass == 0 && ok) {
+        // the run's Q moves to TMEM (in order behind the MMAs that read the run before's), its slot is free again
+        tc_fence_after();
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk)
+            tc_cp_256b(tmem_base + SL::kQt + kk * 8, dq + (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4));
+          tc_commit(bar_qfree(slot));
+        }
+        __syncwarp();
+        issued = true;
+      }
       for (int t = 0; t < nt && ok; ++t) {
-        const int st = stage0 + kr.i, buf = pass * 2 + tb.i;
+        const int st = stage0 + kr.i, buf = pass + tb.i;
         ok = mbar_wait_warp(bar_kfull(st), (uint32_t)kr.phase, ctl);
         if (ok) ok = mbar_wait_warp(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
         if (!ok) break;
         tc_fence_after();
         const uint64_t dk = umma_desc(sbase + SL::kK + st * SL::kTileBytes);
-        // pass 1: rows = query rows (A = Q), columns = tokens (B = K); pass 2: swapped
-        const uint64_t da = pass == 0 ? dq : dk, db = pass == 0 ? dk : dq;
         const uint32_t d_tmem = tmem_base + (uint32_t)buf * kTile;
         if (elect_one()) {
+          // pass 1: rows = query rows (A = Q, in TMEM), columns = tokens (B = K); pass 2: A = K, B = Q
+          // (the start-address field counts 16-byte units: 64-element half, then 32 B per K step)
+          if (pass == 0) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            // the start-address field counts 16-byte units: 64-element half, then 32 B per K step
-            const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-            tc_mma_bf16(d_tmem, da + off, db + off, idesc, kk > 0);
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
+              tc_mma_bf16_ts(d_tmem, tmem_base + SL::kQt + kk * 8, dk + off, idesc, kk > 0);
+            }
+          } else {
+#pragma unroll
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
+              tc_mma_bf16(d_tmem, dk + off, dq + off, idesc, kk > 0);
+            }
           }
           tc_commit(bar_kempty(st));            // the K stage may be refilled once these MMAs are done
           tc_commit(bar_tfull(buf));            // ... and the accumulator is then complete
-          if (t + 1 == nt) tc_commit(bar_qfree(slot));
+          if (pass != 0 && t + 1 == nt) tc_commit(bar_qfree(slot));
         }
         __syncwarp();
         issued = true;
         kr.next(stages);
-        tb.next(2);
+        tb.next(bufs);
       }
     }
     // no MMA may be in flight when the TMEM columns and the shared memory are given back
