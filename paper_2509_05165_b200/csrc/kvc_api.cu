@@ -54,7 +54,7 @@ kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q
     if (s == KVC_OK) return launch_score_augment(P, scores, parts, row_tiles, tiles_per_head, vnorm, st);
     if (s != KVC_ERR_UNSUPPORTED) return s;      // a real failure; UNSUPPORTED = strides TMA cannot take
   }
-  return launch_score_generic(P, gm, q, k, scores, vnorm, ws, ws_bytes, st);
+  return launch_score_generic(P, gm, q, k, scores, vnorm, device_status, ws, ws_bytes, st);
 }
 
 // Scoring as the entry points run it: status word and value norms carved from the score workspace.
@@ -291,7 +291,6 @@ kvc_status kvc_score(const kvc_desc* d, const void* const* q, const void* const*
   if ((s = check_device()) != KVC_OK) return s;
   // conditions detected on the device are reported in a word behind the scratch (kvc_score_status_offset)
   int* status = reinterpret_cast<int*>(reinterpret_cast<char*>(ws) + score_scratch_bytes(P));
-  KVC_CUDA(cudaMemsetAsync(status, 0, sizeof(int), (cudaStream_t)stream));
   return run_score(P, gm, qp, kp, nullptr, scores, status, ws, (cudaStream_t)stream);
 }
 
@@ -308,7 +307,6 @@ kvc_status kvc_score_weighted(const kvc_desc* d, const void* const* q, const voi
   if ((s = check_ws(ws, ws_bytes, score_workspace_bytes(P))) != KVC_OK) return s;
   if ((s = check_device()) != KVC_OK) return s;
   int* status = reinterpret_cast<int*>(reinterpret_cast<char*>(ws) + score_scratch_bytes(P));
-  KVC_CUDA(cudaMemsetAsync(status, 0, sizeof(int), (cudaStream_t)stream));
   return run_score(P, gm, qp, kp, &vp, scores, status, ws, (cudaStream_t)stream);
 }
 
@@ -412,7 +410,6 @@ kvc_status kvc_compress(const kvc_desc* d, const void* const* q, const void* con
   float* composite = composite_out ? composite_out : reinterpret_cast<float*>(w + lay.composite);
   const size_t stage_bytes = lay.alloc - lay.stage;
 
-  if (device_status) KVC_CUDA(cudaMemsetAsync(device_status, 0, sizeof(int32_t), st));
   if ((s = run_score(P, gm, qp, kp, &vp, scores, device_status, w + lay.stage, st)) != KVC_OK) return s;
   if ((s = launch_compose(P, scores, idx, composite, w + lay.stage, stage_bytes, st)) != KVC_OK) return s;
   if ((s = launch_allocate(P, composite, budget, 1, P.min_keep, n_keep, reinterpret_cast<long long*>(offsets),
@@ -511,7 +508,6 @@ kvc_status kvc_compress_unstructured(const kvc_desc* d, const void* const* q, co
   float* sorted = reinterpret_cast<float*>(w + lay.scores);
   const size_t stage_bytes = lay.alloc - lay.stage;
 
-  if (device_status) KVC_CUDA(cudaMemsetAsync(device_status, 0, sizeof(int32_t), st));
   if ((s = run_score(P, gm, qp, kp, &vp, scores, device_status, w + lay.stage, st)) != KVC_OK) return s;
   if ((s = run_select_unstructured(P, scores, budget_entries, idx, n_keep, reinterpret_cast<long long*>(offsets),
                                    sorted, w, lay, st)) != KVC_OK) return s;

@@ -94,6 +94,7 @@ inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 size_t score_workspace_bytes(const Problem& P);
 // Eqs. 3, 14-16: writes scores [L, Bt, Hkv, N].
 // vnorm: nullptr, or ||v|| per (layer, sequence, KV head, token), laid out like scores (App. A.1.3).
+// device_status (may be null) is cleared by the first of its kernels.
 kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k,
                         float* scores, const float* vnorm, int* device_status, void* ws, size_t ws_bytes,
                         cudaStream_t st);
@@ -101,7 +102,7 @@ kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q
 // contiguous GQA groups, window of at most 128 rows).
 size_t score_generic_workspace_bytes(const Problem& P);
 kvc_status launch_score_generic(const Problem& P, const GroupMap& gm, const LayerPtrs& q,
-                                const LayerPtrs& k, float* scores, const float* vnorm, void* ws,
+                                const LayerPtrs& k, float* scores, const float* vnorm, int* device_status, void* ws,
                                 size_t ws_bytes, cudaStream_t st);
 // Eq. 16 in place; before it, with `row_tiles` > 1, the group aggregate (Eq. 15) of every KV head
 // from its row tiles' partial aggregates `parts` [row_tiles][L*Bt*Hkv][N], in tile order.

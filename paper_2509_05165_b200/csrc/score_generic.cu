@@ -292,12 +292,13 @@ __device__ __forceinline__ void stage4(float* dst, const __nv_bfloat16* row, int
 template <typename T, int D>
 __global__ void __launch_bounds__(kLogitThreads, 1)
 score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, float* __restrict__ dots, int row_tiles,
-                    int tok_tiles, int items) {
+                    int tok_tiles, int items, int* __restrict__ status) {
   constexpr int kPitch = D + 4, kVec = D / 4;
   extern __shared__ __align__(16) float gsm[];
   float* const Qs = gsm;
   float* const Ks = gsm + kTileRow * kPitch;                   // two buffers
   grid_dependency_wait();
+  if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;      // (nothing here can fail on the device)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tok = (warp & 1) * 64 + (lane & 7);               // tokens tok + 8 i
   const int row = (warp >> 1) * 32 + (lane >> 3);             // rows row + 4 j
@@ -540,6 +541,79 @@ score_emit_logits_kernel(LogitParams P, GroupMap gm, const float* __restrict__ d
   }
 }
 
+// The kernel below for up to kAugHeads = 8 (4) KV heads: a thread has all heads' group aggregates of its token in registers, reads
+// the row tiles' parts of all heads together and writes every score once.  Bound by HBM / L2: parts once, scores once.
+// (28 layers, 4 heads, 4 row tiles, N = 131072: 129 -> 56 us; 32 layers, 8 heads, 16 row tiles, N = 4096: 43 -> 19.)
+template <int kAugHeads, bool kParts>
+__global__ void __launch_bounds__(256, !kParts ? 6 : kAugHeads == 8 ? 4 : 7)
+score_augment_heads_kernel(float* __restrict__ s, const float* __restrict__ parts, int row_tiles, int tiles_per_head,
+                           int agg_task, int w, const float* __restrict__ vnorm, int G, int agg_group, int augment, int Hkv,
+                           long long N) {
+  grid_dependency_wait();
+  const long long c = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (c >= N) return;
+  const long long at = (long long)blockIdx.y * Hkv * N + c;            // blockIdx.y = (layer, sequence)
+  float* base = s + at;
+  float acc[kAugHeads];
+  if constexpr (kParts) {
+    const long long tile_stride = (long long)gridDim.y * Hkv * N;       // one [L*Bt*Hkv][N] block per row tile
+    const float* p = parts + at;
+    auto fetch = [&](int t, float (&v)[kAugHeads]) {
+#pragma unroll
+      for (int h = 0; h < kAugHeads; ++h) v[h] = h < Hkv ? __ldg(p + t * tile_stride + (long long)h * N) : 0.f;
+    };
+    if (tiles_per_head > 1) {
+#pragma unroll
+      for (int h = 0; h < kAugHeads; ++h) acc[h] = (agg_group == KVC_AGG_MAX) ? -INFINITY : 0.f;
+      for (int j = 0; j < row_tiles / tiles_per_head; ++j) {             // the query heads of the group
+        float ht[kAugHeads];
+        fetch(j * tiles_per_head, ht);
+#pragma unroll 2
+        for (int t = 1; t < tiles_per_head; ++t) {
+          float v[kAugHeads];
+          fetch(j * tiles_per_head + t, v);
+#pragma unroll
+          for (int h = 0; h < kAugHeads; ++h) ht[h] = (agg_task == KVC_AGG_MAX) ? fmaxf(ht[h], v[h]) : ht[h] + v[h];
+        }
+#pragma unroll
+        for (int h = 0; h < kAugHeads; ++h) {
+          if (agg_task == KVC_AGG_MEAN) ht[h] = ht[h] / (float)w;
+          acc[h] = (agg_group == KVC_AGG_MAX) ? fmaxf(acc[h], ht[h]) : acc[h] + ht[h];
+        }
+      }
+    } else {
+      fetch(0, acc);
+#pragma unroll 2
+      for (int t = 1; t < row_tiles; ++t) {
+        float v[kAugHeads];
+        fetch(t, v);
+#pragma unroll
+        for (int h = 0; h < kAugHeads; ++h) acc[h] = (agg_group == KVC_AGG_MAX) ? fmaxf(acc[h], v[h]) : acc[h] + v[h];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < kAugHeads; ++h) if (agg_group == KVC_AGG_MEAN) acc[h] = acc[h] / (float)G;
+  } else {
+#pragma unroll
+    for (int h = 0; h < kAugHeads; ++h) acc[h] = h < Hkv ? base[(long long)h * N] : 0.f;
+  }
+  if (vnorm != nullptr) {
+#pragma unroll
+    for (int h = 0; h < kAugHeads; ++h) if (h < Hkv) acc[h] *= __ldg(vnorm + at + (long long)h * N);
+  }
+  float mean = 0.f;
+  if (augment) {
+    float sum = 0.f;
+#pragma unroll
+    for (int h = 0; h < kAugHeads; ++h) if (h < Hkv) sum += acc[h];
+    mean = sum / (float)Hkv;
+#pragma unroll
+    for (int h = 0; h < kAugHeads; ++h) acc[h] += mean;
+  }
+#pragma unroll
+  for (int h = 0; h < kAugHeads; ++h) if (h < Hkv) base[(long long)h * N] = acc[h];
+}
+
 // Eq. 16: S[h, c] = S_group[h, c] + (1/Hkv) sum_i S_group[i, c], in place.  With row tiles, first
 // Eq. 15 from the tiles' partial aggregates (sum or max over the tile's query heads), in tile order.
 // With vnorm (App. A.1.3), the group aggregate is multiplied by the token's value norm before Eq. 16.
@@ -586,19 +660,6 @@ __global__ void score_augment_kernel(float* __restrict__ s, const float* __restr
     }
   }
   if (!augment) return;
-  if (Hkv <= 8) {
-    // all heads' values at once: the thread waits for memory once (added in ascending head order all the same)
-    float v[8];
-#pragma unroll
-    for (int h = 0; h < 8; ++h) v[h] = h < Hkv ? base[(long long)h * N] : 0.f;
-    float sum = 0.f;
-#pragma unroll
-    for (int h = 0; h < 8; ++h) if (h < Hkv) sum += v[h];
-    const float mean = sum / (float)Hkv;
-#pragma unroll
-    for (int h = 0; h < 8; ++h) if (h < Hkv) base[(long long)h * N] = v[h] + mean;
-    return;
-  }
   float sum = 0.f;
   for (int h = 0; h < Hkv; ++h) sum += base[(long long)h * N];
   const float mean = sum / (float)Hkv;
@@ -659,7 +720,7 @@ LogitPlan logit_plan(const Problem& P) {
 
 template <typename T, int D>
 kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
-                      const LogitPlan& pl, char* ws, cudaStream_t st) {
+                      const LogitPlan& pl, char* ws, int* device_status, cudaStream_t st) {
   constexpr int kSmem = (2 * kTileTok + kTileRow) * (D + 4) * (int)sizeof(float);
   KVC_CUDA(cudaFuncSetAttribute(score_logits_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
   int dev = 0, sms = 0;
@@ -686,7 +747,7 @@ kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, 
     lp.unit0 = (int)u0;
     const long long items = (long long)n * row_tiles * tok_tiles;
     KVC_CUDA(launch_dependent(score_logits_kernel<T, D>, dim3((unsigned)(items < sms ? items : sms)), dim3(kLogitThreads),
-                              (size_t)kSmem, st, lp, gm, q, k, dots, row_tiles, tok_tiles, (int)items));
+                              (size_t)kSmem, st, lp, gm, q, k, dots, row_tiles, tok_tiles, (int)items, device_status));
     KVC_LAUNCH_CHECK("score_logits_kernel");
     KVC_CUDA(launch_dependent(score_row_stats_kernel, dim3((unsigned)((pl.max_rows + 3) / 4), n), dim3(kRowStatWarps * 32),
                               stat_smem, st, lp, gm, (const float*)dots, lse2));
@@ -716,6 +777,15 @@ size_t score_generic_workspace_bytes(const Problem& P) {
 kvc_status launch_score_augment(const Problem& P, float* scores, const float* parts, int row_tiles,
                                 int tiles_per_head, const float* vnorm, cudaStream_t st) {
   if (!P.augment && row_tiles <= 1 && vnorm == nullptr) return KVC_OK;
+  if (P.Hkv <= 8) {
+    const auto kernel = row_tiles > 1 ? (P.Hkv <= 4 ? score_augment_heads_kernel<4, true> : score_augment_heads_kernel<8, true>)
+                                      : score_augment_heads_kernel<8, false>;
+    KVC_CUDA(launch_dependent(kernel, dim3((unsigned)((P.N + 255) / 256), (unsigned)(P.L * P.Bt)), dim3(256), 0,
+                              st, scores, parts, row_tiles, tiles_per_head, P.agg_task, P.w, vnorm, P.max_group, P.agg_group,
+                              P.augment, P.Hkv, P.N));
+    KVC_LAUNCH_CHECK("score_augment_heads_kernel");
+    return KVC_OK;
+  }
   const long long total = (long long)P.L * P.Bt * P.N;
   KVC_CUDA(launch_dependent(score_augment_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st,
                             scores, parts, row_tiles, tiles_per_head, P.agg_task, P.w, vnorm, P.max_group, P.agg_group,
@@ -725,7 +795,7 @@ kvc_status launch_score_augment(const Problem& P, float* scores, const float* pa
 }
 
 kvc_status launch_score_generic(const Problem& P, const GroupMap& gm, const LayerPtrs& q,
-                                const LayerPtrs& k, float* scores, const float* vnorm, void* ws,
+                                const LayerPtrs& k, float* scores, const float* vnorm, int* device_status, void* ws,
                                 size_t ws_bytes, cudaStream_t st) {
   if (ws_bytes < score_generic_workspace_bytes(P)) {
     set_error("score: workspace too small");
@@ -736,13 +806,14 @@ kvc_status launch_score_generic(const Problem& P, const GroupMap& gm, const Laye
     char* w = reinterpret_cast<char*>(ws);
     kvc_status r;
     if (P.dtype == KVC_BF16)
-      r = P.d == 64 ? run_logits<__nv_bfloat16, 64>(P, gm, q, k, scores, pl, w, st)
-                    : run_logits<__nv_bfloat16, 128>(P, gm, q, k, scores, pl, w, st);
+      r = P.d == 64 ? run_logits<__nv_bfloat16, 64>(P, gm, q, k, scores, pl, w, device_status, st)
+                    : run_logits<__nv_bfloat16, 128>(P, gm, q, k, scores, pl, w, device_status, st);
     else
-      r = P.d == 64 ? run_logits<float, 64>(P, gm, q, k, scores, pl, w, st) : run_logits<float, 128>(P, gm, q, k, scores, pl, w, st);
+      r = P.d == 64 ? run_logits<float, 64>(P, gm, q, k, scores, pl, w, device_status, st) : run_logits<float, 128>(P, gm, q, k, scores, pl, w, device_status, st);
     if (r != KVC_OK) return r;
     return launch_score_augment(P, scores, nullptr, 1, 1, vnorm, st);
   }
+  if (device_status) KVC_CUDA(cudaMemsetAsync(device_status, 0, sizeof(int), st));
   const size_t rows = (size_t)P.L * P.Bt * P.Hq * P.w;
   const int nchunks = generic_nchunks(P);
   float2* partial = reinterpret_cast<float2*>(ws);

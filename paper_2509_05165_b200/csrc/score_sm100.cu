@@ -1142,6 +1142,7 @@ struct RefParams {
   int Bt, Hkv, G, HPT, QT, CH, w, d;
   unsigned long long* acc;     // [U][128]: cleared here
   unsigned long long* ovf;     // [U][128][4]: cleared here
+  int* status;                 // the device status word (may be null): cleared here
   long long qs0, qs1, qs2, kvs0, kvs1;
   float sl2e;
 };
@@ -1149,37 +1150,46 @@ struct RefParams {
 __global__ void __launch_bounds__(kRows)
 score_ref_kernel(RefParams P, LayerPtrs qp, LayerPtrs kp, float* __restrict__ ref) {
   grid_dependency_wait();
+  __shared__ __align__(16) uint4 k_row[16];                  // token 0's key
   const int u = blockIdx.x, row = threadIdx.x;
+  const int uh = u / P.QT, qt = u - uh * P.QT;
+  const int lb = uh / P.Hkv, h = uh - lb * P.Hkv;
+  const int l = lb / P.Bt, b = lb - l * P.Bt;
+  const int rows_u = P.CH == 1 ? min(P.HPT, P.G - qt * P.HPT) * P.w : min(kRows, P.w - (qt % P.CH) * kRows);
+  if (row < P.d / 8)
+    k_row[row] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(kp.p[l]) + b * P.kvs0 + h * P.kvs1) + row);
+  // the row's query, 16-byte pieces (rows are 16-byte aligned), all in flight at once
+  uint4 a[16];
+  if (row < rows_u) {
+    const int j = P.CH == 1 ? h * P.G + qt * P.HPT + row / P.w : h * P.G + qt / P.CH;
+    const int m = P.CH == 1 ? row % P.w : (qt % P.CH) * kRows + row;
+    const uint4* q4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(qp.p[l]) + b * P.qs0 + j * P.qs1 + m * P.qs2);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) if (t < P.d / 8) a[t] = __ldg(q4 + t);
+  }
   // the unit's exchange state: empty words
+  if (P.status != nullptr && u == 0 && row == 0) *P.status = 0;
   P.acc[(long long)u * kRows + row] = 0ull;
   {
     ulonglong2* o = reinterpret_cast<ulonglong2*>(P.ovf + ((long long)u * kRows + row) * 4);
     o[0] = make_ulonglong2(0ull, 0ull);
     o[1] = make_ulonglong2(0ull, 0ull);
   }
-  const int uh = u / P.QT, qt = u - uh * P.QT;
-  const int lb = uh / P.Hkv, h = uh - lb * P.Hkv;
-  const int l = lb / P.Bt, b = lb - l * P.Bt;
-  const int rows_u = P.CH == 1 ? min(P.HPT, P.G - qt * P.HPT) * P.w : min(kRows, P.w - (qt % P.CH) * kRows);
+  __syncthreads();
   float r = 0.f;
   if (row < rows_u) {
-    const int j = P.CH == 1 ? h * P.G + qt * P.HPT + row / P.w : h * P.G + qt / P.CH;
-    const int m = P.CH == 1 ? row % P.w : (qt % P.CH) * kRows + row;
-    const __nv_bfloat16* qv = reinterpret_cast<const __nv_bfloat16*>(qp.p[l]) + b * P.qs0 + j * P.qs1 + m * P.qs2;
-    const __nv_bfloat16* kv = reinterpret_cast<const __nv_bfloat16*>(kp.p[l]) + b * P.kvs0 + h * P.kvs1;
-    // 16-byte pieces (rows are 16-byte aligned), all in flight at once; products added in order
-    const uint4* q4 = reinterpret_cast<const uint4*>(qv);
-    const uint4* k4 = reinterpret_cast<const uint4*>(kv);
-    float acc = 0.f;
-#pragma unroll 4
-    for (int t = 0; t < P.d / 8; ++t) {
-      const uint4 a = __ldg(q4 + t), b2 = __ldg(k4 + t);
-      const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b2.x, b2.y, b2.z, b2.w};
+    float acc = 0.f;                                         // products added in order
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        // a bf16 is the upper half of the fp32 with the same value
-        acc = fmaf(__uint_as_float(aw[i] << 16), __uint_as_float(bw[i] << 16), acc);
-        acc = fmaf(__uint_as_float(aw[i] & 0xffff0000u), __uint_as_float(bw[i] & 0xffff0000u), acc);
+    for (int t = 0; t < 16; ++t) {
+      if (t < P.d / 8) {
+        const uint4 k4 = k_row[t];
+        const uint32_t aw[4] = {a[t].x, a[t].y, a[t].z, a[t].w}, bw[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          // a bf16 is the upper half of the fp32 with the same value
+          acc = fmaf(__uint_as_float(aw[i] << 16), __uint_as_float(bw[i] << 16), acc);
+          acc = fmaf(__uint_as_float(aw[i] & 0xffff0000u), __uint_as_float(bw[i] & 0xffff0000u), acc);
+        }
       }
     }
     r = acc * P.sl2e;
@@ -1377,6 +1387,7 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
     RefParams rp;
     rp.acc = fp.acc;
     rp.ovf = fp.ovf;
+    rp.status = device_status;
     rp.Bt = P.Bt; rp.Hkv = P.Hkv; rp.G = G; rp.HPT = pl.HPT; rp.QT = pl.QT; rp.CH = pl.CH; rp.w = P.w; rp.d = P.d;
     rp.qs0 = P.qs[0]; rp.qs1 = P.qs[1]; rp.qs2 = P.qs[2]; rp.kvs0 = P.kvs[0]; rp.kvs1 = P.kvs[1];
     rp.sl2e = P.scale * kLog2eF;

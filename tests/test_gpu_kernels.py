@@ -42,6 +42,7 @@ def test_value_norms_at_tile_edges(dtype, d, N):
     (8, 2, 9, 1), (8, 2, 31, 0),        # columns taken 8 and 16 at a time, the last ones overlapping
     (14, 2, 33, 1), (4, 2, 127, 0),     # ... and 32 at a time; row tiles of three heads and of one
     (2, 1, 129, 1), (4, 2, 256, 0),     # row tiles of 128 rows and one row; of exactly 128
+    (10, 5, 128, 1), (18, 9, 128, 1),   # parts of more KV heads than four, and than eight
 ])
 def test_max_over_windows_of_any_length(Hq, Hkv, w, agg_group):
     """Pass 2 on tiles no mask touches: every way a tile's columns are split into query heads."""
