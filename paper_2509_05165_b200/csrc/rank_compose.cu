@@ -409,38 +409,63 @@ merge_runs_kernel(const uint32_t* __restrict__ keys_in, const int32_t* __restric
 
 // Eq. 19 over the sorted keys: composite[lb, k] = agg_head_h score(keys[lb, h, k]).
 // Mean: heads added in ascending order in fp32, one division at the end.
-// blockIdx.y = (layer, sequence), blockIdx.x over the ranks.  The heads' keys are fetched eight at a
-// time before they are added, so that a thread waits for memory once, not once per head.
-__global__ void compose_kernel(const uint32_t* __restrict__ keys, float* __restrict__ composite,
-                               int Hkv, long long N, int agg_head) {
+// blockIdx.y = (layer, sequence), blockIdx.x over the ranks, kE neighbouring ranks per thread (4 with 16-byte accesses where N
+// is a multiple of 4: 256 segments of 32768 10.3 -> 7.0 us, 112 of 131072 33 -> 15).  The heads' keys are fetched eight at
+// a time before they are added, so that a thread waits for memory once, not once per head.
+template <int kE>
+__global__ void __launch_bounds__(256)
+compose_kernel(const uint32_t* __restrict__ keys, float* __restrict__ composite, int Hkv, long long N, int agg_head) {
   grid_dependency_wait();
-  const long long kk = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int kB = 8;
+  const long long kk = ((long long)blockIdx.x * 256 + threadIdx.x) * kE;
   if (kk >= N) return;
-  const long long lb = blockIdx.y;
-  const uint32_t* p = keys + lb * Hkv * N + kk;
-  float acc = 0.f;
-  for (int h0 = 0; h0 < Hkv; h0 += 8) {
-    uint32_t v[8];
+  const uint32_t* p = keys + (long long)blockIdx.y * Hkv * N + kk;
+  float acc[kE];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = h0 + j < Hkv ? p[(long long)(h0 + j) * N] : 0u;
+  for (int e = 0; e < kE; ++e) acc[e] = 0.f;
+  for (int h0 = 0; h0 < Hkv; h0 += kB) {
+    uint32_t v[kB][kE];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < kB; ++j) {
       if (h0 + j < Hkv) {
-        const float a = key_to_score(v[j]);
-        if (h0 + j == 0) acc = a;
-        else acc = (agg_head == KVC_AGG_MAX) ? fmaxf(acc, a) : __fadd_rn(acc, a);
+        if constexpr (kE == 4) {
+          const uint4 w = __ldg(reinterpret_cast<const uint4*>(p + (long long)(h0 + j) * N));
+          v[j][0] = w.x; v[j][1] = w.y; v[j][2] = w.z; v[j][3] = w.w;
+        } else {
+          v[j][0] = __ldg(p + (long long)(h0 + j) * N);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kB; ++j) {
+      if (h0 + j < Hkv) {
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+          const float a = key_to_score(v[j][e]);
+          if (h0 + j == 0) acc[e] = a;
+          else acc[e] = (agg_head == KVC_AGG_MAX) ? fmaxf(acc[e], a) : __fadd_rn(acc[e], a);
+        }
       }
     }
   }
-  if (agg_head == KVC_AGG_MEAN) acc = __fdiv_rn(acc, (float)Hkv);
-  composite[lb * N + kk] = acc;
+  float* out = composite + (long long)blockIdx.y * N + kk;
+#pragma unroll
+  for (int e = 0; e < kE; ++e) if (agg_head == KVC_AGG_MEAN) acc[e] = __fdiv_rn(acc[e], (float)Hkv);
+  if constexpr (kE == 4) *reinterpret_cast<float4*>(out) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  else *out = acc[0];
 }
 
 // Eq. 18 as fp32: the sorted keys turned back into scores.
-__global__ void sorted_scores_kernel(const uint32_t* __restrict__ keys, float* __restrict__ sorted, long long total) {
+__global__ void __launch_bounds__(256)
+sorted_scores_kernel(const uint32_t* __restrict__ keys, float* __restrict__ sorted, long long total) {
   grid_dependency_wait();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < total) sorted[i] = key_to_score(keys[i]);
+  const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * 4;       // (both arrays start on 256 bytes)
+  if (i + 4 <= total) {
+    const uint4 k = __ldg(reinterpret_cast<const uint4*>(keys + i));
+    *reinterpret_cast<float4*>(sorted + i) = make_float4(key_to_score(k.x), key_to_score(k.y), key_to_score(k.z), key_to_score(k.w));
+  } else {
+    for (long long j = i; j < total; ++j) sorted[j] = key_to_score(keys[j]);
+  }
 }
 
 }  // namespace
@@ -510,7 +535,7 @@ size_t compose_workspace_bytes(const Problem& P) { return sort_regions(P).total;
 kvc_status launch_sorted_scores(const Problem& P, const void* ws, float* sorted, cudaStream_t st) {
   const size_t items = (size_t)P.L * P.Bt * P.Hkv * P.N;
   const uint32_t* keys_b = reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(ws) + sort_regions(P).keys_b);
-  KVC_CUDA(launch_dependent(sorted_scores_kernel, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st,
+  KVC_CUDA(launch_dependent(sorted_scores_kernel, dim3((unsigned)((items + 1023) / 1024)), dim3(256), 0, st,
                             keys_b, sorted, (long long)items));
   KVC_LAUNCH_CHECK("sorted_scores_kernel");
   return KVC_OK;
@@ -569,8 +594,11 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
     }
   }
   if (composite == nullptr) return KVC_OK;      // ranking only (the unstructured variant has no Eq. 19)
-  KVC_CUDA(launch_dependent(compose_kernel, dim3((unsigned)((P.N + 255) / 256), (unsigned)(P.L * P.Bt)), dim3(256), 0, st,
-                            keys_b, composite, P.Hkv, P.N, P.agg_head));
+  const bool vec = P.N % 4 == 0 && (reinterpret_cast<uintptr_t>(composite) & 15u) == 0;
+  const long long per = vec ? 1024 : 256;
+  KVC_CUDA(launch_dependent(vec ? compose_kernel<4> : compose_kernel<1>,
+                            dim3((unsigned)((P.N + per - 1) / per), (unsigned)(P.L * P.Bt)), dim3(256), 0, st,
+                            (const uint32_t*)keys_b, composite, P.Hkv, P.N, P.agg_head));
   KVC_LAUNCH_CHECK("compose_kernel");
   return KVC_OK;
 }

@@ -124,58 +124,98 @@ order_kept_kernel(int32_t* __restrict__ idx, const int32_t* __restrict__ n_keep,
   }
 }
 
-// Head-sharded scoring: the local part of Eq. 16's sum over the KV heads, and the mean added back.
-__global__ void head_sum_kernel(const float* __restrict__ s, float* __restrict__ head_sum, int Hkv, long long N,
-                                long long total) {
+// Head-sharded scoring: the local part of Eq. 16's sum over the KV heads, and the mean added back.  Streams: a thread takes
+// four neighbouring tokens with 16-byte accesses where the rows allow it (kVec: N a multiple of 4), one otherwise;
+// blockIdx.y = (layer, sequence), so that no index has to be divided.  (32 layers, 2 heads, N = 32768, one token per thread and
+// a 64-bit division: 8.0 and 6.3 us, the scaling 3.9; so: 3.7, 3.8 and 2.2.)
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+head_sum_kernel(const float* __restrict__ s, float* __restrict__ head_sum, int Hkv, long long N) {
   grid_dependency_wait();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const long long lb = i / N, c = i - lb * N;
-  const float* base = s + lb * Hkv * N + c;
-  float sum = 0.f;
-  for (int h = 0; h < Hkv; ++h) sum += base[(long long)h * N];
-  head_sum[i] = sum;
+  const long long c = ((long long)blockIdx.x * 256 + threadIdx.x) * (kVec ? 4 : 1);
+  if (c >= N) return;
+  const float* base = s + (long long)blockIdx.y * Hkv * N + c;
+  if constexpr (kVec) {
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int h = 0; h < Hkv; ++h) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(base + (long long)h * N));
+      sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+    }
+    *reinterpret_cast<float4*>(head_sum + (long long)blockIdx.y * N + c) = sum;
+  } else {
+    float sum = 0.f;
+#pragma unroll 4
+    for (int h = 0; h < Hkv; ++h) sum += __ldg(base + (long long)h * N);
+    head_sum[(long long)blockIdx.y * N + c] = sum;
+  }
 }
 
-__global__ void add_head_mean_kernel(float* __restrict__ s, const float* __restrict__ head_sum, int Hkv, float inv_total,
-                                     long long N, long long total) {
+// (blockIdx.z: the head)
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+add_head_mean_kernel(float* __restrict__ s, const float* __restrict__ head_sum, int Hkv, float inv_total, long long N) {
   grid_dependency_wait();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const long long lb = i / N, c = i - lb * N;
-  float* base = s + lb * Hkv * N + c;
-  const float mean = head_sum[i] * inv_total;
-  for (int h = 0; h < Hkv; ++h) base[(long long)h * N] += mean;
+  const long long c = ((long long)blockIdx.x * 256 + threadIdx.x) * (kVec ? 4 : 1);
+  if (c >= N) return;
+  float* at = s + ((long long)blockIdx.y * Hkv + blockIdx.z) * N + c;
+  const float* sum = head_sum + (long long)blockIdx.y * N + c;
+  if constexpr (kVec) {
+    const float4 m = __ldg(reinterpret_cast<const float4*>(sum));
+    float4 v = *reinterpret_cast<const float4*>(at);
+    v.x += m.x * inv_total; v.y += m.y * inv_total; v.z += m.z * inv_total; v.w += m.w * inv_total;
+    *reinterpret_cast<float4*>(at) = v;
+  } else {
+    *at += __ldg(sum) * inv_total;
+  }
 }
 
-__global__ void scale_kernel(float* __restrict__ x, long long n, float f) {
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+scale_kernel(float* __restrict__ x, long long n, float f) {
   grid_dependency_wait();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] *= f;
+  const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * (kVec ? 4 : 1);
+  if (i >= n) return;
+  if constexpr (kVec) {
+    float4 v = *reinterpret_cast<const float4*>(x + i);
+    v.x *= f; v.y *= f; v.z *= f; v.w *= f;
+    *reinterpret_cast<float4*>(x + i) = v;
+  } else {
+    x[i] *= f;
+  }
 }
+
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
 
 kvc_status launch_head_sum(const Problem& P, const float* scores, float* head_sum, cudaStream_t st) {
-  const long long total = (long long)P.L * P.Bt * P.N;
-  KVC_CUDA(launch_dependent(head_sum_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, scores, head_sum,
-                            P.Hkv, P.N, total));
+  const bool vec = P.N % 4 == 0 && aligned16(scores) && aligned16(head_sum);
+  const long long per = vec ? 1024 : 256;
+  KVC_CUDA(launch_dependent(vec ? head_sum_kernel<true> : head_sum_kernel<false>,
+                            dim3((unsigned)((P.N + per - 1) / per), (unsigned)(P.L * P.Bt)), dim3(256), 0, st, scores, head_sum,
+                            P.Hkv, P.N));
   KVC_LAUNCH_CHECK("head_sum_kernel");
   return KVC_OK;
 }
 
 kvc_status launch_add_head_mean(const Problem& P, float* scores, const float* head_sum, int heads_total,
                                 cudaStream_t st) {
-  const long long total = (long long)P.L * P.Bt * P.N;
-  KVC_CUDA(launch_dependent(add_head_mean_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, scores,
-                            head_sum, P.Hkv, 1.0f / (float)heads_total, P.N, total));
+  const bool vec = P.N % 4 == 0 && aligned16(scores) && aligned16(head_sum);
+  const long long per = vec ? 1024 : 256;
+  KVC_CUDA(launch_dependent(vec ? add_head_mean_kernel<true> : add_head_mean_kernel<false>,
+                            dim3((unsigned)((P.N + per - 1) / per), (unsigned)(P.L * P.Bt), (unsigned)P.Hkv), dim3(256), 0, st,
+                            scores, head_sum, P.Hkv, 1.0f / (float)heads_total, P.N));
   KVC_LAUNCH_CHECK("add_head_mean_kernel");
   return KVC_OK;
 }
 
 kvc_status launch_scale(float* x, long long n, float f, cudaStream_t st) {
   if (n <= 0) return KVC_OK;
-  KVC_CUDA(launch_dependent(scale_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, x, n, f));
+  const bool vec = n % 4 == 0 && aligned16(x);
+  const long long per = vec ? 1024 : 256;
+  KVC_CUDA(launch_dependent(vec ? scale_kernel<true> : scale_kernel<false>, dim3((unsigned)((n + per - 1) / per)), dim3(256), 0, st,
+                            x, n, f));
   KVC_LAUNCH_CHECK("scale_kernel");
   return KVC_OK;
 }

@@ -123,3 +123,36 @@ def test_ranking_at_the_switches_of_the_cta_size(N):
     torch.cuda.synchronize()
     Pz.assert_rank_exact(S, idx.cpu().numpy())
     Pz.assert_compose_exact(S, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
+
+
+@pytest.mark.parametrize("N", [1, 1023, 1024, 1030])
+@pytest.mark.parametrize("Hkv", [1, 9])
+def test_streams_of_the_head_sharded_pass_and_composite(N, Hkv):
+    """Rows that allow 16-byte accesses and rows that do not, more heads than one batch of loads.  The sums are taken in
+    head order (exact); the added mean is one product and one sum, possibly fused: one rounding more or less."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    L, Bt = 2, 3
+    desc = kvc.kvc_desc_init(L, Bt, Hkv, Hkv, 64, N, 1, kvc.F32)
+    S = np.random.default_rng(N).random((L, Bt, Hkv, N), dtype=np.float32)
+    scores = torch.from_numpy(S).to(dev)
+    head_sum = torch.empty((L, Bt, N), dtype=torch.float32, device=dev)
+    kvc.kvc_head_sum(desc, scores, head_sum)
+    want = np.zeros((L, Bt, N), dtype=np.float32)
+    for h in range(Hkv):
+        want += S[:, :, h]
+    assert np.array_equal(head_sum.cpu().numpy(), want)
+    kvc.kvc_add_head_mean(desc, scores, head_sum, 2 * Hkv)
+    want_s = S.astype(np.float64) + want[:, :, None].astype(np.float64) / (2 * Hkv)
+    assert np.allclose(scores.cpu().numpy(), want_s, rtol=3 * 2.0 ** -24, atol=0)
+    kvc.kvc_scale(head_sum, 0.5)
+    assert np.array_equal(head_sum.cpu().numpy(), want * np.float32(0.5))
+    idx = torch.empty((L, Bt, Hkv, N), dtype=torch.int32, device=dev)
+    comp = torch.empty((L, Bt, N), dtype=torch.float32, device=dev)
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+    kvc.kvc_compose(desc, scores, idx, comp, ws)
+    torch.cuda.synchronize()
+    s = scores.cpu().numpy()
+    Pz.assert_rank_exact(s, idx.cpu().numpy())
+    Pz.assert_compose_exact(s, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
