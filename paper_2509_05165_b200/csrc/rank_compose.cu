@@ -347,12 +347,19 @@ __device__ __forceinline__ int merge_path_warp(int diag, int na, int nb, const u
   return lo;
 }
 
+// Bound by the latencies of a tile (split search, loads, merge) at four CTAs per SM; a thread reads one key per output, the
+// successor of the one it took.  (Both runs' heads at every step and outputs written to shared memory at a stride of 8:
+// the ranking of 28 segments of 131072, two levels, 118 -> 101 us; with 256 threads of 16 outputs 110, with 1024 of 4 109.)
+// kVec: rows start on 16 bytes (N a multiple of 4): a thread stores its outputs itself, 16 bytes at a time.  Otherwise
+// they go through shared memory once more; a tile's element i sits in slot i + i / kMergeItems there, so that the threads'
+// stretches begin in different banks.
+template <bool kVec>
 __global__ void __launch_bounds__(kMergeThreads)
 merge_runs_kernel(const uint32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in,
                   uint32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out, long long seg_len, long long run,
                   int tiles_per_seg) {
-  __shared__ uint32_t s_key[kMergeTile];
-  __shared__ int32_t s_val[kMergeTile];
+  __shared__ uint32_t s_key[kMergeTile + kMergeThreads];
+  __shared__ int32_t s_val[kMergeTile + kMergeThreads];
   __shared__ int s_split[2];
   grid_dependency_wait();
   const long long seg = blockIdx.x / (unsigned)tiles_per_seg;
@@ -374,36 +381,57 @@ merge_runs_kernel(const uint32_t* __restrict__ keys_in, const int32_t* __restric
   const int a0 = s_split[0], a1 = s_split[1];
   const int b0 = d0 - a0, b1 = d1 - a1;
   const int ca = a1 - a0, cb = b1 - b0;                   // this tile's elements of A, then of B, in shared memory
-  for (int i = tid; i < ca + cb; i += kMergeThreads) {
-    const long long src = base + (i < ca ? (long long)a0 + i : (long long)na + b0 + (i - ca));
-    s_key[i] = keys_in[src];
-    s_val[i] = vals_in[src];
+#pragma unroll
+  for (int k = 0; k < kMergeItems; ++k) {
+    const int i = tid + k * kMergeThreads;
+    if (i < ca + cb) {
+      const long long src = base + (i < ca ? (long long)a0 + i : (long long)na + b0 + (i - ca));
+      s_key[i] = __ldg(keys_in + src);
+      s_val[i] = __ldg(vals_in + src);
+    }
   }
   __syncthreads();
   const int n_out = d1 - d0;
   const int my0 = min(tid * kMergeItems, n_out);
   int ia = merge_path(my0, ca, cb, s_key, s_key + ca);
-  int ib = my0 - ia;
+  int ib = ca + my0 - ia;                                  // (slot of B's next element)
+  const int end_b = ca + cb;
   uint32_t ok[kMergeItems]; int32_t ov[kMergeItems];
+  uint32_t xa = ia < ca ? s_key[ia] : 0xffffffffu, xb = ib < end_b ? s_key[ib] : 0xffffffffu;
 #pragma unroll
   for (int k = 0; k < kMergeItems; ++k) {
-    const bool has_a = ia < ca, has_b = ib < cb;
-    const uint32_t xa = has_a ? s_key[ia] : 0xffffffffu, xb = has_b ? s_key[ca + ib] : 0xffffffffu;
-    const bool take_a = has_a && (!has_b || xa <= xb);
+    const bool take_a = ia < ca && (ib >= end_b || xa <= xb);
     ok[k] = take_a ? xa : xb;
-    ov[k] = take_a ? s_val[ia] : (has_b ? s_val[ca + ib] : 0);
-    if (take_a) ++ia; else ++ib;
+    const int at = take_a ? ia : ib;                       // the next element of the run it came from
+    ov[k] = at < end_b ? s_val[at] : 0;
+    const int nx = at + 1, lim = take_a ? ca : end_b;
+    const uint32_t x = nx < lim ? s_key[nx] : 0xffffffffu;
+    if (take_a) { ia = nx; xa = x; } else { ib = nx; xb = x; }
   }
-  __syncthreads();                                         // everyone has read its inputs: the buffers take the outputs
-#pragma unroll
-  for (int k = 0; k < kMergeItems; ++k) {
-    if (my0 + k < n_out) { s_key[my0 + k] = ok[k]; s_val[my0 + k] = ov[k]; }
-  }
-  __syncthreads();
   const long long dst = base + d0;
-  for (int i = tid; i < n_out; i += kMergeThreads) {
-    keys_out[dst + i] = s_key[i];
-    vals_out[dst + i] = s_val[i];
+  if (kVec) {
+    if (my0 + kMergeItems <= n_out) {
+#pragma unroll
+      for (int k = 0; k < kMergeItems; k += 4) {
+        *reinterpret_cast<uint4*>(keys_out + dst + my0 + k) = make_uint4(ok[k], ok[k + 1], ok[k + 2], ok[k + 3]);
+        *reinterpret_cast<int4*>(vals_out + dst + my0 + k) = make_int4(ov[k], ov[k + 1], ov[k + 2], ov[k + 3]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kMergeItems; ++k)
+        if (my0 + k < n_out) { keys_out[dst + my0 + k] = ok[k]; vals_out[dst + my0 + k] = ov[k]; }
+    }
+  } else {
+    __syncthreads();                                       // everyone has read its inputs: the buffers take the outputs
+    const int slot0 = tid * (kMergeItems + 1);
+#pragma unroll
+    for (int k = 0; k < kMergeItems; ++k) { s_key[slot0 + k] = ok[k]; s_val[slot0 + k] = ov[k]; }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kMergeItems; ++k) {
+      const int i = tid + k * kMergeThreads, slot = i + i / kMergeItems;
+      if (i < n_out) { keys_out[dst + i] = s_key[slot]; vals_out[dst + i] = s_val[slot]; }
+    }
   }
 }
 
@@ -585,7 +613,7 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
       in_b = !in_b;
       uint32_t* k_nxt = in_b ? keys_b : keys_a;
       int32_t* v_nxt = in_b ? idx : vals_a;
-      KVC_CUDA(launch_dependent(merge_runs_kernel, dim3((unsigned)(segments * merge_tiles)), dim3(kMergeThreads), 0, st,
+      KVC_CUDA(launch_dependent(P.N % 4 == 0 ? merge_runs_kernel<true> : merge_runs_kernel<false>, dim3((unsigned)(segments * merge_tiles)), dim3(kMergeThreads), 0, st,
                                 (const uint32_t*)k_cur, (const int32_t*)v_cur, k_nxt, v_nxt, P.N,
                                 (long long)kSegMaxN << level, (int)merge_tiles));
       KVC_LAUNCH_CHECK("merge_runs_kernel");
