@@ -120,13 +120,13 @@ __device__ __forceinline__ void seg_for_keys(const float* s_in, int N, int tid, 
 template <int T, int kIpt>
 __global__ void __launch_bounds__(T, 1024 / T)
 segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ keys_out,
-                    int32_t* __restrict__ idx_out, long long seg_len, int chunks) {
-  // CTA x sorts chunk x % chunks of segment x / chunks: the positions from chunk * kSegMaxN on (a segment of
-  // up to kSegMaxN elements is one chunk; the chunks of a longer one are merged afterwards)
+                    int32_t* __restrict__ idx_out, long long seg_len, int chunks, int chunk_len) {
+  // CTA x sorts chunk x % chunks of segment x / chunks: the positions from chunk * chunk_len on (the chunks of a
+  // segment of several are merged afterwards)
   const long long seg = blockIdx.x / (unsigned)chunks;
   const int chunk = (int)(blockIdx.x - seg * chunks);
-  const long long first = seg * seg_len + (long long)chunk * kSegMaxN;      // of this chunk, in all three arrays
-  const int N = (int)min((long long)kSegMaxN, seg_len - (long long)chunk * kSegMaxN);
+  const long long first = seg * seg_len + (long long)chunk * chunk_len;     // of this chunk, in all three arrays
+  const int N = (int)min((long long)chunk_len, seg_len - (long long)chunk * chunk_len);
   constexpr int kRowShift = T == 1024 ? 12 : T == 512 ? 11 : T == 256 ? 10 : 9;   // log2 of a row of counters in bytes
   static_assert((4 * T) >> kRowShift == 1 && kIpt % 8 == 0 && kIpt <= 32, "rows of counters, groups of places");
   constexpr int kScanWarps = T / 64;                        // the scan runs on the first T / 2 threads
@@ -297,7 +297,7 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   // ---- out: the positions (a slot's position is key_slot of it: the map is its own inverse), and the keys
   uint32_t* k_out = keys_out + first;
   int32_t* i_out = idx_out + first;
-  const int pos0 = chunk * kSegMaxN;
+  const int pos0 = chunk * chunk_len;
   for (int j = tid; j < N; j += T) {
     const uint32_t q = lds_u16(perm + place_slot((uint32_t)j) * 2u);
     i_out[j] = pos0 + (int32_t)key_slot(q);
@@ -306,8 +306,8 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
 }
 
 // ---------------------------------------------------------------------------------------------
-// Segments longer than kSegMaxN: their chunks come sorted from segment_sort_kernel and are merged
-// pairwise, level by level (runs of kSegMaxN << level elements).  A CTA produces kMergeTile
+// Segments of several chunks (see chunking): the chunks come sorted from segment_sort_kernel and are merged
+// pairwise, level by level (runs of the chunks' length << level).  A CTA produces kMergeTile
 // consecutive outputs of one pair of runs A, B: it finds where the tile's first and last output
 // split between A and B (the merge path: a binary search over one diagonal each), brings the two
 // stretches into shared memory, and every thread merges kMergeItems consecutive outputs from its
@@ -498,7 +498,7 @@ sorted_scores_kernel(const uint32_t* __restrict__ keys, float* __restrict__ sort
 
 }  // namespace
 
-typedef void (*SegmentSort)(const float*, uint32_t*, int32_t*, long long, int);
+typedef void (*SegmentSort)(const float*, uint32_t*, int32_t*, long long, int, int);
 struct SegmentPlan {
   SegmentSort kernel;
   int threads;
@@ -545,6 +545,25 @@ static kvc_status segment_sort_prepare(long long N, SegmentPlan* plan) {
   return KVC_OK;
 }
 
+// How segments are cut into chunks: as few as fit an SM each, but while there are no more chunks than half of the SMs
+// (a rank's share of the heads, or a few layers), twice as many, down to 8192 elements: the SMs that would idle take
+// part, for one merge level more.  64 segments of 32768: 59 us as they are, 47 in halves; 8 of 131072: 77 -> 61.
+// (A constant stands for the SMs: the workspace must not depend on the device.)
+struct Chunking {
+  long long len;
+  int count;
+};
+static Chunking chunking(const Problem& P) {
+  constexpr long long kSms = 148;
+  const long long segments = (long long)P.L * P.Bt * P.Hkv;
+  long long c = (P.N + kSegMaxN - 1) / kSegMaxN;
+  const long long least = c;
+  while (segments * c * 2 <= kSms && P.N > c * 8192) c *= 2;
+  if (c == least) return {P.N < kSegMaxN ? P.N : (long long)kSegMaxN, (int)c};
+  const long long len = ((P.N + c - 1) / c + kMergeTile / 2 - 1) / (kMergeTile / 2) * (kMergeTile / 2);   // pairs of runs hold whole tiles
+  return {len, (int)((P.N + len - 1) / len)};
+}
+
 // Scratch of the ranking: the sorted keys [L, Bt, Hkv, N] and, for segments of several chunks, one more
 // buffer of keys and one of positions for the merge levels to alternate with (keys, idx).
 struct SortRegions {
@@ -553,7 +572,7 @@ struct SortRegions {
 static SortRegions sort_regions(const Problem& P) {
   const size_t region = align_up((size_t)P.L * P.Bt * P.Hkv * P.N * 4);
   SortRegions r;
-  if (P.N <= kSegMaxN) { r.keys_a = r.vals_a = 0; r.keys_b = 0; r.total = region; }
+  if (chunking(P).count == 1) { r.keys_a = r.vals_a = 0; r.keys_b = 0; r.total = region; }
   else { r.keys_a = 0; r.vals_a = region; r.keys_b = 2 * region; r.total = 3 * region; }
   return r;
 }
@@ -582,7 +601,8 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
   uint32_t* const keys_b = reinterpret_cast<uint32_t*>(w + reg.keys_b);
   const long long segments = (long long)P.L * P.Bt * P.Hkv;
   SegmentPlan plan;
-  const long long chunk_len = P.N < kSegMaxN ? P.N : (long long)kSegMaxN;
+  const Chunking cut = chunking(P);
+  const long long chunk_len = cut.len;
   const kvc_status seg_state = segment_sort_prepare(chunk_len, &plan);
   if (seg_state != KVC_OK && seg_state != KVC_ERR_UNSUPPORTED) return seg_state;
   if (seg_state != KVC_OK) {
@@ -591,10 +611,10 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
     return KVC_ERR_UNSUPPORTED;
   }
   {
-    // Chunks of up to kSegMaxN elements are sorted inside one SM each: a whole segment in one launch, or,
+    // Chunks are sorted inside one SM each: a whole segment in one launch, or,
     // for longer segments, its chunks, which are then merged pairwise, level by level.  The levels
     // alternate between (keys_a, vals_a) and (keys_b, idx); the last one has to end in the latter.
-    const long long chunks = (P.N + kSegMaxN - 1) / kSegMaxN;
+    const long long chunks = cut.count;
     int levels = 0;
     while ((1LL << levels) < chunks) ++levels;
     const long long merge_tiles = (P.N + kMergeTile - 1) / kMergeTile;
@@ -607,7 +627,8 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
     int32_t* v_cur = in_b ? idx : vals_a;
     const size_t smem = seg_layout(chunk_len, plan.threads).total;
     const unsigned grid = (unsigned)(segments * chunks);
-    KVC_CUDA(launch_dependent(plan.kernel, dim3(grid), dim3(plan.threads), smem, st, scores, k_cur, v_cur, P.N, (int)chunks));
+    KVC_CUDA(launch_dependent(plan.kernel, dim3(grid), dim3(plan.threads), smem, st, scores, k_cur, v_cur, P.N, (int)chunks,
+                              (int)chunk_len));
     KVC_LAUNCH_CHECK("segment_sort_kernel");
     for (int level = 0; level < levels; ++level) {
       in_b = !in_b;
@@ -615,7 +636,7 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
       int32_t* v_nxt = in_b ? idx : vals_a;
       KVC_CUDA(launch_dependent(P.N % 4 == 0 ? merge_runs_kernel<true> : merge_runs_kernel<false>, dim3((unsigned)(segments * merge_tiles)), dim3(kMergeThreads), 0, st,
                                 (const uint32_t*)k_cur, (const int32_t*)v_cur, k_nxt, v_nxt, P.N,
-                                (long long)kSegMaxN << level, (int)merge_tiles));
+                                chunk_len << level, (int)merge_tiles));
       KVC_LAUNCH_CHECK("merge_runs_kernel");
       k_cur = k_nxt;
       v_cur = v_nxt;
