@@ -249,7 +249,8 @@ score_emit_kernel(ScoreParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp,
 // warp and chunk), so the scores are the same bit for bit.  fp32, 16 layers, N = 3001, 32 / 8 heads of 128, w = 32:
 // 1342 us for the two sweeps, 424 us so (the product 335; it cannot take less than 175: 128 multiply-adds a clock and
 // SM).  A larger buffer (96 MB) gains 1 %, smaller ones mean more and shorter launches.
-constexpr int kTileTok = 128, kTileRow = 128, kLogitThreads = 256;
+constexpr int kTileTok = 128, kLogitThreads = 256;
+template <int kTT> constexpr int kLogitTileRows = kTT == 8 ? 128 : 32;
 constexpr size_t kLogitsCap = (size_t)64 << 20;
 constexpr int kMaxLogitChunks = 1024;           // the statistics of a row's chunks meet in shared memory
 
@@ -289,19 +290,22 @@ __device__ __forceinline__ void stage4(float* dst, const __nv_bfloat16* row, int
 // are what a smaller register tile would wait for: an 8-byte read costs the SM 2 clocks where neighbouring lanes read
 // different addresses (the 8 tokens) and 1 where they share one (the 8 rows), 96 for four warps' steps.  (4 x 4 logits
 // with all four products at once: 423 us in the case above.)  Rows are padded by 16 bytes to spread a read over the banks.
-template <typename T, int D>
+// kTT = 2: two tokens per thread, items of 32 rows, for units of few rows and for problems that would leave SMs idle (the tiny
+// fp32 configuration: 8.2 -> 5.7 us).
+template <typename T, int D, int kTT>
 __global__ void __launch_bounds__(kLogitThreads, 1)
 score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, float* __restrict__ dots, int row_tiles,
                     int tok_tiles, int items, int* __restrict__ status) {
-  constexpr int kPitch = D + 4, kVec = D / 4;
+  constexpr int kPitch = D + 4, kVec = D / 4, kTileRow = kLogitTileRows<kTT>;
+  constexpr int kTokGroups = kTileTok / (8 * kTT);             // warps side by side over the tokens
   extern __shared__ __align__(16) float gsm[];
   float* const Qs = gsm;
   float* const Ks = gsm + kTileRow * kPitch;                   // two buffers
   grid_dependency_wait();
   if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;      // (nothing here can fail on the device)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int tok = (warp & 1) * 64 + (lane & 7);               // tokens tok + 8 i
-  const int row = (warp >> 1) * 32 + (lane >> 3);             // rows row + 4 j
+  const int tok = (warp % kTokGroups) * (8 * kTT) + (lane & 7);   // tokens tok + 8 i
+  const int row = (warp / kTokGroups) * 32 + (lane >> 3);     // rows row + 4 j
   const int i0 = (int)((long long)items * blockIdx.x / gridDim.x), i1 = (int)((long long)items * (blockIdx.x + 1) / gridDim.x);
   auto load_k = [&](int item, float* dst) {
     const int ur = item / tok_tiles, tt = item - ur * tok_tiles;
@@ -339,32 +343,32 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 1;" ::: "memory");       // all but the next item's tile
     __syncthreads();
-    if (r0 + (warp >> 1) * 32 < rows) {
+    if (r0 + (warp / kTokGroups) * 32 < rows) {
       const float* kq = buf + tok * kPitch;
       const float* qq = Qs + row * kPitch;
-      unsigned long long acc[8][8];                            // [token][row]: two partial products
-      float first[8][8];                                       // the sum of the first two
+      unsigned long long acc[kTT][8];                            // [token][row]: two partial products
+      float first[kTT][8];                                       // the sum of the first two
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < kTT; ++i)
 #pragma unroll
           for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
 #pragma unroll 4
         for (int v = 0; v < kVec; ++v) {
-          unsigned long long kv[8];
+          unsigned long long kv[kTT];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) kv[i] = *reinterpret_cast<const unsigned long long*>(kq + i * 8 * kPitch + 4 * v + 2 * half);
+          for (int i = 0; i < kTT; ++i) kv[i] = *reinterpret_cast<const unsigned long long*>(kq + i * 8 * kPitch + 4 * v + 2 * half);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const unsigned long long qv = *reinterpret_cast<const unsigned long long*>(qq + j * 4 * kPitch + 4 * v + 2 * half);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i][j] = ffma2(qv, kv[i], acc[i][j]);
+            for (int i = 0; i < kTT; ++i) acc[i][j] = ffma2(qv, kv[i], acc[i][j]);
           }
         }
         if (half == 0) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
+          for (int i = 0; i < kTT; ++i)
 #pragma unroll
             for (int j = 0; j < 8; ++j) { const float2 x = unpack_f2(acc[i][j]); first[i][j] = x.x + x.y; }
         }
@@ -375,7 +379,7 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
       for (int j = 0; j < 8; ++j) {
         if (r0 + row + 4 * j < rows) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
+          for (int i = 0; i < kTT; ++i) {
             const float2 y = unpack_f2(acc[i][j]);
             if (t0 + 8 * i < P.N) out[(long long)(4 * j) * P.np + 8 * i] = first[i][j] + (y.x + y.y);
           }
@@ -718,11 +722,12 @@ LogitPlan logit_plan(const Problem& P) {
   return p;
 }
 
-template <typename T, int D>
-kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
+template <typename T, int D, int kTT>
+kvc_status run_logits_t(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
                       const LogitPlan& pl, char* ws, int* device_status, cudaStream_t st) {
+  constexpr int kTileRow = kLogitTileRows<kTT>;
   constexpr int kSmem = (2 * kTileTok + kTileRow) * (D + 4) * (int)sizeof(float);
-  KVC_CUDA(cudaFuncSetAttribute(score_logits_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+  KVC_CUDA(cudaFuncSetAttribute(score_logits_kernel<T, D, kTT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
   int dev = 0, sms = 0;
   KVC_CUDA(cudaGetDevice(&dev));
   KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -746,7 +751,7 @@ kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, 
     const unsigned n = (unsigned)(pl.units - u0 < pl.units_per_group ? pl.units - u0 : pl.units_per_group);
     lp.unit0 = (int)u0;
     const long long items = (long long)n * row_tiles * tok_tiles;
-    KVC_CUDA(launch_dependent(score_logits_kernel<T, D>, dim3((unsigned)(items < sms ? items : sms)), dim3(kLogitThreads),
+    KVC_CUDA(launch_dependent(score_logits_kernel<T, D, kTT>, dim3((unsigned)(items < sms ? items : sms)), dim3(kLogitThreads),
                               (size_t)kSmem, st, lp, gm, q, k, dots, row_tiles, tok_tiles, (int)items, device_status));
     KVC_LAUNCH_CHECK("score_logits_kernel");
     KVC_CUDA(launch_dependent(score_row_stats_kernel, dim3((unsigned)((pl.max_rows + 3) / 4), n), dim3(kRowStatWarps * 32),
@@ -758,6 +763,16 @@ kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, 
     KVC_LAUNCH_CHECK("score_emit_logits_kernel");
   }
   return KVC_OK;
+}
+
+template <typename T, int D>
+kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
+                      const LogitPlan& pl, char* ws, int* device_status, cudaStream_t st) {
+  // (in items of 32 rows the product reads twice the operands per multiply-add: only where items of 128 rows would be mostly
+  // empty or fewer than the SMs)
+  const long long items = (long long)pl.units_per_group * ((pl.max_rows + 127) / 128) * ((P.N + kTileTok - 1) / kTileTok);
+  if (pl.max_rows <= 32 || items < 148) return run_logits_t<T, D, 2>(P, gm, q, k, scores, pl, ws, device_status, st);
+  return run_logits_t<T, D, 8>(P, gm, q, k, scores, pl, ws, device_status, st);
 }
 
 }  // namespace
