@@ -9,9 +9,16 @@ namespace {
 // 256-byte rows of a bf16 head of 128), so a warp carries 32 / kLpr rows at a time and every lane loads; each lane has
 // kNormRows such rows in flight (one 16-byte load each) before it adds anything, and a warp's rows are consecutive, so
 // that its norms leave in one store.  A warp per row with half of its lanes idle and one load in flight took 807 us for
-// 1.07 GB (1.3 TB/s); this form takes 194 us (5.5 TB/s).  The squares are added in the order they always were:
-// a lane's elements in ascending order, then the lanes by halving distances.
+// 1.07 GB (1.3 TB/s); this form takes 182 us (5.9 TB/s; 191 with plain loads, 4 rows per lane 192).  The squares are
+// added in the order they always were: a lane's elements in ascending order, then the lanes by halving distances.
 constexpr int kNormRows = 8;
+// (a stream: past L1, L2 fetches 256 bytes at a time)
+__device__ __forceinline__ uint4 ld_once(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
 
 template <typename T, int kLpr>
 __global__ void __launch_bounds__(256)
@@ -31,7 +38,7 @@ value_norm_kernel(LayerPtrs vp, float* __restrict__ vnorm, int Bt, int Hkv, long
 #pragma unroll
     for (int u = 0; u < kNormRows; ++u) {
       const long long c = min(row0 + u * kGroups, N - 1);
-      w[u] = __ldg(reinterpret_cast<const uint4*>(base + c * vs2) + sub);
+      w[u] = ld_once(reinterpret_cast<const uint4*>(base + c * vs2) + sub);
     }
     float mine = 0.f;
 #pragma unroll
