@@ -33,9 +33,11 @@ namespace {
 //   scatter  position -> place = first place + rank.  Every thread read all of its places
 //            before the scan, so the permutation is overwritten in place.
 // (thread, place inside the thread) is the order itself, so every pass is stable, and with the
-// identity as the first order equal keys stay in ascending position.  A digit that all keys of
-// the segment share orders nothing and its pass is left out (scores in [2^-31, 2) share the
-// top one).  After the last pass positions and keys go out through the permutation, coalesced.
+// identity as the first order equal keys stay in ascending position.  The keys are taken relative to the
+// segment's smallest, and a digit that none of them has a bit in orders nothing: its pass is left
+// out (scores within a factor of 32 differ in 7 of the 8 digits, scores within 2 % in 5: 256 segments of
+// 32768 of nearly uniform attention 109 -> 98 us; where no digit falls away the extra step costs
+// 1 us).  After the last pass positions and keys go out through the permutation, coalesced.
 // Global traffic: scores read once, idx and sorted keys written once; one launch.
 constexpr int kSegMaxN = 32768;
 constexpr int kSegBatch = 4;                   // key lookups in flight per thread
@@ -61,7 +63,7 @@ struct SegLayout {
   uint32_t keys;        // uint32[n_pad]: the keys, by position
   uint32_t perm;        // uint16[n_pad]: the key slot (key_slot of the position) at every place
   uint32_t cnt;         // uint16[8][T][2]: thread t's counter of digit d in row d & 7, half d >> 3
-  uint32_t wtot;        // uint32[32]: the scan's warp totals;  uint32: bits that differ between keys
+  uint32_t wtot;        // uint32[64]: the scan's warp totals; before, the warps' smallest keys and the bits set in theirs
   uint32_t total;
 };
 __host__ __device__ inline SegLayout seg_layout(long long N, int T) {
@@ -89,32 +91,26 @@ __device__ __forceinline__ uint32_t seg_key(float f) {
   return ~(b ^ m);
 }
 
-// Every group of 4 consecutive keys of the segment goes to use(i, k0, k1, k2, k3, n): i = position
-// of the first (a multiple of 4), n = how many of the 4 exist.  With 16-byte aligned scores all of
-// a thread's loads are issued before the first use.
-template <int T, int kIpt, typename F>
-__device__ __forceinline__ void seg_for_keys(const float* s_in, int N, int tid, F use) {
+// The thread's keys of the segment, in groups of 4 neighbours: group g holds positions (g * T + tid) * 4 ..  All loads are
+// issued before the first use; 16 bytes at a time where the scores are aligned.  Positions behind the end get key 0.
+template <int T, int kIpt>
+__device__ __forceinline__ void seg_load_keys(const float* s_in, int N, int tid, uint32_t (&k)[kIpt]) {
   constexpr int kGroups = kIpt / 4;
-  const bool wide = (reinterpret_cast<uintptr_t>(s_in) & 15u) == 0 && N >= 4;
-  if (wide) {
-    const int last = (N & ~3) - 4;                           // first position of the last whole group
-    float4 v[kGroups];
+  const bool wide = (reinterpret_cast<uintptr_t>(s_in) & 15u) == 0;
+  float v[kIpt];
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) v[g] = *reinterpret_cast<const float4*>(s_in + min((g * T + tid) * 4, last));
+  for (int g = 0; g < kGroups; ++g) {
+    const int i = (g * T + tid) * 4;
+    if (wide && i + 4 <= N) {
+      const float4 w = *reinterpret_cast<const float4*>(s_in + i);
+      v[4 * g] = w.x; v[4 * g + 1] = w.y; v[4 * g + 2] = w.z; v[4 * g + 3] = w.w;
+    } else {
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-      const int i = (g * T + tid) * 4;
-      if (i + 4 <= N) use(i, seg_key(v[g].x), seg_key(v[g].y), seg_key(v[g].z), seg_key(v[g].w), 4);
+      for (int e = 0; e < 4; ++e) v[4 * g + e] = s_in[min(i + e, N - 1)];
     }
-    if (tid == 0 && (N & 3)) {
-      const int i = N & ~3;
-      use(i, seg_key(s_in[i]), seg_key(i + 1 < N ? s_in[i + 1] : 0.f), seg_key(i + 2 < N ? s_in[i + 2] : 0.f), seg_key(0.f), N - i);
-    }
-  } else {
-    for (int i = tid * 4; i < N; i += T * 4)
-      use(i, seg_key(s_in[i]), seg_key(i + 1 < N ? s_in[i + 1] : 0.f), seg_key(i + 2 < N ? s_in[i + 2] : 0.f),
-          seg_key(i + 3 < N ? s_in[i + 3] : 0.f), min(4, N - i));
   }
+#pragma unroll
+  for (int j = 0; j < kIpt; ++j) k[j] = (((j >> 2) * T + tid) * 4 + (j & 3)) < N ? seg_key(v[j]) : 0u;
 }
 
 template <int T, int kIpt>
@@ -147,22 +143,31 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   grid_dependency_wait();
   const float* s_in = scores + first;
 
-  // ---- the keys, once; the identity as the first order; which bits differ anywhere in the segment
-  uint32_t diff = 0;
+  // ---- the keys, once, relative to the smallest of the segment: scores that lie close together then share their upper
+  //      digits, on whichever side of a power of two they lie.  The identity as the first order; which bits are set anywhere
+  uint32_t diff = 0, kmin = 0xffffffffu;
   {
-    const uint32_t ref = seg_key(s_in[0]);
-    if (tid == 0) sts_u32(wtot + 128, 0u);
-    seg_for_keys<T, kIpt>(s_in, N, tid, [&](int i, uint32_t k0, uint32_t k1, uint32_t k2, uint32_t k3, int n) {
-      const uint32_t sw = ((uint32_t)i >> 5) & 31u;          // the four stay inside their 16 bytes; the table is padded
-      sts_u32(keys + (((uint32_t)i) ^ sw) * 4u, k0);
-      sts_u32(keys + (((uint32_t)i + 1u) ^ sw) * 4u, k1);
-      sts_u32(keys + (((uint32_t)i + 2u) ^ sw) * 4u, k2);
-      sts_u32(keys + (((uint32_t)i + 3u) ^ sw) * 4u, k3);
-      diff |= k0 ^ ref;
-      if (n > 1) diff |= k1 ^ ref;
-      if (n > 2) diff |= k2 ^ ref;
-      if (n > 3) diff |= k3 ^ ref;
-    });
+    uint32_t k[kIpt];
+    seg_load_keys<T, kIpt>(s_in, N, tid, k);
+#pragma unroll
+    for (int j = 0; j < kIpt; ++j) if ((((j >> 2) * T + tid) * 4 + (j & 3)) < N) kmin = min(kmin, k[j]);
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    if (lane == 0) sts_u32(wtot + warp * 4, kmin);
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, lane < T / 32 ? lds_u32(wtot + lane * 4) : 0xffffffffu);
+#pragma unroll
+    for (int g = 0; g < kIpt / 4; ++g) {
+      const int i = (g * T + tid) * 4;
+      if (i < N) {
+        const uint32_t sw = ((uint32_t)i >> 5) & 31u;        // the four stay inside their 16 bytes; the table is padded
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t rel = k[4 * g + e] - kmin;
+          sts_u32(keys + (((uint32_t)(i + e)) ^ sw) * 4u, rel);
+          if (i + e < N) diff |= rel;
+        }
+      }
+    }
     // (the permutation holds key slots, not positions: a lookup needs no translation)
 #pragma unroll
     for (int q = 0; q < kIpt / 8; ++q) {
@@ -176,10 +181,9 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
       }
     }
     diff = __reduce_or_sync(0xffffffffu, diff);
+    if (lane == 0) sts_u32(wtot + 128 + warp * 4, diff);
     __syncthreads();
-    if (lane == 0 && diff != 0) atomicOr(reinterpret_cast<uint32_t*>(seg_smem + lay.wtot + 128), diff);
-    __syncthreads();
-    diff = lds_u32(wtot + 128);
+    diff = __reduce_or_sync(0xffffffffu, lane < T / 32 ? lds_u32(wtot + 128 + lane * 4) : 0u);
   }
 
 #pragma unroll 1
@@ -301,7 +305,7 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   for (int j = tid; j < N; j += T) {
     const uint32_t q = lds_u16(perm + place_slot((uint32_t)j) * 2u);
     i_out[j] = pos0 + (int32_t)key_slot(q);
-    k_out[j] = lds_u32(keys + q * 4u);
+    k_out[j] = lds_u32(keys + q * 4u) + kmin;
   }
 }
 
