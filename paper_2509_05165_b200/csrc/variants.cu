@@ -77,15 +77,19 @@ kvc_status launch_norm_t(const Problem& P, const LayerPtrs& v, float* vnorm, cud
   return KVC_OK;
 }
 
-// One CTA per (layer, sequence, head): marks the kept positions in a bitmap (global scratch, one
-// bit per token), then writes the marked positions back in ascending order.
+// One CTA per (layer, sequence, head): marks the kept positions in a bitmap (one bit per token; in shared memory up to
+// kOrderSharedN tokens, else in global scratch), then writes the marked positions back in ascending order.  Bound by latency:
+// marks in shared memory do not travel to L2 (256 heads of 16384, a quarter kept: 13.7 -> 8.6 us).
 constexpr int kOrderThreads = 512;
+constexpr long long kOrderSharedN = 262144;   // 32 KB of marks: the most that leaves every SM room for several CTAs
 
+template <bool kShared>
 __global__ void __launch_bounds__(kOrderThreads)
 order_kept_kernel(int32_t* __restrict__ idx, const int32_t* __restrict__ n_keep, uint32_t* __restrict__ bitmap,
                   int L, int Bt, int Hkv, long long N, int per_head) {
   __shared__ uint32_t warp_tot[kOrderThreads / 32];
   __shared__ uint32_t carry;
+  extern __shared__ uint32_t order_bits[];
   grid_dependency_wait();
   const long long seg = blockIdx.x;                   // (l * Bt + b) * Hkv + h
   const int h = (int)(seg % Hkv);
@@ -94,12 +98,15 @@ order_kept_kernel(int32_t* __restrict__ idx, const int32_t* __restrict__ n_keep,
   const long long n = per_head ? n_keep[((long long)b * L + l) * Hkv + h] : n_keep[(long long)b * L + l];
   int32_t* row = idx + seg * N;
   const long long words = (N + 31) / 32;
-  uint32_t* bits = bitmap + seg * words;
+  uint32_t* bits = kShared ? order_bits : bitmap + seg * words;
   for (long long i = threadIdx.x; i < words; i += kOrderThreads) bits[i] = 0u;
   __syncthreads();
-  for (long long k = threadIdx.x; k < n; k += kOrderThreads) {
-    const int32_t c = row[k];
-    atomicOr(&bits[c >> 5], 1u << (c & 31));
+  for (long long k0 = threadIdx.x; k0 < n; k0 += 4 * kOrderThreads) {
+    int32_t c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = k0 + i * kOrderThreads < n ? row[k0 + i * kOrderThreads] : -1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) if (c[i] >= 0) atomicOr(&bits[c[i] >> 5], 1u << (c[i] & 31));
   }
   if (threadIdx.x == 0) carry = 0u;
   __syncthreads();
@@ -244,7 +251,10 @@ kvc_status launch_order_kept(const Problem& P, int32_t* idx, const int32_t* n_ke
     return KVC_ERR_WORKSPACE;
   }
   const long long segs = (long long)P.L * P.Bt * P.Hkv;
-  KVC_CUDA(launch_dependent(order_kept_kernel, dim3((unsigned)segs), dim3(kOrderThreads), 0, st, idx, n_keep,
+  const bool shared = P.N <= kOrderSharedN;
+  const size_t smem = shared ? (size_t)((P.N + 31) / 32) * sizeof(uint32_t) : 0;
+  KVC_CUDA(launch_dependent(shared ? order_kept_kernel<true> : order_kept_kernel<false>, dim3((unsigned)segs), dim3(kOrderThreads),
+                            smem, st, idx, n_keep,
                             reinterpret_cast<uint32_t*>(ws), P.L, P.Bt, P.Hkv, P.N, per_head ? 1 : 0));
   KVC_LAUNCH_CHECK("order_kept_kernel");
   return KVC_OK;

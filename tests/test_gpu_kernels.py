@@ -156,3 +156,26 @@ def test_streams_of_the_head_sharded_pass_and_composite(N, Hkv):
     s = scores.cpu().numpy()
     Pz.assert_rank_exact(s, idx.cpu().numpy())
     Pz.assert_compose_exact(s, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
+
+
+@pytest.mark.parametrize("N", [31, 16385, 262144, 262145])
+def test_position_order_with_the_bitmap_in_either_memory(N):
+    """Marks in shared memory (up to 262144 tokens) and in the workspace; more words than threads, a partial last word."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    L, Hkv = 2, 2
+    desc = kvc.kvc_desc_init(L, 1, Hkv, Hkv, 64, N, 1, kvc.F32)
+    g = np.random.default_rng(N)
+    perm = np.stack([np.stack([g.permutation(N) for _ in range(Hkv)]) for _ in range(L)])[:, None].astype(np.int32)
+    n_keep = np.array([[N // 3, N - 1]], dtype=np.int32)
+    idx = torch.from_numpy(perm.copy()).to(dev)
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+    kvc.kvc_order_kept(desc, idx, torch.from_numpy(n_keep).to(dev), ws)
+    torch.cuda.synchronize()
+    got = idx.cpu().numpy()
+    for l in range(L):
+        n = int(n_keep[0, l])
+        want = perm[l, 0].copy()
+        want[:, :n] = np.sort(want[:, :n], axis=-1)
+        assert np.array_equal(got[l, 0], want)
