@@ -247,9 +247,9 @@ score_emit_kernel(ScoreParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp,
 // the statistics and the emission then read them.  Units are taken in groups that fill the buffer.  Every sum is
 // taken in the order of the sweeps (four partial products per logit, the butterfly over 32 tokens, 8 such steps per
 // warp and chunk), so the scores are the same bit for bit.  fp32, 16 layers, N = 3001, 32 / 8 heads of 128, w = 32:
-// 1342 us for the two sweeps, 424 us so (the product 335; it cannot take less than 175: 128 multiply-adds a clock and
+// 1342 us for the two sweeps, 417 us so (the product 314; it cannot take less than 175: 128 multiply-adds a clock and
 // SM).  A larger buffer (96 MB) gains 1 %, smaller ones mean more and shorter launches.
-constexpr int kTileTok = 128, kLogitThreads = 256;
+constexpr int kTileTok = 128, kHalfTok = kTileTok / 2, kLogitThreads = 256;
 template <int kTT> constexpr int kLogitTileRows = kTT == 8 ? 128 : 32;
 constexpr size_t kLogitsCap = (size_t)64 << 20;
 constexpr int kMaxLogitChunks = 1024;           // the statistics of a row's chunks meet in shared memory
@@ -284,8 +284,10 @@ __device__ __forceinline__ void stage4(float* dst, const __nv_bfloat16* row, int
 }
 
 // dots[unit - unit0][row][token] = <q row, k token>.  Work items are (unit, 128 rows, 128 tokens), tokens fastest, dealt
-// to the CTAs in even stretches, so that a CTA keeps its Q rows and streams K tiles through two buffers.  8 x 8 logits
-// per thread; the four partial products of a logit are taken two at a time (a packed pair), in two sweeps over the
+// to the CTAs in even stretches, so that a CTA keeps its Q rows and streams K tiles through two buffers.  The tokens of an
+// item are two halves of four warps, one on each scheduler, that wait for each other only where the Q rows change, and there
+// the second half starts one sweep later: one half multiplies while the other stores and waits for its tile (325 -> 314 us
+// in the case above; 320 without the delayed start).  8 x 8 logits per thread; the four partial products of a logit are taken two at a time (a packed pair), in two sweeps over the
 // tile.  Bound by the multiply-adds (128 clocks of a scheduler per warp and step of two elements); the operand reads
 // are what a smaller register tile would wait for: an 8-byte read costs the SM 2 clocks where neighbouring lanes read
 // different addresses (the 8 tokens) and 1 where they share one (the 8 rows), 96 for four warps' steps.  (4 x 4 logits
@@ -297,15 +299,16 @@ __global__ void __launch_bounds__(kLogitThreads, 1)
 score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, float* __restrict__ dots, int row_tiles,
                     int tok_tiles, int items, int* __restrict__ status) {
   constexpr int kPitch = D + 4, kVec = D / 4, kTileRow = kLogitTileRows<kTT>;
-  constexpr int kTokGroups = kTileTok / (8 * kTT);             // warps side by side over the tokens
+  constexpr int kTokGroups = kHalfTok / (8 * kTT);             // a half's warps side by side over its tokens
   extern __shared__ __align__(16) float gsm[];
   float* const Qs = gsm;
   float* const Ks = gsm + kTileRow * kPitch;                   // two buffers
   grid_dependency_wait();
   if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;      // (nothing here can fail on the device)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int tok = (warp % kTokGroups) * (8 * kTT) + (lane & 7);   // tokens tok + 8 i
-  const int row = (warp / kTokGroups) * 32 + (lane >> 3);     // rows row + 4 j
+  const int half_id = warp >> 2, ht = threadIdx.x & 127;      // four warps, one on each scheduler
+  const int tok = half_id * kHalfTok + (warp & 3) % kTokGroups * (8 * kTT) + (lane & 7);   // tokens tok + 8 i
+  const int row0 = (warp & 3) / kTokGroups * 32, row = row0 + (lane >> 3);   // rows row + 4 j
   const int i0 = (int)((long long)items * blockIdx.x / gridDim.x), i1 = (int)((long long)items * (blockIdx.x + 1) / gridDim.x);
   auto load_k = [&](int item, float* dst) {
     const int ur = item / tok_tiles, tt = item - ur * tok_tiles;
@@ -313,18 +316,19 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
     const int h = unit % P.Hkv, lb = unit / P.Hkv;
     const T* base = reinterpret_cast<const T*>(kp.p[lb / P.Bt]) + (lb % P.Bt) * P.kvs0 + h * P.kvs1;
 #pragma unroll 4
-    for (int i = threadIdx.x; i < kTileTok * kVec; i += kLogitThreads) {
-      const int t = i / kVec, v = i % kVec;
+    for (int i = ht; i < kHalfTok * kVec; i += kLogitThreads / 2) {
+      const int t = half_id * kHalfTok + i / kVec, v = i % kVec;
       stage4(dst + t * kPitch + 4 * v, base + min((long long)tt * kTileTok + t, P.N - 1) * P.kvs2, v);
     }
   };
   if (i0 < i1) load_k(i0, Ks);
-  asm volatile("cp.async.commit_group;" ::: "memory");
   int cur = -1, rows = 0, r0 = 0;                              // the (unit, rows) whose Q is here
   for (int item = i0; item < i1; ++item) {
     float* const buf = Ks + ((item - i0) & 1) * (kTileTok * kPitch);
     const int ur = item / tok_tiles, tt = item - ur * tok_tiles;
-    if (ur != cur) {
+    const bool fresh = ur != cur;
+    if (fresh) {
+      if (cur >= 0) __syncthreads();                           // the Q rows here have been read
       cur = ur;
       const int unit = P.unit0 + ur / row_tiles;
       const int h = unit % P.Hkv, lb = unit / P.Hkv;
@@ -337,19 +341,26 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
         const int j = gm.qh[gm.begin[h] + rr / P.w];
         stage4(Qs + (i / kVec) * kPitch + 4 * v, base + j * P.qs1 + (long long)(rr % P.w) * P.qs2, v);
       }
-      asm volatile("cp.async.commit_group;" ::: "memory");
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+    } else {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + half_id) : "memory");
     }
+    // this half's tile is here, and the one before has been read
     if (item + 1 < i1) load_k(item + 1, Ks + ((item + 1 - i0) & 1) * (kTileTok * kPitch));
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");       // all but the next item's tile
-    __syncthreads();
-    if (r0 + (warp / kTokGroups) * 32 < rows) {
+    const bool delay = kTT == 8 && fresh && item + 1 < i1;     // (the same in all threads; with a single item it only costs)
+    if (delay && half_id == 1) asm volatile("bar.sync 3, 256;" ::: "memory");
+    if (r0 + row0 >= rows) {
+      if (delay && half_id == 0) asm volatile("bar.arrive 3, 256;" ::: "memory");
+    } else {
       const float* kq = buf + tok * kPitch;
       const float* qq = Qs + row * kPitch;
       unsigned long long acc[kTT][8];                            // [token][row]: two partial products
       float first[kTT][8];                                       // the sum of the first two
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
+        if (half == 1 && delay && half_id == 0) asm volatile("bar.arrive 3, 256;" ::: "memory");
 #pragma unroll
         for (int i = 0; i < kTT; ++i)
 #pragma unroll
@@ -386,7 +397,6 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
         }
       }
     }
-    __syncthreads();                                           // this tile and these Q rows have been read
   }
 }
 
