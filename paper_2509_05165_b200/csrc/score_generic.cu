@@ -247,7 +247,7 @@ score_emit_kernel(ScoreParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp,
 // the statistics and the emission then read them.  Units are taken in groups that fill the buffer.  Every sum is
 // taken in the order of the sweeps (four partial products per logit, the butterfly over 32 tokens, 8 such steps per
 // warp and chunk), so the scores are the same bit for bit.  fp32, 16 layers, N = 3001, 32 / 8 heads of 128, w = 32:
-// 1342 us for the two sweeps, 417 us so (the product 314; it cannot take less than 175: 128 multiply-adds a clock and
+// 1342 us for the two sweeps, 406 us so (the product 314; it cannot take less than 175: 128 multiply-adds a clock and
 // SM).  A larger buffer (96 MB) gains 1 %, smaller ones mean more and shorter launches.
 constexpr int kTileTok = 128, kHalfTok = kTileTok / 2, kLogitThreads = 256;
 template <int kTT> constexpr int kLogitTileRows = kTT == 8 ? 128 : 32;
@@ -400,8 +400,12 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
   }
 }
 
-// The log-sum-exp (base 2) of four rows of a unit.  Eight lanes per row; a warp takes 8 steps of 32 tokens, 128 apart,
-// as a warp of score_stats_kernel does; the four "warps" of a chunk and then the chunks are folded as there.
+// The log-sum-exp (base 2) of four rows of a unit.  Eight lanes per row, four neighbouring tokens each; a warp takes 8 steps
+// of 32 tokens, 128 apart, as a warp of score_stats_kernel does; the four "warps" of a chunk and then the chunks are folded
+// as there.  Bound by the load / shuffle unit: 16-byte loads (8 per lane, 4 lines each, where 4-byte ones were 32), and the 8
+// steps' butterflies together: at each distance a lane passes on half of its steps and keeps the sums of the others, so that lane
+// i ends with step i (28 shuffles for the sums, 7 for the maxima; one step at a time takes 24 and 24 with one token per lane
+// and load).  The additions are those of the butterfly.  (49 million logits: 65 -> 55 us.)
 constexpr int kRowStatWarps = 4;
 __global__ void __launch_bounds__(kRowStatWarps * 32)
 score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dots, float* __restrict__ lse2) {
@@ -416,46 +420,79 @@ score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dot
   const int r = min(r0 + rl, rows - 1);
   const float* src = dots + ((long long)blockIdx.y * P.max_rows + r) * P.np;
   const long long vis = min(P.N - 1, P.q_pos0 + r % P.w);      // the last token the row sees
+  __shared__ __align__(16) float step_max[kRowStatWarps][4][kChunkIters];
+  __shared__ __align__(16) float2 step_sum[kRowStatWarps][4][kChunkIters];   // (factor of the sum so far, sum of the step)
   for (int p = warp; p < 4 * P.nchunks; p += kRowStatWarps) {
-    const long long base = (long long)(p >> 2) * (kChunkIters * kThreads) + (p & 3) * 32 + sub;
+    const long long base = (long long)(p >> 2) * (kChunkIters * kThreads) + (p & 3) * 32 + 4 * sub;
     const float* at = src + base;
     float s[kChunkIters][4];
-    if (base + (kChunkIters - 1) * kThreads + 24 <= vis) {     // all of them are there and seen
+    if (base + (kChunkIters - 1) * kThreads + 3 <= vis) {      // all of them are there and seen
 #pragma unroll
-      for (int it = 0; it < kChunkIters; ++it)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) s[it][i] = __ldg(at + it * kThreads + 8 * i);
-#pragma unroll
-      for (int it = 0; it < kChunkIters; ++it)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) s[it][i] = s[it][i] * P.scale_log2e;
+      for (int it = 0; it < kChunkIters; ++it) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(at + it * kThreads));
+        s[it][0] = x.x * P.scale_log2e; s[it][1] = x.y * P.scale_log2e; s[it][2] = x.z * P.scale_log2e; s[it][3] = x.w * P.scale_log2e;
+      }
     } else {
       const int left = (int)max(-1LL, min(vis - base, (long long)kChunkIters * kThreads));   // offsets up to here count
 #pragma unroll
-      for (int it = 0; it < kChunkIters; ++it)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          s[it][i] = it * kThreads + 8 * i <= left ? __ldg(at + it * kThreads + 8 * i) * P.scale_log2e : -INFINITY;
-    }
-    float m = -INFINITY, lsum = 0.f;
-#pragma unroll
-    for (int it = 0; it < kChunkIters; ++it) {
-      float m_w = fmaxf(fmaxf(s[it][0], s[it][1]), fmaxf(s[it][2], s[it][3]));
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) m_w = fmaxf(m_w, __shfl_xor_sync(0xffffffffu, m_w, o));
-      const float m_new = fmaxf(m, m_w);
-      float e[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) e[i] = (m_new == -INFINITY) ? 0.f : exp2f(s[it][i] - m_new);
-      float l_w = (e[0] + e[2]) + (e[1] + e[3]);               // distances 16 and 8 of the butterfly
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) l_w += __shfl_xor_sync(0xffffffffu, l_w, o);
-      if (m_new > -INFINITY) {
-        lsum = lsum * exp2f(m - m_new) + l_w;
-        m = m_new;
+      for (int it = 0; it < kChunkIters; ++it) {
+        const int o = it * kThreads;
+        const float4 x = o <= left ? __ldg(reinterpret_cast<const float4*>(at + o)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        s[it][0] = o <= left ? x.x * P.scale_log2e : -INFINITY;
+        s[it][1] = o + 1 <= left ? x.y * P.scale_log2e : -INFINITY;
+        s[it][2] = o + 2 <= left ? x.z * P.scale_log2e : -INFINITY;
+        s[it][3] = o + 3 <= left ? x.w * P.scale_log2e : -INFINITY;
       }
     }
-    if (sub == 0) st_sm[p * 4 + rl] = make_float2(m, lsum);
+    // the maximum of step `sub`, then of the steps up to it
+    float mw[kChunkIters];
+#pragma unroll
+    for (int it = 0; it < kChunkIters; ++it) mw[it] = fmaxf(fmaxf(s[it][0], s[it][1]), fmaxf(s[it][2], s[it][3]));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const bool up = sub & o;
+#pragma unroll
+      for (int k = 0; k < o; ++k)
+        mw[k] = fmaxf(up ? mw[k + o] : mw[k], __shfl_xor_sync(0xffffffffu, up ? mw[k] : mw[k + o], o));
+    }
+    float m = mw[0];
+#pragma unroll
+    for (int o = 1; o < kChunkIters; o <<= 1) {
+      const float x = __shfl_up_sync(0xffffffffu, m, o, kChunkIters);
+      m = fmaxf(m, x);                                         // (a lane without a source gets its own)
+    }
+    const float m_below = __shfl_up_sync(0xffffffffu, m, 1, kChunkIters), m_before = sub ? m_below : -INFINITY;
+    step_max[warp][rl][sub] = m;
+    __syncwarp();
+    float ms[kChunkIters];
+#pragma unroll
+    for (int it = 0; it < kChunkIters; it += 4) *reinterpret_cast<float4*>(ms + it) = *reinterpret_cast<const float4*>(&step_max[warp][rl][it]);
+#pragma unroll
+    for (int it = 0; it < kChunkIters; ++it)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[it][i] = (ms[it] == -INFINITY) ? 0.f : exp2f(s[it][i] - ms[it]);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {                          // distances 16, 8, 4 of the butterfly
+      const bool up = sub & o;
+#pragma unroll
+      for (int k = 0; k < o; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          s[k][i] = (up ? s[k + o][i] : s[k][i]) + __shfl_xor_sync(0xffffffffu, up ? s[k][i] : s[k + o][i], o);
+    }
+    const float l_w = (s[0][0] + s[0][2]) + (s[0][1] + s[0][3]);   // 2 and 1
+    step_sum[warp][rl][sub] = make_float2(m == -INFINITY ? 0.f : exp2f(m_before - m), l_w);
+    __syncwarp();
+    if (sub == kChunkIters - 1) {                              // (its maximum is that of all steps)
+      float lsum = 0.f;
+#pragma unroll
+      for (int it = 0; it < kChunkIters; ++it) {
+        const float2 x = step_sum[warp][rl][it];
+        lsum = fmaf(lsum, x.x, x.y);
+      }
+      st_sm[p * 4 + rl] = make_float2(m, lsum);
+    }
+    __syncwarp();
   }
   __syncthreads();
   // per chunk: the four warps' statistics
