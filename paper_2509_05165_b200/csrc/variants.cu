@@ -81,7 +81,9 @@ kvc_status launch_norm_t(const Problem& P, const LayerPtrs& v, float* vnorm, cud
 // kOrderSharedN tokens, else in global scratch), then writes the marked positions back in ascending order.  Bound by latency:
 // marks in shared memory do not travel to L2 (256 heads of 16384, a quarter kept: 13.7 -> 8.6 us).
 constexpr int kOrderThreads = 512;
-constexpr long long kOrderSharedN = 262144;   // 32 KB of marks: the most that leaves every SM room for several CTAs
+// 32 KB of marks: four CTAs of 512 threads per SM fill it and fit, without a launch attribute.  (64 heads, a quarter kept, at the
+// line: 66 us in shared memory for 262144 tokens, 97 us in the workspace for 262148.)
+constexpr long long kOrderSharedN = 262144;
 
 template <bool kShared>
 __global__ void __launch_bounds__(kOrderThreads)
