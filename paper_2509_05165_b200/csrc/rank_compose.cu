@@ -354,7 +354,7 @@ __device__ __forceinline__ int merge_path_warp(int diag, int na, int nb, const u
 // Bound by the latencies of a tile (split search, loads, merge) at four CTAs per SM; a thread reads one key per output, the
 // successor of the one it took.  (Both runs' heads at every step and outputs written to shared memory at a stride of 8:
 // the ranking of 28 segments of 131072, two levels, 118 -> 101 us; with 256 threads of 16 outputs 110, with 1024 of 4 109.)
-// kVec: rows start on 16 bytes (N a multiple of 4): a thread stores its outputs itself, 16 bytes at a time.  Otherwise
+// kVec: rows start on 16 bytes (N a multiple of 4, both output arrays aligned): a thread stores its outputs itself, 16 bytes at a time.  Otherwise
 // they go through shared memory once more; a tile's element i sits in slot i + i / kMergeItems there, so that the threads'
 // stretches begin in different banks.
 template <bool kVec>
@@ -638,7 +638,10 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
       in_b = !in_b;
       uint32_t* k_nxt = in_b ? keys_b : keys_a;
       int32_t* v_nxt = in_b ? idx : vals_a;
-      KVC_CUDA(launch_dependent(P.N % 4 == 0 ? merge_runs_kernel<true> : merge_runs_kernel<false>, dim3((unsigned)(segments * merge_tiles)), dim3(kMergeThreads), 0, st,
+      // 16-byte stores where a segment's rows start on 16 bytes; the last level's positions go to the caller's idx, which may
+      // start anywhere (the buffers of the workspace start on 256 bytes)
+      const bool vec = P.N % 4 == 0 && (reinterpret_cast<uintptr_t>(v_nxt) & 15u) == 0;
+      KVC_CUDA(launch_dependent(vec ? merge_runs_kernel<true> : merge_runs_kernel<false>, dim3((unsigned)(segments * merge_tiles)), dim3(kMergeThreads), 0, st,
                                 (const uint32_t*)k_cur, (const int32_t*)v_cur, k_nxt, v_nxt, P.N,
                                 chunk_len << level, (int)merge_tiles));
       KVC_LAUNCH_CHECK("merge_runs_kernel");

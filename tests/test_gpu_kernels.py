@@ -179,3 +179,31 @@ def test_position_order_with_the_bitmap_in_either_memory(N):
         want = perm[l, 0].copy()
         want[:, :n] = np.sort(want[:, :n], axis=-1)
         assert np.array_equal(got[l, 0], want)
+
+
+@pytest.mark.parametrize("L,Hkv,N", [(1, 2, 65536), (2, 4, 32768), (2, 4, 16384)])
+def test_ranking_into_arrays_that_start_on_four_bytes(L, Hkv, N):
+    """Segments of several chunks (eight, four and two: the last merge writes the caller's idx): scores, idx and composite
+    need the alignment of their elements only."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    desc = kvc.kvc_desc_init(L, 1, Hkv, Hkv, 64, N, 1, kvc.F32)
+    n = L * Hkv * N
+    S = np.random.default_rng(N).random(n, dtype=np.float32)
+    S[: n // 2] = np.round(S[: n // 2] * 7) / 8
+    scores = torch.empty(n + 1, dtype=torch.float32, device=dev)[1:]
+    idx_buf = torch.full((n + 2,), -1, dtype=torch.int32, device=dev)
+    comp_buf = torch.full((L * N + 2,), -1.0, dtype=torch.float32, device=dev)
+    idx, comp = idx_buf[1:n + 1], comp_buf[1:L * N + 1]
+    assert [t.data_ptr() % 16 for t in (scores, idx, comp)] == [4, 4, 4]
+    scores.copy_(torch.from_numpy(S))
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+    kvc.kvc_compose(desc, scores, idx, comp, ws)
+    torch.cuda.synchronize()
+    S, got = S.reshape(L, 1, Hkv, N), idx_buf.cpu().numpy()
+    assert got[0] == -1 and got[-1] == -1
+    Pz.assert_rank_exact(S, got[1:-1].reshape(S.shape))
+    got_c = comp_buf.cpu().numpy()
+    assert got_c[0] == -1 and got_c[-1] == -1
+    Pz.assert_compose_exact(S, got[1:-1].reshape(S.shape), got_c[1:-1].reshape(L, 1, N), desc.agg_head)
