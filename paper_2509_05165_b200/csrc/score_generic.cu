@@ -407,6 +407,7 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
 // i ends with step i (28 shuffles for the sums, 7 for the maxima; one step at a time takes 24 and 24 with one token per lane
 // and load).  The additions are those of the butterfly.  (49 million logits: 65 -> 55 us.)
 constexpr int kRowStatWarps = 4;
+constexpr size_t kRowStatStatic = kRowStatWarps * 4 * kChunkIters * (sizeof(float) + sizeof(float2));   // its step_max and step_sum
 __global__ void __launch_bounds__(kRowStatWarps * 32)
 score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dots, float* __restrict__ lse2) {
   extern __shared__ float2 st_sm[];                            // [4 * nchunks][4 rows]
@@ -789,7 +790,7 @@ kvc_status run_logits_t(const Problem& P, const GroupMap& gm, const LayerPtrs& q
   lp.agg_task = P.agg_task; lp.agg_group = P.agg_group;
   lp.nchunks = (int)((P.N + kChunkIters * kThreads - 1) / (kChunkIters * kThreads));
   const size_t stat_smem = (size_t)lp.nchunks * 16 * sizeof(float2);
-  if (stat_smem > 48 * 1024)
+  if (stat_smem + kRowStatStatic > 48 * 1024)                   // (what a launch may have without the attribute, static bytes included)
     KVC_CUDA(cudaFuncSetAttribute(score_row_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   kMaxLogitChunks * 16 * (int)sizeof(float2)));
   float* dots = reinterpret_cast<float*>(ws);

@@ -1,4 +1,8 @@
 """Single kernels at the edges of their tiles, against the oracle on the same seeded inputs."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -207,3 +211,31 @@ def test_ranking_into_arrays_that_start_on_four_bytes(L, Hkv, N):
     got_c = comp_buf.cpu().numpy()
     assert got_c[0] == -1 and got_c[-1] == -1
     Pz.assert_compose_exact(S, got[1:-1].reshape(S.shape), got_c[1:-1].reshape(L, 1, N), desc.agg_head)
+
+
+_STATISTICS_LENGTHS = """
+import sys; sys.path.insert(0, "tests")
+import torch
+import paper_2509_05165_b200 as kvc
+from paper_2509_05165_b200 import workloads as W
+import parity as Pz
+for N in (380928, 380929, 393216, 393217):
+    cfg = W.WorkloadConfig("statistics", 1, 2, 1, 64, N, 1, dtype="f32", elem_std=1.0, hh_frac=0.0)
+    wl = W.make_workload(cfg, torch.device("cuda:0"))
+    desc = kvc.desc_from_config(cfg)
+    scores = torch.empty((1, 1, 1, N), dtype=torch.float32, device="cuda:0")
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device="cuda:0")
+    kvc.kvc_score(desc, wl.q, wl.k, scores, ws)
+    torch.cuda.synchronize()
+    Pz.assert_scores_close(scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
+"""
+
+
+def test_statistics_that_just_need_the_larger_shared_memory():
+    """The statistics of 372 to 385 chunks take 47 616 to 49 280 bytes beside the kernel's own 1536, on both sides of the 49 152 a
+    launch may have without an attribute.  In a process of its own and in ascending order: the attribute, once set, stays."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _STATISTICS_LENGTHS], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
