@@ -994,8 +994,13 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
       const uint32_t idesc = umma_idesc(pass == 0 ? kTile : (c.template rows<kLong>(P) + 31) / 32 * 32);
       qr.next(slots);
+      if (pass == 0 && ok && issued)
+        // the MMAs of the run before read the Q columns: their last tile has to be complete.  (The tensor pipe runs an MMA
+        // behind the copies issued before it, as PTX guarantees for tcgen05.cp -> tcgen05.mma, but it promises nothing for a copy
+        // issued behind an MMA.)  The accumulator that the tile fills is free later still, so the first MMA below waits longer.
+        ok = mbar_wait_warp(bar_tfull(0), (uint32_t)(tb.phase ^ 1), ctl);
       if (pass == 0 && ok) {
-        // the run's Q moves to TMEM (in order behind the MMAs that read the run before's), its slot is free again
+        // the run's Q moves to TMEM, its slot is free again
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
