@@ -74,7 +74,7 @@ void oracle_attention_rows(const float* q, const float* k, int64_t N, int32_t d,
                            int32_t w, double scale, int64_t q_pos0, double* A) {
   for (int32_t m = 0; m < w; ++m) {
     double* row = A + (int64_t)m * N;
-    int64_t last = q_pos0 + m; /* last visible key */
+    int64_t last = q_pos0 >= N ? N - 1 : q_pos0 + m; /* last visible key (the sum must not overflow) */
     int64_t n_vis = last >= N - 1 ? N : last + 1;
     if (n_vis < 0) n_vis = 0;
     /* logits s_c = scale * <q_m, k_c> */

@@ -109,7 +109,8 @@ kvc_status resolve(const kvc_desc* d, Problem* P, GroupMap* gm) {
   KVC_REQUIRE(d->reserved_ == 0, KVC_ERR_INVALID_ARG, "reserved_ must be 0");
 
   P->L = d->n_layers; P->Bt = d->batch; P->Hq = d->n_q_heads; P->Hkv = d->n_kv_heads;
-  P->d = d->head_dim; P->w = d->window; P->N = d->n_ctx; P->q_pos0 = d->q_pos0;
+  P->d = d->head_dim; P->w = d->window; P->N = d->n_ctx;
+  P->q_pos0 = d->q_pos0 < d->n_ctx ? d->q_pos0 : d->n_ctx;      // (any value from N on is no mask; q_pos0 + row must not overflow)
   P->dtype = d->dtype; P->elem_bytes = (d->dtype == KVC_BF16) ? 2 : 4;
   P->scale = (d->scale > 0.f) ? d->scale : 1.0f / sqrtf((float)d->head_dim);
   P->agg_task = d->agg_task; P->agg_group = d->agg_group; P->agg_head = d->agg_head;

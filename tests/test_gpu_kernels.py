@@ -239,3 +239,19 @@ def test_statistics_that_just_need_the_larger_shared_memory():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", _STATISTICS_LENGTHS], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("dtype,w", [("bf16", 16), ("bf16", 200), ("f32", 16)])
+def test_positions_far_behind_the_context_mask_nothing(dtype, w):
+    """The largest position there is gives what the first one behind the context gives, bit for bit (full tiles and a partial one)."""
+    cfg = W.WorkloadConfig("far", 1, 4, 2, 64, 333, w, dtype=dtype, elem_std=1.0)
+    dev, wl, desc = _setup(cfg, q_pos0=333)
+    out = alloc_outputs(desc, 1, wl.k[0].dtype, dev)
+    kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
+    want = out.scores.clone()
+    for q_pos0 in (2 ** 40, 2 ** 63 - 1):
+        desc.q_pos0 = q_pos0
+        kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
+        torch.cuda.synchronize()
+        assert torch.equal(out.scores, want)
+    Pz.assert_scores_close(want.cpu().numpy(), Pz.oracle_scores(wl, desc))

@@ -52,6 +52,15 @@ def test_rows_sum_to_one_through_mean_pooling(oracle):
         np.testing.assert_allclose(S.sum(axis=1), 2 * np.ones(Hkv), rtol=1e-12)
 
 
+def test_every_position_behind_the_context_masks_nothing(oracle):
+    r = _rng(31)
+    q = r.standard_normal((2, 3, 8)).astype(np.float32)
+    k = r.standard_normal((1, 20, 8)).astype(np.float32)
+    want = oracle.score_layer(q, k, 0.5, 20)
+    for q_pos0 in (21, 2 ** 40, 2 ** 63 - 1):
+        assert np.array_equal(oracle.score_layer(q, k, 0.5, q_pos0), want)
+
+
 def test_attention_rows_are_distributions_with_causal_support(oracle):
     r = _rng(3)
     w, d, N, q_pos0 = 6, 4, 20, 11
