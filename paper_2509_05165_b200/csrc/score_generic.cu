@@ -252,7 +252,6 @@ score_emit_kernel(ScoreParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp,
 constexpr int kTileTok = 128, kHalfTok = kTileTok / 2, kLogitThreads = 256;
 template <int kTT> constexpr int kLogitTileRows = kTT == 8 ? 128 : 32;
 constexpr size_t kLogitsCap = (size_t)64 << 20;
-constexpr int kMaxLogitChunks = 1024;           // the statistics of a row's chunks meet in shared memory
 
 struct LogitParams {
   int Bt, Hkv, w, max_rows;                     // max_rows: of a unit (the largest group's)
@@ -406,11 +405,14 @@ score_logits_kernel(LogitParams P, GroupMap gm, LayerPtrs qp, LayerPtrs kp, floa
 // steps' butterflies together: at each distance a lane passes on half of its steps and keeps the sums of the others, so that lane
 // i ends with step i (28 shuffles for the sums, 7 for the maxima; one step at a time takes 24 and 24 with one token per lane
 // and load).  The additions are those of the butterfly.  (49 million logits: 65 -> 55 us.)
+// kSplit: blockIdx.z takes per_slice of the chunks only and leaves their statistics in `partial` [row][chunk] for
+// score_fold_stats_kernel (see LogitPlan).
 constexpr int kRowStatWarps = 4;
-constexpr size_t kRowStatStatic = kRowStatWarps * 4 * kChunkIters * (sizeof(float) + sizeof(float2));   // its step_max and step_sum
+template <bool kSplit>
 __global__ void __launch_bounds__(kRowStatWarps * 32)
-score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dots, float* __restrict__ lse2) {
-  extern __shared__ float2 st_sm[];                            // [4 * nchunks][4 rows]
+score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dots, float* __restrict__ lse2,
+                       float2* __restrict__ partial, int per_slice) {
+  extern __shared__ float2 st_sm[];                            // [4 * chunks][4 rows]
   grid_dependency_wait();
   const int unit = P.unit0 + blockIdx.y;
   const int h = unit % P.Hkv;
@@ -423,8 +425,10 @@ score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dot
   const long long vis = min(P.N - 1, P.q_pos0 + r % P.w);      // the last token the row sees
   __shared__ __align__(16) float step_max[kRowStatWarps][4][kChunkIters];
   __shared__ __align__(16) float2 step_sum[kRowStatWarps][4][kChunkIters];   // (factor of the sum so far, sum of the step)
-  for (int p = warp; p < 4 * P.nchunks; p += kRowStatWarps) {
-    const long long base = (long long)(p >> 2) * (kChunkIters * kThreads) + (p & 3) * 32 + 4 * sub;
+  const int chunk0 = kSplit ? (int)blockIdx.z * per_slice : 0;
+  const int chunks = kSplit ? min(per_slice, P.nchunks - chunk0) : P.nchunks;
+  for (int p = warp; p < 4 * chunks; p += kRowStatWarps) {
+    const long long base = (long long)(chunk0 + (p >> 2)) * (kChunkIters * kThreads) + (p & 3) * 32 + 4 * sub;
     const float* at = src + base;
     float s[kChunkIters][4];
     if (base + (kChunkIters - 1) * kThreads + 3 <= vis) {      // all of them are there and seen
@@ -497,7 +501,7 @@ score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dot
   }
   __syncthreads();
   // per chunk: the four warps' statistics
-  for (int i = threadIdx.x; i < P.nchunks * 4; i += kRowStatWarps * 32) {
+  for (int i = threadIdx.x; i < chunks * 4; i += kRowStatWarps * 32) {
     const int ch = i >> 2, rr = i & 3;
     float M = -INFINITY;
 #pragma unroll
@@ -510,8 +514,13 @@ score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dot
         Lsum += v.y * exp2f(v.x - M);
       }
     }
-    st_sm[ch * 16 + rr] = make_float2(M, Lsum);                // (read by nobody else: slot wv = 0 of this chunk and row)
+    if (kSplit) {
+      if (r0 + rr < rows) partial[((long long)blockIdx.y * P.max_rows + r0 + rr) * P.nchunks + chunk0 + ch] = make_float2(M, Lsum);
+    } else {
+      st_sm[ch * 16 + rr] = make_float2(M, Lsum);              // (read by nobody else: slot wv = 0 of this chunk and row)
+    }
   }
+  if (kSplit) return;
   __syncthreads();
   if (threadIdx.x < 4 && r0 + threadIdx.x < rows) {
     float M = -INFINITY;
@@ -523,6 +532,29 @@ score_row_stats_kernel(LogitParams P, GroupMap gm, const float* __restrict__ dot
     }
     lse2[(long long)blockIdx.y * P.max_rows + r0 + threadIdx.x] = M + log2f(Lsum);
   }
+}
+
+// The chunks' statistics of a row folded to its log-sum-exp, a warp per row: the lanes fetch 32 chunks at a time, the sum is
+// taken in the order of the chunks, as score_row_stats_kernel takes it.
+__global__ void __launch_bounds__(kThreads)
+score_fold_stats_kernel(LogitParams P, GroupMap gm, const float2* __restrict__ partial, float* __restrict__ lse2) {
+  grid_dependency_wait();
+  const int h = (P.unit0 + blockIdx.y) % P.Hkv;
+  const int row = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= (gm.begin[h + 1] - gm.begin[h]) * P.w) return;
+  const float2* src = partial + ((long long)blockIdx.y * P.max_rows + row) * P.nchunks;
+  float M = -INFINITY;
+  for (int i = lane; i < P.nchunks; i += 32) M = fmaxf(M, __ldg(&src[i].x));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  float Lsum = 0.f;
+  for (int i0 = 0; i0 < P.nchunks; i0 += 32) {
+    const float2 v = i0 + lane < P.nchunks ? __ldg(src + i0 + lane) : make_float2(-INFINITY, 0.f);
+    const float f = exp2f(v.x - M);                            // (0 where no key is seen, and there the sum is 0 too)
+#pragma unroll
+    for (int i = 0; i < 32; ++i) Lsum += __shfl_sync(0xffffffffu, v.y, i) * __shfl_sync(0xffffffffu, f, i);
+  }
+  if (lane == 0) lse2[(long long)blockIdx.y * P.max_rows + row] = M + log2f(Lsum);
 }
 
 // Eqs. 14-15 from the kept logits: four tokens per thread, 16 rows in flight.  kMean: agg_task is the mean.
@@ -744,12 +776,13 @@ kvc_status run(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const L
   return KVC_OK;
 }
 
-// How the units are cut into groups whose logits fit the buffer; units_per_group = 0: one unit alone does not fit (or the
-// problem belongs to the tensor cores and gets here only when its strides do not suit them): the two sweeps.
+// How the units are cut into groups whose logits fit the buffer; units_per_group = 0: the two sweeps, because one unit alone does
+// not fit, or because the problem belongs to the tensor cores and gets here only when its strides do not suit them.
 struct LogitPlan {
   long long np, units;
   int max_rows, units_per_group;
-  size_t dots_bytes, lse_bytes;
+  int slices, per_slice;        // of the statistics: how many CTAs share the chunks of a row, and the chunks of each
+  size_t dots_bytes, lse_bytes, partial_bytes;
 };
 LogitPlan logit_plan(const Problem& P) {
   LogitPlan p;
@@ -760,13 +793,27 @@ LogitPlan logit_plan(const Problem& P) {
   const long long nchunks = (P.N + kChunkIters * kThreads - 1) / (kChunkIters * kThreads);
   p.max_rows = (int)rows;
   p.units_per_group = 0;
-  p.dots_bytes = p.lse_bytes = 0;
-  if (unit_bytes > (long long)kLogitsCap || nchunks > kMaxLogitChunks || score_sm100_shape_ok(P)) return p;
+  p.slices = 1;
+  p.per_slice = (int)nchunks;
+  p.dots_bytes = p.lse_bytes = p.partial_bytes = 0;
+  if (unit_bytes > (long long)kLogitsCap || score_sm100_shape_ok(P)) return p;
   const long long per = (long long)kLogitsCap / unit_bytes < 65535 ? (long long)kLogitsCap / unit_bytes : 65535;
   const long long groups = (p.units + per - 1) / per;
   p.units_per_group = (int)((p.units + groups - 1) / groups);   // groups of even size
   p.dots_bytes = align_up((size_t)p.units_per_group * unit_bytes);
   p.lse_bytes = align_up((size_t)p.units_per_group * rows * sizeof(float));
+  // A CTA of the statistics takes four rows over the whole context; where these CTAs are few and the context is long, slices of
+  // the chunks instead, about eight CTAs per SM, for one small launch more.  (A constant stands for the SMs: the workspace must not
+  // depend on the device.  fp32, heads of 64: 32 rows of 65536 tokens 107 -> 27 us per call, 16 units of 64 rows of 262144 tokens
+  // 8740 -> 2388; with 4 chunks it costs what it gains; half and twice as many slices are within 1 %.)
+  constexpr long long kStatCtas = 8 * 148;
+  const long long ctas = (long long)p.units_per_group * ((rows + 3) / 4);
+  if (ctas * 2 <= kStatCtas && nchunks >= 5) {
+    const long long want = kStatCtas / ctas;
+    p.per_slice = (int)((nchunks + want - 1) / want);
+    p.slices = (int)((nchunks + p.per_slice - 1) / p.per_slice);
+    p.partial_bytes = align_up((size_t)p.units_per_group * rows * nchunks * sizeof(float2));
+  }
   return p;
 }
 
@@ -789,12 +836,13 @@ kvc_status run_logits_t(const Problem& P, const GroupMap& gm, const LayerPtrs& q
   lp.scale_log2e = P.scale * kLog2e;
   lp.agg_task = P.agg_task; lp.agg_group = P.agg_group;
   lp.nchunks = (int)((P.N + kChunkIters * kThreads - 1) / (kChunkIters * kThreads));
-  const size_t stat_smem = (size_t)lp.nchunks * 16 * sizeof(float2);
-  if (stat_smem + kRowStatStatic > 48 * 1024)                   // (what a launch may have without the attribute, static bytes included)
-    KVC_CUDA(cudaFuncSetAttribute(score_row_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  kMaxLogitChunks * 16 * (int)sizeof(float2)));
+  const auto stat_kernel = pl.slices > 1 ? score_row_stats_kernel<true> : score_row_stats_kernel<false>;
+  // (at most 28 chunks: unsliced with 5 and more of them are only groups of 593 CTAs and more, whose logits fill the buffer with
+  // 28 290 tokens a row; slices hold a 1184th of the buffer each, rounded up)
+  const size_t stat_smem = (size_t)pl.per_slice * 16 * sizeof(float2);
   float* dots = reinterpret_cast<float*>(ws);
   float* lse2 = reinterpret_cast<float*>(ws + pl.dots_bytes);
+  float2* partial = reinterpret_cast<float2*>(ws + pl.dots_bytes + pl.lse_bytes);
   for (long long u0 = 0; u0 < pl.units; u0 += pl.units_per_group) {
     const unsigned n = (unsigned)(pl.units - u0 < pl.units_per_group ? pl.units - u0 : pl.units_per_group);
     lp.unit0 = (int)u0;
@@ -802,9 +850,14 @@ kvc_status run_logits_t(const Problem& P, const GroupMap& gm, const LayerPtrs& q
     KVC_CUDA(launch_dependent(score_logits_kernel<T, D, kTT>, dim3((unsigned)(items < sms ? items : sms)), dim3(kLogitThreads),
                               (size_t)kSmem, st, lp, gm, q, k, dots, row_tiles, tok_tiles, (int)items, device_status));
     KVC_LAUNCH_CHECK("score_logits_kernel");
-    KVC_CUDA(launch_dependent(score_row_stats_kernel, dim3((unsigned)((pl.max_rows + 3) / 4), n), dim3(kRowStatWarps * 32),
-                              stat_smem, st, lp, gm, (const float*)dots, lse2));
+    KVC_CUDA(launch_dependent(stat_kernel, dim3((unsigned)((pl.max_rows + 3) / 4), n, (unsigned)pl.slices),
+                              dim3(kRowStatWarps * 32), stat_smem, st, lp, gm, (const float*)dots, lse2, partial, pl.per_slice));
     KVC_LAUNCH_CHECK("score_row_stats_kernel");
+    if (pl.slices > 1) {
+      KVC_CUDA(launch_dependent(score_fold_stats_kernel, dim3((unsigned)((pl.max_rows + kThreads / 32 - 1) / (kThreads / 32)), n),
+                                dim3(kThreads), 0, st, lp, gm, (const float2*)partial, lse2));
+      KVC_LAUNCH_CHECK("score_fold_stats_kernel");
+    }
     KVC_CUDA(launch_dependent(P.agg_task == KVC_AGG_MEAN ? score_emit_logits_kernel<true> : score_emit_logits_kernel<false>,
                               dim3((unsigned)((P.N + 4 * kThreads - 1) / (4 * kThreads)), n), dim3(kThreads), 0, st, lp, gm,
                               (const float*)dots, (const float*)lse2, scores));
@@ -832,7 +885,7 @@ static int generic_nchunks(const Problem& P) {
 
 size_t score_generic_workspace_bytes(const Problem& P) {
   const LogitPlan pl = logit_plan(P);
-  if (pl.units_per_group > 0) return pl.dots_bytes + pl.lse_bytes;
+  if (pl.units_per_group > 0) return pl.dots_bytes + pl.lse_bytes + pl.partial_bytes;
   const size_t rows = (size_t)P.L * P.Bt * P.Hq * P.w;
   return align_up(rows * generic_nchunks(P) * sizeof(float2)) + align_up(rows * sizeof(float));
 }

@@ -1,8 +1,4 @@
 """Single kernels at the edges of their tiles, against the oracle on the same seeded inputs."""
-import os
-import subprocess
-import sys
-
 import numpy as np
 import pytest
 import torch
@@ -213,32 +209,19 @@ def test_ranking_into_arrays_that_start_on_four_bytes(L, Hkv, N):
     Pz.assert_compose_exact(S, got[1:-1].reshape(S.shape), got_c[1:-1].reshape(L, 1, N), desc.agg_head)
 
 
-_STATISTICS_LENGTHS = """
-import sys; sys.path.insert(0, "tests")
-import torch
-import paper_2509_05165_b200 as kvc
-from paper_2509_05165_b200 import workloads as W
-import parity as Pz
-for N in (380928, 380929, 393216, 393217):
-    cfg = W.WorkloadConfig("statistics", 1, 2, 1, 64, N, 1, dtype="f32", elem_std=1.0, hh_frac=0.0)
-    wl = W.make_workload(cfg, torch.device("cuda:0"))
-    desc = kvc.desc_from_config(cfg)
-    scores = torch.empty((1, 1, 1, N), dtype=torch.float32, device="cuda:0")
-    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device="cuda:0")
-    kvc.kvc_score(desc, wl.q, wl.k, scores, ws)
+@pytest.mark.parametrize("L,Hq,Hkv,w,N", [
+    (1, 2, 1, 1, 4096), (1, 2, 1, 1, 4097),        # the statistics of four chunks in one piece, of five in slices
+    (2, 6, 3, 3, 9000),                            # six rows: a second CTA of rows in every slice
+    (1, 4, 1, 160, 20001),                         # 640 rows, 160 CTAs: slices of three chunks, the last one shorter
+    (1, 2, 1, 1, 380929), (1, 2, 1, 1, 1050000),   # slices of one chunk; the log-sum-exp of more chunks than a warp
+])
+def test_scoring_of_long_contexts_on_the_cuda_cores(L, Hq, Hkv, w, N):
+    cfg = W.WorkloadConfig("long", L, Hq, Hkv, 64, N, w, dtype="f32", elem_std=1.0, hh_frac=0.0)
+    dev, wl, desc = _setup(cfg)
+    out = alloc_outputs(desc, 1, wl.k[0].dtype, dev)
+    kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
     torch.cuda.synchronize()
-    Pz.assert_scores_close(scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
-"""
-
-
-def test_statistics_that_just_need_the_larger_shared_memory():
-    """The statistics of 372 to 385 chunks take 47 616 to 49 280 bytes beside the kernel's own 1536, on both sides of the 49 152 a
-    launch may have without an attribute.  In a process of its own and in ascending order: the attribute, once set, stays."""
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    r = subprocess.run([sys.executable, "-c", _STATISTICS_LENGTHS], cwd=root, capture_output=True, text=True, timeout=300)
-    assert r.returncode == 0, r.stderr[-2000:]
+    Pz.assert_scores_close(out.scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
 
 
 @pytest.mark.parametrize("dtype,w", [("bf16", 16), ("bf16", 200), ("f32", 16)])
