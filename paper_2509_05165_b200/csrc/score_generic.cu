@@ -776,8 +776,27 @@ kvc_status run(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const L
   return KVC_OK;
 }
 
+// Few rows over many tokens: the two sweeps.  They are bound by reading K twice then, while the product multiplies 32 rows whatever
+// there are, and for bf16 its operands wait for their conversion.  The line rises with the tokens (short contexts of
+// few units do not fill the SMs with sweeps).  Product over sweeps, fp32 with one query head per KV head: 256K tokens of 64,
+// 2 rows 1.16, 3 rows 1.05, 4 rows 0.96; of 128, 1 row 1.12, 2 rows 1.03, 3 rows 0.96; with two query heads 0.89 and
+// less.  bf16: 256K tokens of 64, 5 rows 1.12, 8 rows 0.88, two heads of 1 row 1.23, of 3 rows 0.95; 1M tokens, 8 rows 1.22,
+// two heads of 4 rows 1.05, of 6 rows 0.91, four heads of 1 row 1.02, of 2 rows 0.90.
+bool few_rows(const Problem& P) {
+  struct Line { long long tokens; int rows; };
+  static constexpr Line kBf16[] = {{2048 << 10, 13}, {768 << 10, 10}, {352 << 10, 8}, {224 << 10, 6}, {112 << 10, 3}};
+  static constexpr Line kF32[] = {{3072 << 10, 5}, {352 << 10, 4}, {224 << 10, 3}, {112 << 10, 2}};
+  const long long tokens = (long long)P.L * P.Bt * P.Hkv * P.N, rows = (long long)P.max_group * P.w;
+  if (P.dtype == KVC_BF16) {
+    for (const Line& at : kBf16) if (tokens >= at.tokens) return rows + 2 * (P.max_group - 1) <= at.rows;
+  } else if (P.max_group == 1) {
+    for (const Line& at : kF32) if (tokens >= at.tokens) return rows * (P.d / 64) <= at.rows;
+  }
+  return false;
+}
+
 // How the units are cut into groups whose logits fit the buffer; units_per_group = 0: the two sweeps, because one unit alone does
-// not fit, or because the problem belongs to the tensor cores and gets here only when its strides do not suit them.
+// not fit, has few rows, or because the problem belongs to the tensor cores and gets here only when its strides do not suit them.
 struct LogitPlan {
   long long np, units;
   int max_rows, units_per_group;
@@ -796,7 +815,7 @@ LogitPlan logit_plan(const Problem& P) {
   p.slices = 1;
   p.per_slice = (int)nchunks;
   p.dots_bytes = p.lse_bytes = p.partial_bytes = 0;
-  if (unit_bytes > (long long)kLogitsCap || score_sm100_shape_ok(P)) return p;
+  if (unit_bytes > (long long)kLogitsCap || score_sm100_shape_ok(P) || few_rows(P)) return p;
   const long long per = (long long)kLogitsCap / unit_bytes < 65535 ? (long long)kLogitsCap / unit_bytes : 65535;
   const long long groups = (p.units + per - 1) / per;
   p.units_per_group = (int)((p.units + groups - 1) / groups);   // groups of even size

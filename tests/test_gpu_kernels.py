@@ -214,10 +214,28 @@ def test_ranking_into_arrays_that_start_on_four_bytes(L, Hkv, N):
     (2, 6, 3, 3, 9000),                            # six rows: a second CTA of rows in every slice
     (1, 4, 1, 160, 20001),                         # 640 rows, 160 CTAs: slices of three chunks, the last one shorter
     (1, 2, 1, 1, 380929), (1, 2, 1, 1, 1050000),   # slices of one chunk; the log-sum-exp of more chunks than a warp
+    (1, 1, 1, 2, 114687), (1, 1, 1, 2, 114688),    # few rows: kept logits, and the two sweeps from here on
+    (1, 1, 1, 4, 360448), (1, 1, 1, 5, 360448),    # ... the most rows for the sweeps, and one more
 ])
 def test_scoring_of_long_contexts_on_the_cuda_cores(L, Hq, Hkv, w, N):
     cfg = W.WorkloadConfig("long", L, Hq, Hkv, 64, N, w, dtype="f32", elem_std=1.0, hh_frac=0.0)
     dev, wl, desc = _setup(cfg)
+    out = alloc_outputs(desc, 1, wl.k[0].dtype, dev)
+    kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
+    torch.cuda.synchronize()
+    Pz.assert_scores_close(out.scores.cpu().numpy(), Pz.oracle_scores(wl, desc))
+
+
+@pytest.mark.parametrize("G,w", [(1, 6), (1, 7), (2, 2), (3, 1)])
+def test_few_rows_of_bf16_with_an_explicit_map(G, w):
+    """Two units of 131072 tokens: up to 6 rows of one query head, 2 of two heads go to the two sweeps."""
+    import ctypes
+    N, Hkv = 131072, 2
+    cfg = W.WorkloadConfig("few", 1, G * Hkv, Hkv, 64, N, w, dtype="bf16", elem_std=1.0, hh_frac=0.0)
+    dev, wl, desc = _setup(cfg)
+    members = (ctypes.c_int32 * (G * Hkv))(*[(j + 1) % Hkv for j in range(G * Hkv)])
+    desc.q_to_kv = ctypes.cast(members, ctypes.POINTER(ctypes.c_int32))
+    assert not kvc.kvc_score_uses_tensor_cores(desc)
     out = alloc_outputs(desc, 1, wl.k[0].dtype, dev)
     kvc.kvc_score(desc, wl.q, wl.k, out.scores, out.workspace)
     torch.cuda.synchronize()
