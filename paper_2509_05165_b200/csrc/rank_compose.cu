@@ -353,12 +353,13 @@ __device__ __forceinline__ int merge_path_warp(int diag, int na, int nb, const u
 
 // Bound by the latencies of a tile (split search, loads, merge) at four CTAs per SM; a thread reads one key per output, the
 // successor of the one it took.  (Both runs' heads at every step and outputs written to shared memory at a stride of 8:
-// the ranking of 28 segments of 131072, two levels, 118 -> 101 us; with 256 threads of 16 outputs 110, with 1024 of 4 109.)
+// the ranking of 28 segments of 131072, two levels, 118 -> 101 us; with 256 threads of 16 outputs 110, with 1024 of 4 109.
+// Left to itself the compiler takes 40 registers where kVec is false, and three CTAs fit: 112 segments of 131071 492 us, 458 so.)
 // kVec: rows start on 16 bytes (N a multiple of 4, both output arrays aligned): a thread stores its outputs itself, 16 bytes at a time.  Otherwise
 // they go through shared memory once more; a tile's element i sits in slot i + i / kMergeItems there, so that the threads'
 // stretches begin in different banks.
 template <bool kVec>
-__global__ void __launch_bounds__(kMergeThreads)
+__global__ void __launch_bounds__(kMergeThreads, 4)
 merge_runs_kernel(const uint32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in,
                   uint32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out, long long seg_len, long long run,
                   int tiles_per_seg) {
