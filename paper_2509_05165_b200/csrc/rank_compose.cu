@@ -113,16 +113,10 @@ __device__ __forceinline__ void seg_load_keys(const float* s_in, int N, int tid,
   for (int j = 0; j < kIpt; ++j) k[j] = (((j >> 2) * T + tid) * 4 + (j & 3)) < N ? seg_key(v[j]) : 0u;
 }
 
+// N elements, from `first` on in all three arrays; their positions count from pos0.
 template <int T, int kIpt>
-__global__ void __launch_bounds__(T, 1024 / T)
-segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ keys_out,
-                    int32_t* __restrict__ idx_out, long long seg_len, int chunks, int chunk_len) {
-  // CTA x sorts chunk x % chunks of segment x / chunks: the positions from chunk * chunk_len on (the chunks of a
-  // segment of several are merged afterwards)
-  const long long seg = blockIdx.x / (unsigned)chunks;
-  const int chunk = (int)(blockIdx.x - seg * chunks);
-  const long long first = seg * seg_len + (long long)chunk * chunk_len;     // of this chunk, in all three arrays
-  const int N = (int)min((long long)chunk_len, seg_len - (long long)chunk * chunk_len);
+__device__ __forceinline__ void segment_sort(const float* __restrict__ scores, uint32_t* __restrict__ keys_out,
+                                             int32_t* __restrict__ idx_out, long long first, int N, int pos0) {
   constexpr int kRowShift = T == 1024 ? 12 : T == 512 ? 11 : T == 256 ? 10 : 9;   // log2 of a row of counters in bytes
   static_assert((4 * T) >> kRowShift == 1 && kIpt % 8 == 0 && kIpt <= 32, "rows of counters, groups of places");
   constexpr int kScanWarps = T / 64;                        // the scan runs on the first T / 2 threads
@@ -301,12 +295,28 @@ segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ key
   // ---- out: the positions (a slot's position is key_slot of it: the map is its own inverse), and the keys
   uint32_t* k_out = keys_out + first;
   int32_t* i_out = idx_out + first;
-  const int pos0 = chunk * chunk_len;
   for (int j = tid; j < N; j += T) {
     const uint32_t q = lds_u16(perm + place_slot((uint32_t)j) * 2u);
     i_out[j] = pos0 + (int32_t)key_slot(q);
     k_out[j] = lds_u32(keys + q * 4u) + kmin;
   }
+}
+
+// CTA x sorts chunk x % chunks of segment x / chunks: the positions from chunk * chunk_len on (the chunks of a
+// segment of several are merged afterwards).  kShort: the last chunk of a segment is at most half as long as kIpt places
+// per thread are made for; with them a few warps would do all of its work (the ranking of 80 segments of 40000: 125 -> 101 us,
+// of 32772: 106 -> 93).
+template <int T, int kIpt, bool kShort = false>
+__global__ void __launch_bounds__(T, 1024 / T)
+segment_sort_kernel(const float* __restrict__ scores, uint32_t* __restrict__ keys_out,
+                    int32_t* __restrict__ idx_out, long long seg_len, int chunks, int chunk_len) {
+  const long long seg = blockIdx.x / (unsigned)chunks;
+  const int chunk = (int)(blockIdx.x - seg * chunks), pos0 = chunk * chunk_len;
+  const long long first = seg * seg_len + pos0;
+  const int N = (int)min((long long)chunk_len, seg_len - pos0);
+  if (kShort && N <= T * 8) segment_sort<T, 8>(scores, keys_out, idx_out, first, N, pos0);
+  else if (kShort && N <= T * 16) segment_sort<T, 16>(scores, keys_out, idx_out, first, N, pos0);
+  else segment_sort<T, kIpt>(scores, keys_out, idx_out, first, N, pos0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -515,7 +525,7 @@ struct SegmentPlan {
 // with 128 x 32 (31.7 tested).  Beyond, 24 or 32 places, which move the most elements per SM: 1024 segments of 5003: 92 with
 // 256 x 24, 108 with 512 x 16, 113 with 256 x 32 (116 before); 256 of 8192: 33.7 with 256 x 32, 35.3 with 512 x 16; of 16384: 60 with
 // 512 x 32, of which two fit an SM, 71 with 1024 x 16 (98 before).
-static SegmentPlan segment_plan(long long N) {
+static SegmentPlan segment_plan(long long N, bool short_last) {
   if (N <= 1024) return {segment_sort_kernel<128, 8>, 128};
   if (N <= 2048) return {segment_sort_kernel<128, 16>, 128};
   if (N <= 4096) return {segment_sort_kernel<256, 16>, 256};
@@ -524,26 +534,28 @@ static SegmentPlan segment_plan(long long N) {
   if (N <= 12288) return {segment_sort_kernel<512, 24>, 512};
   if (N <= 16384) return {segment_sort_kernel<512, 32>, 512};
   if (N <= 24576) return {segment_sort_kernel<1024, 24>, 1024};
+  if (short_last) return {segment_sort_kernel<1024, 32, true>, 1024};
   return {segment_sort_kernel<1024, 32>, 1024};
 }
 
-// Can a segment of N elements be sorted inside one SM here?  Sets the shared-memory attribute once
+// Can a segment (or, of several, a chunk) of N elements be sorted inside one SM here?  Sets the shared-memory attribute once
 // per device (it is per device), under a lock.
-static kvc_status segment_sort_prepare(long long N, SegmentPlan* plan) {
+static kvc_status segment_sort_prepare(long long N, bool short_last, SegmentPlan* plan) {
   if (N > kSegMaxN) return KVC_ERR_UNSUPPORTED;
   static std::mutex mu;
   static int optin[kMaxDevices];           // 0: not looked at, else the device's opt-in bytes (or -1)
   int dev = 0;
   KVC_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return KVC_ERR_UNSUPPORTED;
-  *plan = segment_plan(N);
+  *plan = segment_plan(N, short_last);
   const size_t need = seg_layout(N, plan->threads).total;
   std::lock_guard<std::mutex> lock(mu);
   if (optin[dev] == 0) {
     int bytes = 0;
     KVC_CUDA(cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     for (long long n : {1024LL, 2048LL, 4096LL, 6144LL, 8192LL, 12288LL, 16384LL, 24576LL, (long long)kSegMaxN})
-      KVC_CUDA(cudaFuncSetAttribute(segment_plan(n).kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+      for (bool s : {false, true})
+        KVC_CUDA(cudaFuncSetAttribute(segment_plan(n, s).kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     optin[dev] = bytes > 0 ? bytes : -1;
   }
   if (optin[dev] < 0 || need > (size_t)optin[dev]) return KVC_ERR_UNSUPPORTED;
@@ -608,11 +620,13 @@ kvc_status launch_compose(const Problem& P, const float* scores, int32_t* idx, f
   SegmentPlan plan;
   const Chunking cut = chunking(P);
   const long long chunk_len = cut.len;
-  const kvc_status seg_state = segment_sort_prepare(chunk_len, &plan);
+  // (only where it is short: the copy for both takes a percent longer on whole chunks)
+  const bool short_last = P.N - (cut.count - 1) * chunk_len <= kSegMaxN / 2;
+  const kvc_status seg_state = segment_sort_prepare(chunk_len, short_last, &plan);
   if (seg_state != KVC_OK && seg_state != KVC_ERR_UNSUPPORTED) return seg_state;
   if (seg_state != KVC_OK) {
     set_error("compose: this device cannot give a CTA the %zu bytes of shared memory the ranking needs",
-              (size_t)seg_layout(chunk_len, segment_plan(chunk_len).threads).total);
+              (size_t)seg_layout(chunk_len, segment_plan(chunk_len, short_last).threads).total);
     return KVC_ERR_UNSUPPORTED;
   }
   {

@@ -125,6 +125,34 @@ def test_ranking_at_the_switches_of_the_cta_size(N):
     Pz.assert_compose_exact(S, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
 
 
+def _rank_many_segments(N):
+    """Eq. 17 on 80 segments (so many that none is cut for the sake of idle SMs) of five kinds of scores in turn."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    L, Hkv = 10, 8
+    desc = kvc.kvc_desc_init(L, 1, Hkv, Hkv, 64, N, 1, kvc.F32)
+    g = np.random.default_rng(N)
+    x = g.random((5, N), dtype=np.float32)
+    kinds = np.stack([x[0], np.round(x[1] * 5) / 8, (1 + x[2] * 1e-4) / N, np.full(N, 0.25), np.exp(-80 * x[4])]).astype(np.float32)
+    S = kinds[np.arange(L * Hkv) % 5].reshape(L, 1, Hkv, N)
+    idx = torch.empty((L, 1, Hkv, N), dtype=torch.int32, device=dev)
+    comp = torch.empty((L, 1, N), dtype=torch.float32, device=dev)
+    ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+    kvc.kvc_compose(desc, torch.from_numpy(S).to(dev), idx, comp, ws)
+    torch.cuda.synchronize()
+    got = idx.cpu().numpy().reshape(L * Hkv, N)
+    Pz.assert_rank_exact(kinds, got[:5])
+    assert np.array_equal(got, got[:5][np.arange(L * Hkv) % 5])
+    Pz.assert_compose_exact(S, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
+
+
+@pytest.mark.parametrize("N", [32769, 40960, 40961, 49152, 49153, 65537])
+def test_ranking_of_segments_with_a_short_last_chunk(N):
+    """Last chunks of one element, of the most for 8 and for 16 places per thread, and of one more."""
+    _rank_many_segments(N)
+
+
 @pytest.mark.parametrize("N", [1, 1023, 1024, 1030])
 @pytest.mark.parametrize("Hkv", [1, 9])
 def test_streams_of_the_head_sharded_pass_and_composite(N, Hkv):
