@@ -838,13 +838,10 @@ LogitPlan logit_plan(const Problem& P) {
 
 template <typename T, int D, int kTT>
 kvc_status run_logits_t(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
-                      const LogitPlan& pl, char* ws, int* device_status, cudaStream_t st) {
+                      const LogitPlan& pl, int sms, char* ws, int* device_status, cudaStream_t st) {
   constexpr int kTileRow = kLogitTileRows<kTT>;
   constexpr int kSmem = (2 * kTileTok + kTileRow) * (D + 4) * (int)sizeof(float);
   KVC_CUDA(cudaFuncSetAttribute(score_logits_kernel<T, D, kTT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-  int dev = 0, sms = 0;
-  KVC_CUDA(cudaGetDevice(&dev));
-  KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int row_tiles = (pl.max_rows + kTileRow - 1) / kTileRow;
   const int tok_tiles = (int)((P.N + kTileTok - 1) / kTileTok);
   LogitParams lp;
@@ -888,11 +885,14 @@ kvc_status run_logits_t(const Problem& P, const GroupMap& gm, const LayerPtrs& q
 template <typename T, int D>
 kvc_status run_logits(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, float* scores,
                       const LogitPlan& pl, char* ws, int* device_status, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  KVC_CUDA(cudaGetDevice(&dev));
+  KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   // (in items of 32 rows the product reads twice the operands per multiply-add: only where items of 128 rows would be mostly
   // empty or fewer than the SMs)
   const long long items = (long long)pl.units_per_group * ((pl.max_rows + 127) / 128) * ((P.N + kTileTok - 1) / kTileTok);
-  if (pl.max_rows <= 32 || items < 148) return run_logits_t<T, D, 2>(P, gm, q, k, scores, pl, ws, device_status, st);
-  return run_logits_t<T, D, 8>(P, gm, q, k, scores, pl, ws, device_status, st);
+  if (pl.max_rows <= 32 || items < sms) return run_logits_t<T, D, 2>(P, gm, q, k, scores, pl, sms, ws, device_status, st);
+  return run_logits_t<T, D, 8>(P, gm, q, k, scores, pl, sms, ws, device_status, st);
 }
 
 }  // namespace
