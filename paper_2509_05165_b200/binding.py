@@ -129,8 +129,11 @@ def _stream(stream) -> C.c_void_p:
     if stream is None:
         if not torch.cuda.is_initialized() and not torch.cuda.is_available():
             return C.c_void_p(None)      # argument errors are still reported; nothing can launch
-        # (the raw handle: building a Stream object takes longer than a kernel launch)
-        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # (the raw handle where this torch has it: building a Stream object takes longer than a kernel launch)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return C.c_void_p(raw(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 

@@ -145,3 +145,17 @@ def test_test_hooks_take_and_restore_their_settings_without_a_device():
     kvc.kvc_debug_select_hooks()                 # automatic choice, default bound
     kvc.kvc_debug_score_hooks(1000000, 3)
     kvc.kvc_debug_score_hooks()                  # default wait bound, nothing withheld
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_with_and_without_the_raw_handle(monkeypatch, raw):
+    """The handle of the current stream, on a torch that has the call for it and on one that has not."""
+    import types
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=4096))
+    if raw:
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 4096 + dev, raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert binding._stream(None).value == 4096
