@@ -18,6 +18,8 @@
  *   - Work is enqueued on `stream` (a cudaStream_t passed as void*, NULL = the default stream);
  *     calls return without synchronising.  The return value reports errors the host can see
  *     (bad arguments, a failed launch); kvc_last_error() then holds a message.
+ *   - Q, K, V, K' and V' start on 16 bytes (see the layouts below); every other array needs the
+ *     alignment of its elements only.
  *   - Inputs are never modified.  Indices are 0-based.  Sequences of a batch are independent:
  *     each has its own pool and its own budget (the paper has no batch dimension).
  *   - Finite inputs are a precondition; NaN/Inf in Q or K give unspecified scores.

@@ -2,7 +2,7 @@
 //
 // This is the shape-agnostic path: fp32 or bf16 inputs, head_dim 64 or 128, any window length,
 // any GQA map.  Where the logits of a (layer, sequence, KV head) fit a bounded buffer they are computed once and kept
-// (second part of this file); otherwise it makes two sweeps over K.  Sweep 1 produces, for every query row, the
+// (second part of this file); otherwise, and for few rows over many tokens, it makes two sweeps over K.  Sweep 1 produces, for every query row, the
 // log-sum-exp of its logits over the visible keys (per-chunk partials, then a combine kernel).
 // Sweep 2 recomputes the logits and emits exp(s - lse) -- the softmax weight of Eq. 3 -- reduced
 // over the window rows (Eq. 14) and over the query heads of the KV head (Eq. 15).  A last kernel

@@ -32,10 +32,11 @@
 //                        exp(max_m(s_m - lse_m)): one exponential per query head, not per row.
 //
 // A unit is a (layer, sequence, KV head, row tile): the G x w window rows of a KV head are cut
-// into row tiles of at most 128 rows (whole query heads), so that any GQA group / window size
-// with w <= 128 runs here (w = 8, 16, 32, 64, 128 as compile-time specialisations, any other
-// length through one variant that reads it at run time); with more than one row tile the
-// pass-2 results are partial group aggregates that the Eq. 16 kernel combines in a fixed order.
+// into row tiles of at most 128 rows: whole query heads where w <= 128 (w = 8, 16, 32, 64, 128 as
+// compile-time specialisations, any other length through one variant that reads it at run time),
+// pieces of one query head for longer windows, so that any GQA group and window runs here; with
+// more than one row tile the pass-2 results are partial aggregates that the Eq. 16 kernel combines
+// in a fixed order.
 //
 // The two passes of a CTA are two pipelines of their own (copies -> K stages and Q slots -> MMAs ->
 // accumulators -> epilogue) over the same list of runs; they share nothing but the issue slots and the
@@ -57,9 +58,12 @@
 // scoring of the 8B shape at 32K: 684 -> 656 us).  With one producer and one K and Q ring for both passes,
 // every one of these warps had to follow both passes tile by tile, 1100 (issuers) to 1500 (producer) clocks
 // of bookkeeping out of the 2160 that a pair of tiles took; with a pipeline per pass a pair takes 1890 (32K: 656 ->
-// 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers).  What bounds it now is the board's power:
-// at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds, and copies of the kernel with work left
-// out are faster by that work's energy (an eighth of the MMAs -25 %, of the exponentials -5 %, of the maxima -5 %).
+// 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers).  (Those are a back-to-back run's times at its
+// 1.4 GHz; a capture of 4 layers at 1.7 GHz has 2370 clocks per pair, start and drain included.)
+// No unit is saturated: tensor pipe and special-function pipe are half busy, DRAM less.  A copy of the kernel with an
+// eighth of the MMAs, exponentials and maxima still takes 455 of 715 us, so more than half of the time is the K tiles' way
+// into shared memory, once per pass and row tile, and their hand-over from role to role.  Run back to back the board's
+// power adds a sixth: at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds (560 -> 660 us).
 #include <cuda.h>
 
 #include <atomic>

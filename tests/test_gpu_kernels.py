@@ -108,7 +108,8 @@ def test_selection_at_the_limits_of_its_kernel(L, Hkv, N, kind):
 
 @pytest.mark.parametrize("N", [8, 1024, 1025, 2048, 2049, 6144, 6145, 12288, 12289, 16384, 16385, 24576, 24577])
 def test_ranking_at_the_switches_of_the_cta_size(N):
-    """Eq. 17 on random and heavily tied scores: full and barely started CTAs of every size."""
+    """Eq. 17 on random and heavily tied scores of two segments: CTAs of every size up to 8192 elements, full and barely started;
+    longer segments are cut into chunks of about that for the sake of idle SMs (in two, three and four here) and merged."""
     cfg = W.WorkloadConfig("rank_switch", 1, 2, 2, 64, N, 1, dtype="f32", elem_std=1.0)
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -145,6 +146,12 @@ def _rank_many_segments(N):
     Pz.assert_rank_exact(kinds, got[:5])
     assert np.array_equal(got, got[:5][np.arange(L * Hkv) % 5])
     Pz.assert_compose_exact(S, idx.cpu().numpy(), comp.cpu().numpy(), desc.agg_head)
+
+
+@pytest.mark.parametrize("N", [8193, 12288, 12289, 16384, 16385, 24576, 24577, 32767, 32768])
+def test_ranking_at_the_switches_of_the_larger_cta_sizes(N):
+    """Segments in one chunk each: 512 and 1024 threads with 24 and 32 places, full and barely started."""
+    _rank_many_segments(N)
 
 
 @pytest.mark.parametrize("N", [32769, 40960, 40961, 49152, 49153, 65537])
