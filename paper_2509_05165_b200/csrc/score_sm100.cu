@@ -449,9 +449,9 @@ struct SmemLayout : Rings<D> {
                                                                // -log-sum-exp of the pass-2 unit
   static constexpr int kStats = kNegLse + kRows * 4;           // 2 x 128 rows x float2: the upper half's statistics
   static constexpr int kTotal = kStats + 2 * kRows * 8;
-  // TMEM columns: the accumulator of pass 1, the two of pass 2, pass 1's Q
+  // TMEM columns: the accumulator of pass 1, the two of pass 2, pass 1's Q (two sets)
   static constexpr int kAcc1 = 0, kAcc2 = kTile, kQt = 3 * kTile;
-  static_assert(kQt + D / 2 <= 512, "TMEM columns");
+  static_assert(kQt + 2 * (D / 2) <= 512, "TMEM columns");
   static_assert(kCtl % 8 == 0 && kNegLse % 16 == 0 && kStats % 8 == 0 && kTotal <= 232448, "shared-memory layout");
 };
 
@@ -998,18 +998,18 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
       const uint32_t idesc = umma_idesc(pass == 0 ? kTile : (c.template rows<kLong>(P) + 31) / 32 * 32);
       qr.next(slots);
-      if (pass == 0 && ok && issued)
-        // the MMAs of the run before read the Q columns: their last tile has to be complete.  (The tensor pipe runs an MMA
-        // behind the copies issued before it, as PTX guarantees for tcgen05.cp -> tcgen05.mma, but it promises nothing for a copy
-        // issued behind an MMA.)  The accumulator that the tile fills is free later still, so the first MMA below waits longer.
-        ok = mbar_wait_warp(bar_tfull(0), (uint32_t)(tb.phase ^ 1), ctl);
+      const uint32_t q_tmem = tmem_base + SL::kQt + (uint32_t)(k & 1) * (D / 2);   // pass 1
       if (pass == 0 && ok) {
-        // the run's Q moves to TMEM, its slot is free again
+        // The run's Q moves to TMEM, its slot is free again.  Two sets of columns in turn: PTX runs an MMA behind the copies issued
+        // before it (tcgen05.cp -> tcgen05.mma), but promises nothing for a copy issued behind an MMA, and the MMAs of the run
+        // before may still read their set.  Those of the run before that, which read this one, are complete: the first tile of the
+        // run before was issued only when the epilogue had emptied the accumulator of their last tile.  (One set, and a wait for
+        // the last MMAs in front of the copy: 448 rows per token at 128K 4457 -> 4491 us per pass, 500-row windows 1225 -> 1234.)
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk)
-            tc_cp_256b(tmem_base + SL::kQt + kk * 8, dq + (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4));
+            tc_cp_256b(q_tmem + kk * 8, dq + (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4));
           tc_commit(bar_qfree(slot));
         }
         __syncwarp();
@@ -1030,7 +1030,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-              tc_mma_bf16_ts(d_tmem, tmem_base + SL::kQt + kk * 8, dk + off, idesc, kk > 0);
+              tc_mma_bf16_ts(d_tmem, q_tmem + kk * 8, dk + off, idesc, kk > 0);
             }
           } else {
 #pragma unroll
