@@ -59,7 +59,7 @@
 // every one of these warps had to follow both passes tile by tile, 1100 (issuers) to 1500 (producer) clocks
 // of bookkeeping out of the 2160 that a pair of tiles took; with a pipeline per pass a pair takes 1890 (32K: 656 ->
 // 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers).  (Those are a back-to-back run's times at its
-// 1.4 GHz; a capture of 4 layers at 1.7 GHz has 2370 clocks per pair, start and drain included.)
+// 1.4 GHz; a capture of 4 layers at 1.8 GHz has 2380 clocks per pair, start and drain included.)
 // No unit is saturated: tensor pipe and special-function pipe are half busy, DRAM less.  A copy of the kernel with an
 // eighth of the MMAs, exponentials and maxima still takes 455 of 715 us, so more than half of the time is the K tiles' way
 // into shared memory, once per pass and row tile, and their hand-over from role to role.  Run back to back the board's
