@@ -39,11 +39,9 @@
 // in a fixed order.
 //
 // The two passes of a CTA are two pipelines of their own (copies -> K stages and Q slots -> MMAs ->
-// accumulators -> epilogue) over the same list of runs; they share nothing but the issue slots and the
-// tensor pipe.  Pass 1 has its Q, the row operand, in TMEM (copied there once per run) and one
-// accumulator, which its epilogue empties at once: a quarter of the MMAs' operand reads leave shared
-// memory, whose data banks are busy four fifths of the time (500-row windows: 1303 -> 1277 us per pass;
-// the 8B shape gains 0.2 %).  Pass 2 goes as fast as the statistics arrive; pass 1 is held to at most
+// accumulators -> epilogue) over the same list of runs; they share nothing but the issue slots, the
+// tensor pipe and shared memory.  Pass 1 has its Q, the row operand, in TMEM (copied there once per run) and one
+// accumulator, which its epilogue empties at once.  Pass 2 goes as fast as the statistics arrive; pass 1 is held to at most
 // `lead` tiles ahead of it (two runs where a unit has no more runs than there are CTAs: 38 MB of K at
 // 148 CTAs, which L2 still holds), exactly what the statistics need: they need every run of a unit, and
 // the other CTAs' runs of it lie that far ahead at most, so the CTAs cannot wait for each other in a
@@ -52,18 +50,25 @@
 //
 // Warp roles (512 threads): warp 0 = TMA producer of pass 1 (K, Q, L2 prefetch), warp 3 = of pass 2; warp
 // 1 = MMA issuer of pass 1 and TMEM owner, warp 2 = of pass 2; warps 4-7 = pass-2 epilogue; warps 8-15 = pass-1
-// epilogue (two groups of four warps, each takes one half of every tile's columns).  The four single warps
+// epilogue, two groups of four warps.  The four single warps
 // run their loops with all lanes and elect a lane for each MMA, commit or copy: from one lane of a diverged
-// warp every such instruction first moves its operands to uniform registers, about 50 clocks per MMA (the
-// scoring of the 8B shape at 32K: 684 -> 656 us).  With one producer and one K and Q ring for both passes,
-// every one of these warps had to follow both passes tile by tile, 1100 (issuers) to 1500 (producer) clocks
-// of bookkeeping out of the 2160 that a pair of tiles took; with a pipeline per pass a pair takes 1890 (32K: 656 ->
-// 600 us; window 64 and GQA group 7 at 128K: 1140 -> 960 us for 7 layers).  (Those are a back-to-back run's times at its
-// 1.4 GHz; a capture of 4 layers at 1.8 GHz has 2380 clocks per pair, start and drain included.)
-// No unit is saturated: tensor pipe and special-function pipe are half busy, DRAM less.  A copy of the kernel with an
-// eighth of the MMAs, exponentials and maxima still takes 455 of 715 us, so more than half of the time is the K tiles' way
-// into shared memory, once per pass and row tile, and their hand-over from role to role.  Run back to back the board's
-// power adds a sixth: at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds (560 -> 660 us).
+// warp every such instruction first moves its operands to uniform registers, about 50 clocks per MMA.
+//
+// What bounds it, in clocks per pair of tiles (128 rows x 128 tokens, heads of 128, both passes): tensor pipe and
+// special-function pipe 1024 each; shared memory most: K copied in 512, Q (written twice, read once, per run) 192, pass 1's
+// operand reads 256, pass 2's 512 (both operands come from there: a 128 x 128 x 16 MMA reads 8 KB in its 64 clocks), and 270 for
+// the -log-sum-exps that every tile of pass 2 reads (a 16-byte load by all lanes of one address takes 2.1 clocks of the SM):
+// 1742 of the 1890 that a pair took.  Hence:
+//   - one row tile per unit: the pass-2 epilogue keeps a run's 128 -log-sum-exps in registers (216 per thread, taken from the
+//     single warps and from pass 1 by setmaxnreg) and reads them once per run: 8B shape at 32K 1078 -> 1060 us per pass, at 8K
+//     1 %, 4 sequences of 5003 with heads of 64 442 -> 430.
+//   - several row tiles: a work unit has two of them, which share every K tile in shared memory (256 instead of 512).  Pass 1's
+//     two groups then take a row tile each, a tile's 128 columns at once in registers (168 per thread), where with one row tile
+//     each takes half of the columns of every tile and both are at the exponentials, and at everything else, at the same
+//     time: window 64, GQA group 7 at 128K 4400 -> 4280 us per pass, 500-row windows 1203 -> 1158; 1690 clocks per pair.
+// Registers decide the rest: a warp's 128 exponentials take 1134 clocks when the compiler has room to overlap them and 2125
+// when it has not (it then waits for every pair), so in the second form the logits die in their exponentials.
+// Run back to back the board's power adds a sixth: at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds.
 #include <cuda.h>
 
 #include <atomic>
@@ -76,6 +81,14 @@ namespace {
 
 constexpr int kTile = 128;            // tokens per tile = MMA M = MMA N
 constexpr int kFastThreads = 512;
+// Registers per thread of the warpgroups, out of the 128 that the kernel starts with: the single warps, the pass-2 epilogue
+// and the pass-1 epilogue's two groups.  With one row tile pass 2 keeps a run's -log-sum-exps, with two pass 1 a whole tile's logits.
+// (A kernel that moves registers must not call functions out of line: ptxas 12.9 crashes on it, so the cold paths are inlined.)
+constexpr int kRegsStart = 128;
+template <int kRT> struct Regs;
+template <> struct Regs<1> { static constexpr int kSingle = 56, kP2 = 216, kP1 = 120; };
+template <> struct Regs<2> { static constexpr int kSingle = 64, kP2 = 112, kP1 = 168; };
+
 constexpr int kRows = 128;            // query rows per unit handled by one MMA (R <= 128)
 constexpr int kMinRunTiles = 4;       // tiles per run; runs are longer only where a unit would otherwise have more than 255
 constexpr int kPrefetch = 2;          // pass-1 tiles prefetched into L2 ahead of their load
@@ -99,14 +112,15 @@ struct FastParams {
   float* scores;               // [L*Bt*Hkv][N], or with QT > 1 the partial aggregates [QT][L*Bt*Hkv][N]
   int L, Bt, Hkv, G;
   int HPT, QT, w;              // query heads per row tile, row tiles per KV head, window rows per query head
+  int QP;                      // work units per KV head: QT, or with two row tiles per unit ceil(QT / 2)
   int CH;                      // row tiles per query head: 1, or ceil(w / 128) for windows longer than 128 rows
                                // (then HPT = 1 and row tile q holds rows (q % CH) * 128 .. of query head q / CH)
   long long N, q_pos0;
   int U, NT, RPU, grid;        // units, tiles per unit, runs per unit, CTAs
   int RT;                      // tiles per run
   int step_u, step_j;          // grid = step_u * RPU + step_j: how a CTA's next run moves (unit, run in unit)
-  int step_l, step_b, step_h, step_q;  // step_u = ((step_l * Bt + step_b) * Hkv + step_h) * QT + step_q
-  unsigned int total_runs;     // U * RPU
+  int step_l, step_b, step_h, step_q;  // step_u = ((step_l * Bt + step_b) * Hkv + step_h) * QP + step_q
+  unsigned int total_runs;     // runs of all work units
   int lead;                    // tiles by which pass 1 may be ahead of pass 2 (their K copies)
   float sl2e;                  // scale * log2(e)
   int agg_group;
@@ -153,16 +167,16 @@ struct Ctl {
 };
 // Called from the slow part of every wait loop: has this CTA, or any other, given up, or has this
 // wait lasted longer than the bound?  (Then it marks the CTA as aborted.)
-__device__ __noinline__ bool give_up(volatile Ctl* ctl, unsigned long long t0) {
+__device__ __forceinline__ bool give_up(volatile Ctl* ctl, unsigned long long t0) {
   if (ctl->abort) return true;
   const int* gs = ctl->grid_status;
   if (gs != nullptr && *reinterpret_cast<const volatile int*>(gs) != 0) { ctl->abort = 1; return true; }
   if (globaltimer_ns() - t0 > ctl->limit_ns) { ctl->abort = 1; return true; }
   return false;
 }
-// Bounded wait.  Returns false when the CTA has given up (see give_up).  The retry loop is kept
-// out of line: the kernel's hot loops have to stay small enough for the instruction cache.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
+// Bounded wait.  Returns false when the CTA has given up (see give_up).  The retry loop is for
+// the rare case.
+__device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
   const unsigned long long t0 = globaltimer_ns();
   uint32_t spins = 0;
   while (!mbar_try(bar, parity)) {
@@ -182,7 +196,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, ctl));
 }
 // Pass 1 may copy tile `pos` once fewer than `lead` tiles lie between it and pass 2 (bounded; one answer per warp).
-__device__ __noinline__ bool wait_lead_slow(int pos, int lead, volatile Ctl* ctl) {
+__device__ __forceinline__ bool wait_lead_slow(int pos, int lead, volatile Ctl* ctl) {
   const unsigned long long t0 = globaltimer_ns();
   uint32_t spins = 0;
   while (pos - ctl->p2_tiles >= lead) {
@@ -202,7 +216,7 @@ __device__ __forceinline__ bool elect_one() {
 }
 // The same for a copy or an MMA that has been issued and therefore completes whatever the rest
 // of the grid does: only the time bound ends this wait early, not the abort flag.
-__device__ __noinline__ bool mbar_wait_issued(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
+__device__ __forceinline__ bool mbar_wait_issued(uint32_t bar, uint32_t parity, volatile Ctl* ctl) {
   const unsigned long long t0 = globaltimer_ns();
   uint32_t spins = 0;
   while (!mbar_try(bar, parity)) {
@@ -276,6 +290,22 @@ __device__ __forceinline__ void tc_wait_ld(uint32_t (&r)[32]) {
         "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
       :: "memory");
 }
+// The same for 16 columns.
+__device__ __forceinline__ void tc_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tc_wait_ld(uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.wait::ld.sync.aligned;"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+      :: "memory");
+}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -309,6 +339,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
+}
+// The registers per thread of the calling warpgroup.
+template <int N> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_set() {
+  if constexpr (N > kRegsStart) regs_inc<N>(); else if constexpr (N < kRegsStart) regs_dec<N>();
 }
 __device__ __forceinline__ void named_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
@@ -367,41 +403,50 @@ __device__ __forceinline__ void combine(float& M, float& Ls, float m, float l) {
 // exponentials in the special-function pipe.
 // ------------------------------------------------------------------------------------------------
 struct RunCursor {
-  int u, j;         // unit, run inside the unit
-  int l, b, h, q;   // the unit's layer, sequence, KV head, row tile
+  int j;            // run inside the work unit
+  int l, b, h, q;   // the work unit's layer, sequence, KV head, and which of the KV head's work units it is
   __device__ __forceinline__ void init(const FastParams& P) {
-    u = (int)(blockIdx.x / (unsigned int)P.RPU);
+    const int u = (int)(blockIdx.x / (unsigned int)P.RPU);
     j = (int)(blockIdx.x - (unsigned int)u * (unsigned int)P.RPU);
-    const int uh = u / P.QT;
-    q = u - uh * P.QT;
+    const int uh = u / P.QP;
+    q = u - uh * P.QP;
     const int lb = uh / P.Hkv;
     h = uh - lb * P.Hkv;
     l = lb / P.Bt;
     b = lb - l * P.Bt;
   }
-  // window rows of this unit's row tile (whole query heads; the last tile of a KV head may be short)
+  // row tiles of this work unit (kRT, but for a KV head's last one)
+  template <int kRT>
+  __device__ __forceinline__ int row_tiles(const FastParams& P) const { return kRT == 1 ? 1 : min(kRT, P.QT - q * kRT); }
+  // window rows of its row tile rt (whole query heads; the last tile of a KV head may be short)
   // (kLong: the instantiation that also handles windows longer than 128 rows, CH > 1; everywhere else
   // that case is compiled out of the hot loops)
-  template <bool kLong>
-  __device__ __forceinline__ int rows(const FastParams& P) const {
-    return (!kLong || P.CH == 1) ? min(P.HPT, P.G - q * P.HPT) * P.w : min(kRows, P.w - (q % P.CH) * kRows);
+  template <bool kLong, int kRT>
+  __device__ __forceinline__ int rows(const FastParams& P, int rt) const {
+    const int qt = q * kRT + rt;
+    return (!kLong || P.CH == 1) ? min(P.HPT, P.G - qt * P.HPT) * P.w : min(kRows, P.w - (qt % P.CH) * kRows);
   }
-  // first window row of this row tile inside its query head, and the tile's first query head in the group
-  template <bool kLong>
-  __device__ __forceinline__ int row0(const FastParams& P) const { return (!kLong || P.CH == 1) ? 0 : (q % P.CH) * kRows; }
-  template <bool kLong>
-  __device__ __forceinline__ int head0(const FastParams& P) const { return (!kLong || P.CH == 1) ? q * P.HPT : q / P.CH; }
-  // index of the (layer, sequence, KV head)
+  // first window row of the row tile inside its query head, and the tile's first query head in the group
+  template <bool kLong, int kRT>
+  __device__ __forceinline__ int row0(const FastParams& P, int rt) const {
+    return (!kLong || P.CH == 1) ? 0 : ((q * kRT + rt) % P.CH) * kRows;
+  }
+  template <bool kLong, int kRT>
+  __device__ __forceinline__ int head0(const FastParams& P, int rt) const {
+    return (!kLong || P.CH == 1) ? (q * kRT + rt) * P.HPT : (q * kRT + rt) / P.CH;
+  }
+  // index of the (layer, sequence, KV head), and of the unit (layer, sequence, KV head, row tile)
   __device__ __forceinline__ int kv_unit(const FastParams& P) const { return (l * P.Bt + b) * P.Hkv + h; }
+  template <int kRT>
+  __device__ __forceinline__ int unit(const FastParams& P, int rt) const { return kv_unit(P) * P.QT + q * kRT + rt; }
   __device__ __forceinline__ int tiles(const FastParams& P) const { return min(P.RT, P.NT - j * P.RT); }
   __device__ __forceinline__ int first_token(const FastParams& P) const { return j * P.RT * kTile; }
   __device__ __forceinline__ void next(const FastParams& P) {
     j += P.step_j;
     int c = 0;
     if (j >= P.RPU) { j -= P.RPU; c = 1; }
-    u += P.step_u + c;
     q += P.step_q + c; c = 0;
-    if (q >= P.QT) { q -= P.QT; c = 1; }
+    if (q >= P.QP) { q -= P.QP; c = 1; }
     h += P.step_h + c; c = 0;
     if (h >= P.Hkv) { h -= P.Hkv; c = 1; }
     b += P.step_b + c; c = 0;
@@ -423,13 +468,15 @@ template <int K1, int K2, int Q1, int Q2>
 struct RingSizes {
   static constexpr int kK1 = K1, kK2 = K2, kQ1 = Q1, kQ2 = Q2;
 };
-template <int D> struct Rings;
-template <> struct Rings<128> : RingSizes<3, 2, 1, 1> {};
-template <> struct Rings<64> : RingSizes<5, 5, 2, 2> {};
+template <int D, int kRT> struct Rings;
+template <> struct Rings<128, 1> : RingSizes<3, 2, 1, 1> {};
+template <> struct Rings<64, 1> : RingSizes<5, 5, 2, 2> {};
+template <> struct Rings<128, 2> : RingSizes<2, 2, 1, 2> {};
+template <> struct Rings<64, 2> : RingSizes<4, 4, 2, 4> {};
 
-template <int D>
-struct SmemLayout : Rings<D> {
-  using R = Rings<D>;
+template <int D, int kRT>
+struct SmemLayout : Rings<D, kRT> {
+  using R = Rings<D, kRT>;
   static constexpr int kHalves = D / 64;
   static constexpr int kTileBytes = kTile * D * 2;
   static constexpr int kStages = R::kK1 + R::kK2, kSlots = R::kQ1 + R::kQ2;
@@ -445,10 +492,10 @@ struct SmemLayout : Rings<D> {
   static constexpr int kBarMmaDone = kBarQFree + 8 * kSlots;   // 2 x 8
   static constexpr int kTmemSlot = kBarMmaDone + 16;           // 4 B (+ padding)
   static constexpr int kCtl = kTmemSlot + 8;                   // Ctl, 24 B
-  static constexpr int kNegLse = (kCtl + 24 + 15) / 16 * 16;   // 128 floats, read as 16-byte vectors:
-                                                               // -log-sum-exp of the pass-2 unit
-  static constexpr int kStats = kNegLse + kRows * 4;           // 2 x 128 rows x float2: the upper half's statistics
-  static constexpr int kTotal = kStats + 2 * kRows * 8;
+  static constexpr int kNegLse = (kCtl + 24 + 15) / 16 * 16;   // kRT x 128 floats, read as 16-byte vectors:
+                                                               // -log-sum-exp of the pass-2 unit's rows
+  static constexpr int kStats = kNegLse + kRT * kRows * 4;     // one row tile: 2 x 128 rows x float2: the upper half's statistics
+  static constexpr int kTotal = kStats + (kRT == 1 ? 2 * kRows * 8 : 0);
   // TMEM columns: the accumulator of pass 1, the two of pass 2, pass 1's Q (two sets)
   static constexpr int kAcc1 = 0, kAcc2 = kTile, kQt = 3 * kTile;
   static_assert(kQt + 2 * (D / 2) <= 512, "TMEM columns");
@@ -462,7 +509,7 @@ constexpr unsigned long long kAccArrival = 1ull << 56, kAccOverflow = 1ull << 48
 constexpr unsigned long long kAccSumMask = kAccOverflow - 1;
 
 // Bounded poll of a row's pushed statistics until all `runs` runs of the unit have arrived.
-__device__ __noinline__ unsigned long long poll_acc_slow(const unsigned long long* src, unsigned int runs,
+__device__ __forceinline__ unsigned long long poll_acc_slow(const unsigned long long* src, unsigned int runs,
                                                          volatile Ctl* ctl) {
   const unsigned long long t0 = globaltimer_ns();
   uint32_t spins = 0;
@@ -474,14 +521,32 @@ __device__ __noinline__ unsigned long long poll_acc_slow(const unsigned long lon
   return v;
 }
 
+// Pass 1: a run's sum of one row, 2^(logit - M) over its tokens = Ls.  The short way: rescaled to the row's fixed
+// reference and added to the row's 64-bit word (integer addition: the total does not depend on the order).
+__device__ __forceinline__ void send_sum(const FastParams& P, int unit, int run, int row, float row_ref, float M, float Ls) {
+  unsigned long long* word = P.acc + (long long)unit * kRows + row;
+  const float lv = lg2(Ls) + (M - row_ref);                     // log2 of the contribution
+  if (!(Ls > 0.f)) {
+    red_add_relaxed_u64(word, kAccArrival);
+  } else if (lv < kAccLimitLog2) {
+    red_add_relaxed_u64(word, kAccArrival + __float2ull_rn(ex2(lv + (float)kAccFracBits)));
+  } else {
+    // it does not fit: the run's record and its bit in the row's bitmap, then the arrival with
+    // release semantics, so that both are visible to whoever acquires the complete word
+    P.partial[((long long)unit * P.RPU + run) * kRows + row] = make_float2(M, Ls);
+    red_or_relaxed_u64(P.ovf + ((long long)unit * kRows + row) * 4 + (run >> 6), 1ull << (run & 63));
+    red_add_release_u64(word, kAccArrival + kAccOverflow);
+  }
+}
+
 // ------------------------------------------------------------------------------------------------
-// Cold paths, out of line: tiles that touch the causal boundary or the end of the context, and
+// Cold paths: tiles that touch the causal boundary or the end of the context, and
 // the aggregator variants other than the paper's defaults.
 // ------------------------------------------------------------------------------------------------
 
 // Pass 1, 64 columns (tokens c_first ..) of this thread's query row, with masking: the row's
 // (reference, sum) follows the running maximum.  Reads the accumulator itself.
-__device__ __noinline__ void p1_masked_half(uint32_t taddr, long long c_first, long long row_vis, float sl2e,
+__device__ __forceinline__ void p1_masked_half(uint32_t taddr, long long c_first, long long row_vis, float sl2e,
                                             float* mref_io, float* lsum_io) {
   float mref = *mref_io, lsum = *lsum_io;
 #pragma unroll 1
@@ -520,7 +585,7 @@ __device__ __noinline__ void p1_masked_half(uint32_t taddr, long long c_first, l
 // masking.  Returns the group aggregate before the division of the mean.  W is the window length
 // where it is one of the specialised powers of two, 0 where it is only known at run time (`w`).
 template <int W, bool kTaskMean>
-__device__ __noinline__ float p2_generic_tile(uint32_t taddr, const float* neg_lse, int n_chunks, int R, float sl2e,
+__device__ __forceinline__ float p2_generic_tile(uint32_t taddr, const float* neg_lse, int n_chunks, int R, float sl2e,
                                               bool full, long long m_min, int agg_group, int w) {
   float gacc = (agg_group == KVC_AGG_MAX) ? -INFINITY : 0.f;
   float hacc = kTaskMean ? 0.f : -INFINITY;
@@ -587,7 +652,7 @@ __device__ __forceinline__ void tc_ld_cols(uint32_t taddr, uint32_t (&r)[kC]) {
 // masked tiles still are, the scoring of the 8B shape at 16K takes 886 us with w = 24, 2071 with 49 and 4097 with 100; so it
 // takes 386, 649 and 1240.)  Returns the group aggregate before the division of the mean.
 template <int kC>
-__device__ __noinline__ float p2_odd_tile(uint32_t taddr, const float* neg_lse, int R, int w, float sl2e, bool gmax) {
+__device__ __forceinline__ float p2_odd_tile(uint32_t taddr, const float* neg_lse, int R, int w, float sl2e, bool gmax) {
   float gacc = gmax ? -INFINITY : 0.f;
 #pragma unroll 1
   for (int h0 = 0; h0 < R; h0 += w) {
@@ -612,7 +677,7 @@ __device__ __noinline__ float p2_odd_tile(uint32_t taddr, const float* neg_lse, 
 // than 128 rows), with masking: rows below m_min do not see the token.  Returns the tile's part of
 // Eq. 14 for the token: the largest attention weight, or the sum of the weights, over these rows.
 template <bool kTaskMean>
-__device__ __noinline__ float p2_long_tile(uint32_t taddr, const float* neg_lse, int n_chunks, int R, float sl2e,
+__device__ __forceinline__ float p2_long_tile(uint32_t taddr, const float* neg_lse, int n_chunks, int R, float sl2e,
                                            bool full, long long m_min) {
   float hacc = kTaskMean ? 0.f : -INFINITY;
 #pragma unroll 1
@@ -634,10 +699,10 @@ __device__ __noinline__ float p2_long_tile(uint32_t taddr, const float* neg_lse,
 // ------------------------------------------------------------------------------------------------
 // The kernel
 // ------------------------------------------------------------------------------------------------
-template <int D, int W, bool kTaskMean>
+template <int D, int W, bool kTaskMean, int kRT>
 __global__ void __launch_bounds__(kFastThreads, 1)
 score_sm100_kernel(const __grid_constant__ FastParams P) {
-  using SL = SmemLayout<D>;
+  using SL = SmemLayout<D, kRT>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -656,7 +721,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < SL::kStages; ++s) { mbar_init(bar_kfull(s), 1); mbar_init(bar_kempty(s), 1); }
     // the accumulators of pass 1 are read by eight warps (two column halves), those of pass 2 by four
-    for (int b = 0; b < 3; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), b == 0 ? 8 : 4); }
+    for (int b = 0; b < 3; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), b == 0 && kRT == 1 ? 8 : 4); }
+    if (kRT == 2) mbar_init(bar_tfull(3), 1);
     for (int q = 0; q < SL::kSlots; ++q) { mbar_init(bar_qfull(q), 1); mbar_init(bar_qfree(q), 1); }
     mbar_init(bar_mma_done(0), 1); mbar_init(bar_mma_done(1), 1);
     ctl->abort = 0;
@@ -682,15 +748,139 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     if (threadIdx.x == 0 && P.status) atomicCAS(P.status, 0, (int)KVC_ERR_CUDA);
     my_runs = 0;               // nothing is computed; the teardown below still frees the TMEM columns
   }
+  constexpr bool kKeep = kRT == 1 && W > 0 && !kTaskMean;   // pass 2 keeps a run's -log-sum-exps in registers
   constexpr bool kLong = (W == 0);   // only the run-time window variant has windows longer than 128 rows
   // the whole box arrives (rows outside the tensor as zeros)
   const uint32_t q_bytes = (uint32_t)((!kLong || P.CH == 1) ? P.HPT * P.w : kRows) * D * 2;
   const long long vis_all = min(P.N - 1, P.q_pos0);          // tokens up to here are seen by every row
 
-  // (The order of the roles in the code is not neutral: their hot loops share the instruction caches,
-  // and this order measured fastest.)
-  if (warp >= 8) {
-    // ============================== pass-1 epilogue ============================================
+  static_assert(Regs<kRT>::kSingle + Regs<kRT>::kP2 + 2 * Regs<kRT>::kP1 <= 4 * kRegsStart, "registers");
+  if constexpr (kRT == 2 || kKeep) { if (warp < 4) regs_set<Regs<kRT>::kSingle>(); }
+  if (kRT == 2 && warp >= 8) {
+    if constexpr (kRT == 2) {
+    // ============================== pass-1 epilogue, two row tiles =============================
+    // A group per row tile, the tiles of the two in turn.  A tile's 128 columns go to registers at once and the accumulator is free.
+    regs_set<Regs<kRT>::kP1>();
+    const int group = (warp - 8) >> 2;                // which of a work unit's row tiles
+    const int quarter = warp & 3;                     // TMEM lane quarter this warp may read
+    const int row = quarter * 32 + lane;              // TMEM lane = query row
+    const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + SL::kAcc1;
+    const int row_m = row % (W > 0 ? W : P.w);        // the row inside its query head (windows of up to 128 rows)
+    const unsigned long long scale2 = pack2(P.sl2e, P.sl2e);
+    const int bar = group * 3;
+    uint32_t n1 = 0;
+    bool ok = true;
+    const int vis_plain = (int)vis_all - (kTile - 1); // a tile whose first token is at most this has no mask (N < 2^30)
+    RunCursor c;
+    c.init(P);
+    for (int k = 0; k < my_runs; ++k, c.next(P)) {
+      if (group >= c.template row_tiles<kRT>(P)) continue;
+      const int unit = c.template unit<kRT>(P, group);
+      const bool row_used = row < c.template rows<kLong, kRT>(P, group);
+      const float row_ref = __ldg(P.ref + (long long)unit * kRows + row);
+      float mref[2] = {-INFINITY, -INFINITY}, lsum[2] = {0.f, 0.f};    // per half of the columns: sum over the run so far of 2^(logit - mref)
+      // 32 logits against a reference: packed arithmetic, four partial sums
+      auto sum_chunk = [&](const uint32_t (&r)[32], const float ref) {
+        const unsigned long long neg_ref = pack2(-ref, -ref);
+        unsigned long long acc0 = 0ull, acc1 = 0ull;        // +0.0f twice
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          const unsigned long long y0 = fma2(pack2u(r[i], r[i + 1]), scale2, neg_ref);
+          const unsigned long long y1 = fma2(pack2u(r[i + 2], r[i + 3]), scale2, neg_ref);
+          float a, b, c, d;
+          unpack2(y0, a, b);
+          unpack2(y1, c, d);
+          acc0 = add2(acc0, pack2(ex2(a), ex2(b)));
+          acc1 = add2(acc1, pack2(ex2(c), ex2(d)));
+        }
+        float s0, s1, s2, s3;
+        unpack2(acc0, s0, s1);
+        unpack2(acc1, s2, s3);
+        return (s0 + s1) + (s2 + s3);
+      };
+      auto max_chunk = [&](const uint32_t (&r)[32]) {
+        float a = __uint_as_float(r[0]), b = __uint_as_float(r[1]);
+#pragma unroll
+        for (int i = 2; i < 30; i += 4) {
+          a = max3(a, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+          b = max3(b, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+        }
+        a = max3(a, __uint_as_float(r[30]), __uint_as_float(r[31]));
+        return fmaxf(a, b);
+      };
+      const int nt = c.tiles(P);
+      int tok0 = c.first_token(P);
+      for (int t = 0; t < nt; ++t, tok0 += kTile) {
+        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(bar), n1 & 1u, ctl));
+        ++n1;
+        if (!ok) continue;
+        tc_fence_after();
+        if (tok0 <= vis_plain) {
+          uint32_t r0[32], r1[32], r2[32], r3[32];
+          tc_ld32_nowait(taddr, r0);
+          tc_ld32_nowait(taddr + 32, r1);
+          tc_ld32_nowait(taddr + 64, r2);
+          tc_ld32_nowait(taddr + 96, r3);
+          tc_wait_ld(r0); tc_wait_ld(r1); tc_wait_ld(r2); tc_wait_ld(r3);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_tempty(0));
+          if (mref[0] == -INFINITY) { mref[0] = __uint_as_float(r0[0]) * P.sl2e; mref[1] = __uint_as_float(r2[0]) * P.sl2e; }
+          const float top = fmaxf(fmaxf(max_chunk(r0), max_chunk(r1)), fmaxf(max_chunk(r2), max_chunk(r3)));
+          if (!__any_sync(0xffffffffu, row_used && !(fmaf(top, P.sl2e, -fminf(mref[0], mref[1])) < 58.5f))) {
+            lsum[0] += sum_chunk(r0, mref[0]);
+            lsum[0] += sum_chunk(r1, mref[0]);
+            lsum[1] += sum_chunk(r2, mref[1]);
+            lsum[1] += sum_chunk(r3, mref[1]);
+          } else {
+            uint32_t copy[128];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { copy[i] = r0[i]; copy[32 + i] = r1[i]; copy[64 + i] = r2[i]; copy[96 + i] = r3[i]; }
+#pragma unroll 1
+            for (int ch = 0; ch < 4; ++ch) {
+              float m = ch < 2 ? mref[0] : mref[1], l = ch < 2 ? lsum[0] : lsum[1];
+#pragma unroll 1
+              for (int attempt = 0; attempt < 8; ++attempt) {
+                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 1
+                for (int i = 0; i < 32; i += 4) {
+                  const uint32_t* p = copy + ch * 32 + i;
+                  s0 += ex2(fmaf(__uint_as_float(p[0]), P.sl2e, -m));
+                  s1 += ex2(fmaf(__uint_as_float(p[1]), P.sl2e, -m));
+                  s2 += ex2(fmaf(__uint_as_float(p[2]), P.sl2e, -m));
+                  s3 += ex2(fmaf(__uint_as_float(p[3]), P.sl2e, -m));
+                }
+                const float sum = (s0 + s1) + (s2 + s3);
+                if (sum < kRescaleLimit) { l += sum; break; }    // (false for inf / NaN as well)
+                m += 64.f;
+                l *= 5.421010862427522e-20f;                     // 2^-64
+              }
+              if (ch < 2) { mref[0] = m; lsum[0] = l; } else { mref[1] = m; lsum[1] = l; }
+            }
+          }
+        } else {
+          const long long row_vis = min(P.N - 1, P.q_pos0 + ((!kLong || P.CH == 1) ? row_m : c.template row0<kLong, kRT>(P, group) + row));
+#pragma unroll 1
+          for (int h = 0; h < 2; ++h) {
+            float m2 = h == 0 ? mref[0] : mref[1], l2 = h == 0 ? lsum[0] : lsum[1];
+            p1_masked_half(taddr + h * 64, (long long)tok0 + h * 64, row_vis, P.sl2e, &m2, &l2);
+            if (h == 0) { mref[0] = m2; lsum[0] = l2; } else { mref[1] = m2; lsum[1] = l2; }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_tempty(0));
+        }
+      }
+      if (ok && unit != P.withhold_unit) {
+        float M = row_used ? mref[0] : -INFINITY, Ls = row_used ? lsum[0] : 0.f;
+        combine(M, Ls, row_used ? mref[1] : -INFINITY, row_used ? lsum[1] : 0.f);
+        send_sum(P, unit, c.j, row, row_ref, M, Ls);
+      }
+    }
+    }
+  } else if (kRT == 1 && warp >= 8) {
+    // ============================== pass-1 epilogue, one row tile ==============================
+    if constexpr (kKeep) regs_set<Regs<1>::kP1>();
     const int half = (warp - 8) >> 2;                 // which 64 columns (tokens) of every tile
     const int quarter = warp & 3;                     // TMEM lane quarter this warp may read
     const int row = quarter * 32 + lane;              // TMEM lane = query row
@@ -699,9 +889,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     const int row_m = row % (W > 0 ? W : P.w);        // the row inside its query head (windows of up to 128 rows)
     const unsigned long long scale2 = pack2(P.sl2e, P.sl2e);
 
-    int n1 = 0;
+    uint32_t n1 = 0;
     float mref = -INFINITY, lsum = 0.f;               // sum over the run so far of 2^(logit - mref)
-    float row_ref = 0.f;                              // the row's reference exponent for the pushed sum
     bool ok = true;
 
     // 32 unmasked logits against the row's current reference: no maximum, packed arithmetic.
@@ -733,79 +922,74 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
       }
     };
 
-    RunCursor c;
-    c.init(P);
-    for (int k = 0; k < my_runs; ++k, c.next(P)) {
-      const bool row_used = row < c.template rows<kLong>(P);
-      if (half == 0) row_ref = __ldg(P.ref + (long long)c.u * kRows + row);   // used at the run's end
-      const int nt = c.tiles(P);
-      int tok0 = c.first_token(P);                      // first token of the tile
-      for (int t = 0; t < nt; ++t, tok0 += kTile) {
-        // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
-        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(0), (uint32_t)(n1 & 1), ctl));
-        ++n1;
-        if (!ok) continue;
-        tc_fence_after();
-        const uint32_t taddr = lane_addr + SL::kAcc1 + half * 64;
-        if (tok0 + kTile - 1 <= vis_all) {              // no masking anywhere in the tile
-          uint32_t ra[32], rb[32];
-          tc_ld32_nowait(taddr, ra);
-          tc_ld32_nowait(taddr + 32, rb);
-          tc_wait_ld(ra);
-          tc_wait_ld(rb);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_tempty(0));    // the accumulator is in registers now
-          if (row_used) { fast_chunk(ra); fast_chunk(rb); }
-        } else {
-          float m2 = mref, l2 = lsum;                     // (the whole warp takes part in the TMEM loads)
-          const long long row_vis = min(P.N - 1, P.q_pos0 + ((!kLong || P.CH == 1) ? row_m : c.template row0<kLong>(P) + row));   // last key this row sees
-          p1_masked_half(taddr, (long long)tok0 + half * 64, row_vis, P.sl2e, &m2, &l2);
-          if (row_used) { mref = m2; lsum = l2; }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_tempty(0));
-        }
-      }
-      // the end of the run: the two halves of every row meet through shared memory (two buffers in turn); the lower
-      // half's warps send the run's sum of every row, the upper half's go on to the next run
-      const int par = k & 1;
+    // The end of a run: the two halves of every row meet through shared memory (two buffers in turn); the lower
+    // half's warps send the run's sum of every row, the upper half's go on.  n: runs before this one.
+    auto exchange = [&](const int n, const bool row_used, const float row_ref, const int unit, const int run) {
+      const int par = n & 1;
       if (half == 1) {
-        if (k >= 2) named_bar(5 + par, 256);              // the buffer has been read
+        if (n >= 2) named_bar(5 + par, 256);              // the buffer has been read
         stage[par * kRows] = make_float2(row_used ? mref : -INFINITY, row_used ? lsum : 0.f);
         named_bar_arrive(3 + par, 256);
       } else {
         named_bar(3 + par, 256);
         const float2 other = stage[par * kRows];
-        if (k + 2 < my_runs) named_bar_arrive(5 + par, 256);
-        if (ok && c.u != P.withhold_unit) {
+        if (n + 2 < my_runs) named_bar_arrive(5 + par, 256);
+        if (ok && unit != P.withhold_unit) {
           float M = row_used ? mref : -INFINITY, Ls = row_used ? lsum : 0.f;
           combine(M, Ls, other.x, other.y);
-          // the short way: add the run's sum, rescaled to the row's fixed reference, to the row's
-          // 64-bit word (integer addition: the total does not depend on the order)
-          unsigned long long* word = P.acc + (long long)c.u * kRows + row;
-          const float lv = lg2(Ls) + (M - row_ref);                     // log2 of the contribution
-          if (!(Ls > 0.f)) {
-            red_add_relaxed_u64(word, kAccArrival);
-          } else if (lv < kAccLimitLog2) {
-            red_add_relaxed_u64(word, kAccArrival + __float2ull_rn(ex2(lv + (float)kAccFracBits)));
-          } else {
-            // it does not fit: the run's record and its bit in the row's bitmap, then the arrival with
-            // release semantics, so that both are visible to whoever acquires the complete word
-            P.partial[((long long)c.u * P.RPU + c.j) * kRows + row] = make_float2(M, Ls);
-            red_or_relaxed_u64(P.ovf + ((long long)c.u * kRows + row) * 4 + (c.j >> 6), 1ull << (c.j & 63));
-            red_add_release_u64(word, kAccArrival + kAccOverflow);
-          }
+          send_sum(P, unit, run, row, row_ref, M, Ls);
         }
       }
       mref = -INFINITY; lsum = 0.f;
+    };
+
+    const int vis_plain = (int)vis_all - (kTile - 1);     // a tile whose first token is at most this has no mask (N < 2^30)
+    RunCursor c;
+    c.init(P);
+    for (int k = 0; k < my_runs; ++k, c.next(P)) {
+      const int unit = c.template unit<1>(P, 0);
+      const bool row_used = row < c.template rows<kLong, 1>(P, 0);
+      float row_ref = 0.f;                              // the row's reference exponent for the pushed sum: used at the run's end
+      if (half == 0) row_ref = __ldg(P.ref + (long long)unit * kRows + row);
+      const int nt = c.tiles(P);
+      int tok0 = c.first_token(P);                      // first token of the tile
+      for (int t = 0; t < nt; ++t, tok0 += kTile) {
+        // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
+        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_tfull(0), n1 & 1u, ctl));
+        ++n1;
+        if (ok) {
+          tc_fence_after();
+          const uint32_t taddr = lane_addr + SL::kAcc1 + half * 64;
+          if (tok0 <= vis_plain) {
+            uint32_t ra[32], rb[32];
+            tc_ld32_nowait(taddr, ra);
+            tc_ld32_nowait(taddr + 32, rb);
+            tc_wait_ld(ra);
+            tc_wait_ld(rb);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_tempty(0));  // the accumulator is in registers now
+            if (row_used) { fast_chunk(ra); fast_chunk(rb); }
+          } else {
+            float m2 = mref, l2 = lsum;                 // (the whole warp takes part in the TMEM loads)
+            const long long row_vis = min(P.N - 1, P.q_pos0 + ((!kLong || P.CH == 1) ? row_m : c.template row0<kLong, 1>(P, 0) + row));   // last key this row sees
+            p1_masked_half(taddr, (long long)tok0 + half * 64, row_vis, P.sl2e, &m2, &l2);
+            if (row_used) { mref = m2; lsum = l2; }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_tempty(0));
+          }
+        }
+      }
+      exchange(k, row_used, row_ref, unit, c.j);
     }
   } else if (warp >= 4 && warp < 8) {
     // ============================== pass-2 epilogue ============================================
+    if constexpr (kRT == 2 || kKeep) regs_set<Regs<kRT>::kP2>();
     const int quarter = warp & 3;
     const int trow = quarter * 32 + lane;             // TMEM lane = token inside the tile; also 0..127 in the group
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    float* neg_lse = reinterpret_cast<float*>(smem + SL::kNegLse);
+    float* neg_lse_of = reinterpret_cast<float*>(smem + SL::kNegLse);
     const unsigned long long scale2 = pack2(P.sl2e, P.sl2e);
     int n2 = 0;
     bool ok = true;
@@ -816,73 +1000,101 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     const int n_ctx = (int)P.N;
     RunCursor cu;
     cu.init(P);
-    unsigned long long early_word = 0ull;             // a coming run's pushed word and reference, fetched ahead
-    float early_ref = 0.f;
-    if (my_runs > 0) {
-      early_word = ld_relaxed_u64(P.acc + (long long)cu.u * kRows + trow);
-      early_ref = __ldg(P.ref + (long long)cu.u * kRows + trow);
-    }
+    unsigned long long early_word[kRT];               // a coming run's pushed words and references, fetched ahead
+    float early_ref[kRT];
+    auto fetch_early = [&]() {
+#pragma unroll
+      for (int rt = 0; rt < kRT; ++rt) {
+        early_word[rt] = 0ull; early_ref[rt] = 0.f;
+        if (kRT == 1 || rt < cu.template row_tiles<kRT>(P)) {
+          const long long at = (long long)cu.template unit<kRT>(P, rt) * kRows + trow;
+          early_word[rt] = ld_relaxed_u64(P.acc + at);
+          early_ref[rt] = __ldg(P.ref + at);
+        }
+      }
+    };
+    if (my_runs > 0) fetch_early();
     for (int k = 0; k < my_runs; ++k) {
-      const int rows_u = cu.template rows<kLong>(P);
-      const int n_chunks = (rows_u + 31) / 32;
-      const int row0 = cu.template row0<kLong>(P);
-      // where the unit's scores (or partial aggregates) go
-      float* const score_row = P.scores + ((long long)cu.q * ((long long)P.L * P.Bt * P.Hkv) + cu.kv_unit(P)) * P.N;
+      const int nrt = cu.template row_tiles<kRT>(P);
+      int rows_of[kRT], row0_of[kRT];
+      float* score_row_of[kRT];                        // where the units' scores (or partial aggregates) go
+#pragma unroll
+      for (int rt = 0; rt < kRT; ++rt) {
+        const int r1 = kRT == 1 ? 0 : min(rt, nrt - 1);
+        rows_of[rt] = cu.template rows<kLong, kRT>(P, r1);
+        row0_of[rt] = cu.template row0<kLong, kRT>(P, r1);
+        score_row_of[rt] = P.scores + ((long long)(cu.q * kRT + r1) * ((long long)P.L * P.Bt * P.Hkv) + cu.kv_unit(P)) * P.N;
+      }
       const int nt = cu.tiles(P);
       int tok0 = cu.first_token(P);                    // first token of the tile
+      ulonglong2 nl_regs[kKeep ? 32 : 1];           // one row tile: its rows' -log-sum-exps
       {
-        // a new run: its unit's log-sum-exp.  The short way: the row's pushed word, complete once
+        // a new run: its units' log-sum-exps.  The short way: the row's pushed word, complete once
         // every run of the unit has arrived (fetched a tile or two ago; polled if it was not
         // complete then).  If a run's sum did not fit, the runs' records decide.
-        float lse = 0.f;
-        if (ok && trow < rows_u) {
-          bool pushed = false;
-          {
-            unsigned long long word = early_word;
-            if ((unsigned int)(word >> 56) != (unsigned int)P.RPU)
-              word = poll_acc_slow(P.acc + (long long)cu.u * kRows + trow, (unsigned int)P.RPU, ctl);
-            const unsigned long long sum = word & kAccSumMask;
-            if (((word >> 48) & 0xffull) == 0 && sum != 0) {
-              lse = early_ref + lg2((float)sum) - (float)kAccFracBits;
-              pushed = true;
-            }
-          }
-          if (!pushed) {
-            // the long way: all runs have arrived (the count in the word); those whose sum did not fit
-            // wrote a record and set their bit before their release.  Fold them, in run order (the same
-            // order for every reader), into the fixed-point sum of the others.
-            asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            const unsigned long long word = ld_relaxed_u64(P.acc + (long long)cu.u * kRows + trow);
-            const unsigned long long sum = word & kAccSumMask;
-            float M = -INFINITY, Ls = 0.f;
-            if (sum != 0) { M = early_ref; Ls = (float)sum * 9.5367431640625e-07f; }       // 2^-20
-            const float2* rec = P.partial + (long long)cu.u * P.RPU * kRows + trow;
-            const unsigned long long* bits_of = P.ovf + ((long long)cu.u * kRows + trow) * 4;
-#pragma unroll 1
-            for (int wi = 0; wi < 4; ++wi) {
-              unsigned long long bits = __ldcg(bits_of + wi);
-              while (bits) {
-                const int j = wi * 64 + __ffsll((long long)bits) - 1;
-                bits &= bits - 1;
-                const float2 v = __ldcg(rec + (long long)j * kRows);
-                combine(M, Ls, v.x, v.y);
+        float lse_of[kRT];
+#pragma unroll
+        for (int rt = 0; rt < kRT; ++rt) {
+          float lse = 0.f;
+          if (ok && (kRT == 1 || rt < nrt) && trow < rows_of[rt]) {
+            const int unit = cu.template unit<kRT>(P, rt);
+            bool pushed = false;
+            {
+              unsigned long long word = early_word[rt];
+              if ((unsigned int)(word >> 56) != (unsigned int)P.RPU)
+                word = poll_acc_slow(P.acc + (long long)unit * kRows + trow, (unsigned int)P.RPU, ctl);
+              const unsigned long long sum = word & kAccSumMask;
+              if (((word >> 48) & 0xffull) == 0 && sum != 0) {
+                lse = early_ref[rt] + lg2((float)sum) - (float)kAccFracBits;
+                pushed = true;
               }
             }
-            lse = M + log2f(Ls);
+            if (!pushed) {
+              // the long way: all runs have arrived (the count in the word); those whose sum did not fit
+              // wrote a record and set their bit before their release.  Fold them, in run order (the same
+              // order for every reader), into the fixed-point sum of the others.
+              asm volatile("fence.acq_rel.gpu;" ::: "memory");
+              const unsigned long long word = ld_relaxed_u64(P.acc + (long long)unit * kRows + trow);
+              const unsigned long long sum = word & kAccSumMask;
+              float M = -INFINITY, Ls = 0.f;
+              if (sum != 0) { M = early_ref[rt]; Ls = (float)sum * 9.5367431640625e-07f; }       // 2^-20
+              const float2* rec = P.partial + (long long)unit * P.RPU * kRows + trow;
+              const unsigned long long* bits_of = P.ovf + ((long long)unit * kRows + trow) * 4;
+#pragma unroll 1
+              for (int wi = 0; wi < 4; ++wi) {
+                unsigned long long bits = __ldcg(bits_of + wi);
+                while (bits) {
+                  const int j = wi * 64 + __ffsll((long long)bits) - 1;
+                  bits &= bits - 1;
+                  const float2 v = __ldcg(rec + (long long)j * kRows);
+                  combine(M, Ls, v.x, v.y);
+                }
+              }
+              lse = M + log2f(Ls);
+            }
           }
+          lse_of[rt] = lse;
         }
         named_bar(1, 128);                             // everyone is done with the previous unit's values
-        neg_lse[trow] = (trow < rows_u) ? -lse : -INFINITY;    // (a row that is not there never wins a maximum)
+#pragma unroll
+        for (int rt = 0; rt < kRT; ++rt)               // (a row that is not there never wins a maximum)
+          neg_lse_of[rt * kRows + trow] = (trow < rows_of[rt]) ? -lse_of[rt] : -INFINITY;
         named_bar(1, 128);
+        if constexpr (kKeep) {
+          const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(neg_lse_of);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) nl_regs[i] = l2[i];
+        }
         ok = !__any_sync(0xffffffffu, ctl->abort != 0) && ok;
       }
       cu.next(P);
       for (int t = 0; t < nt; ++t, tok0 += kTile) {
-      if (t == max(nt - 2, 0) && k + 1 < my_runs) {
-        // the next run's word and reference: in flight while the rest of this run is computed
-        early_word = ld_relaxed_u64(P.acc + (long long)cu.u * kRows + trow);
-        early_ref = __ldg(P.ref + (long long)cu.u * kRows + trow);
-      }
+      // the next run's words and references: in flight while the rest of this run (two accumulators) is computed
+      if (t == max(nt - 2 / kRT, 0) && k + 1 < my_runs) fetch_early();
+      for (int rt = 0; rt < nrt; ++rt) {
+      const int rows_u = kRT == 1 || rt == 0 ? rows_of[0] : rows_of[kRT - 1];
+      const int n_chunks = (rows_u + 31) / 32;
+      const float* const neg_lse = neg_lse_of + rt * kRows;
       const int buf = 1 + (n2 & 1);
       const uint32_t tmem_col = SL::kAcc2 + (uint32_t)(n2 & 1) * kTile;
       // (the TMEM loads below are warp-wide instructions: the decision has to be the warp's)
@@ -900,59 +1112,88 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         // column-by-column loop of the masked tiles)
         gacc = gmax ? -INFINITY : 0.f;
         float hacc = -INFINITY;
-        uint32_t r[32];
-        tc_ld32_nowait(lane_addr + tmem_col, r);
-        auto chunk = [&](const int j, const bool last) {
-          // the rows' -log-sum-exp for this chunk, fetched while the accumulator load is in flight
-          ulonglong2 nl[8];
-          {
-            const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(neg_lse + j * 32);
+        const uint32_t acc = lane_addr + tmem_col;
+        // 16 columns: the largest log2 of their weights goes to hacc; with W = 8, 16 whole heads end here
+        auto part = [&](const uint32_t* r, const ulonglong2* nl, const int col) {
+          float x[16];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) nl[i] = l2[i];
-          }
-          tc_wait_ld(r);
-          float x[32];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
+          for (int i = 0; i < 4; ++i) {
             const unsigned long long y0 = fma2(pack2u(r[4 * i], r[4 * i + 1]), scale2, nl[i].x);
             const unsigned long long y1 = fma2(pack2u(r[4 * i + 2], r[4 * i + 3]), scale2, nl[i].y);
-            unpack2(y0, x[4 * i], x[4 * i + 1]);                     // log2 of the attention weights
+            unpack2(y0, x[4 * i], x[4 * i + 1]);
             unpack2(y1, x[4 * i + 2], x[4 * i + 3]);
           }
-          if (!last) {
-            tc_ld32_nowait(lane_addr + tmem_col + (j + 1) * 32, r);
-          } else {
-            tc_fence_before();                                        // the accumulator has been read
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_tempty(buf));
-          }
           if (W == 8 || W == 16) {
-            constexpr int kW = W > 0 ? W : 32;
+            constexpr int kW = W == 8 ? 8 : 16;
 #pragma unroll
-            for (int h0 = 0; h0 < 32; h0 += kW) {
+            for (int h0 = 0; h0 < 16; h0 += kW) {
               float a = fmaxf(x[h0], x[h0 + 1]);
 #pragma unroll
               for (int i = 2; i < kW; i += 2) a = max3(a, x[h0 + i], x[h0 + i + 1]);
-              if (j * 32 + h0 < rows_u) {
+              if (col + h0 < rows_u) {
                 const float s_task = ex2(a);
                 gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
               }
             }
-            return;
+          } else {
+            float a = max3(x[0], x[1], x[2]), b = max3(x[3], x[4], x[5]);
+            a = max3(a, x[6], x[7]); b = max3(b, x[8], x[9]);
+            a = max3(a, x[10], x[11]); b = max3(b, x[12], x[13]);
+            a = max3(a, x[14], x[15]);
+            hacc = max3(hacc, a, b);
           }
-          float a = x[0], b = x[1];
-#pragma unroll
-          for (int i = 2; i < 30; i += 4) { a = max3(a, x[i], x[i + 1]); b = max3(b, x[i + 2], x[i + 3]); }
-          hacc = max3(hacc, a, b);
-          hacc = max3(hacc, x[30], x[31]);
-          if (W > 0 && ((j + 1) * 32) % (W > 0 ? W : 1) == 0) {
+        };
+        auto head_end = [&](const int j) {                               // behind chunk j of 32 columns
+          if (W > 16 && ((j + 1) * 32) % (W > 0 ? W : 1) == 0) {
             const float s_task = ex2(hacc);
             gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
             hacc = -INFINITY;
           }
         };
+        auto emptied = [&]() {                                           // the accumulator has been read
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_tempty(buf));
+        };
+        if constexpr (kKeep) {
+          // a chunk of 32 columns is fetched while the one before it is worked on
+          uint32_t ra[32], rb[32];
+          tc_ld32_nowait(acc, ra);
+          auto chunk = [&](const int j, uint32_t (&r)[32], uint32_t (&r_next)[32]) {
+            tc_wait_ld(r);
+            if (j + 1 < n_chunks) tc_ld32_nowait(acc + j * 32 + 32, r_next); else emptied();
+            part(r, nl_regs + 8 * j, j * 32);
+            part(r + 16, nl_regs + 8 * j + 4, j * 32 + 16);
+            head_end(j);
+          };
+          chunk(0, ra, rb);
+          if (n_chunks > 1) chunk(1, rb, ra);
+          if (n_chunks > 2) chunk(2, ra, rb);
+          if (n_chunks > 3) chunk(3, rb, ra);
+        } else {
+          // the same with half chunks, whose -log-sum-exps come from shared memory
+          uint32_t ra[16], rb[16];
+          ulonglong2 na[4], nb[4];
+          auto load_nl = [&](ulonglong2 (&nl)[4], const int col) {
+            const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(neg_lse + col);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) nl[i] = l2[i];
+          };
+          tc_ld16_nowait(acc, ra);
+          load_nl(na, 0);
 #pragma unroll 1
-        for (int j = 0; j < n_chunks; ++j) chunk(j, j + 1 == n_chunks);
+          for (int j = 0; j < n_chunks; ++j) {
+            load_nl(nb, j * 32 + 16);
+            tc_wait_ld(ra);
+            tc_ld16_nowait(acc + j * 32 + 16, rb);
+            part(ra, na, j * 32);
+            if (j + 1 < n_chunks) load_nl(na, j * 32 + 32);
+            tc_wait_ld(rb);
+            if (j + 1 < n_chunks) tc_ld16_nowait(acc + j * 32 + 32, ra); else emptied();
+            part(rb, nb, j * 32 + 16);
+            head_end(j);
+          }
+        }
         if (W == 0) gacc = ex2(hacc);                                  // the head's maximum over these rows
       } else if (!kTaskMean && W == 0 && full && P.w >= 8) {
         gacc = P.w >= 32 ? p2_odd_tile<32>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
@@ -965,7 +1206,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         // a window longer than 128 rows: the tile holds rows row0 .. of one query head and yields
         // that head's partial Eq. 14 (the maximum, or the sum, over these rows)
         gacc = p2_long_tile<kTaskMean>(lane_addr + tmem_col, neg_lse, n_chunks, rows_u, P.sl2e, full,
-                                       (long long)c - P.q_pos0 - row0);
+                                       (long long)c - P.q_pos0 - (kRT == 1 || rt == 0 ? row0_of[0] : row0_of[kRT - 1]));
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty(buf));
@@ -977,7 +1218,8 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         if (lane == 0) mbar_arrive(bar_tempty(buf));
       }
       // one row tile: the group aggregate itself; several: this tile's part of it
-      if (c < n_ctx) score_row[c] = gacc * inv_g;
+      if (c < n_ctx) (kRT == 1 || rt == 0 ? score_row_of[0] : score_row_of[kRT - 1])[c] = gacc * inv_g;
+      }
       }
     }
   } else if (warp == 1 || warp == 2) {
@@ -991,62 +1233,82 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     bool ok = true, issued = false;
     RunCursor c;
     c.init(P);
+    int visits = 0;                                    // row tiles begun
     for (int k = 0; k < my_runs && ok; ++k, c.next(P)) {
-      const int nt = c.tiles(P);
-      const int slot = slot0 + qr.i;
-      ok = mbar_wait_warp(bar_qfull(slot), (uint32_t)qr.phase, ctl);
-      const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
-      const uint32_t idesc = umma_idesc(pass == 0 ? kTile : (c.template rows<kLong>(P) + 31) / 32 * 32);
-      qr.next(slots);
-      const uint32_t q_tmem = tmem_base + SL::kQt + (uint32_t)(k & 1) * (D / 2);   // pass 1
-      if (pass == 0 && ok) {
-        // The run's Q moves to TMEM, its slot is free again.  Two sets of columns in turn: PTX runs an MMA behind the copies issued
-        // before it (tcgen05.cp -> tcgen05.mma), but promises nothing for a copy issued behind an MMA, and the MMAs of the run
-        // before may still read their set.  Those of the run before that, which read this one, are complete: the first tile of the
-        // run before was issued only when the epilogue had emptied the accumulator of their last tile.  (One set, and a wait for
-        // the last MMAs in front of the copy: 448 rows per token at 128K 4457 -> 4491 us per pass, 500-row windows 1225 -> 1234.)
-        tc_fence_after();
-        if (elect_one()) {
+      const int nt = c.tiles(P), nrt = c.template row_tiles<kRT>(P);
+      int slot_of[kRT];
+      uint64_t dq_of[kRT];
+      uint32_t idesc_of[kRT], q_tmem_of[kRT];
+      // a row tile's Q has arrived; for pass 1 it moves on to TMEM
+      auto begin_q = [&](const int rt) {
+        const int slot = slot0 + qr.i;
+        ok = mbar_wait_warp(bar_qfull(slot), (uint32_t)qr.phase, ctl);
+        const uint64_t dq = umma_desc(sbase + SL::kQ + slot * SL::kTileBytes);
+        qr.next(slots);
+        const uint32_t q_tmem = tmem_base + SL::kQt + (uint32_t)(visits & 1) * (D / 2);   // pass 1
+        ++visits;
+        slot_of[rt] = slot; dq_of[rt] = dq; q_tmem_of[rt] = q_tmem;
+        idesc_of[rt] = umma_idesc(pass == 0 ? kTile : (c.template rows<kLong, kRT>(P, rt) + 31) / 32 * 32);
+        if (pass == 0 && ok) {
+          // Its slot is free again then.  Two sets of columns in turn: PTX runs an MMA behind the copies issued
+          // before it (tcgen05.cp -> tcgen05.mma), but promises nothing for a copy issued behind an MMA, and the MMAs of the row
+          // tile before may still read their set.  Those of the one before that, which read this set, are complete: an MMA of
+          // another row tile has been issued since, and only when the epilogue had emptied the accumulator of their last tile.
+          // (One set, and a wait for the last MMAs in front of the copy: 448 rows per token at 128K 4457 -> 4491 us per pass,
+          // 500-row windows 1225 -> 1234.)
+          tc_fence_after();
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk)
-            tc_cp_256b(q_tmem + kk * 8, dq + (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4));
-          tc_commit(bar_qfree(slot));
-        }
-        __syncwarp();
-        issued = true;
-      }
-      for (int t = 0; t < nt && ok; ++t) {
-        const int st = stage0 + kr.i, buf = pass + tb.i;
-        ok = mbar_wait_warp(bar_kfull(st), (uint32_t)kr.phase, ctl);
-        if (ok) ok = mbar_wait_warp(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t dk = umma_desc(sbase + SL::kK + st * SL::kTileBytes);
-        const uint32_t d_tmem = tmem_base + (uint32_t)buf * kTile;
-        if (elect_one()) {
-          // pass 1: rows = query rows (A = Q, in TMEM), columns = tokens (B = K); pass 2: A = K, B = Q
-          // (the start-address field counts 16-byte units: 64-element half, then 32 B per K step)
-          if (pass == 0) {
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-              const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-              tc_mma_bf16_ts(d_tmem, q_tmem + kk * 8, dk + off, idesc, kk > 0);
-            }
-          } else {
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-              const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
-              tc_mma_bf16(d_tmem, dk + off, dq + off, idesc, kk > 0);
-            }
+            for (int kk = 0; kk < D / 16; ++kk)
+              tc_cp_256b(q_tmem + kk * 8, dq + (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4));
+            tc_commit(bar_qfree(slot));
           }
-          tc_commit(bar_kempty(st));            // the K stage may be refilled once these MMAs are done
-          tc_commit(bar_tfull(buf));            // ... and the accumulator is then complete
-          if (pass != 0 && t + 1 == nt) tc_commit(bar_qfree(slot));
+          __syncwarp();
+          issued = true;
         }
-        __syncwarp();
-        issued = true;
+      };
+      begin_q(0);
+      for (int t = 0; t < nt && ok; ++t) {
+        const int st = stage0 + kr.i;
+        ok = mbar_wait_warp(bar_kfull(st), (uint32_t)kr.phase, ctl);
+        const uint64_t dk = umma_desc(sbase + SL::kK + st * SL::kTileBytes);
+        for (int rt = 0; rt < nrt && ok; ++rt) {
+          // (the second row tile's Q only now: its TMEM columns are those of the run before until the MMAs above are issued)
+          if (kRT == 2 && rt == 1 && t == 0) begin_q(kRT - 1);
+          const int buf = pass + tb.i;
+          if (ok) ok = mbar_wait_warp(bar_tempty(buf), (uint32_t)(tb.phase ^ 1), ctl);
+          if (!ok) break;
+          tc_fence_after();
+          const bool first = kRT == 1 || rt == 0;
+          const uint64_t dq = first ? dq_of[0] : dq_of[kRT - 1];
+          const uint32_t q_tmem = first ? q_tmem_of[0] : q_tmem_of[kRT - 1];
+          const uint32_t idesc = first ? idesc_of[0] : idesc_of[kRT - 1];
+          const uint32_t d_tmem = tmem_base + (uint32_t)buf * kTile;
+          if (elect_one()) {
+            // pass 1: rows = query rows (A = Q, in TMEM), columns = tokens (B = K); pass 2: A = K, B = Q
+            // (the start-address field counts 16-byte units: 64-element half, then 32 B per K step)
+            if (pass == 0) {
+#pragma unroll
+              for (int kk = 0; kk < D / 16; ++kk) {
+                const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
+                tc_mma_bf16_ts(d_tmem, q_tmem + kk * 8, dk + off, idesc, kk > 0);
+              }
+            } else {
+#pragma unroll
+              for (int kk = 0; kk < D / 16; ++kk) {
+                const uint64_t off = (uint64_t)(((kk >> 2) * (kTile * 128) + (kk & 3) * 32) >> 4);
+                tc_mma_bf16(d_tmem, dk + off, dq + off, idesc, kk > 0);
+              }
+            }
+            if (rt + 1 == nrt) tc_commit(bar_kempty(st));   // the K stage may be refilled once these MMAs are done
+            tc_commit(bar_tfull(kRT == 2 && pass == 0 && rt == 1 ? 3 : buf));   // ... and the accumulator is then complete
+            if (pass != 0 && t + 1 == nt) tc_commit(bar_qfree(first ? slot_of[0] : slot_of[kRT - 1]));
+          }
+          __syncwarp();
+          issued = true;
+          tb.next(bufs);
+        }
         kr.next(stages);
-        tb.next(bufs);
       }
     }
     // no MMA may be in flight when the TMEM columns and the shared memory are given back
@@ -1100,18 +1362,22 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
         ++pos;
         if (t == 0) {
           // the run's Q (after its first K tile: with a single slot it has to wait for the MMAs of the run before)
-          const int slot = slot0 + qr.i;
-          ok = mbar_wait_warp(bar_qfree(slot), (uint32_t)(qr.phase ^ 1), ctl);
-          if (!ok) break;
-          if (elect_one()) {
-            mbar_expect_tx(bar_qfull(slot), q_bytes);
-            for (int hf = 0; hf < SL::kHalves; ++hf)
-              tma_load_4d(sbase + SL::kQ + slot * SL::kTileBytes + hf * (kTile * 128), P.q_maps + c.l, bar_qfull(slot), hf * 64,
-                          c.template row0<kLong>(P), c.h * P.G + c.template head0<kLong>(P), c.b, pol_keep);
+          const int nrt = c.template row_tiles<kRT>(P);
+          for (int rt = 0; rt < nrt; ++rt) {
+            const int slot = slot0 + qr.i;
+            ok = mbar_wait_warp(bar_qfree(slot), (uint32_t)(qr.phase ^ 1), ctl);
+            if (!ok) break;
+            if (elect_one()) {
+              mbar_expect_tx(bar_qfull(slot), q_bytes);
+              for (int hf = 0; hf < SL::kHalves; ++hf)
+                tma_load_4d(sbase + SL::kQ + slot * SL::kTileBytes + hf * (kTile * 128), P.q_maps + c.l, bar_qfull(slot), hf * 64,
+                            c.template row0<kLong, kRT>(P, rt), c.h * P.G + c.template head0<kLong, kRT>(P, rt), c.b, pol_keep);
+            }
+            __syncwarp();
+            qr.next(slots);
+            ++nq;
           }
-          __syncwarp();
-          qr.next(slots);
-          ++nq;
+          if (!ok) break;
         }
       }
       c = nx;
@@ -1255,10 +1521,14 @@ bool encode_map(CUtensorMap* m, const void* base, int rank, const long long* dim
 struct FastPlan {
   int U, NT, RPU, grid, RT;
   int HPT, QT, CH;             // query heads per row tile, row tiles per KV head, row tiles per query head
+  int RTU, QP;                 // row tiles per work unit, work units per KV head
   long long total_runs;
   int lead;
   size_t off_partial, off_parts, off_acc, off_ovf, off_ref, off_total;
 };
+
+// Window lengths with a specialisation of their own.
+constexpr bool window_special(int w) { return w == 8 || w == 16 || w == 32 || w == 64 || w == 128; }
 
 // sms <= 0: no device yet (host-only size query) -- the workspace does not depend on it
 void make_plan(const Problem& P, int sms, FastPlan* pl) {
@@ -1277,14 +1547,27 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   pl->RT = kMinRunTiles;
   if ((pl->NT + pl->RT - 1) / pl->RT > 255) pl->RT = (pl->NT + 254) / 255;   // the arrivals of a unit are counted in 8 bits
   pl->RPU = (pl->NT + pl->RT - 1) / pl->RT;
-  pl->total_runs = (long long)pl->U * pl->RPU;
+  // Two row tiles per work unit share every K tile, but a run takes twice as long until its sums are out, and so do the first
+  // run's and the last one's lead: 5 to 7 us, which have to be earned back.  (Scoring of 28 layers with 2 KV heads of 128, window 64,
+  // GQA group 4: 6 pairs of runs per CTA 68.3 us one row tile at a time, 75.9 in pairs; 12: 127.2 and 126.9; 24: 246.4 and
+  // 240.3; 16 layers of one KV head, window 300: 10 pairs 101 and 106, 21 187 and 186, 42 366 and 355.)  With heads of 64 shared
+  // memory does not bound the kernel: 32K tokens of the first shape 201 and 213 us; except for windows longer than 128 rows
+  // (window 200: 7 pairs per CTA 68 and 67, 14 125 and 114, 55 443 and 399).  A run-time window of up to 128 rows gains
+  // nothing (49 rows, 24 pairs: 276 and 276), nor does the task mean, whose pass 2 goes column by column.
+  pl->RTU = 1;
+  if (pl->QT > 1 && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
+    const long long pair_runs = (long long)P.L * P.Bt * P.Hkv * ((pl->QT + 1) / 2) * pl->RPU;
+    if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0) pl->RTU = 2;
+  }
+  pl->QP = (pl->QT + pl->RTU - 1) / pl->RTU;
+  pl->total_runs = (long long)P.L * P.Bt * P.Hkv * pl->QP * pl->RPU;
   pl->grid = sms > 0 ? (int)(pl->total_runs < sms ? pl->total_runs : sms) : 1;
   // Pass 2 of a run starts once every run of its unit has been through pass 1: at other CTAs these lie at most
   // (grid + RPU - 2) / grid runs later in their order.  Pass 1 must be allowed that far ahead of pass 2 (or the CTAs
   // would wait for each other), and no further: the rows in between should still be in L2 when pass 2 reads them.
   pl->lead = (1 + (pl->grid + pl->RPU - 2) / pl->grid) * pl->RT;
   size_t off = 0;
-  pl->off_partial = off; off += align_up((size_t)pl->total_runs * kRows * sizeof(float2));
+  pl->off_partial = off; off += align_up((size_t)pl->U * pl->RPU * kRows * sizeof(float2));
   pl->off_acc = off; off += align_up((size_t)pl->U * kRows * sizeof(unsigned long long));
   pl->off_ovf = off; off += align_up((size_t)pl->U * kRows * 4 * sizeof(unsigned long long));
   pl->off_ref = off; off += align_up((size_t)pl->U * kRows * sizeof(float));
@@ -1311,18 +1594,18 @@ std::mutex g_launch_mutex;
 // The kernel's CTAs wait for one another, so all of them have to be resident at once: one per
 // SM with the opt-in amount of shared memory.  Checked once per device and instantiation (the
 // attribute is per device); KVC_ERR_UNSUPPORTED sends the caller to the CUDA-core path.
-template <int D, int W, bool M>
+template <int D, int W, bool M, int kRT>
 kvc_status prepare_t(int grid) {
-  using SL = SmemLayout<D>;
+  using SL = SmemLayout<D, kRT>;
   static signed char state[kMaxDevices];      // 0: not looked at, 1: fits, -1: does not
   int dev = 0;
   KVC_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return KVC_ERR_UNSUPPORTED;
   std::lock_guard<std::mutex> lock(g_launch_mutex);
   if (state[dev] == 0) {
-    KVC_CUDA(cudaFuncSetAttribute(score_sm100_kernel<D, W, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kTotal));
+    KVC_CUDA(cudaFuncSetAttribute(score_sm100_kernel<D, W, M, kRT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kTotal));
     int per_sm = 0, sms = 0;
-    KVC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_sm100_kernel<D, W, M>, kFastThreads,
+    KVC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_sm100_kernel<D, W, M, kRT>, kFastThreads,
                                                            (size_t)SL::kTotal));
     KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     state[dev] = (per_sm >= 1 && sms >= 1) ? 1 : -1;
@@ -1331,26 +1614,34 @@ kvc_status prepare_t(int grid) {
   return state[dev] == 1 ? KVC_OK : KVC_ERR_UNSUPPORTED;
 }
 
-template <int D, int W, bool M>
+template <int D, int W, bool M, int kRT>
 kvc_status launch_t(const FastParams& fp, int grid, cudaStream_t st) {
-  using SL = SmemLayout<D>;
-  const kvc_status s = prepare_t<D, W, M>(grid);
+  using SL = SmemLayout<D, kRT>;
+  const kvc_status s = prepare_t<D, W, M, kRT>(grid);
   if (s != KVC_OK) return s;
-  KVC_CUDA(launch_dependent(score_sm100_kernel<D, W, M>, dim3(grid), dim3(kFastThreads), (size_t)SL::kTotal, st, fp));
+  KVC_CUDA(launch_dependent(score_sm100_kernel<D, W, M, kRT>, dim3(grid), dim3(kFastThreads), (size_t)SL::kTotal, st, fp));
   KVC_LAUNCH_CHECK("score_sm100_kernel");
   return KVC_OK;
 }
 
-template <int D, bool M>
+template <int D, bool M, int kRT>
 kvc_status launch_w(int W, const FastParams& fp, int grid, cudaStream_t st) {
   switch (W) {
-    case 8: return launch_t<D, 8, M>(fp, grid, st);
-    case 16: return launch_t<D, 16, M>(fp, grid, st);
-    case 32: return launch_t<D, 32, M>(fp, grid, st);
-    case 64: return launch_t<D, 64, M>(fp, grid, st);
-    case 128: return launch_t<D, 128, M>(fp, grid, st);
-    default: return launch_t<D, 0, M>(fp, grid, st);      // any other window length: known at run time only
+    case 8: return launch_t<D, 8, M, kRT>(fp, grid, st);
+    case 16: return launch_t<D, 16, M, kRT>(fp, grid, st);
+    case 32: return launch_t<D, 32, M, kRT>(fp, grid, st);
+    case 64: return launch_t<D, 64, M, kRT>(fp, grid, st);
+    case 128: return launch_t<D, 128, M, kRT>(fp, grid, st);
+    default: return launch_t<D, 0, M, kRT>(fp, grid, st);      // any other window length: known at run time only
   }
+}
+
+// (two row tiles: only what make_plan sends here)
+template <int D>
+kvc_status launch_d(bool mean, int row_tiles, int W, const FastParams& fp, int grid, cudaStream_t st) {
+  if (row_tiles == 1) return mean ? launch_w<D, true, 1>(W, fp, grid, st) : launch_w<D, false, 1>(W, fp, grid, st);
+  if constexpr (D == 128) return launch_w<D, false, 2>(W, fp, grid, st);
+  else return launch_t<D, 0, false, 2>(fp, grid, st);
 }
 
 }  // namespace
@@ -1364,7 +1655,7 @@ bool score_sm100_shape_ok(const Problem& P) {
   FastPlan pl;
   make_plan(P, 0, &pl);
   if ((long long)P.L * P.Bt * P.Hkv * pl.QT > (1 << 24)) return false;
-  if ((pl.total_runs + 8192) * pl.RT >= (1LL << 31)) return false;   // 32-bit sequence indices
+  if (((long long)pl.U * pl.RPU + 8192) * pl.RT >= (1LL << 31)) return false;   // 32-bit sequence indices
   return true;
 }
 
@@ -1424,22 +1715,21 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
   *row_tiles_out = pl.QT;
   *tiles_per_head_out = pl.CH;
   fp.L = P.L; fp.Bt = P.Bt; fp.Hkv = P.Hkv; fp.G = G;
-  fp.HPT = pl.HPT; fp.QT = pl.QT; fp.CH = pl.CH; fp.w = P.w;
+  fp.HPT = pl.HPT; fp.QT = pl.QT; fp.QP = pl.QP; fp.CH = pl.CH; fp.w = P.w;
   fp.N = P.N; fp.q_pos0 = P.q_pos0;
   fp.U = pl.U; fp.NT = pl.NT; fp.RPU = pl.RPU; fp.RT = pl.RT; fp.grid = pl.grid;
   fp.total_runs = (unsigned int)pl.total_runs; fp.lead = pl.lead;
   fp.step_u = pl.grid / pl.RPU; fp.step_j = pl.grid % pl.RPU;
-  fp.step_q = fp.step_u % pl.QT;
-  fp.step_h = (fp.step_u / pl.QT) % P.Hkv;
-  fp.step_b = (fp.step_u / pl.QT / P.Hkv) % P.Bt;
-  fp.step_l = fp.step_u / pl.QT / P.Hkv / P.Bt;
+  fp.step_q = fp.step_u % pl.QP;
+  fp.step_h = (fp.step_u / pl.QP) % P.Hkv;
+  fp.step_b = (fp.step_u / pl.QP / P.Hkv) % P.Bt;
+  fp.step_l = fp.step_u / pl.QP / P.Hkv / P.Bt;
   fp.sl2e = P.scale * kLog2eF;
   fp.agg_group = P.agg_group;
   fp.wait_limit_ns = g_wait_limit_ns.load();
   fp.withhold_unit = g_withhold_unit.load();
   const bool mean = P.agg_task == KVC_AGG_MEAN;
-  if (P.d == 128) return mean ? launch_w<128, true>(P.w, fp, pl.grid, st) : launch_w<128, false>(P.w, fp, pl.grid, st);
-  return mean ? launch_w<64, true>(P.w, fp, pl.grid, st) : launch_w<64, false>(P.w, fp, pl.grid, st);
+  return P.d == 128 ? launch_d<128>(mean, pl.RTU, P.w, fp, pl.grid, st) : launch_d<64>(mean, pl.RTU, P.w, fp, pl.grid, st);
 }
 
 }  // namespace kvc

@@ -6,7 +6,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 import paper_2509_05165_b200 as kvc
-from paper_2509_05165_b200 import workloads as W
+from paper_2509_05165_b200 import binding, workloads as W
 from paper_2509_05165_b200.binding import alloc_outputs
 
 import parity as Pz
@@ -291,3 +291,43 @@ def test_positions_far_behind_the_context_mask_nothing(dtype, w):
         torch.cuda.synchronize()
         assert torch.equal(out.scores, want)
     Pz.assert_scores_close(want.cpu().numpy(), Pz.oracle_scores(wl, desc))
+
+
+@pytest.mark.parametrize("Hq,Hkv,w,d,N,L,batch,q_pos0,scale", [
+    (16, 8, 128, 128, 5, 64, 8, None, 0.0),      # two row tiles per KV head, contexts of five tokens, ...
+    (16, 8, 128, 128, 129, 64, 8, None, 0.0),    # ... of a tile and a token, the mask in both
+    (24, 8, 128, 128, 1024, 24, 4, 5000, 0.0),   # three row tiles: the last work unit has one; whole runs, no mask
+    (40, 8, 128, 128, 777, 24, 4, 300, 0.0),     # five row tiles, the mask inside
+    (36, 2, 8, 128, 640, 80, 10, None, 0.0),     # sixteen heads of 8 rows in the first row tile, two in the second
+    (18, 2, 16, 128, 640, 80, 10, None, 0.0),    # eight heads of 16 rows, one
+    (14, 2, 32, 128, 1537, 64, 8, 0, 0.0),       # four heads of 32 rows, three; row m sees tokens up to m only
+    (16, 4, 64, 128, 1500, 64, 4, None, 2.0),    # logits more than 40 nats above a run's first: the references move
+    (4, 2, 300, 128, 700, 64, 6, 5000, 0.0),     # long windows: three row tiles per head, the last one short
+    (6, 3, 200, 64, 2049, 32, 4, None, 4.0),     # heads of 64, two row tiles per head
+])
+def test_row_tiles_in_pairs_give_the_scores_of_one_at_a_time(Hq, Hkv, w, d, N, L, batch, q_pos0, scale):
+    """Large problems take the row tiles of a KV head two at a time over the same keys, small ones one at a time: the scores of
+    all layers together are, bit for bit, those of every layer by itself (which the parity tests hold against the oracle)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(7)
+    q = [torch.randn((batch, Hq, w, d), generator=gen, device=dev).to(torch.bfloat16) for _ in range(L)]
+    k = [torch.randn((batch, Hkv, N, d), generator=gen, device=dev).to(torch.bfloat16) for _ in range(L)]
+
+    def scores(layers):
+        desc = binding.kvc_desc_init(len(layers), batch, Hq, Hkv, d, N, w, binding.BF16)
+        desc.scale = scale
+        if q_pos0 is not None:
+            desc.q_pos0 = q_pos0
+        assert kvc.kvc_score_uses_tensor_cores(desc)
+        out = torch.empty((len(layers), batch, Hkv, N), device=dev)
+        ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
+        kvc.kvc_score(desc, [q[i] for i in layers], [k[i] for i in layers], out, ws)
+        return out
+
+    together = scores(list(range(L)))
+    for i in range(0, L, max(1, L // 6)):
+        alone = scores([i])
+        assert torch.isfinite(alone).all()
+        assert torch.equal(together[i].view(torch.int32), alone[0].view(torch.int32)), i
