@@ -43,16 +43,20 @@ size_t score_workspace_bytes(const Problem& P) {
   return n;
 }
 
-kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k,
-                        float* scores, const float* vnorm, int* device_status, void* ws, size_t ws_bytes,
+kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, const LayerPtrs* v,
+                        float* scores, float* vnorm, int* device_status, void* ws, size_t ws_bytes,
                         cudaStream_t st) {
   if (score_sm100_supported(P)) {
     const float* parts = nullptr;
     int row_tiles = 1, tiles_per_head = 1;
-    const kvc_status s = launch_score_sm100(P, q, k, scores, device_status, ws, ws_bytes, st, &parts, &row_tiles,
+    const kvc_status s = launch_score_sm100(P, q, k, v, scores, vnorm, device_status, ws, ws_bytes, st, &parts, &row_tiles,
                                             &tiles_per_head);
     if (s == KVC_OK) return launch_score_augment(P, scores, parts, row_tiles, tiles_per_head, vnorm, st);
     if (s != KVC_ERR_UNSUPPORTED) return s;      // a real failure; UNSUPPORTED = strides TMA cannot take
+  }
+  if (vnorm != nullptr) {
+    const kvc_status s = launch_value_norm(P, *v, vnorm, st);
+    if (s != KVC_OK) return s;
   }
   return launch_score_generic(P, gm, q, k, scores, vnorm, device_status, ws, ws_bytes, st);
 }
@@ -62,13 +66,8 @@ static kvc_status run_score(const Problem& P, const GroupMap& gm, const LayerPtr
                             const LayerPtrs* v, float* scores, int* device_status, void* ws, cudaStream_t st) {
   char* w = reinterpret_cast<char*>(ws);
   const size_t scratch = score_scratch_bytes(P);
-  float* vnorm = nullptr;
-  if (P.value_norm) {
-    vnorm = reinterpret_cast<float*>(w + scratch + 256);
-    const kvc_status s = launch_value_norm(P, *v, vnorm, st);
-    if (s != KVC_OK) return s;
-  }
-  return launch_score(P, gm, q, k, scores, vnorm, device_status, ws, scratch, st);
+  float* vnorm = P.value_norm ? reinterpret_cast<float*>(w + scratch + 256) : nullptr;
+  return launch_score(P, gm, q, k, v, scores, vnorm, device_status, ws, scratch, st);
 }
 
 namespace {

@@ -93,10 +93,10 @@ inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 // Scratch bytes the scoring step needs.
 size_t score_workspace_bytes(const Problem& P);
 // Eqs. 3, 14-16: writes scores [L, Bt, Hkv, N].
-// vnorm: nullptr, or ||v|| per (layer, sequence, KV head, token), laid out like scores (App. A.1.3).
+// vnorm: nullptr, or the place for ||v|| per (layer, sequence, KV head, token), laid out like scores (App. A.1.3); v is not null then.
 // device_status (may be null) is cleared by the first of its kernels.
-kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k,
-                        float* scores, const float* vnorm, int* device_status, void* ws, size_t ws_bytes,
+kvc_status launch_score(const Problem& P, const GroupMap& gm, const LayerPtrs& q, const LayerPtrs& k, const LayerPtrs* v,
+                        float* scores, float* vnorm, int* device_status, void* ws, size_t ws_bytes,
                         cudaStream_t st);
 // The two implementations behind it: CUDA cores (any supported shape) and tcgen05 (bf16 with
 // contiguous GQA groups, any window).
@@ -114,8 +114,9 @@ kvc_status launch_score_augment(const Problem& P, float* scores, const float* pa
 bool score_sm100_shape_ok(const Problem& P);
 bool score_sm100_supported(const Problem& P);
 size_t score_sm100_workspace_bytes(const Problem& P);
-kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerPtrs& k, float* scores,
-                              int* device_status, void* ws, size_t ws_bytes, cudaStream_t st,
+// With vnorm, the value norms come out of the same launch.
+kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerPtrs& k, const LayerPtrs* v, float* scores,
+                              float* vnorm, int* device_status, void* ws, size_t ws_bytes, cudaStream_t st,
                               const float** parts_out, int* row_tiles_out, int* tiles_per_head_out);
 
 // ---- rank + compose ---------------------------------------------------------------------------

@@ -75,6 +75,7 @@
 #include <mutex>
 
 #include "kvc_internal.cuh"
+#include "value_norm.cuh"
 
 namespace kvc {
 namespace {
@@ -125,6 +126,11 @@ struct FastParams {
   float sl2e;                  // scale * log2(e)
   int agg_group;
   unsigned long long wait_limit_ns;   // bound of every device-side wait
+  // the value norms, by the CTAs from `grid` on (see value_norm_cta): V^(l), their place, V's strides in elements
+  LayerPtrs v;
+  float* vnorm;
+  long long vs0, vs1, vs2;
+  int norm_ctas;               // 0: none
   int withhold_unit;           // test hook: the statistics of this unit are never sent (-1: none), so that
                                // the waits for them run into their bound
 };
@@ -697,6 +703,63 @@ __device__ __forceinline__ float p2_long_tile(uint32_t taddr, const float* neg_l
 }
 
 // ------------------------------------------------------------------------------------------------
+// Value norms (App. A.1.3) on CTAs of their own in the scoring launch: they wait for HBM, the scoring CTAs for their SMs, so the
+// two overlap where a kernel before the scoring had to be waited for (see norm_share).  A lane's pieces of the rows go through
+// shared memory, kNormStages blocks of rows ahead: 192 KB in flight per SM (two blocks in registers reach half of the rate: the
+// loads of both are waited for together).
+// ------------------------------------------------------------------------------------------------
+constexpr int kNormStages = 3;
+template <int D>
+__device__ __forceinline__ void value_norm_cta(const FastParams& P, uint32_t sbase) {
+  constexpr int kLpr = D / 8, kGroups = 32 / kLpr, kBlock = kNormBlock<kLpr>, kWarps = kFastThreads / 32;
+  static_assert(kNormStages * kNormRows * kFastThreads * 16 <= 14 * 16384, "shared memory");
+  unsigned long long policy;                               // (V goes through L2 once; K has to stay there)
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  const int lane = threadIdx.x & 31, sub = lane & (kLpr - 1), grp = lane / kLpr;
+  const int segs = P.L * P.Bt * P.Hkv, per_seg = (int)((P.N + kBlock - 1) / kBlock);
+  const int stride = P.norm_ctas * kWarps, step_seg = stride / per_seg, step_blk = stride % per_seg;
+  const int id = (int)(blockIdx.x - P.grid) * kWarps + (int)(threadIdx.x >> 5);
+  struct At {
+    int seg, blk;
+    __device__ __forceinline__ void next(int step_seg, int step_blk, int per_seg) {
+      blk += step_blk;
+      seg += step_seg;
+      if (blk >= per_seg) { blk -= per_seg; ++seg; }
+    }
+  } ahead = {id / per_seg, id % per_seg}, at = ahead;
+  const uint32_t mine = sbase + threadIdx.x * 16;          // piece u of stage s: + (s * kNormRows + u) * kFastThreads * 16
+  auto fetch = [&](int stage) {
+    if (ahead.seg < segs) {
+      const int h = ahead.seg % P.Hkv, lb = ahead.seg / P.Hkv, b = lb % P.Bt, l = lb / P.Bt;
+      const __nv_bfloat16* base = reinterpret_cast<const __nv_bfloat16*>(P.v.p[l]) + b * P.vs0 + h * P.vs1 + sub * 8;
+      const int first = ahead.blk * kBlock + grp, last = (int)P.N - 1;     // (N < 2^30)
+#pragma unroll
+      for (int u = 0; u < kNormRows; ++u) {
+        const __nv_bfloat16* src = base + min(first + u * kGroups, last) * P.vs2;
+        asm volatile("cp.async.cg.shared.global.L2::cache_hint.L2::256B [%0], [%1], 16, %2;"
+                     ::"r"(mine + (uint32_t)(stage * kNormRows + u) * (kFastThreads * 16)), "l"(src), "l"(policy) : "memory");
+      }
+      ahead.next(step_seg, step_blk, per_seg);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");   // (empty behind the end: the count of groups stays that of the stages)
+  };
+#pragma unroll
+  for (int s = 0; s < kNormStages; ++s) fetch(s);
+  for (int stage = 0; at.seg < segs; at.next(step_seg, step_blk, per_seg)) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kNormStages - 1) : "memory");
+    uint4 w[kNormRows];                                    // (a lane reads back what it copied itself)
+#pragma unroll
+    for (int u = 0; u < kNormRows; ++u)
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[u].x), "=r"(w[u].y), "=r"(w[u].z), "=r"(w[u].w)
+                   : "r"(mine + (uint32_t)(stage * kNormRows + u) * (kFastThreads * 16)) : "memory");
+    norm_store<__nv_bfloat16, kLpr>(w, P.vnorm + (long long)at.seg * P.N, (long long)at.blk * kBlock, P.N);
+    fetch(stage);
+    if (++stage == kNormStages) stage = 0;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// ------------------------------------------------------------------------------------------------
 // The kernel
 // ------------------------------------------------------------------------------------------------
 template <int D, int W, bool kTaskMean, int kRT>
@@ -705,6 +768,11 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
   using SL = SmemLayout<D, kRT>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
+  if (blockIdx.x >= (unsigned int)P.grid) {       // (the value norms' CTAs: nothing of the rest is theirs)
+    grid_dependency_wait();
+    value_norm_cta<D>(P, sbase);
+    return;
+  }
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   volatile Ctl* ctl = reinterpret_cast<volatile Ctl*>(smem + SL::kCtl);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + SL::kTmemSlot);
@@ -1523,12 +1591,31 @@ struct FastPlan {
   int HPT, QT, CH;             // query heads per row tile, row tiles per KV head, row tiles per query head
   int RTU, QP;                 // row tiles per work unit, work units per KV head
   long long total_runs;
-  int lead;
+  int lead, norm_ctas;
   size_t off_partial, off_parts, off_acc, off_ovf, off_ref, off_total;
 };
 
 // Window lengths with a specialisation of their own.
 constexpr bool window_special(int w) { return w == 8 || w == 16 || w == 32 || w == 64 || w == 128; }
+
+// How many of the SMs take the value norms: as many as make both parts take the same time, in clocks: a scoring CTA has whole
+// runs, kPairClocks per pair of tiles; an SM that only reads gets kNormBytes per clock.  (8B shape with value norms, us per pass
+// with the norms before the scoring, and beside it at 25, 32, 40, 50 bytes per clock: 1000 tokens 86.6, 80.6, 81.7, 76.1, 75.4;
+// 4096: 219, 218, 208, 206, 209; 16384 with the other options 805, 760, 735, 755, 781; 32768: 1542, 1488, 1453, 1491, 1535; two
+// sequences of 8192 with heads of 64: 525, 521, 494, 487, 517.)
+constexpr double kPairClocks128 = 1800., kPairClocks64 = 1550., kNormBytes = 36.;
+int norm_share(const Problem& P, const FastPlan& pl, int sms) {
+  const double bytes = (double)P.L * P.Bt * P.Hkv * (double)P.N * P.d * P.elem_bytes;
+  const double run = pl.RT * pl.RTU * (P.d == 128 ? kPairClocks128 : kPairClocks64);
+  int best = 1;
+  double best_t = 1e300;
+  for (int n = 1; n < sms; ++n) {
+    const double score = (double)((pl.total_runs + sms - n - 1) / (sms - n)) * run, norm = bytes / (n * kNormBytes);
+    const double t = score > norm ? score : norm;
+    if (t < best_t) { best_t = t; best = n; }
+  }
+  return best;
+}
 
 // sms <= 0: no device yet (host-only size query) -- the workspace does not depend on it
 void make_plan(const Problem& P, int sms, FastPlan* pl) {
@@ -1561,7 +1648,8 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   }
   pl->QP = (pl->QT + pl->RTU - 1) / pl->RTU;
   pl->total_runs = (long long)P.L * P.Bt * P.Hkv * pl->QP * pl->RPU;
-  pl->grid = sms > 0 ? (int)(pl->total_runs < sms ? pl->total_runs : sms) : 1;
+  pl->norm_ctas = P.value_norm && sms > 1 ? norm_share(P, *pl, sms) : 0;
+  pl->grid = sms > 0 ? (int)(pl->total_runs < sms - pl->norm_ctas ? pl->total_runs : sms - pl->norm_ctas) : 1;
   // Pass 2 of a run starts once every run of its unit has been through pass 1: at other CTAs these lie at most
   // (grid + RPU - 2) / grid runs later in their order.  Pass 1 must be allowed that far ahead of pass 2 (or the CTAs
   // would wait for each other), and no further: the rows in between should still be in L2 when pass 2 reads them.
@@ -1619,7 +1707,7 @@ kvc_status launch_t(const FastParams& fp, int grid, cudaStream_t st) {
   using SL = SmemLayout<D, kRT>;
   const kvc_status s = prepare_t<D, W, M, kRT>(grid);
   if (s != KVC_OK) return s;
-  KVC_CUDA(launch_dependent(score_sm100_kernel<D, W, M, kRT>, dim3(grid), dim3(kFastThreads), (size_t)SL::kTotal, st, fp));
+  KVC_CUDA(launch_dependent(score_sm100_kernel<D, W, M, kRT>, dim3(grid + fp.norm_ctas), dim3(kFastThreads), (size_t)SL::kTotal, st, fp));
   KVC_LAUNCH_CHECK("score_sm100_kernel");
   return KVC_OK;
 }
@@ -1670,8 +1758,8 @@ size_t score_sm100_workspace_bytes(const Problem& P) {
 
 // Returns KVC_ERR_UNSUPPORTED (without setting an error) when the tensor maps cannot be encoded
 // for these strides; the caller then uses the CUDA-core path.
-kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerPtrs& k, float* scores,
-                              int* device_status, void* ws, size_t ws_bytes, cudaStream_t st,
+kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerPtrs& k, const LayerPtrs* v, float* scores,
+                              float* vnorm, int* device_status, void* ws, size_t ws_bytes, cudaStream_t st,
                               const float** parts_out, int* row_tiles_out, int* tiles_per_head_out) {
   const int sms = sm_count();
   if (sms < 1) return KVC_ERR_UNSUPPORTED;
@@ -1726,6 +1814,16 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
   fp.step_l = fp.step_u / pl.QP / P.Hkv / P.Bt;
   fp.sl2e = P.scale * kLog2eF;
   fp.agg_group = P.agg_group;
+  fp.norm_ctas = vnorm != nullptr ? pl.norm_ctas : 0;
+  if (vnorm != nullptr && fp.norm_ctas == 0) {         // (a device of one SM)
+    const kvc_status s = launch_value_norm(P, *v, vnorm, st);
+    if (s != KVC_OK) return s;
+  }
+  if (fp.norm_ctas > 0) {
+    fp.v = *v;
+    fp.vnorm = vnorm;
+    fp.vs0 = P.kvs[0]; fp.vs1 = P.kvs[1]; fp.vs2 = P.kvs[2];
+  }
   fp.wait_limit_ns = g_wait_limit_ns.load();
   fp.withhold_unit = g_withhold_unit.load();
   const bool mean = P.agg_task == KVC_AGG_MEAN;

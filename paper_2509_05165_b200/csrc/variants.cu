@@ -1,17 +1,11 @@
 // Kernels of the options beyond the default pipeline: the value norms of the v-norm variant
 // (App. A.1.3) and the position order of the kept tokens.
 #include "kvc_internal.cuh"
+#include "value_norm.cuh"
 
 namespace kvc {
 namespace {
 
-// ||v|| of every value row.  Bound by HBM: V is read once.  A row is kLpr = row bytes / 16 lanes wide (16 for the
-// 256-byte rows of a bf16 head of 128), so a warp carries 32 / kLpr rows at a time and every lane loads; each lane has
-// kNormRows such rows in flight (one 16-byte load each) before it adds anything, and a warp's rows are consecutive, so
-// that its norms leave in one store.  A warp per row with half of its lanes idle and one load in flight took 807 us for
-// 1.07 GB (1.3 TB/s); this form takes 182 us (5.9 TB/s; 191 with plain loads, 4 rows per lane 192).  The squares are
-// added in the order they always were: a lane's elements in ascending order, then the lanes by halving distances.
-constexpr int kNormRows = 8;
 // (a stream: past L1, L2 fetches 256 bytes at a time)
 __device__ __forceinline__ uint4 ld_once(const uint4* p) {
   uint4 v;
@@ -20,15 +14,17 @@ __device__ __forceinline__ uint4 ld_once(const uint4* p) {
   return v;
 }
 
+// ||v|| of every value row, where the scoring kernel does not take it along (fp32, explicit maps, strides it cannot take).  Bound
+// by HBM: V is read once.  A warp per row with half of its lanes idle and one load in flight took 807 us for
+// 1.07 GB (1.3 TB/s); this form takes 182 us (5.9 TB/s; 191 with plain loads, 4 rows per lane 192).
 template <typename T, int kLpr>
 __global__ void __launch_bounds__(256)
 value_norm_kernel(LayerPtrs vp, float* __restrict__ vnorm, int Bt, int Hkv, long long segs, long long N, long long vs0,
                   long long vs1, long long vs2) {
   grid_dependency_wait();
   constexpr int kGroups = 32 / kLpr;                         // rows a warp loads at once
-  static_assert(kNormRows <= kLpr, "a lane of the row's group holds each norm");
   const int lane = threadIdx.x & 31, sub = lane & (kLpr - 1), grp = lane / kLpr;
-  const long long row0 = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * (kNormRows * kGroups) + grp;
+  const long long first = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * kNormBlock<kLpr>;
   for (long long seg = blockIdx.y; seg < segs; seg += gridDim.y) {      // (l * Bt + b) * Hkv + h
     const int h = (int)(seg % Hkv);
     const int b = (int)(seg / Hkv % Bt);
@@ -37,38 +33,16 @@ value_norm_kernel(LayerPtrs vp, float* __restrict__ vnorm, int Bt, int Hkv, long
     uint4 w[kNormRows];
 #pragma unroll
     for (int u = 0; u < kNormRows; ++u) {
-      const long long c = min(row0 + u * kGroups, N - 1);
+      const long long c = min(first + grp + u * kGroups, N - 1);
       w[u] = ld_once(reinterpret_cast<const uint4*>(base + c * vs2) + sub);
     }
-    float mine = 0.f;
-#pragma unroll
-    for (int u = 0; u < kNormRows; ++u) {
-      const uint32_t ws[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
-      float acc = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (sizeof(T) == 2) {
-          // a bf16 is the upper half of the fp32 with the same value
-          const float lo = __uint_as_float(ws[i] << 16), hi = __uint_as_float(ws[i] & 0xffff0000u);
-          acc = fmaf(lo, lo, acc);
-          acc = fmaf(hi, hi, acc);
-        } else {
-          const float x = __uint_as_float(ws[i]);
-          acc = fmaf(x, x, acc);
-        }
-      }
-#pragma unroll
-      for (int o = kLpr / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (sub == u) mine = acc;
-    }
-    const long long c = row0 + sub * kGroups;
-    if (sub < kNormRows && c < N) vnorm[seg * N + c] = sqrtf(mine);
+    norm_store<T, kLpr>(w, vnorm + seg * N, first, N);
   }
 }
 
 template <typename T, int kLpr>
 kvc_status launch_norm_t(const Problem& P, const LayerPtrs& v, float* vnorm, cudaStream_t st) {
-  const long long per_cta = 8LL * kNormRows * (32 / kLpr);
+  const long long per_cta = 8LL * kNormBlock<kLpr>;
   const long long segs = (long long)P.L * P.Bt * P.Hkv;
   const dim3 grid((unsigned)((P.N + per_cta - 1) / per_cta), (unsigned)(segs < 65535 ? segs : 65535));
   KVC_CUDA(launch_dependent(value_norm_kernel<T, kLpr>, grid, dim3(256), 0, st, v, vnorm, P.Bt, P.Hkv, segs, P.N,

@@ -331,3 +331,40 @@ def test_row_tiles_in_pairs_give_the_scores_of_one_at_a_time(Hq, Hkv, w, d, N, L
         alone = scores([i])
         assert torch.isfinite(alone).all()
         assert torch.equal(together[i].view(torch.int32), alone[0].view(torch.int32)), i
+
+
+@pytest.mark.parametrize("L,batch,Hkv,d,N,w,pad", [
+    (3, 2, 5, 128, 17, 4, 0),        # fewer blocks of rows than warps that take them
+    (2, 3, 4, 64, 1033, 32, 64),     # rows apart in memory, a short last block per segment
+    (24, 4, 8, 128, 515, 16, 0),     # many segments per warp
+    (1, 1, 2, 128, 40007, 32, 128),  # one long segment after the other
+    (20, 2, 4, 128, 2100, 130, 0),   # row tiles in pairs beside the norms
+])
+def test_value_norms_beside_the_scoring(L, batch, Hkv, d, N, w, pad):
+    """The norms that the scoring launch takes along: weighted scores are the plain ones times the norms of the value rows (the
+    norm's squares are added in fp32 with errors below 1e-6)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(3)
+
+    def rand(*shape):
+        return torch.randn(shape, generator=gen, device=dev).to(torch.bfloat16)
+
+    q = [rand(batch, 2 * Hkv, w, d) for _ in range(L)]
+    k = [rand(batch, Hkv, N, d + pad)[..., :d] for _ in range(L)]
+    v = [(rand(batch, Hkv, N, d + pad) * (1 + i))[..., :d] for i in range(L)]
+    desc = binding.kvc_desc_init(L, batch, 2 * Hkv, Hkv, d, N, w, binding.BF16)
+    desc.augment_head_mean = 0
+    desc.q_pos0 = N
+    for i, s in enumerate(k[0].stride()[:3]):
+        desc.kv_stride[i] = s
+    assert kvc.kvc_score_uses_tensor_cores(desc)
+    plain, weighted = (torch.empty((L, batch, Hkv, N), device=dev) for _ in range(2))
+    kvc.kvc_score(desc, q, k, plain, torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev))
+    desc.value_norm = 1
+    ws = torch.full((kvc.kvc_workspace_size(desc, 0),), 0xff, dtype=torch.uint8, device=dev)
+    kvc.kvc_score_weighted(desc, q, k, v, weighted, ws)
+    want = torch.stack([p.double() * x.double().norm(dim=-1) for p, x in zip(plain, v)])
+    assert torch.isfinite(weighted).all()
+    assert ((weighted.double() - want).abs() <= 1e-6 * want.abs()).all()
