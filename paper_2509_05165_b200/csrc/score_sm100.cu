@@ -54,18 +54,22 @@
 // run their loops with all lanes and elect a lane for each MMA, commit or copy: from one lane of a diverged
 // warp every such instruction first moves its operands to uniform registers, about 50 clocks per MMA.
 //
-// What bounds it, in clocks per pair of tiles (128 rows x 128 tokens, heads of 128, both passes): tensor pipe and
-// special-function pipe 1024 each; shared memory most: K copied in 512, Q (written twice, read once, per run) 192, pass 1's
-// operand reads 256, pass 2's 512 (both operands come from there: a 128 x 128 x 16 MMA reads 8 KB in its 64 clocks), and 270 for
-// the -log-sum-exps that every tile of pass 2 reads (a 16-byte load by all lanes of one address takes 2.1 clocks of the SM):
-// 1742 of the 1890 that a pair took.  Hence:
+// What bounds it (waits counted in an instrumented copy, heads of 128, clocks per pair of tiles = 128 rows x 128 tokens in both
+// passes): the two epilogues.  Tensor pipe and special-function pipe have 1024 clocks of work each, DRAM, L2 and the data banks of
+// shared memory are at half or less.  With one row tile per unit a pair took 1890: pass 1's epilogue was busy for 1700 of them
+// (1150 to 1250 of exponentials, both warps of a scheduler at once, and the rest, barrier, TMEM load, the exchange of the halves,
+// at once as well), pass 2's for 1540, because each of its 32-column chunks waited for an accumulator load and for eight
+// 16-byte reads of -log-sum-exps, which queue behind pass 1's exponentials (all lanes reading one address: 2.1 clocks of the
+// SM each, 270 per tile).  Hence:
 //   - one row tile per unit: the pass-2 epilogue keeps a run's 128 -log-sum-exps in registers (216 per thread, taken from the
-//     single warps and from pass 1 by setmaxnreg) and reads them once per run: 8B shape at 32K 1078 -> 1060 us per pass, at 8K
-//     1 %, 4 sequences of 5003 with heads of 64 442 -> 430.
-//   - several row tiles: a work unit has two of them, which share every K tile in shared memory (256 instead of 512).  Pass 1's
-//     two groups then take a row tile each, a tile's 128 columns at once in registers (168 per thread), where with one row tile
-//     each takes half of the columns of every tile and both are at the exponentials, and at everything else, at the same
-//     time: window 64, GQA group 7 at 128K 4400 -> 4280 us per pass, 500-row windows 1203 -> 1158; 1690 clocks per pair.
+//     single warps and from pass 1 by setmaxnreg), reads them once per run, and loads a chunk while it works on the one before:
+//     8B shape at 32K 1078 -> 1060 us per pass, at 8K 1 %, 4 sequences of 5003 with heads of 64 442 -> 430.  Pass 1's epilogue
+//     is what is left: 1750 of 1800 clocks.
+//   - several row tiles: a work unit has two of them, which share every K tile in shared memory.  Pass 1's
+//     two groups then take a row tile each, a tile's 128 columns at once in registers (168 per thread): half of the rounds of
+//     barrier and load, and the groups are out of phase, where with one row tile each takes half of the columns of every tile.
+//     Pass 2 takes 16 columns at a time, the next 16 in flight.  Window 64, GQA group 7 at 128K 4400 -> 4280 us per pass, 500-row
+//     windows 1203 -> 1158; 1690 clocks per pair, of which pass 2's epilogue is busy for 1530.
 // Registers decide the rest: a warp's 128 exponentials take 1134 clocks when the compiler has room to overlap them and 2125
 // when it has not (it then waits for every pair), so in the second form the logits die in their exponentials.
 // Run back to back the board's power adds a sixth: at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds.
@@ -1637,10 +1641,10 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   // Two row tiles per work unit share every K tile, but a run takes twice as long until its sums are out, and so do the first
   // run's and the last one's lead: 5 to 7 us, which have to be earned back.  (Scoring of 28 layers with 2 KV heads of 128, window 64,
   // GQA group 4: 6 pairs of runs per CTA 68.3 us one row tile at a time, 75.9 in pairs; 12: 127.2 and 126.9; 24: 246.4 and
-  // 240.3; 16 layers of one KV head, window 300: 10 pairs 101 and 106, 21 187 and 186, 42 366 and 355.)  With heads of 64 shared
-  // memory does not bound the kernel: 32K tokens of the first shape 201 and 213 us; except for windows longer than 128 rows
+  // 240.3; 16 layers of one KV head, window 300: 10 pairs 101 and 106, 21 187 and 186, 42 366 and 355.)  With heads of 64 pairs are
+  // slower (32K tokens of the first shape 201 and 213 us) except for windows longer than 128 rows
   // (window 200: 7 pairs per CTA 68 and 67, 14 125 and 114, 55 443 and 399).  A run-time window of up to 128 rows gains
-  // nothing (49 rows, 24 pairs: 276 and 276), nor does the task mean, whose pass 2 goes column by column.
+  // nothing (49 rows, 24 pairs: 276 and 276); the task mean, whose pass 2 goes column by column, stays one row tile at a time.
   pl->RTU = 1;
   if (pl->QT > 1 && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
     const long long pair_runs = (long long)P.L * P.Bt * P.Hkv * ((pl->QT + 1) / 2) * pl->RPU;
