@@ -1645,10 +1645,14 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   // slower (32K tokens of the first shape 201 and 213 us) except for windows longer than 128 rows
   // (window 200: 7 pairs per CTA 68 and 67, 14 125 and 114, 55 443 and 399).  A run-time window of up to 128 rows gains
   // nothing (49 rows, 24 pairs: 276 and 276); the task mean, whose pass 2 goes column by column, stays one row tile at a time.
+  // So do long windows whose causal mask runs through more than a fiftieth of the tiles: masked tiles go column by column as well, and a
+  // run of them on two row tiles holds its whole unit up (8B shape, 500 rows at the end of 4096 tokens 408 us one at a time, 481 in
+  // pairs, 8192: 672 and 711, 16384: 1231 and 1250; four units of 60000: 528 and 512).
   pl->RTU = 1;
   if (pl->QT > 1 && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
     const long long pair_runs = (long long)P.L * P.Bt * P.Hkv * ((pl->QT + 1) / 2) * pl->RPU;
-    if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0) pl->RTU = 2;
+    const long long masked = P.q_pos0 < P.N - 1 ? (P.N - 1 - P.q_pos0) / kTile + 1 : 0;      // tiles that the mask touches
+    if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0 && (P.w <= kRows || masked * 50 <= pl->NT)) pl->RTU = 2;
   }
   pl->QP = (pl->QT + pl->RTU - 1) / pl->RTU;
   pl->total_runs = (long long)P.L * P.Bt * P.Hkv * pl->QP * pl->RPU;
@@ -1656,8 +1660,11 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   pl->grid = sms > 0 ? (int)(pl->total_runs < sms - pl->norm_ctas ? pl->total_runs : sms - pl->norm_ctas) : 1;
   // Pass 2 of a run starts once every run of its unit has been through pass 1: at other CTAs these lie at most
   // (grid + RPU - 2) / grid runs later in their order.  Pass 1 must be allowed that far ahead of pass 2 (or the CTAs
-  // would wait for each other), and no further: the rows in between should still be in L2 when pass 2 reads them.
-  pl->lead = (1 + (pl->grid + pl->RPU - 2) / pl->grid) * pl->RT;
+  // would wait for each other), and no further: the rows in between should still be in L2 when pass 2 reads them.  Two runs further
+  // for windows longer than 128 rows: a head's row tiles read the same rows anyway, and the runs are uneven (the short last row tile of
+  // a head, masked tiles).  (500 rows: 65536 tokens 692 -> 583 us, 60000 615 -> 512, one row tile at a time 579 -> 528; 4096 tokens without a
+  // mask the same.  Window 64, GQA group 7 at 128K 1 % slower with one run more, so not there.)
+  pl->lead = (1 + (pl->grid + pl->RPU - 2) / pl->grid) * pl->RT + (pl->CH > 1 ? 2 * pl->RT : 0);
   size_t off = 0;
   pl->off_partial = off; off += align_up((size_t)pl->U * pl->RPU * kRows * sizeof(float2));
   pl->off_acc = off; off += align_up((size_t)pl->U * kRows * sizeof(unsigned long long));

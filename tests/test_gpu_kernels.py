@@ -304,6 +304,8 @@ def test_positions_far_behind_the_context_mask_nothing(dtype, w):
     (16, 4, 64, 128, 1500, 64, 4, None, 2.0),    # logits more than 40 nats above a run's first: the references move
     (4, 2, 300, 128, 700, 64, 6, 5000, 0.0),     # long windows: three row tiles per head, the last one short
     (6, 3, 200, 64, 2049, 32, 4, None, 4.0),     # heads of 64, two row tiles per head
+    (6, 3, 200, 64, 2049, 32, 4, 5000, 4.0),     # the same without a mask (through more than a fiftieth of the tiles it keeps them single)
+    (2, 1, 200, 64, 40000, 8, 1, None, 0.0),     # ... and with one through fewer
 ])
 def test_row_tiles_in_pairs_give_the_scores_of_one_at_a_time(Hq, Hkv, w, d, N, L, batch, q_pos0, scale):
     """Large problems take the row tiles of a KV head two at a time over the same keys, small ones one at a time: the scores of
