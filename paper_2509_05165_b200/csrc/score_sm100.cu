@@ -766,7 +766,7 @@ __device__ __forceinline__ void value_norm_cta(const FastParams& P, uint32_t sba
 // ------------------------------------------------------------------------------------------------
 // The kernel
 // ------------------------------------------------------------------------------------------------
-template <int D, int W, bool kTaskMean, int kRT>
+template <int D, int W, bool kTaskMean, int kRT, bool kKeep>
 __global__ void __launch_bounds__(kFastThreads, 1)
 score_sm100_kernel(const __grid_constant__ FastParams P) {
   using SL = SmemLayout<D, kRT>;
@@ -820,7 +820,7 @@ score_sm100_kernel(const __grid_constant__ FastParams P) {
     if (threadIdx.x == 0 && P.status) atomicCAS(P.status, 0, (int)KVC_ERR_CUDA);
     my_runs = 0;               // nothing is computed; the teardown below still frees the TMEM columns
   }
-  constexpr bool kKeep = kRT == 1 && W > 0 && !kTaskMean;   // pass 2 keeps a run's -log-sum-exps in registers
+  static_assert(!kKeep || (kRT == 1 && W > 0 && !kTaskMean), "pass 2 keeps a run's -log-sum-exps in registers");
   constexpr bool kLong = (W == 0);   // only the run-time window variant has windows longer than 128 rows
   // the whole box arrives (rows outside the tensor as zeros)
   const uint32_t q_bytes = (uint32_t)((!kLong || P.CH == 1) ? P.HPT * P.w : kRows) * D * 2;
@@ -1644,12 +1644,12 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   // 240.3; 16 layers of one KV head, window 300: 10 pairs 101 and 106, 21 187 and 186, 42 366 and 355.)  With heads of 64 pairs are
   // slower (32K tokens of the first shape 201 and 213 us) except for windows longer than 128 rows
   // (window 200: 7 pairs per CTA 68 and 67, 14 125 and 114, 55 443 and 399).  A run-time window of up to 128 rows gains
-  // nothing (49 rows, 24 pairs: 276 and 276); the task mean, whose pass 2 goes column by column, stays one row tile at a time.
+  // nothing (49 rows, 24 pairs: 276 and 276); with three, five or seven row tiles the one left over costs what the pairs gain; the task mean, whose pass 2 goes column by column, stays one row tile at a time.
   // So do long windows whose causal mask runs through more than a fiftieth of the tiles: masked tiles go column by column as well, and a
   // run of them on two row tiles holds its whole unit up (8B shape, 500 rows at the end of 4096 tokens 408 us one at a time, 481 in
   // pairs, 8192: 672 and 711, 16384: 1231 and 1250; four units of 60000: 528 and 512).
   pl->RTU = 1;
-  if (pl->QT > 1 && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
+  if (pl->QT > 1 && (pl->QT % 2 == 0 || pl->QT > 8) && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
     const long long pair_runs = (long long)P.L * P.Bt * P.Hkv * ((pl->QT + 1) / 2) * pl->RPU;
     const long long masked = P.q_pos0 < P.N - 1 ? (P.N - 1 - P.q_pos0) / kTile + 1 : 0;      // tiles that the mask touches
     if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0 && (P.w <= kRows || masked * 50 <= pl->NT)) pl->RTU = 2;
@@ -1693,7 +1693,7 @@ std::mutex g_launch_mutex;
 // The kernel's CTAs wait for one another, so all of them have to be resident at once: one per
 // SM with the opt-in amount of shared memory.  Checked once per device and instantiation (the
 // attribute is per device); KVC_ERR_UNSUPPORTED sends the caller to the CUDA-core path.
-template <int D, int W, bool M, int kRT>
+template <int D, int W, bool M, int kRT, bool kKeep>
 kvc_status prepare_t(int grid) {
   using SL = SmemLayout<D, kRT>;
   static signed char state[kMaxDevices];      // 0: not looked at, 1: fits, -1: does not
@@ -1702,9 +1702,9 @@ kvc_status prepare_t(int grid) {
   if (dev < 0 || dev >= kMaxDevices) return KVC_ERR_UNSUPPORTED;
   std::lock_guard<std::mutex> lock(g_launch_mutex);
   if (state[dev] == 0) {
-    KVC_CUDA(cudaFuncSetAttribute(score_sm100_kernel<D, W, M, kRT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kTotal));
+    KVC_CUDA(cudaFuncSetAttribute(score_sm100_kernel<D, W, M, kRT, kKeep>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kTotal));
     int per_sm = 0, sms = 0;
-    KVC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_sm100_kernel<D, W, M, kRT>, kFastThreads,
+    KVC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_sm100_kernel<D, W, M, kRT, kKeep>, kFastThreads,
                                                            (size_t)SL::kTotal));
     KVC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     state[dev] = (per_sm >= 1 && sms >= 1) ? 1 : -1;
@@ -1713,34 +1713,37 @@ kvc_status prepare_t(int grid) {
   return state[dev] == 1 ? KVC_OK : KVC_ERR_UNSUPPORTED;
 }
 
-template <int D, int W, bool M, int kRT>
+template <int D, int W, bool M, int kRT, bool kKeep>
 kvc_status launch_t(const FastParams& fp, int grid, cudaStream_t st) {
   using SL = SmemLayout<D, kRT>;
-  const kvc_status s = prepare_t<D, W, M, kRT>(grid);
+  const kvc_status s = prepare_t<D, W, M, kRT, kKeep>(grid);
   if (s != KVC_OK) return s;
-  KVC_CUDA(launch_dependent(score_sm100_kernel<D, W, M, kRT>, dim3(grid + fp.norm_ctas), dim3(kFastThreads), (size_t)SL::kTotal, st, fp));
+  KVC_CUDA(launch_dependent(score_sm100_kernel<D, W, M, kRT, kKeep>, dim3(grid + fp.norm_ctas), dim3(kFastThreads), (size_t)SL::kTotal, st, fp));
   KVC_LAUNCH_CHECK("score_sm100_kernel");
   return KVC_OK;
 }
 
-template <int D, bool M, int kRT>
+template <int D, bool M, int kRT, bool kKeep>
 kvc_status launch_w(int W, const FastParams& fp, int grid, cudaStream_t st) {
   switch (W) {
-    case 8: return launch_t<D, 8, M, kRT>(fp, grid, st);
-    case 16: return launch_t<D, 16, M, kRT>(fp, grid, st);
-    case 32: return launch_t<D, 32, M, kRT>(fp, grid, st);
-    case 64: return launch_t<D, 64, M, kRT>(fp, grid, st);
-    case 128: return launch_t<D, 128, M, kRT>(fp, grid, st);
-    default: return launch_t<D, 0, M, kRT>(fp, grid, st);      // any other window length: known at run time only
+    case 8: return launch_t<D, 8, M, kRT, kKeep>(fp, grid, st);
+    case 16: return launch_t<D, 16, M, kRT, kKeep>(fp, grid, st);
+    case 32: return launch_t<D, 32, M, kRT, kKeep>(fp, grid, st);
+    case 64: return launch_t<D, 64, M, kRT, kKeep>(fp, grid, st);
+    case 128: return launch_t<D, 128, M, kRT, kKeep>(fp, grid, st);
+    default: return launch_t<D, 0, M, kRT, false>(fp, grid, st);      // any other window length: known at run time only
   }
 }
 
 // (two row tiles: only what make_plan sends here)
 template <int D>
-kvc_status launch_d(bool mean, int row_tiles, int W, const FastParams& fp, int grid, cudaStream_t st) {
-  if (row_tiles == 1) return mean ? launch_w<D, true, 1>(W, fp, grid, st) : launch_w<D, false, 1>(W, fp, grid, st);
-  if constexpr (D == 128) return launch_w<D, false, 2>(W, fp, grid, st);
-  else return launch_t<D, 0, false, 2>(fp, grid, st);
+kvc_status launch_d(bool mean, int row_tiles, bool keep, int W, const FastParams& fp, int grid, cudaStream_t st) {
+  if (row_tiles == 1) {
+    if (mean) return launch_w<D, true, 1, false>(W, fp, grid, st);
+    return keep ? launch_w<D, false, 1, true>(W, fp, grid, st) : launch_w<D, false, 1, false>(W, fp, grid, st);
+  }
+  if constexpr (D == 128) return launch_w<D, false, 2, false>(W, fp, grid, st);
+  else return launch_t<D, 0, false, 2, false>(fp, grid, st);
 }
 
 }  // namespace
@@ -1838,7 +1841,12 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
   fp.wait_limit_ns = g_wait_limit_ns.load();
   fp.withhold_unit = g_withhold_unit.load();
   const bool mean = P.agg_task == KVC_AGG_MEAN;
-  return P.d == 128 ? launch_d<128>(mean, pl.RTU, P.w, fp, pl.grid, st) : launch_d<64>(mean, pl.RTU, P.w, fp, pl.grid, st);
+  // Keeping the -log-sum-exps pays on tiles that no mask touches; where more than an eighth of them is masked (by the window, or as
+  // the short last tile) the other form is faster (GQA group 7: window 128, heads of 64, 704 tokens 47.9 and 42.3 us, window 64, 795
+  // tokens 33.7 and 32.2; the 8B shape at 1000 tokens, one of eight, 30.5 and 31.4).
+  const long long plain = ((P.q_pos0 < P.N - 1 ? P.q_pos0 : P.N - 1) + 1) / kTile;
+  const bool keep = (pl.NT - plain) * 8 <= pl.NT;
+  return P.d == 128 ? launch_d<128>(mean, pl.RTU, keep, P.w, fp, pl.grid, st) : launch_d<64>(mean, pl.RTU, keep, P.w, fp, pl.grid, st);
 }
 
 }  // namespace kvc

@@ -296,8 +296,8 @@ def test_positions_far_behind_the_context_mask_nothing(dtype, w):
 @pytest.mark.parametrize("Hq,Hkv,w,d,N,L,batch,q_pos0,scale", [
     (16, 8, 128, 128, 5, 64, 8, None, 0.0),      # two row tiles per KV head, contexts of five tokens, ...
     (16, 8, 128, 128, 129, 64, 8, None, 0.0),    # ... of a tile and a token, the mask in both
-    (24, 8, 128, 128, 1024, 24, 4, 5000, 0.0),   # three row tiles: the last work unit has one; whole runs, no mask
-    (40, 8, 128, 128, 777, 24, 4, 300, 0.0),     # five row tiles, the mask inside
+    (72, 8, 128, 128, 1024, 8, 4, 5000, 0.0),    # nine row tiles: the last work unit has one; whole runs, no mask
+    (88, 8, 128, 128, 777, 8, 4, 300, 0.0),      # eleven row tiles, the mask inside
     (36, 2, 8, 128, 640, 80, 10, None, 0.0),     # sixteen heads of 8 rows in the first row tile, two in the second
     (18, 2, 16, 128, 640, 80, 10, None, 0.0),    # eight heads of 16 rows, one
     (14, 2, 32, 128, 1537, 64, 8, 0, 0.0),       # four heads of 32 rows, three; row m sees tokens up to m only
