@@ -73,6 +73,8 @@ def _load():
     lib.kvc_score_status_offset.restype = C.c_int
     lib.kvc_debug_score_hooks.argtypes = [i64, i32]
     lib.kvc_debug_score_hooks.restype = None
+    lib.kvc_debug_score_plan.argtypes = [dp, i32, vp]
+    lib.kvc_debug_score_plan.restype = C.c_int
     lib.kvc_debug_select_hooks.argtypes = [i32, i32]
     lib.kvc_debug_select_hooks.restype = None
     lib.kvc_score_uses_tensor_cores.argtypes = [dp]
@@ -194,6 +196,13 @@ def kvc_debug_score_hooks(wait_limit_ns: int = 0, withhold_unit: int = -1) -> No
     """Test hook: bound of the scoring kernel's device-side waits, and a unit whose statistics
     are withheld so that those waits expire.  The defaults restore normal operation."""
     _load().kvc_debug_score_hooks(int(wait_limit_ns), int(withhold_unit))
+
+
+def kvc_debug_score_plan(desc: KvcDesc, sms: int) -> dict:
+    """Test hook: how the tensor-core scoring of this problem is laid out on a device of ``sms`` SMs (no device needed)."""
+    out = (C.c_int64 * 6)()
+    _check(_load().kvc_debug_score_plan(C.byref(desc), int(sms), out))
+    return dict(zip(("row_tiles", "ctas", "norm_ctas", "keep", "runs", "lead"), out))
 
 
 def kvc_debug_select_hooks(path: int = 0, max_rounds: int = -1) -> None:

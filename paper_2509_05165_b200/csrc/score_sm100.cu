@@ -1603,6 +1603,7 @@ struct FastPlan {
   int RTU, QP;                 // row tiles per work unit, work units per KV head
   long long total_runs;
   int lead, norm_ctas;
+  bool keep;                   // pass 2 keeps a run's -log-sum-exps in registers
   size_t off_partial, off_parts, off_acc, off_ovf, off_ref, off_total;
 };
 
@@ -1645,22 +1646,31 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   pl->RT = kMinRunTiles;
   if ((pl->NT + pl->RT - 1) / pl->RT > 255) pl->RT = (pl->NT + 254) / 255;   // the arrivals of a unit are counted in 8 bits
   pl->RPU = (pl->NT + pl->RT - 1) / pl->RT;
+  // Tiles that some row does not see whole: the causal mask runs through them, or the context ends in them.
+  const long long masked = pl->NT - ((P.q_pos0 < P.N - 1 ? P.q_pos0 : P.N - 1) + 1) / kTile;
   // Two row tiles per work unit share every K tile, but a run takes twice as long until its sums are out, and so do the first
   // run's and the last one's lead: 5 to 7 us, which have to be earned back.  (Scoring of 28 layers with 2 KV heads of 128, window 64,
   // GQA group 4: 6 pairs of runs per CTA 68.3 us one row tile at a time, 75.9 in pairs; 12: 127.2 and 126.9; 24: 246.4 and
   // 240.3; 16 layers of one KV head, window 300: 10 pairs 101 and 106, 21 187 and 186, 42 366 and 355.)  With heads of 64 pairs are
   // slower (32K tokens of the first shape 201 and 213 us) except for windows longer than 128 rows
   // (window 200: 7 pairs per CTA 68 and 67, 14 125 and 114, 55 443 and 399).  A run-time window of up to 128 rows gains
-  // nothing (49 rows, 24 pairs: 276 and 276); with three, five or seven row tiles the one left over costs what the pairs gain; the task mean, whose pass 2 goes column by column, stays one row tile at a time.
-  // So do long windows whose causal mask runs through more than a fiftieth of the tiles: masked tiles go column by column as well, and a
-  // run of them on two row tiles holds its whole unit up (8B shape, 500 rows at the end of 4096 tokens 408 us one at a time, 481 in
-  // pairs, 8192: 672 and 711, 16384: 1231 and 1250; four units of 60000: 528 and 512).
+  // nothing (49 rows, 24 pairs: 276 and 276); with three, five or seven row tiles the one left over costs what the pairs gain
+  // (window 128, group 7, 32K: 2306 and 2336 us per pass); the task mean, whose pass 2 goes column by column, stays one row tile at a time.
+  // So do contexts of whose tiles more than a fiftieth is masked: masked tiles go column by column as well, and a run of them on two
+  // row tiles holds its whole unit up.  (us per pass of 32 layers, 8 KV heads, one at a time and in pairs: 500 rows at the end of
+  // 4096 tokens 408 and 481, 16384 1231 and 1250, behind 3000 tokens, whose last tile is partial, 1025 and 1062, group 9 behind 1155
+  // tokens, 16 layers, 523 and 622; window 150, heads of 64, behind 3000 tokens 238 and 248; window 128, group 8, 1787 tokens, one
+  // tile masked by the window, 324 and 387.  With less: window 64 at 8192 tokens 470 and 466, at 32768 1772 and 1732; 500 rows
+  // behind 65536 tokens, 4 layers, 1923 and 1824.)
   pl->RTU = 1;
   if (pl->QT > 1 && (pl->QT % 2 == 0 || pl->QT > 8) && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
     const long long pair_runs = (long long)P.L * P.Bt * P.Hkv * ((pl->QT + 1) / 2) * pl->RPU;
-    const long long masked = P.q_pos0 < P.N - 1 ? (P.N - 1 - P.q_pos0) / kTile + 1 : 0;      // tiles that the mask touches
-    if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0 && (P.w <= kRows || masked * 50 <= pl->NT)) pl->RTU = 2;
+    if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0 && masked * 50 <= pl->NT) pl->RTU = 2;
   }
+  // Keeping the -log-sum-exps pays on tiles that are not masked; where more than an eighth of them is, the other form is faster
+  // (GQA group 7: window 128, heads of 64, 704 tokens 47.9 and 42.3 us, window 64, 795 tokens 33.7 and 32.2; the 8B shape at 1000
+  // tokens, one of eight, 30.5 and 31.4).
+  pl->keep = pl->RTU == 1 && P.agg_task == KVC_AGG_MAX && window_special(P.w) && masked * 8 <= pl->NT;
   pl->QP = (pl->QT + pl->RTU - 1) / pl->RTU;
   pl->total_runs = (long long)P.L * P.Bt * P.Hkv * pl->QP * pl->RPU;
   pl->norm_ctas = P.value_norm && sms > 1 ? norm_share(P, *pl, sms) : 0;
@@ -1848,12 +1858,7 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
   fp.wait_limit_ns = g_wait_limit_ns.load();
   fp.withhold_unit = g_withhold_unit.load();
   const bool mean = P.agg_task == KVC_AGG_MEAN;
-  // Keeping the -log-sum-exps pays on tiles that no mask touches; where more than an eighth of them is masked (by the window, or as
-  // the short last tile) the other form is faster (GQA group 7: window 128, heads of 64, 704 tokens 47.9 and 42.3 us, window 64, 795
-  // tokens 33.7 and 32.2; the 8B shape at 1000 tokens, one of eight, 30.5 and 31.4).
-  const long long plain = ((P.q_pos0 < P.N - 1 ? P.q_pos0 : P.N - 1) + 1) / kTile;
-  const bool keep = (pl.NT - plain) * 8 <= pl.NT;
-  return P.d == 128 ? launch_d<128>(mean, pl.RTU, keep, P.w, fp, pl.grid, st) : launch_d<64>(mean, pl.RTU, keep, P.w, fp, pl.grid, st);
+  return P.d == 128 ? launch_d<128>(mean, pl.RTU, pl.keep, P.w, fp, pl.grid, st) : launch_d<64>(mean, pl.RTU, pl.keep, P.w, fp, pl.grid, st);
 }
 
 }  // namespace kvc
@@ -1866,4 +1871,21 @@ extern "C" __attribute__((visibility("default"))) void kvc_debug_score_hooks(int
                                                                              int32_t withhold_unit) {
   kvc::g_wait_limit_ns.store(wait_limit_ns > 0 ? (unsigned long long)wait_limit_ns : kvc::kDefaultWaitLimitNs);
   kvc::g_withhold_unit.store(withhold_unit);
+}
+
+// Test hook: how the scoring of this problem is laid out on a device of `sms` SMs (none needed here): out[0] row tiles per work unit,
+// [1] scoring CTAs, [2] CTAs of the value norms, [3] whether pass 2 keeps a run's -log-sum-exps, [4] work units' runs, [5] tiles by
+// which pass 1 may be ahead.  KVC_ERR_UNSUPPORTED for a problem of the CUDA-core kernels.
+extern "C" __attribute__((visibility("default"))) int kvc_debug_score_plan(const kvc_desc* d, int32_t sms, int64_t* out) {
+  kvc::Problem P;
+  const kvc_status s = kvc::resolve_desc(d, &P);
+  if (s != KVC_OK) return s;
+  if (sms < 1 || !kvc::score_sm100_shape_ok(P)) {
+    kvc::set_error("score plan: not a problem of the tensor-core kernel");
+    return KVC_ERR_UNSUPPORTED;
+  }
+  kvc::FastPlan pl;
+  kvc::make_plan(P, sms, &pl);
+  out[0] = pl.RTU; out[1] = pl.grid; out[2] = pl.norm_ctas; out[3] = pl.keep; out[4] = pl.total_runs; out[5] = pl.lead;
+  return KVC_OK;
 }
