@@ -608,6 +608,7 @@ __device__ __forceinline__ float p2_generic_tile(uint32_t taddr, const float* ne
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
       const int col = j * 32 + i;
+      if (W == 0 && i > 0 && i % 8 == 0 && col >= R) break;              // (one row per head and few heads: most columns are nobody's)
       float xi = fmaf(__uint_as_float(r[i]), sl2e, neg_lse[col]);       // log2 of the attention weight
       bool head_done;
       if (W > 0) {
