@@ -1611,22 +1611,73 @@ struct FastPlan {
 // Window lengths with a specialisation of their own.
 constexpr bool window_special(int w) { return w == 8 || w == 16 || w == 32 || w == 64 || w == 128; }
 
+// Clocks of a scoring CTA per pair of tiles, by what its pass 2 does with the rows of a row tile.  The maximum over a specialised
+// window, or a long one, is bound by pass 1; every other way costs clocks per row.  (Scoring of 98304 tokens x 8 heads of 128, clocks per
+// pair at 1.9 GHz, start included, times 0.74, which makes the first of them 1800: window 32 x 4 heads 1800, 32 x 1 1510, 7 x 4 2290, 7 x
+// 16 5040, 13 x 9 3540, 24 x 4 2530, 49 x 2 2140; mean 32 x 4 2940, 32 x 2 2110, 24 x 4 7930, 13 x 9 9840, 500 rows 2840; a masked tile
+// 2300 to 3800 more.  Heads of 64: 1550, 1390, and 100 to 300 less than heads of 128 elsewhere.)
+constexpr double kMaskedClocks = 3000.;
+double pair_clocks(const Problem& P, const FastPlan& pl) {
+  const bool mean = P.agg_task == KVC_AGG_MEAN;
+  const double rows = P.w > kRows ? kRows : pl.HPT * P.w;
+  double least = P.d == 128 ? 1410. + 3. * rows : 1470. + 0.6 * rows;
+  if (mean && least < 1600.) least = 1600.;
+  double per_row = 0.;
+  if (P.w > kRows) per_row = mean ? 12. : 0.;
+  else if (window_special(P.w)) per_row = mean ? 14. : 0.;
+  else if (mean) per_row = 70.;
+  else per_row = P.w < 8 ? 32. : P.w < 16 ? 20. : P.w < 32 ? 14. : 7.;
+  const double clocks = 1250. + per_row * rows;
+  return clocks > least ? clocks : least;
+}
+
 // How many of the SMs take the value norms: as many as make both parts take the same time, in clocks: a scoring CTA has whole
-// runs, kPairClocks per pair of tiles; an SM that only reads gets kNormBytes per clock.  (8B shape with value norms, us per pass
+// runs; an SM that only reads gets kNormBytes per clock.  (8B shape with value norms, us per pass
 // with the norms before the scoring, and beside it at 25, 32, 40, 50 bytes per clock: 1000 tokens 86.6, 80.6, 81.7, 76.1, 75.4;
 // 4096: 219, 218, 208, 206, 209; 16384 with the other options 805, 760, 735, 755, 781; 32768: 1542, 1488, 1453, 1491, 1535; two
-// sequences of 8192 with heads of 64: 525, 521, 494, 487, 517.)
-constexpr double kPairClocks128 = 1800., kPairClocks64 = 1550., kNormBytes = 36.;
-int norm_share(const Problem& P, const FastPlan& pl, int sms) {
-  const double bytes = (double)P.L * P.Bt * P.Hkv * (double)P.N * P.d * P.elem_bytes;
-  const double run = pl.RT * pl.RTU * (P.d == 128 ? kPairClocks128 : kPairClocks64);
-  int best = 1;
-  double best_t = 1e300;
-  for (int n = 1; n < sms; ++n) {
-    const double score = (double)((pl.total_runs + sms - n - 1) / (sms - n)) * run, norm = bytes / (n * kNormBytes);
-    const double t = score > norm ? score : norm;
+// sequences of 8192 with heads of 64: 525, 521, 494, 487, 517.  36 lies between the best two.)
+// 0, for the kernel of their own, where that is expected to be as fast: it reads 25 bytes per clock and SM and takes 2 to 3 us besides.
+// A unit's masked tiles are its last; a CTA's runs are `grid` apart, so with a common divisor g of grid and runs per unit it meets every
+// g-th run of a unit only, and some CTA the masked ones all the time (500 rows at the end of 4096 tokens, value norms, 16 layers: 635
+// us at a grid without such a divisor, 1214 at one of a multiple of eight).  The worst CTA counts.
+// Windows longer than 128 rows, whose row tiles find their K in L2 for longer, lose 4 % to V going through it (300 rows behind 65536
+// tokens, 3 layers: 1158 us with the kernel of its own, 1224 with six SMs beside the scoring).
+constexpr double kNormBytes = 36., kNormAloneBytes = 25., kNormAloneClocks = 4500.;
+int norm_share(const Problem& P, const FastPlan& pl, int sms, long long masked) {
+  const long long block = P.d == 128 ? kNormBlock<16> : kNormBlock<8>;            // (rows are read by whole blocks)
+  const double bytes = (double)P.L * P.Bt * P.Hkv * (double)((P.N + block - 1) / block * block) * P.d * P.elem_bytes;
+  const double plain = pl.RTU * pair_clocks(P, pl) * pl.NT / pl.RPU;              // of a run
+  auto score = [&](int grid) {
+    int g = grid, b = pl.RPU;
+    while (b != 0) { const int r = g % b; g = b; b = r; }
+    // the masked tiles of the runs j = RPU - 1 - c, RPU - 1 - c - g, ...: the last run's class c = 0 has the most, or c = 1 where the
+    // last run is a short one
+    long long worst = 0;
+    for (int c = 0; c < 2 && c < g; ++c) {
+      long long sum = 0;
+      for (int j = pl.RPU - 1 - c; j >= 0; j -= g) {
+        const long long first = (long long)j * pl.RT, end = first + pl.RT < pl.NT ? first + pl.RT : pl.NT, from = pl.NT - masked;
+        if (end <= from) break;
+        sum += end - (first > from ? first : from);
+      }
+      worst = sum > worst ? sum : worst;
+    }
+    return (double)((pl.total_runs + grid - 1) / grid) * (plain + pl.RTU * kMaskedClocks * (double)worst * g / pl.RPU);
+  };
+  // where an even scoring and the norms would take the same time; the best whole number is next to it, or the largest that costs no
+  // CTA another run
+  const double all = (double)pl.total_runs * (plain + pl.RTU * kMaskedClocks * (double)masked / pl.RPU);
+  const int even = (int)(sms / (1. + all * kNormBytes / bytes));
+  int best = 0;
+  double best_t = score(sms) + bytes / (sms * kNormAloneBytes) + kNormAloneClocks;
+  auto consider = [&](int n) {
+    if (n < 1 || n >= sms) return;
+    const double beside = score(sms - n), norm = bytes / (n * kNormBytes), t = (beside > norm ? beside : norm) * (P.w > kRows ? 1.04 : 1.01);
     if (t < best_t) { best_t = t; best = n; }
-  }
+  };
+  for (int n = even - 3; n <= even + 12; ++n) consider(n);
+  const long long most = (pl.total_runs + sms - even - 1) / (sms - even);
+  for (long long k = most > 2 ? most - 2 : 1; k <= most + 1; ++k) consider(sms - (int)((pl.total_runs + k - 1) / k));
   return best;
 }
 
@@ -1674,7 +1725,7 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   pl->keep = pl->RTU == 1 && P.agg_task == KVC_AGG_MAX && window_special(P.w) && masked * 8 <= pl->NT;
   pl->QP = (pl->QT + pl->RTU - 1) / pl->RTU;
   pl->total_runs = (long long)P.L * P.Bt * P.Hkv * pl->QP * pl->RPU;
-  pl->norm_ctas = P.value_norm && sms > 1 ? norm_share(P, *pl, sms) : 0;
+  pl->norm_ctas = P.value_norm && sms > 1 ? norm_share(P, *pl, sms, masked) : 0;
   pl->grid = sms > 0 ? (int)(pl->total_runs < sms - pl->norm_ctas ? pl->total_runs : sms - pl->norm_ctas) : 1;
   // Pass 2 of a run starts once every run of its unit has been through pass 1: at other CTAs these lie at most
   // (grid + RPU - 2) / grid runs later in their order.  Pass 1 must be allowed that far ahead of pass 2 (or the CTAs
@@ -1847,7 +1898,7 @@ kvc_status launch_score_sm100(const Problem& P, const LayerPtrs& q, const LayerP
   fp.sl2e = P.scale * kLog2eF;
   fp.agg_group = P.agg_group;
   fp.norm_ctas = vnorm != nullptr ? pl.norm_ctas : 0;
-  if (vnorm != nullptr && fp.norm_ctas == 0) {         // (a device of one SM)
+  if (vnorm != nullptr && fp.norm_ctas == 0) {         // (see norm_share)
     const kvc_status s = launch_value_norm(P, *v, vnorm, st);
     if (s != KVC_OK) return s;
   }

@@ -39,6 +39,26 @@ def test_row_tiles_go_in_pairs_where_few_tiles_are_masked(q_heads, kv_heads, d, 
     assert kvc.kvc_debug_score_plan(_desc(q_heads, kv_heads, d, n_ctx, w, layers, after=after), SMS)["row_tiles"] == pairs
 
 
+def test_value_norms_take_fewer_sms_from_dearer_scorings():
+    """Of 148 SMs, at 16K tokens of the 8B shape: a scoring that takes k times as long per logit can spare about 1 / k as many."""
+    def share(w, **options):
+        return kvc.kvc_debug_score_plan(_desc(32, 8, 128, 16384, w, 32, value_norm=1, **options), SMS)["norm_ctas"]
+
+    assert 40 <= share(32) <= 56
+    assert 32 <= share(24) <= 44                                     # column blocks of a run-time window
+    assert 28 <= share(32, agg_task=kvc.AGG_MEAN) <= 38              # a second exponential per logit
+    assert 10 <= share(24, agg_task=kvc.AGG_MEAN) <= 18              # column by column
+    assert share(32, agg_task=kvc.AGG_MEAN) < share(24) < share(32)
+    # none where the norms are a small part and V would go through the L2 that the K tiles wait in
+    assert kvc.kvc_debug_score_plan(_desc(32, 8, 128, 65536, 300, 3, after=True, value_norm=1), SMS)["norm_ctas"] == 0
+
+
+def test_value_norms_leave_the_scoring_no_grid_that_meets_masked_tiles_all_the_time():
+    """500 rows at the end of 4096 tokens: the last two of a unit's eight runs are masked; an odd grid meets all eight in turn."""
+    plan = kvc.kvc_debug_score_plan(_desc(32, 8, 128, 4096, 500, 16, value_norm=1), SMS)
+    assert plan["norm_ctas"] > 0 and plan["ctas"] % 2 == 1
+
+
 def test_every_layout_fits_the_device():
     """All CTAs are resident at once (they wait for one another), no scoring CTA is without a run, and pass 1 may run ahead as far as
     the statistics of a unit are spread over the CTAs."""
