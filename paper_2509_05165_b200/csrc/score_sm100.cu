@@ -1179,7 +1179,7 @@ __device__ __forceinline__ void score_cta(const FastParams& P, uint8_t* smem) {
         gacc = gmax ? -INFINITY : 0.f;
         float hacc = -INFINITY;
         const uint32_t acc = lane_addr + tmem_col;
-        // 16 columns: the largest log2 of their weights goes to hacc; with W = 8, 16 whole heads end here
+        // 16 columns: the largest log2 of their weights goes to hacc; with W = 16 a head ends here
         auto part = [&](const uint32_t* r, const ulonglong2* nl, const int col) {
           float x[16];
 #pragma unroll
@@ -1189,17 +1189,13 @@ __device__ __forceinline__ void score_cta(const FastParams& P, uint8_t* smem) {
             unpack2(y0, x[4 * i], x[4 * i + 1]);
             unpack2(y1, x[4 * i + 2], x[4 * i + 3]);
           }
-          if (W == 8 || W == 16) {
-            constexpr int kW = W == 8 ? 8 : 16;
+          if (W == 16) {
+            float a = fmaxf(x[0], x[1]);
 #pragma unroll
-            for (int h0 = 0; h0 < 16; h0 += kW) {
-              float a = fmaxf(x[h0], x[h0 + 1]);
-#pragma unroll
-              for (int i = 2; i < kW; i += 2) a = max3(a, x[h0 + i], x[h0 + i + 1]);
-              if (col + h0 < rows_u) {
-                const float s_task = ex2(a);
-                gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
-              }
+            for (int i = 2; i < 16; i += 2) a = max3(a, x[i], x[i + 1]);
+            if (col < rows_u) {
+              const float s_task = ex2(a);
+              gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
             }
           } else {
             float a = max3(x[0], x[1], x[2]), b = max3(x[3], x[4], x[5]);
@@ -1236,6 +1232,36 @@ __device__ __forceinline__ void score_cta(const FastParams& P, uint8_t* smem) {
           if (n_chunks > 1) chunk(1, rb, ra);
           if (n_chunks > 2) chunk(2, ra, rb);
           if (n_chunks > 3) chunk(3, rb, ra);
+        } else if constexpr (W == 8) {
+          // whole chunks, the next one behind the arithmetic: every head ends with an exponential, which half chunks, and the form
+          // above (it spills), only put off (heads of 128, 128 rows, 20000 tokens, 6 layers: 84.3 us kept, 85.5 in halves, 81.0 so)
+          uint32_t r[32];
+          tc_ld32_nowait(acc, r);
+#pragma unroll 1
+          for (int j = 0; j < n_chunks; ++j) {
+            ulonglong2 nl[8];
+            const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(neg_lse + j * 32);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) nl[i] = l2[i];
+            tc_wait_ld(r);
+            float x[32];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              unpack2(fma2(pack2u(r[4 * i], r[4 * i + 1]), scale2, nl[i].x), x[4 * i], x[4 * i + 1]);
+              unpack2(fma2(pack2u(r[4 * i + 2], r[4 * i + 3]), scale2, nl[i].y), x[4 * i + 2], x[4 * i + 3]);
+            }
+            if (j + 1 < n_chunks) tc_ld32_nowait(acc + j * 32 + 32, r); else emptied();
+#pragma unroll
+            for (int h0 = 0; h0 < 32; h0 += 8) {
+              float a = fmaxf(x[h0], x[h0 + 1]);
+#pragma unroll
+              for (int i = 2; i < 8; i += 2) a = max3(a, x[h0 + i], x[h0 + i + 1]);
+              if (j * 32 + h0 < rows_u) {
+                const float s_task = ex2(a);
+                gacc = gmax ? fmaxf(gacc, s_task) : gacc + s_task;
+              }
+            }
+          }
         } else {
           // the same with half chunks, whose -log-sum-exps come from shared memory
           uint32_t ra[16], rb[16];
@@ -1722,7 +1748,7 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   // Keeping the -log-sum-exps pays on tiles that are not masked; where more than an eighth of them is, the other form is faster
   // (GQA group 7: window 128, heads of 64, 704 tokens 47.9 and 42.3 us, window 64, 795 tokens 33.7 and 32.2; the 8B shape at 1000
   // tokens, one of eight, 30.5 and 31.4).
-  pl->keep = pl->RTU == 1 && P.agg_task == KVC_AGG_MAX && window_special(P.w) && masked * 8 <= pl->NT;
+  pl->keep = pl->RTU == 1 && P.agg_task == KVC_AGG_MAX && window_special(P.w) && P.w > 8 && masked * 8 <= pl->NT;
   pl->QP = (pl->QT + pl->RTU - 1) / pl->RTU;
   pl->total_runs = (long long)P.L * P.Bt * P.Hkv * pl->QP * pl->RPU;
   pl->norm_ctas = P.value_norm && sms > 1 ? norm_share(P, *pl, sms, masked) : 0;
@@ -1795,7 +1821,7 @@ kvc_status launch_t(const FastParams& fp, int grid, cudaStream_t st) {
 template <int D, bool M, int kRT, bool kKeep>
 kvc_status launch_w(int W, const FastParams& fp, int grid, cudaStream_t st) {
   switch (W) {
-    case 8: return launch_t<D, 8, M, kRT, kKeep>(fp, grid, st);
+    case 8: return launch_t<D, 8, M, kRT, false>(fp, grid, st);
     case 16: return launch_t<D, 16, M, kRT, kKeep>(fp, grid, st);
     case 32: return launch_t<D, 32, M, kRT, kKeep>(fp, grid, st);
     case 64: return launch_t<D, 64, M, kRT, kKeep>(fp, grid, st);
