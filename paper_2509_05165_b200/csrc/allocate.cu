@@ -265,9 +265,7 @@ constexpr int kSelDefaultRounds = 40;     // sampling rounds and exact steps tog
 
 struct SelectShared {
   uint32_t hist[kSelBins];                      // block sizes of the samples per bin
-  // where the rows' pooled entries start (a 64-bit division per entry of the last step otherwise: 16 rows of 3001 9.5 -> 8.8 us, 32 of 1000
-  // 9.5 -> 9.0, of 32768 11.5 -> 11.2; the steps of a thread's searches taken together instead: up to 0.4 us slower)
-  long long base[kSelMaxRows];                  // where the rows' pooled entries start
+  long long base[kSelMaxRows];                  // where the rows' pooled entries start (for the searches)
   int lo[kSelMaxRows], hi[kSelMaxRows];         // the rows' windows: positions < lo are better than T, >= hi worse
   int gt[kSelMaxRows], ge[kSelMaxRows];         // the answer: entries better than T, and at least as good
   int off[kSelMaxRows + 1];                     // running sum of the window lengths (last step)
@@ -410,6 +408,8 @@ select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr
   const int tpr = 1 << tshift, sshift = tshift + 2;
   static_assert(kSelItems == 4, "sshift");
   const int r = tid >> tshift, sub = tid & (tpr - 1);  // this thread's row and its place among the row's threads
+  const int rr0 = r < R ? r : 0, rl0 = rr0 / hpr;
+  const float* row = composite + (((long long)rl0 * Bt + b) * hpr + (rr0 - rl0 * hpr)) * N + floor;
   if (tid < R) {
     const int rl = tid / hpr;                          // (32-bit: the 64-bit division of row_start is slow)
     sh.base[tid] = (((long long)rl * Bt + b) * hpr + (tid - rl * hpr)) * N + floor;
@@ -423,7 +423,6 @@ select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr
     sh.slack = sh.taken = sh.new_width = 0u;
   }
   __syncthreads();
-  const float* row = composite + sh.base[r < R ? r : 0];
   grid_dependency_wait();                              // (everything above overlapped the end of the kernel before this one)
   if (budget > 0 && M > 0) {
     bool found = false;                                // sh.gt / sh.ge hold the answer
@@ -558,7 +557,11 @@ select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr
             }
             at[i] = x;
             wgt[i] = 1u;
-            key[i] = score_to_key(composite[sh.base[x] + sh.lo[x] + (e - sh.off[x])]);
+            // (32-bit, and none for whole layers: 64-bit divisions cost 32 rows of 1000 0.5 us; the starts out of shared memory, which
+            // the code of the rounds before pays for, cost ties and long rows up to 0.8: 16 rows of 3001 with ties 13.6 -> 12.8, 28 of
+            // 131072 13.5 -> 13.2, but a single row of 1000 5.0 -> 5.3)
+            const int xl = hpr == 1 ? x : x / hpr;
+            key[i] = score_to_key(composite[(((long long)xl * Bt + b) * hpr + (x - xl * hpr)) * N + floor + sh.lo[x] + (e - sh.off[x])]);
           }
         }
 #pragma unroll
