@@ -293,21 +293,34 @@ def test_positions_far_behind_the_context_mask_nothing(dtype, w):
     Pz.assert_scores_close(want.cpu().numpy(), Pz.oracle_scores(wl, desc))
 
 
-@pytest.mark.parametrize("Hq,Hkv,w,d,N,L,batch,q_pos0,scale", [
-    (16, 8, 128, 128, 5, 64, 8, None, 0.0),      # two row tiles per KV head, contexts of five tokens, ...
-    (16, 8, 128, 128, 129, 64, 8, None, 0.0),    # ... of a tile and a token, the mask in both
-    (72, 8, 128, 128, 1024, 8, 4, 5000, 0.0),    # nine row tiles: the last work unit has one; whole runs, no mask
-    (88, 8, 128, 128, 777, 8, 4, 300, 0.0),      # eleven row tiles, the mask inside
-    (36, 2, 8, 128, 640, 80, 10, None, 0.0),     # sixteen heads of 8 rows in the first row tile, two in the second
-    (18, 2, 16, 128, 640, 80, 10, None, 0.0),    # eight heads of 16 rows, one
-    (14, 2, 32, 128, 1537, 64, 8, 0, 0.0),       # four heads of 32 rows, three; row m sees tokens up to m only
-    (16, 4, 64, 128, 1500, 64, 4, None, 2.0),    # logits more than 40 nats above a run's first: the references move
-    (4, 2, 300, 128, 700, 64, 6, 5000, 0.0),     # long windows: three row tiles per head, the last one short
-    (6, 3, 200, 64, 2049, 32, 4, None, 4.0),     # heads of 64, two row tiles per head
-    (6, 3, 200, 64, 2049, 32, 4, 5000, 4.0),     # the same without a mask (through more than a fiftieth of the tiles it keeps them single)
-    (2, 1, 200, 64, 40000, 8, 1, None, 0.0),     # ... and with one through fewer
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("Hq,Hkv,w,d,N,L,batch,q_pos0,scale,pairs", [
+    # in pairs (on 148 SMs)
+    (72, 8, 128, 128, 1024, 10, 4, 5000, 0.0, 2),    # nine row tiles: the last work unit has one; whole runs, no mask
+    (88, 8, 128, 128, 6400, 3, 2, 6300, 0.0, 2),     # eleven row tiles, the mask in the last tile
+    (36, 2, 8, 128, 8192, 24, 4, None, 0.0, 2),      # sixteen heads of 8 rows in the first row tile, two in the second
+    (18, 2, 16, 128, 8192, 24, 4, None, 0.0, 2),     # eight heads of 16 rows, one
+    (14, 2, 32, 128, 6528, 32, 4, 6450, 0.0, 2),     # four heads of 32 rows, three
+    (16, 4, 64, 128, 6400, 20, 3, None, 2.0, 2),     # logits more than 40 nats above a run's first: the references move
+    (4, 2, 300, 128, 8192, 8, 4, 8150, 0.0, 2),      # long windows: three row tiles per head, the last one short
+    (6, 3, 200, 64, 2048, 32, 4, 5000, 4.0, 2),      # heads of 64, two row tiles per head
+    (2, 1, 200, 64, 40000, 8, 1, None, 0.0, 2),      # the mask in three of 313 tiles
+    # one at a time: the mask, or the end of the context, in more than a fiftieth of the tiles
+    (16, 8, 128, 128, 5, 64, 8, None, 0.0, 1),       # contexts of five tokens
+    (16, 8, 128, 128, 129, 64, 8, None, 0.0, 1),     # of a tile and a token
+    (88, 8, 128, 128, 777, 8, 4, 300, 0.0, 1),
+    (36, 2, 8, 128, 640, 80, 10, None, 0.0, 1),
+    (18, 2, 16, 128, 640, 80, 10, None, 0.0, 1),
+    (14, 2, 32, 128, 1537, 64, 8, 0, 0.0, 1),        # row m sees tokens up to m only
+    (16, 4, 64, 128, 1500, 64, 4, None, 2.0, 1),
+    (4, 2, 300, 128, 700, 64, 6, 5000, 0.0, 1),
+    (6, 3, 200, 64, 2049, 32, 4, None, 4.0, 1),
+    (6, 3, 200, 64, 2049, 32, 4, 5000, 4.0, 1),
 ])
-def test_row_tiles_in_pairs_give_the_scores_of_one_at_a_time(Hq, Hkv, w, d, N, L, batch, q_pos0, scale):
+def test_row_tiles_in_pairs_give_the_scores_of_one_at_a_time(Hq, Hkv, w, d, N, L, batch, q_pos0, scale, pairs):
     """Large problems take the row tiles of a KV head two at a time over the same keys, small ones one at a time: the scores of
     all layers together are, bit for bit, those of every layer by itself (which the parity tests hold against the oracle)."""
     if not torch.cuda.is_available():
@@ -317,32 +330,41 @@ def test_row_tiles_in_pairs_give_the_scores_of_one_at_a_time(Hq, Hkv, w, d, N, L
     q = [torch.randn((batch, Hq, w, d), generator=gen, device=dev).to(torch.bfloat16) for _ in range(L)]
     k = [torch.randn((batch, Hkv, N, d), generator=gen, device=dev).to(torch.bfloat16) for _ in range(L)]
 
-    def scores(layers):
-        desc = binding.kvc_desc_init(len(layers), batch, Hq, Hkv, d, N, w, binding.BF16)
+    def scores(layers, b, group, row_tiles):
+        desc = binding.kvc_desc_init(len(layers), len(b), Hq, Hkv, d, N, w, binding.BF16)
         desc.scale = scale
+        desc.agg_group = group
         if q_pos0 is not None:
             desc.q_pos0 = q_pos0
         assert kvc.kvc_score_uses_tensor_cores(desc)
-        out = torch.empty((len(layers), batch, Hkv, N), device=dev)
+        if _sms() == 148:
+            assert kvc.kvc_debug_score_plan(desc, 148)["row_tiles"] == row_tiles
+        out = torch.empty((len(layers), len(b), Hkv, N), device=dev)
         ws = torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev)
-        kvc.kvc_score(desc, [q[i] for i in layers], [k[i] for i in layers], out, ws)
+        kvc.kvc_score(desc, [q[i][b] for i in layers], [k[i][b] for i in layers], out, ws)
         return out
 
-    together = scores(list(range(L)))
-    for i in range(0, L, max(1, L // 6)):
-        alone = scores([i])
-        assert torch.isfinite(alone).all()
-        assert torch.equal(together[i].view(torch.int32), alone[0].view(torch.int32)), i
+    for group in (kvc.AGG_MEAN, kvc.AGG_MAX):
+        together = scores(list(range(L)), list(range(batch)), group, pairs)
+        for i in range(0, L, max(1, L // 6)):
+            b = i % batch
+            alone = scores([i], [b], group, 1)
+            assert torch.isfinite(alone).all()
+            assert torch.equal(together[i, b].view(torch.int32), alone[0, 0].view(torch.int32)), (i, b)
 
 
-@pytest.mark.parametrize("L,batch,Hkv,d,N,w,pad", [
-    (3, 2, 5, 128, 17, 4, 0),        # fewer blocks of rows than warps that take them
-    (2, 3, 4, 64, 1033, 32, 64),     # rows apart in memory, a short last block per segment
-    (24, 4, 8, 128, 515, 16, 0),     # many segments per warp
-    (1, 1, 2, 128, 40007, 32, 128),  # one long segment after the other
-    (20, 2, 4, 128, 2100, 130, 0),   # row tiles in pairs beside the norms
+# pairs, beside: row tiles per work unit, and whether the norms' CTAs are in the scoring launch (on 148 SMs)
+@pytest.mark.parametrize("L,batch,Hkv,d,N,w,pad,pairs,beside", [
+    (3, 2, 5, 128, 17, 4, 0, 1, True),         # fewer blocks of rows than warps that take them
+    (2, 3, 4, 64, 1033, 32, 64, 1, True),      # rows apart in memory, a short last block per segment
+    (24, 4, 8, 128, 515, 16, 0, 1, True),      # many segments per warp
+    (1, 1, 2, 128, 40007, 32, 128, 1, True),   # one long segment after the other
+    (20, 2, 4, 128, 2100, 130, 0, 1, True),
+    (40, 2, 8, 128, 2560, 128, 64, 2, True),   # row tiles in pairs beside the norms
+    (28, 1, 4, 128, 3200, 500, 0, 2, True),    # ... of a long window
+    (16, 1, 8, 128, 4096, 500, 0, 2, False),   # row tiles in pairs, the norms in their own kernel
 ])
-def test_value_norms_beside_the_scoring(L, batch, Hkv, d, N, w, pad):
+def test_value_norms_beside_the_scoring(L, batch, Hkv, d, N, w, pad, pairs, beside):
     """The norms that the scoring launch takes along: weighted scores are the plain ones times the norms of the value rows (the
     norm's squares are added in fp32 with errors below 1e-6)."""
     if not torch.cuda.is_available():
@@ -365,6 +387,9 @@ def test_value_norms_beside_the_scoring(L, batch, Hkv, d, N, w, pad):
     plain, weighted = (torch.empty((L, batch, Hkv, N), device=dev) for _ in range(2))
     kvc.kvc_score(desc, q, k, plain, torch.empty(kvc.kvc_workspace_size(desc, 0), dtype=torch.uint8, device=dev))
     desc.value_norm = 1
+    if _sms() == 148:
+        plan = kvc.kvc_debug_score_plan(desc, 148)
+        assert plan["row_tiles"] == pairs and (plan["norm_ctas"] > 0) == beside
     ws = torch.full((kvc.kvc_workspace_size(desc, 0),), 0xff, dtype=torch.uint8, device=dev)
     kvc.kvc_score_weighted(desc, q, k, v, weighted, ws)
     want = torch.stack([p.double() * x.double().norm(dim=-1) for p, x in zip(plain, v)])
