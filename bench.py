@@ -284,7 +284,7 @@ def aggregate_tokens_per_s(cfg, world, ms_per_step):
     return cfg.batch * cfg.n_ctx * world / (ms_per_step * 1e-3)
 
 
-SCORE_SOURCE = os.path.join(ROOT, "paper_2509_05165_b200", "csrc", "score_sm100.cu")
+SCORE_SOURCES = [os.path.join(ROOT, "paper_2509_05165_b200", "csrc", f) for f in ("score_sm100.cu", "value_norm.cuh")]
 SCORE_PROFILE = os.path.join(ROOT, "profiles", "score_sm100_llama8b_32k_L4.txt")
 
 
@@ -292,7 +292,7 @@ def score_traffic_bytes(cfg):
     """DRAM traffic of one launch of the scoring kernel on this workload, from the ncu capture summarised in
     profiles/ (dram__bytes_read.sum + dram__bytes_write.sum of a 4-layer capture of the same shape, scaled to
     the workload's layers: the traffic is proportional to them).  None for any other shape, and None as soon
-    as the kernel's source is no longer the one the capture was taken on (the summary records its hash)."""
+    as the kernel's sources are no longer the ones the capture was taken on (the summary records their hash)."""
     if not cfg.name.startswith("llama8b_32k") or cfg.n_ctx != 32768 or cfg.batch != 1:
         return None
     try:
@@ -301,7 +301,7 @@ def score_traffic_bytes(cfg):
         rd = int(re.search(r"dram_bytes_read_per_launch:\s*(\d+)", text).group(1))
         wr = int(re.search(r"dram_bytes_write_per_launch:\s*(\d+)", text).group(1))
         layers = int(re.search(r"capture_layers:\s*(\d+)", text).group(1))
-        if hashlib.sha256(open(SCORE_SOURCE, "rb").read()).hexdigest() != sha:
+        if hashlib.sha256(b"".join(open(f, "rb").read() for f in SCORE_SOURCES)).hexdigest() != sha:
             return None
         return (rd + wr) * cfg.n_layers // layers
     except Exception:  # noqa: BLE001

@@ -45,7 +45,9 @@
 // `lead` tiles ahead of it (two runs where a unit has no more runs than there are CTAs: 38 MB of K at
 // 148 CTAs, which L2 still holds), exactly what the statistics need: they need every run of a unit, and
 // the other CTAs' runs of it lie that far ahead at most, so the CTAs cannot wait for each other in a
-// circle while all of them are resident (the host checks that they can be).  Every wait (mbarrier or
+// circle while all of them are resident (the host checks that they can be).  Windows longer than 128 rows get
+// two runs more: 77 MB of copies, but the row tiles of a KV head follow one another and copy the same rows (a group of 4 with 500 rows
+// 16 times: 5 MB of K, or one head's where the context is long, 34 MB at 128K).  Every wait (mbarrier or
 // global word) is bounded; on expiry the kernel records KVC_ERR_TIMEOUT, stops computing and drains.
 //
 // Warp roles (512 threads): warp 0 = TMA producer of pass 1 (K, Q, L2 prefetch), warp 3 = of pass 2; warp
@@ -63,7 +65,7 @@
 // SM each, 270 per tile).  Hence:
 //   - one row tile per unit: the pass-2 epilogue keeps a run's 128 -log-sum-exps in registers (216 per thread, taken from the
 //     single warps and from pass 1 by setmaxnreg), reads them once per run, and loads a chunk while it works on the one before:
-//     8B shape at 32K 1078 -> 1060 us per pass, at 8K 1 %, 4 sequences of 5003 with heads of 64 442 -> 430.  Pass 1's epilogue
+//     8B shape at 32K 1078 -> 1060 us per pass, 4 sequences of 5003 with heads of 64 442 -> 430 (8K and less within 1 %).  Pass 1's epilogue
 //     is what is left: 1750 of 1800 clocks.
 //   - several row tiles: a work unit has two of them, which share every K tile in shared memory.  Pass 1's
 //     two groups then take a row tile each, a tile's 128 columns at once in registers (168 per thread): half of the rounds of
@@ -72,7 +74,8 @@
 //     windows 1203 -> 1158; 1690 clocks per pair, of which pass 2's epilogue is busy for 1530.
 // Registers decide the rest: a warp's 128 exponentials take 1134 clocks when the compiler has room to overlap them and 2125
 // when it has not (it then waits for every pair), so in the second form the logits die in their exponentials.
-// Run back to back the board's power adds a sixth: at 1000 W the clock falls from 1.9 to 1.4 GHz within tens of milliseconds.
+// Power is the rest: the 8B shape's scoring at 32K takes 573 us for 50 ms from rest and 690 to 710 back to back, where the clock reads 1.17 to
+// 1.21 GHz: 830 K clocks, 435 us at 1.9 GHz.  (The same clocks in 573 us are 1.45 GHz; the reading, 1.965, lags by 0.1 s.)
 #include <cuda.h>
 
 #include <atomic>
@@ -641,13 +644,8 @@ __device__ __forceinline__ void tc_ld_cols(uint32_t taddr, uint32_t (&r)[kC]) {
     tc_ld32_nowait(taddr, r);
     tc_wait_ld(r);
   } else if constexpr (kC == 16) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
+    tc_ld16_nowait(taddr, r);
+    tc_wait_ld(r);
   } else {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
@@ -1732,8 +1730,10 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   // 240.3; 16 layers of one KV head, window 300: 10 pairs 101 and 106, 21 187 and 186, 42 366 and 355.)  With heads of 64 pairs are
   // slower (32K tokens of the first shape 201 and 213 us) except for windows longer than 128 rows
   // (window 200: 7 pairs per CTA 68 and 67, 14 125 and 114, 55 443 and 399).  A run-time window of up to 128 rows gains
-  // nothing (49 rows, 24 pairs: 276 and 276); with three, five or seven row tiles the one left over costs what the pairs gain
-  // (window 128, group 7, 32K: 2306 and 2336 us per pass); the task mean, whose pass 2 goes column by column, stays one row tile at a time.
+  // nothing (49 rows, 24 pairs: 276 and 276).  Of few row tiles an odd one left over costs what the pairs gain (us per pass one at a time
+  // and in pairs: 7 row tiles 2306 and 2336, 9 1411 and 1425, 11 1685 and 1695, 13 1007 and 1021, 9 of 300 rows 724 and 736; 21 of 300 rows 772
+  // and 749; heads of 64, 9 of 300 rows 300 and 292, 21 619 and 576).  The task mean, whose pass 2 goes column by column, stays one row tile
+  // at a time.
   // So do contexts of whose tiles more than a fiftieth is masked: masked tiles go column by column as well, and a run of them on two
   // row tiles holds its whole unit up.  (us per pass of 32 layers, 8 KV heads, one at a time and in pairs: 500 rows at the end of
   // 4096 tokens 408 and 481, 16384 1231 and 1250, behind 3000 tokens, whose last tile is partial, 1025 and 1062, group 9 behind 1155
@@ -1741,7 +1741,7 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   // tile masked by the window, 324 and 387.  With less: window 64 at 8192 tokens 470 and 466, at 32768 1772 and 1732; 500 rows
   // behind 65536 tokens, 4 layers, 1923 and 1824.)
   pl->RTU = 1;
-  if (pl->QT > 1 && (pl->QT % 2 == 0 || pl->QT > 8) && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
+  if (pl->QT > 1 && (pl->QT % 2 == 0 || pl->QT > (P.d == 128 ? 16 : 8)) && P.agg_task == KVC_AGG_MAX && (P.w > kRows || (P.d == 128 && window_special(P.w)))) {
     const long long pair_runs = (long long)P.L * P.Bt * P.Hkv * ((pl->QT + 1) / 2) * pl->RPU;
     if (pair_runs >= (long long)sms * (P.d == 128 ? 20 : 8) && sms > 0 && masked * 50 <= pl->NT) pl->RTU = 2;
   }
@@ -1755,7 +1755,7 @@ void make_plan(const Problem& P, int sms, FastPlan* pl) {
   pl->grid = sms > 0 ? (int)(pl->total_runs < sms - pl->norm_ctas ? pl->total_runs : sms - pl->norm_ctas) : 1;
   // Pass 2 of a run starts once every run of its unit has been through pass 1: at other CTAs these lie at most
   // (grid + RPU - 2) / grid runs later in their order.  Pass 1 must be allowed that far ahead of pass 2 (or the CTAs
-  // would wait for each other), and no further: the rows in between should still be in L2 when pass 2 reads them.  Two runs further
+  // would wait for each other), and further only there: the rows in between should still be in L2 when pass 2 reads them.  Two runs further
   // for windows longer than 128 rows: a head's row tiles read the same rows anyway, and the runs are uneven (the short last row tile of
   // a head, masked tiles).  (500 rows: 65536 tokens 692 -> 583 us, 60000 615 -> 512, one row tile at a time 579 -> 528; 4096 tokens without a
   // mask the same.  Window 64, GQA group 7 at 128K 1 % slower with one run more, so not there.)

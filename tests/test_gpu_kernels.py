@@ -299,8 +299,8 @@ def _sms():
 
 @pytest.mark.parametrize("Hq,Hkv,w,d,N,L,batch,q_pos0,scale,pairs", [
     # in pairs (on 148 SMs)
-    (72, 8, 128, 128, 1024, 10, 4, 5000, 0.0, 2),    # nine row tiles: the last work unit has one; whole runs, no mask
-    (88, 8, 128, 128, 6400, 3, 2, 6300, 0.0, 2),     # eleven row tiles, the mask in the last tile
+    (136, 8, 128, 128, 1024, 6, 4, 5000, 0.0, 2),    # seventeen row tiles: the last work unit has one; whole runs, no mask
+    (152, 8, 128, 128, 6400, 2, 2, 6300, 0.0, 2),    # nineteen row tiles, the mask in the last tile
     (36, 2, 8, 128, 8192, 24, 4, None, 0.0, 2),      # sixteen heads of 8 rows in the first row tile, two in the second
     (18, 2, 16, 128, 8192, 24, 4, None, 0.0, 2),     # eight heads of 16 rows, one
     (14, 2, 32, 128, 6528, 32, 4, 6450, 0.0, 2),     # four heads of 32 rows, three

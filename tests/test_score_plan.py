@@ -33,6 +33,9 @@ def _desc(q_heads, kv_heads, d, n_ctx, w, layers, batch=1, after=False, **option
     (28, 4, 128, 131072, 64, 28, False, 2),
     (32, 8, 64, 8192, 300, 16, True, 2),
     (56, 8, 128, 32768, 128, 16, False, 1),      # seven row tiles
+    (36, 4, 128, 32768, 128, 16, False, 1),      # nine ...
+    (12, 4, 64, 8192, 300, 16, True, 2),         # ... of heads of 64
+    (28, 4, 128, 32768, 300, 4, True, 2),        # twenty-one
     (32, 8, 128, 32768, 49, 32, False, 1),       # a run-time window
 ])
 def test_row_tiles_go_in_pairs_where_few_tiles_are_masked(q_heads, kv_heads, d, n_ctx, w, layers, after, pairs):
