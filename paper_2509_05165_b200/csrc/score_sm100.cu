@@ -682,6 +682,13 @@ __device__ __forceinline__ float p2_odd_tile(uint32_t taddr, const float* neg_ls
   return gacc;
 }
 
+// The same out of line, for windows of 9 to 15 rows: where pass 2 bounds the kernel they are 1 to 3 % faster so (20000 tokens, heads of 64:
+// at worst 1.05 of the time before all of these went into the kernel's body, 1.025 called), longer windows 1 to 2 % slower.
+template <int kC>
+__device__ __noinline__ float p2_odd_tile_called(uint32_t taddr, const float* neg_lse, int R, int w, float sl2e, bool gmax) {
+  return p2_odd_tile<kC>(taddr, neg_lse, R, w, sl2e, gmax);
+}
+
 // Pass 2, one token against the R rows of one query head that this row tile holds (windows longer
 // than 128 rows), with masking: rows below m_min do not see the token.  Returns the tile's part of
 // Eq. 14 for the token: the largest attention weight, or the sum of the weights, over these rows.
@@ -1285,10 +1292,10 @@ __device__ __forceinline__ void score_cta(const FastParams& P, uint8_t* smem) {
           }
         }
         if (W == 0) gacc = ex2(hacc);                                  // the head's maximum over these rows
-      } else if (!kTaskMean && W == 0 && full && P.w >= 8) {
+      } else if (!kTaskMean && W == 0 && kRT == 1 && full && P.w >= 8) {
         gacc = P.w >= 32 ? p2_odd_tile<32>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
              : P.w >= 16 ? p2_odd_tile<16>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
-                         : p2_odd_tile<8>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax);
+                         : p2_odd_tile_called<8>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty(buf));
@@ -1659,14 +1666,15 @@ double pair_clocks(const Problem& P, const FastPlan& pl) {
 // runs; an SM that only reads gets kNormBytes per clock.  (8B shape with value norms, us per pass
 // with the norms before the scoring, and beside it at 25, 32, 40, 50 bytes per clock: 1000 tokens 86.6, 80.6, 81.7, 76.1, 75.4;
 // 4096: 219, 218, 208, 206, 209; 16384 with the other options 805, 760, 735, 755, 781; 32768: 1542, 1488, 1453, 1491, 1535; two
-// sequences of 8192 with heads of 64: 525, 521, 494, 487, 517.  36 lies between the best two.)
+// sequences of 8192 with heads of 64: 525, 521, 494, 487, 517.  With the prices above, at 36, 34, 32: 4096 tokens 211, 209, 207; 16384 761,
+// 748, 745; 32768 1489, 1464, 1451; 16 layers of GQA group 7, window 64, 20000 tokens 519, 508, 511.)
 // 0, for the kernel of their own, where that is expected to be as fast: it reads 25 bytes per clock and SM and takes 2 to 3 us besides.
 // A unit's masked tiles are its last; a CTA's runs are `grid` apart, so with a common divisor g of grid and runs per unit it meets every
 // g-th run of a unit only, and some CTA the masked ones all the time (500 rows at the end of 4096 tokens, value norms, 16 layers: 635
 // us at a grid without such a divisor, 1214 at one of a multiple of eight).  The worst CTA counts.
 // Windows longer than 128 rows, whose row tiles find their K in L2 for longer, lose 4 % to V going through it (300 rows behind 65536
 // tokens, 3 layers: 1158 us with the kernel of its own, 1224 with six SMs beside the scoring).
-constexpr double kNormBytes = 36., kNormAloneBytes = 25., kNormAloneClocks = 4500.;
+constexpr double kNormBytes = 32., kNormAloneBytes = 25., kNormAloneClocks = 4500.;
 int norm_share(const Problem& P, const FastPlan& pl, int sms, long long masked) {
   const long long block = P.d == 128 ? kNormBlock<16> : kNormBlock<8>;            // (rows are read by whole blocks)
   const double bytes = (double)P.L * P.Bt * P.Hkv * (double)((P.N + block - 1) / block * block) * P.d * P.elem_bytes;
