@@ -395,6 +395,9 @@ __device__ inline void locate_in_windows(const float* __restrict__ composite, Se
 }
 
 // (the host keeps R * (N - floor) below 2^32)
+// kFew: up to kSelFewRows rows, which take their start out of shared memory throughout
+constexpr int kSelFewRows = 8;
+template <bool kFew>
 __global__ void __launch_bounds__(kSelThreads)
 select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr, long long N, long long floor,
                      long long budget, int max_rounds, int32_t* __restrict__ n_keep,
@@ -408,7 +411,7 @@ select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr
   const int tpr = 1 << tshift, sshift = tshift + 2;
   static_assert(kSelItems == 4, "sshift");
   const int r = tid >> tshift, sub = tid & (tpr - 1);  // this thread's row and its place among the row's threads
-  const int rr0 = r < R ? r : 0, rl0 = rr0 / hpr;
+  const int rr0 = r < R ? r : 0, rl0 = kFew ? 0 : rr0 / hpr;
   const float* row = composite + (((long long)rl0 * Bt + b) * hpr + (rr0 - rl0 * hpr)) * N + floor;
   if (tid < R) {
     const int rl = tid / hpr;                          // (32-bit: the 64-bit division of row_start is slow)
@@ -423,6 +426,7 @@ select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr
     sh.slack = sh.taken = sh.new_width = 0u;
   }
   __syncthreads();
+  if (kFew) row = composite + sh.base[rr0];
   grid_dependency_wait();                              // (everything above overlapped the end of the kernel before this one)
   if (budget > 0 && M > 0) {
     bool found = false;                                // sh.gt / sh.ge hold the answer
@@ -557,11 +561,12 @@ select_sorted_kernel(const float* __restrict__ composite, int R, int Bt, int hpr
             }
             at[i] = x;
             wgt[i] = 1u;
-            // (32-bit, and none for whole layers: 64-bit divisions cost 32 rows of 1000 0.5 us; the starts out of shared memory, which
-            // the code of the rounds before pays for, cost ties and long rows up to 0.8: 16 rows of 3001 with ties 13.6 -> 12.8, 28 of
-            // 131072 13.5 -> 13.2, but a single row of 1000 5.0 -> 5.3)
-            const int xl = hpr == 1 ? x : x / hpr;
-            key[i] = score_to_key(composite[(((long long)xl * Bt + b) * hpr + (x - xl * hpr)) * N + floor + sh.lo[x] + (e - sh.off[x])]);
+            // (32-bit, and none for whole layers: 64-bit divisions cost 32 rows of 1000 0.5 us.  The starts out of shared memory are
+            // faster for few rows, one of 1000 5.0 us and 5.3, but cost ties and long rows up to 0.8: 16 rows of 3001 with ties 13.6 and
+            // 12.8, 28 of 131072 13.5 and 13.2.)
+            const int xl = kFew || hpr == 1 ? x : x / hpr;
+            const long long from = kFew ? sh.base[x] : (((long long)xl * Bt + b) * hpr + (x - xl * hpr)) * N + floor;
+            key[i] = score_to_key(composite[from + sh.lo[x] + (e - sh.off[x])]);
           }
         }
 #pragma unroll
@@ -677,7 +682,7 @@ kvc_status launch_allocate(const Problem& P, const float* composite, long long b
   if (path != SelectPath::kHistograms && R <= kSelMaxRows && (long long)R * (P.N - min_keep) < (1LL << 32)) {
     const int hook_rounds = g_select_rounds.load();
     const int rounds = hook_rounds >= 0 ? hook_rounds : kSelDefaultRounds;
-    KVC_CUDA(launch_dependent(select_sorted_kernel, dim3(P.Bt), dim3(kSelThreads), 0, st, composite, R, P.Bt,
+    KVC_CUDA(launch_dependent(R <= kSelFewRows ? select_sorted_kernel<true> : select_sorted_kernel<false>, dim3(P.Bt), dim3(kSelThreads), 0, st, composite, R, P.Bt,
                               heads_per_row, P.N, min_keep, rest, rounds, n_keep, offsets));
     KVC_LAUNCH_CHECK("select_sorted_kernel");
     return KVC_OK;
