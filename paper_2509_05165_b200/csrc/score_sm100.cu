@@ -1292,10 +1292,15 @@ __device__ __forceinline__ void score_cta(const FastParams& P, uint8_t* smem) {
           }
         }
         if (W == 0) gacc = ex2(hacc);                                  // the head's maximum over these rows
-      } else if (!kTaskMean && W == 0 && kRT == 1 && full && P.w >= 8) {
+      } else if (!kTaskMean && W == 0 && full && P.w >= 8) {
+        // (row tiles in pairs never come here, yet their kernel with heads of 64 is 15 % slower where ptxas does not see it)
+        const auto short_blocks = [&]() {
+          if constexpr (kRT == 1) return p2_odd_tile_called<8>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax);
+          else return p2_odd_tile<8>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax);
+        };
         gacc = P.w >= 32 ? p2_odd_tile<32>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
              : P.w >= 16 ? p2_odd_tile<16>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax)
-                         : p2_odd_tile_called<8>(lane_addr + tmem_col, neg_lse, rows_u, P.w, P.sl2e, gmax);
+                         : short_blocks();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty(buf));
